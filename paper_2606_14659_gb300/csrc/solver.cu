@@ -1014,32 +1014,108 @@ int launch_lz_eig(int f32, Unit* units, double* S, int nunits, cudaStream_t s) {
 // ----------------------------------------------------------------------------
 // Ritz vector and thick-restart basis (per row, in place): y = Q s_0 into Y;
 // q_i <- Q s_i for i < kk; the residual direction moves to W[kk & 1] so that
-// the next cycle's first step reads it.
+// the next cycle's first step reads it.  A unit whose cycle cap this cycle
+// reaches is not restarted: only y is formed.
+//
+// Bound: HBM in FP32 (K vectors read, kk + 1 written), the FP64 rate in FP64
+// ((kk + 1) K FMAs a row).  The coefficients are converted to the vector type
+// once per CTA and kept in shared memory, NA at a time (a row of YSTR values per
+// basis vector, read as broadcasts): a basis value is loaded once and updates NA
+// accumulators, RITZ_R rows per thread.  Every output sums over the basis vectors
+// in ascending order.
+// Before, every row thread fetched and converted each coefficient itself (an FP64
+// conversion per coefficient and warp): 2.36 ms for 40 FP32 vectors of 3.7M rows and
+// 9 outputs, 3.08 ms for 16 FP64 vectors; the Fiedler pair of that mesh took 437 ms
+// and takes 373 ms with this form.
 // ----------------------------------------------------------------------------
+#define YSTR 20  // RSB_MAXKEEP + 1, rounded up to 16 bytes
+
+// The coefficients of y and of the kk kept vectors, in the vector type.
 template <typename V, bool CO>
-__device__ __forceinline__ void lz_ritz_t(const LzArgs<V>& a, int tix) {
+__device__ __forceinline__ void ritz_stage(const double* Ym, int K, int kk, V* Ys) {
+  for (int idx = threadIdx.x; idx < K * (kk + 1); idx += RSB_BLOCK) {
+    const int l = idx / (kk + 1), i = idx % (kk + 1);
+    Ys[l * YSTR + i] = V(ldc<CO>(Ym + l * RSB_MAXM + i));
+  }
+  __syncthreads();
+}
+
+// NA outputs of RR rows (rows r0 + rr * RSB_BLOCK; ok[rr]: inside the tile) from
+// the vectors q + l * ld.
+template <typename V, int NA, int RR>
+__device__ __forceinline__ void ritz_rows(const V* q, long long ld, int K, const V* Ys,
+                                          const bool (&ok)[RR], V (&acc)[NA][RR]) {
+#pragma unroll
+  for (int i = 0; i < NA; ++i)
+#pragma unroll
+    for (int rr = 0; rr < RR; ++rr) acc[i][rr] = V(0);
+  constexpr int LU = 16 / (RR * (int)sizeof(V) / 4);  // basis vectors in flight
+  for (int l0 = 0; l0 < K; l0 += LU) {
+    V qv[LU][RR];
+#pragma unroll
+    for (int u = 0; u < LU; ++u)
+#pragma unroll
+      for (int rr = 0; rr < RR; ++rr)
+        qv[u][rr] = (ok[rr] && l0 + u < K) ? q[(long long)(l0 + u) * ld + rr * RSB_BLOCK] : V(0);
+#pragma unroll
+    for (int u = 0; u < LU; ++u)
+      if (l0 + u < K) {
+#pragma unroll
+        for (int i = 0; i < NA; ++i) {
+          const V c = Ys[(l0 + u) * YSTR + i];
+#pragma unroll
+          for (int rr = 0; rr < RR; ++rr) acc[i][rr] += c * qv[u][rr];
+        }
+      }
+  }
+}
+
+// rows of one tile: q points at row row0 of vector 0 (global or shared memory)
+template <typename V, int NA, int RR>
+__device__ __forceinline__ void ritz_tile(V* q, long long ld, int K, int kk, int nr, const V* Ys,
+                                          V* y) {
+  for (int b = 0; b < nr; b += RR * RSB_BLOCK) {
+    const int r0 = b + threadIdx.x;
+    bool ok[RR];
+#pragma unroll
+    for (int rr = 0; rr < RR; ++rr) ok[rr] = r0 + rr * RSB_BLOCK < nr;
+    V acc[NA][RR];
+    ritz_rows<V, NA, RR>(q + r0, ld, K, Ys, ok, acc);
+#pragma unroll
+    for (int rr = 0; rr < RR; ++rr)
+      if (ok[rr]) {
+        y[r0 + rr * RSB_BLOCK] = acc[0][rr];
+#pragma unroll
+        for (int i = 0; i < NA; ++i)
+          if (i < kk) q[(long long)i * ld + r0 + rr * RSB_BLOCK] = acc[i][rr];
+      }
+  }
+}
+
+// The number of accumulators: y alone, up to the default 8 kept vectors, or all.
+template <typename V>
+__device__ __forceinline__ void ritz_dispatch(V* q, long long ld, int K, int kk, int nr,
+                                              const V* Ys, V* y) {
+  constexpr int RR = sizeof(V) == 4 ? 4 : 2;
+  if (kk == 0) ritz_tile<V, 1, RR>(q, ld, K, kk, nr, Ys, y);
+  else if (kk <= 8) ritz_tile<V, 9, RR>(q, ld, K, kk, nr, Ys, y);
+  else ritz_tile<V, RSB_MAXKEEP + 1, RR / 2>(q, ld, K, kk, nr, Ys, y);
+}
+
+template <typename V, bool CO>
+__device__ __forceinline__ void lz_ritz_t(const LzArgs<V>& a, int tix, V* Ys) {
   const Tile t = a.tiles[tix];
   const Unit& u = a.units[t.unit];
   if (ldc<CO>(&u.status) != U_ACTIVE) return;
   const int K = ldc<CO>(&u.msteps);
-  const int kk = ldc<CO>(&u.kk);
-  const double* Ym = unit_S(a.S, t.unit) + RSB_MAXM * RSB_MAXM;
+  // the last cycle under the cap ends converged or capped: nothing is kept
+  const int kk = ldc<CO>(&u.cycles) + 1 >= u.maxcycles ? 0 : ldc<CO>(&u.kk);
+  ritz_stage<V, CO>(unit_S(a.S, t.unit) + RSB_MAXM * RSB_MAXM, K, kk, Ys);
+  ritz_dispatch<V>(a.Q + t.row0, a.N, K, kk, t.row1 - t.row0, Ys, a.Y + t.row0);
   const V* wl = (K & 1) ? a.W1 : a.W0;
   V* wn = (kk & 1) ? a.W1 : a.W0;
-  for (int r = t.row0 + threadIdx.x; r < t.row1; r += RSB_BLOCK) {
-    V q[RSB_MAXM];
-#pragma unroll
-    for (int l = 0; l < RSB_MAXM; ++l) q[l] = l < K ? a.Q[(long long)l * a.N + r] : V(0);
-    for (int i = 0; i <= kk; ++i) {
-      V acc = V(0);
-#pragma unroll
-      for (int l = 0; l < RSB_MAXM; ++l)
-        if (l < K) acc += V(ldc<CO>(Ym + l * RSB_MAXM + i)) * q[l];
-      if (i == 0) a.Y[r] = acc;
-      if (i < kk) a.Q[(long long)i * a.N + r] = acc;
-    }
-    if (kk > 0 && wn != wl) wn[r] = wl[r];
-  }
+  if (kk > 0 && wn != wl)
+    for (int r = t.row0 + threadIdx.x; r < t.row1; r += RSB_BLOCK) wn[r] = wl[r];
   if (CO && a.pb_a && threadIdx.x == 0)
     atomicAdd(a.pb_a, (unsigned long long)(t.row1 - t.row0) * sizeof(V) * (K + kk + 1));
 }
@@ -1195,7 +1271,8 @@ __device__ __forceinline__ void proj3_t(const LzArgs<V>& a, const V* y, int tix,
 
 template <typename V>
 __global__ void __launch_bounds__(RSB_BLOCK) k_lz_ritz(LzArgs<V> a) {
-  lz_ritz_t<V, false>(a, blockIdx.x);
+  __shared__ __align__(16) V Ys[RSB_MAXM * YSTR];
+  lz_ritz_t<V, false>(a, blockIdx.x, Ys);
 }
 template <typename V>
 __global__ void __launch_bounds__(RSB_BLOCK) k_lz_resid(LzArgs<V> a, const V* __restrict__ y,
@@ -1250,7 +1327,10 @@ __global__ void __launch_bounds__(RSB_BLOCK, 2)
   }
   for (int u = blockIdx.x; u < nunits; u += G) lz_eig_u<V, true>(a.units[u], unit_S(a.S, u), sh.J);
   if (!grid_sync(gb, G)) return;
-  for (int t = blockIdx.x; t < ntiles; t += G) lz_ritz_t<V, true>(a, t);
+  for (int t = blockIdx.x; t < ntiles; t += G) {
+    lz_ritz_t<V, true>(a, t, ws);  // RSB_MAXM * YSTR <= SUBROWS values
+    __syncthreads();
+  }
   if (!grid_sync(gb, G)) return;
   for (int t = blockIdx.x; t < ntiles; t += G) lz_resid_t<V, true>(a, a.Y, 0, t, sm, out);
   if (!grid_sync(gb, G)) return;
@@ -1523,38 +1603,21 @@ __device__ __forceinline__ void res_coef(const double* out, int nc, double isn, 
 }
 
 // Ritz vector y = Q s_0 into Y and the kept vectors q_i <- Q s_i (i < kk) in
-// shared memory; the residual direction moves to W[kk & 1].
+// shared memory (lz_ritz_t on the resident basis); the residual direction moves
+// to W[kk & 1].
 template <typename V>
 __device__ void res_ritz(const LzArgs<V>& a, const Tile& t, const Unit& u, V* Qs, int trs,
                          V* Ys) {
   if (ldc<true>(&u.status) != U_ACTIVE) return;
   const int nr = t.row1 - t.row0;
   const int K = ldc<true>(&u.msteps);
-  const int kk = ldc<true>(&u.kk);
-  const double* Ym = unit_S(a.S, t.unit) + RSB_MAXM * RSB_MAXM;
-  constexpr int YS = RSB_MAXKEEP + 1;
-  for (int idx = threadIdx.x; idx < K * (kk + 1); idx += RSB_BLOCK) {
-    const int l = idx / (kk + 1), i = idx % (kk + 1);
-    Ys[l * YS + i] = V(__ldcg(Ym + l * RSB_MAXM + i));
-  }
-  __syncthreads();
+  const int kk = ldc<true>(&u.cycles) + 1 >= u.maxcycles ? 0 : ldc<true>(&u.kk);
+  ritz_stage<V, true>(unit_S(a.S, t.unit) + RSB_MAXM * RSB_MAXM, K, kk, Ys);
+  ritz_dispatch<V>(Qs, trs, K, kk, nr, Ys, a.Y + t.row0);
   const V* wl = (K & 1) ? a.W1 : a.W0;
   V* wn = (kk & 1) ? a.W1 : a.W0;
-  for (int rl = threadIdx.x; rl < nr; rl += RSB_BLOCK) {
-    const int r = t.row0 + rl;
-    V q[RSB_MAXM];
-#pragma unroll
-    for (int l = 0; l < RSB_MAXM; ++l) q[l] = l < K ? Qs[(size_t)l * trs + rl] : V(0);
-    for (int i = 0; i <= kk; ++i) {
-      V acc = V(0);
-#pragma unroll
-      for (int l = 0; l < RSB_MAXM; ++l)
-        if (l < K) acc += Ys[l * YS + i] * q[l];
-      if (i == 0) a.Y[r] = acc;
-      if (i < kk) Qs[(size_t)i * trs + rl] = acc;
-    }
-    if (kk > 0 && wn != wl) wn[r] = __ldcg(wl + r);
-  }
+  if (kk > 0 && wn != wl)
+    for (int r = t.row0 + threadIdx.x; r < t.row1; r += RSB_BLOCK) wn[r] = __ldcg(wl + r);
   if (a.pb_a && threadIdx.x == 0)
     atomicAdd(a.pb_a, (unsigned long long)nr * sizeof(V) * (K + kk + 1));
 }
