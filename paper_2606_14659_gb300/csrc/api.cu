@@ -284,6 +284,7 @@ struct Ctx {
   DevBuf gs_count, gs_cursor, gs_bptr, gs_bucket, gs_ev32, gs_len, gs_rowptr, gs_w, gs_misc;
   DevBuf part_concat;
   int trmax = 0;    // largest tile of the level being solved, rows
+  int ntmax = 0;    // most tiles of one of its units
   std::vector<DevBuf> stage;  // staged host inputs
   int* h_pinned = nullptr;
 };
@@ -511,6 +512,12 @@ static int max_tile_rows(const std::vector<Tile>& tiles) {
   return m;
 }
 
+static int max_unit_tiles(const std::vector<Unit>& units) {
+  int m = 0;
+  for (const Unit& u : units) m = std::max(m, u.ntile);
+  return m;
+}
+
 // mesh_rows[i]: the element count of the mesh unit i belongs to (empty: the
 // units are parts of one mesh, whose rows they cover)
 static void make_tiles(std::vector<Unit>& units, std::vector<Tile>& tiles, int rmin = RSB_MINR,
@@ -623,6 +630,7 @@ static int solve_candidate(Ctx& c, const LevelGraph& G, const Tile* tiles, int n
   int rc;
   SolveBufs B;
   B.trmax = c.trmax;
+  B.ntmax = c.ntmax;
   B.D[0] = nd > 0 ? dptr<double>(c.cand[0]) : nullptr;
   B.D[1] = nd > 1 ? dptr<double>(c.cand[1]) : nullptr;
   Counters* cn = dptr<Counters>(c.counters);
@@ -754,6 +762,7 @@ static int split_units(Ctx& c, const LevelGraph& G, std::vector<Unit>& hunits,
   RSB_CK(cudaMemcpyAsync(units, hunits.data(), sizeof(Unit) * nunits, cudaMemcpyHostToDevice, c.s));
   RSB_CK(cudaMemcpyAsync(tiles, htiles.data(), sizeof(Tile) * ntiles, cudaMemcpyHostToDevice, c.s));
   c.trmax = max_tile_rows(htiles);
+  c.ntmax = max_unit_tiles(hunits);
   const uint64_t* ckey = dptr<uint64_t>(c.ckey);
   double* partials = dptr<double>(c.partials);
   int64_t maxn = 0;
@@ -1442,6 +1451,7 @@ extern "C" int rsb_fiedler(const rsb_csr* g, const rsb_options* opt, double* lam
   std::vector<Tile> htiles;
   make_tiles(hunits, htiles, o.tile_rows > 0 ? o.tile_rows : RSB_MINR);
   c.trmax = max_tile_rows(htiles);
+  c.ntmax = max_unit_tiles(hunits);
   const int ntiles = (int)htiles.size();
   if ((rc = devbuf_reserve(c.units, sizeof(Unit))) ||
       (rc = devbuf_reserve(c.tiles, sizeof(Tile) * ntiles)) ||

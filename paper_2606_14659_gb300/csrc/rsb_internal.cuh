@@ -422,6 +422,14 @@ __device__ __forceinline__ void final_reduce(const double* partials, long long s
     if (on) {
       const double* p = partials + (long long)c * stride + t0;
       int t = s;
+      for (; t + 56 < nt; t += 64) {  // two blocks' loads in flight
+        const double a0 = __ldcg(p + t), a1 = __ldcg(p + t + 8);
+        const double a2 = __ldcg(p + t + 16), a3 = __ldcg(p + t + 24);
+        const double b0 = __ldcg(p + t + 32), b1 = __ldcg(p + t + 40);
+        const double b2 = __ldcg(p + t + 48), b3 = __ldcg(p + t + 56);
+        acc += (a0 + a1) + (a2 + a3);
+        acc += (b0 + b1) + (b2 + b3);
+      }
       for (; t + 24 < nt; t += 32) {
         const double a0 = __ldcg(p + t), a1 = __ldcg(p + t + 8);
         const double a2 = __ldcg(p + t + 16), a3 = __ldcg(p + t + 24);
@@ -433,6 +441,55 @@ __device__ __forceinline__ void final_reduce(const double* partials, long long s
     acc += __shfl_xor_sync(0xffffffffu, acc, 2);
     acc += __shfl_xor_sync(0xffffffffu, acc, 1);
     if (on && s == 0) out[c] = acc;
+  }
+  __syncthreads();
+}
+
+// final_reduce for up to RED_FEW coefficients (the norms and projections of a
+// step), the same sums in the same order.  With one coefficient final_reduce
+// leaves a chain of nt / 32 dependent load rounds and nt / 8 FP64 additions to
+// eight lanes (15 us for 973 tiles); here every thread of the CTA forms the
+// four-tile sums of some (tile block, lane) at once, so that one round of loads
+// and nt / 32 additions are left on the chain.  sp: shared scratch of
+// RED_FEW_DOUBLES(nc) doubles.
+#define RED_FEW 5
+#define RED_FEW_DOUBLES(nc) ((nc) * (RSB_MAXTILES_PER_UNIT / 32) * 8)
+__device__ __forceinline__ void final_reduce_few(const double* partials, long long stride, int t0,
+                                                 int nt, int nc, double* out, double* sp) {
+  const int nq = nt > 24 ? (nt - 25) / 32 + 1 : 0;  // 32-tile blocks with a full lane
+  for (int idx = threadIdx.x; idx < nc * nq * 8; idx += RSB_BLOCK) {
+    const int s = idx & 7, cq = idx >> 3;
+    const int c = cq / nq, q = cq - c * nq;
+    const int t = 32 * q + s;
+    if (t + 24 < nt) {
+      const double* p = partials + (long long)c * stride + t0 + t;
+      const double a0 = __ldcg(p), a1 = __ldcg(p + 8), a2 = __ldcg(p + 16), a3 = __ldcg(p + 24);
+      sp[idx] = (a0 + a1) + (a2 + a3);
+    }
+  }
+  const int c = threadIdx.x >> 5, s = threadIdx.x & 31;
+  const bool on = c < nc && s < 8;
+  const int fb = on && nt > 24 + s ? (nt - 25 - s) / 32 + 1 : 0;  // full blocks of this lane
+  double r[4] = {0.0, 0.0, 0.0, 0.0};
+  if (on) {
+    const double* p = partials + (long long)c * stride + t0;
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      if (s + 32 * fb + 8 * i < nt) r[i] = __ldcg(p + s + 32 * fb + 8 * i);
+  }
+  __syncthreads();
+  if (c < nc) {
+    double acc = 0.0;
+    if (on) {
+      for (int q = 0; q < fb; ++q) acc += sp[(c * nq + q) * 8 + s];
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        if (s + 32 * fb + 8 * i < nt) acc += r[i];
+    }
+    acc += __shfl_xor_sync(0xffffffffu, acc, 4);
+    acc += __shfl_xor_sync(0xffffffffu, acc, 2);
+    acc += __shfl_xor_sync(0xffffffffu, acc, 1);
+    if (s == 0) out[c] = acc;
   }
   __syncthreads();
 }
@@ -625,5 +682,6 @@ struct SolveBufs {
   void* bu = nullptr;            // block Lanczos: per-unit block state
   int64_t N = 0;
   int trmax = 0;                 // largest tile of the level, rows
+  int ntmax = 0;                 // most tiles of a unit of the level
   int maxcycles = 0;             // cycle cap of the current solve
 };

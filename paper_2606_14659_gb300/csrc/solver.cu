@@ -295,6 +295,7 @@ __device__ __forceinline__ void lz_a_t(const LzArgs<V>& a, int j, int tix, V* ws
   }
   store_dots<V>(a, nc, acc, tix);
   if (a.pb_a) prof_add(a.pb_a, pbytes);
+  if constexpr (!CO) return;  // k_lz_close reduces
   if (last_cta(&u.cnt, u.ntile)) {
     final_reduce(a.partials, a.stride, u.tile0, u.ntile, nc, out);
     if (threadIdx.x == 0) {
@@ -340,6 +341,7 @@ __device__ __forceinline__ void lz_b_t(const LzArgs<V>& a, int j, int tix, V* ws
   }
   store_dots<V>(a, nc, acc, tix);
   if (a.pb_b) prof_add(a.pb_b, pbytes);
+  if constexpr (!CO) return;  // k_lz_close reduces
   if (last_cta(&u.cnt, u.ntile)) {
     final_reduce(a.partials, a.stride, u.tile0, u.ntile, nc, out);
     if (threadIdx.x == 0) {
@@ -358,7 +360,7 @@ __device__ __forceinline__ void lz_b_t(const LzArgs<V>& a, int j, int tix, V* ws
 
 template <typename V, bool CO>
 __device__ __forceinline__ void lz_c_t(const LzArgs<V>& a, int j, double breakdown, int tix,
-                                       V* cv, double* sm, double* out) {
+                                       V* cv, double* sm, double* out, double* sp) {
   const Tile t = a.tiles[tix];
   Unit& u = a.units[t.unit];
   if (ldc<CO>(&u.status) != U_ACTIVE || j >= ldc<CO>(&u.msteps) || j < ldc<CO>(&u.j0)) return;
@@ -390,7 +392,7 @@ __device__ __forceinline__ void lz_c_t(const LzArgs<V>& a, int j, double breakdo
   const double sum = block_total(acc, sm);
   if (threadIdx.x == 0) a.partials[tix] = sum;
   if (last_cta(&u.cnt, u.ntile)) {
-    final_reduce(a.partials, a.stride, u.tile0, u.ntile, 1, out);
+    final_reduce_few(a.partials, a.stride, u.tile0, u.ntile, 1, out, sp);
     if (threadIdx.x == 0) {
       const double b = sqrt(out[0]);
       u.beta[j + 1] = b;
@@ -422,7 +424,8 @@ __global__ void __launch_bounds__(RSB_BLOCK) k_lz_c(LzArgs<V> a, int j, double b
   __shared__ double sm[RSB_WARPS];
   __shared__ V cv[RSB_MAXC];
   __shared__ double out[1];
-  lz_c_t<V, false>(a, j, breakdown, blockIdx.x, cv, sm, out);
+  __shared__ double sp[RED_FEW_DOUBLES(1)];
+  lz_c_t<V, false>(a, j, breakdown, blockIdx.x, cv, sm, out, sp);
 }
 
 // ----------------------------------------------------------------------------
@@ -541,51 +544,75 @@ __global__ void __launch_bounds__(RSB_BLOCK) k_lz_a1(LzArgs<V> a, int j, int nsu
 // part), from the reduced totals av = [a_b (b < nb), v.v] and gz = [g_b
 // (b < nb), v.z] of src, scaled here in place to v = src / nu (inu = 1 / nu)
 // and u0 = 1/sqrt(n) on its entry; sc[0..2] = rho, q_j.z, alpha and
-// sk[0..j) = S_kj come back in shared memory.  S is read for columns < j;
-// column and row j are written when write_s.  The streaming kernel and the
-// resident kernel both call this, so both modes produce the same numbers.
-template <bool CO>
-__device__ void d2_finish(double* av, double* gz, int nb, int nd, int j, double inu, double isn,
-                          double* Sm, bool write_s, double* sc, double* sk) {
-  if (threadIdx.x == 0) {
-    for (int b = 0; b < nb; ++b) av[b] *= inu;
-    av[nb] *= inu * inu;
-    gz[nb] *= inu;
-    av[0] *= isn;
-    gz[0] *= isn;
+// sk[0..j) = S_kj come back in shared memory.  Ss: columns < j of S (row k at
+// k * RSB_MAXM; S is symmetric).  The streaming kernel and the resident kernel
+// both call this, so both modes produce the same numbers.
+// On GB300 an FP64 warp instruction holds its SM sub-partition for 64 cycles
+// however many lanes are active, so no sum is left to one lane: a.a and a.g
+// are taken by one warp in a butterfly, every S_k.a by four lanes of the other
+// warps.  (These are corrections of size |a| ~ 1e-7 to v.v, v.z and g.)  With
+// the sums on single threads this took 11 us at j = 39, now 2 us.
+__device__ __forceinline__ void d2_finish(double* av, double* gz, int nb, int nd, int j, double inu,
+                                          double isn, const double* Ss, double* sc, double* sk) {
+  const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
+  if (tid <= nb) {
+    double x = av[tid] * (tid < nb ? inu : inu * inu);
+    if (tid == 0) x *= isn;
+    av[tid] = x;
+  } else if (tid >= 64 && tid - 64 <= nb) {
+    const int b = tid - 64;
+    if (b == 0) gz[0] *= isn;
+    if (b == nb) gz[nb] *= inu;
+  }
+  __syncthreads();
+  const double* aq = av + 1 + nd;  // a on q_0..q_{j-1}
+  if (w == 7) {
     double aa = 0.0, ag = 0.0;
-    for (int b = 0; b < nb; ++b) {
-      aa += av[b] * av[b];
-      ag += av[b] * gz[b];
+    for (int b = lane; b < nb; b += 32) {
+      aa = fma(av[b], av[b], aa);
+      ag = fma(av[b], gz[b], ag);
     }
+    aa = warp_sum(aa);
+    ag = warp_sum(ag);
     const double rho2 = av[nb] - aa;
     // v has unit norm and |a| is at rounding level after its first pass; a
     // non-positive rho^2 means v lies in span(B) to working precision
     const double rho = rho2 > 0.0 ? sqrt(rho2) : 1e-300;
-    sc[0] = rho;
-    sc[1] = (gz[nb] - ag) / rho;  // q_j.z
+    const double qz = (gz[nb] - ag) / rho;
+    if (lane == 0) {
+      sc[0] = rho;
+      sc[1] = qz;  // q_j.z
+    }
+  } else {
+    // warps 0..4 cover k < 40, four lanes per k
+    const int k = 8 * w + (lane & 7), part = lane >> 3;
+    double sa = 0.0;
+    if (k < j)
+      for (int i = part; i < j; i += 4) sa = fma(Ss[i * RSB_MAXM + k], aq[i], sa);
+    sa += __shfl_xor_sync(0xffffffffu, sa, 8);
+    sa += __shfl_xor_sync(0xffffffffu, sa, 16);
+    if (k < j && part == 0) sk[k] = gz[1 + nd + k] - sa;
   }
   __syncthreads();
   const double rho = sc[0];
-  const double* aq = av + 1 + nd;  // a on q_0..q_{j-1}
-  for (int k = threadIdx.x; k < j; k += RSB_BLOCK) {
-    double sa_k = 0.0;
-    for (int i = 0; i < j; ++i) sa_k += ldc<CO>(Sm + k * RSB_MAXM + i) * aq[i];
-    sk[k] = (gz[1 + nd + k] - sa_k) / rho;
-  }
+  if (tid < j) sk[tid] = sk[tid] / rho;
   __syncthreads();
-  if (threadIdx.x == 0) {
+  if (w == 7) {
     double sig = 0.0;
-    for (int k = 0; k < j; ++k) sig += sk[k] * aq[k];
-    sc[2] = (sc[1] - sig) / rho;
-    if (write_s) Sm[j * RSB_MAXM + j] = sc[2];
+    for (int k = lane; k < j; k += 32) sig = fma(sk[k], aq[k], sig);
+    sig = warp_sum(sig);
+    if (lane == 0) sc[2] = (sc[1] - sig) / rho;
   }
-  if (write_s)
-    for (int k = threadIdx.x; k < j; k += RSB_BLOCK) {
-      Sm[k * RSB_MAXM + j] = sk[k];
-      Sm[j * RSB_MAXM + k] = sk[k];
-    }
   __syncthreads();
+}
+
+// Column and row j of S from the finished step D2.
+__device__ __forceinline__ void d2_store_S(double* Sm, int j, const double* sc, const double* sk) {
+  for (int k = threadIdx.x; k <= j; k += RSB_BLOCK) {
+    const double v = k < j ? sk[k] : sc[2];
+    Sm[k * RSB_MAXM + j] = v;
+    Sm[j * RSB_MAXM + k] = v;
+  }
 }
 
 // ----------------------------------------------------------------------------
@@ -594,7 +621,7 @@ __device__ void d2_finish(double* av, double* gz, int nb, int nd, int j, double 
 // synchronization Gram-Schmidt and GMRES algorithms", 2020).  v = src / nu_j
 // has been projected once against B = [u0, D, q_0..q_{j-1}]; z = L v (D1).
 // One staged pass over q_0..q_{j-1}, src and z takes a = B^T v, g = B^T z,
-// v.v and v.z; the unit's last CTA then forms
+// v.v and v.z; k_lz_close then forms
 //   rho = sqrt(v.v - a.a)                  q_j = (v - B a) / rho
 //   L q_j = (z - L B a) / rho, where L B a lies in span(B, q_j) up to
 //   rounding (L u0 = 0; D holds eigenvector approximations; L q_i for i < j
@@ -609,9 +636,8 @@ __global__ void __launch_bounds__(RSB_BLOCK, 4) k_lz_d2(LzArgs<V> a, int j, Grid
   extern __shared__ __align__(128) unsigned char d2_sh[];
   constexpr int AL = BulkRows<V>::AL, CRB = BulkRows<V>::CRB;
   __shared__ __align__(8) uint64_t bar[ST_NB];
-  __shared__ double out[2 * RSB_MAXC + 2];
   const Tile t = a.tiles[blockIdx.x];
-  Unit& u = a.units[t.unit];
+  const Unit& u = a.units[t.unit];
   if (u.status != U_ACTIVE || j >= u.msteps || j < u.j0) return;
   V* Qb = reinterpret_cast<V*>(d2_sh);  // [ST_NB][j + 2][CRB]: q_0..q_{j-1}, src, z
   const int nd = u.nd;
@@ -680,24 +706,107 @@ __global__ void __launch_bounds__(RSB_BLOCK, 4) k_lz_d2(LzArgs<V> a, int j, Grid
     store_dots<V>(a2, nc, az, blockIdx.x);
   }
   if (a.pb_a2) prof_add(a.pb_a2, pbytes);
-  if (last_cta(&u.cnt, u.ntile)) {
-    final_reduce(a.partials, a.stride, u.tile0, u.ntile, nc, out);
-    final_reduce(a.partials + (long long)nc * a.stride, a.stride, u.tile0, u.ntile, nc, out + nc);
-    const double inu = 1.0 / (j == u.j0 ? u.beta0 : u.beta[j]);
-    __shared__ double sc[3], sk[RSB_MAXM];
-    d2_finish<false>(out, out + nc, nb, nd, j, inu, u.isn, unit_S(a.S, t.unit), true, sc, sk);
-    const double rho = sc[0];
-    if (threadIdx.x == 0) {
-      u.alpha[j] = sc[2];
-      // D3: q_j = src / (nu rho) - sum_b (a_b / rho) b,
-      //     w = z / rho - sum_b (g_b / rho) b - (q_j.z / rho) q_j
-      u.dz_src = inu / rho;
-      u.dz_z = 1.0 / rho;
-      u.dz_qz = sc[1] / rho;
+}
+
+// ----------------------------------------------------------------------------
+// Closing of a step's dots (streaming path): the sums over the unit's tiles, then
+//   CLOSE_A: c1 (FP64 step A);  CLOSE_B: c2 and column j of S (FP64 step B);
+//   CLOSE_D2: d2_finish and the coefficients of D3.
+// The tiles' partials of one unit are nt x 2 (j + 2) FP64 values: at 973 tiles and
+// j = 39 their additions alone keep one SM's FP64 pipe busy for 20 us, which the
+// last CTA of the dots kernel used to spend while the chip idled (45 us with its
+// chain of loads).  So a kernel of its own spreads the coefficients over
+// close_ctas() CTAs of the unit: one for a unit of few tiles, one per 32
+// coefficients (a warp sums four, as in final_reduce) up to 192 tiles, one per
+// four (final_reduce_few) above.  The order of every sum stays final_reduce's.
+// ----------------------------------------------------------------------------
+enum { CLOSE_A = 0, CLOSE_B = 1, CLOSE_D2 = 2 };
+
+__host__ __device__ inline int close_per_cta(int nt, int ncoef) {
+  return nt <= 32 ? ncoef : nt <= 192 ? 32 : 4;
+}
+__host__ __device__ inline int close_ctas(int nt, int ncoef) {
+  const int per = close_per_cta(nt, ncoef);
+  return (ncoef + per - 1) / per;
+}
+template <int MODE>
+__host__ __device__ inline int close_ncoef(int nd, int j) {
+  return MODE == CLOSE_D2 ? 2 * (2 + nd + j) : 2 + nd + j;
+}
+
+template <typename V, int MODE>
+__global__ void __launch_bounds__(RSB_BLOCK) k_lz_close(LzArgs<V> a, int j, int G) {
+  __shared__ double out[2 * RSB_MAXC + 2];
+  __shared__ double sp[RED_FEW_DOUBLES(4)];
+  const int ui = (int)(blockIdx.x / (unsigned)G), g = (int)(blockIdx.x - (unsigned)ui * G);
+  Unit& u = a.units[ui];
+  if (u.status != U_ACTIVE || j >= u.msteps || j < u.j0) return;
+  const int nd = u.nd, nt = u.ntile;
+  const int ncoef = close_ncoef<MODE>(nd, j);
+  const int per = close_per_cta(nt, ncoef), gu = close_ctas(nt, ncoef);
+  if (g >= gu) return;
+  const int c0 = g * per, n = min(per, ncoef - c0);
+  const double* P = a.partials + (long long)c0 * a.stride;
+  double* Sm = unit_S(a.S, ui);
+  __shared__ double Ss[MODE == CLOSE_D2 ? RSB_MAXM * RSB_MAXM : 1];
+  __shared__ double inu_sh;
+  if constexpr (MODE == CLOSE_D2) {
+    for (int idx = threadIdx.x; idx < j * RSB_MAXM; idx += RSB_BLOCK) Ss[idx] = Sm[idx];
+    if (threadIdx.x == 0) inu_sh = 1.0 / (j == u.j0 ? u.beta0 : u.beta[j]);
+  }
+  if (per == 4) {
+    final_reduce_few(P, a.stride, u.tile0, nt, n, out, sp);
+  } else {
+    // final_reduce takes up to RSB_MAXC + 5 coefficients at once
+    for (int k = 0; k < n; k += 32)
+      final_reduce(P + (long long)k * a.stride, a.stride, u.tile0, nt, min(32, n - k), out + k);
+  }
+  if constexpr (MODE == CLOSE_A) {
+    for (int k = threadIdx.x; k < n; k += RSB_BLOCK)
+      u.c1[c0 + k] = c0 + k == 0 ? out[k] * u.isn : out[k];
+  } else if constexpr (MODE == CLOSE_B) {
+    for (int k = threadIdx.x; k < n; k += RSB_BLOCK) {
+      const int c = c0 + k;
+      u.c2[c] = c == 0 ? out[k] * u.isn : out[k];
+      if (c > nd) {
+        const double v = u.c1[c] + out[k];
+        Sm[(c - 1 - nd) * RSB_MAXM + j] = v;
+        Sm[j * RSB_MAXM + c - 1 - nd] = v;
+      }
     }
-    for (int b = threadIdx.x; b < nb; b += RSB_BLOCK) {
-      u.c2[b] = out[b] / rho;
-      u.c1[b] = out[nc + b] / rho;
+  } else {
+    const int nb = 1 + nd + j, nc = nb + 1;
+    if (gu > 1) {  // the totals meet in c2 (a, v.v) and c1 (g, v.z); the last CTA goes on
+      for (int k = threadIdx.x; k < n; k += RSB_BLOCK) {
+        const int c = c0 + k;
+        if (c < nc) u.c2[c] = out[k];
+        else u.c1[c - nc] = out[k];
+      }
+      if (!last_cta(&u.cnt, gu)) return;
+      for (int c = threadIdx.x; c < ncoef; c += RSB_BLOCK)
+        out[c] = __ldcg(c < nc ? u.c2 + c : u.c1 + (c - nc));
+    }
+    __shared__ double sc[3], sk[RSB_MAXM];
+    __syncthreads();
+    const double inu = inu_sh;
+    d2_finish(out, out + nc, nb, nd, j, inu, u.isn, Ss, sc, sk);
+    d2_store_S(Sm, j, sc, sk);
+    const double rho = sc[0];
+    // D3: q_j = src / (nu rho) - sum_b (a_b / rho) b,
+    //     w = z / rho - sum_b (g_b / rho) b - (q_j.z / rho) q_j
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (w == 4) {
+      if (lane == 0) u.alpha[j] = sc[2];
+      const double x = (lane == 0 ? inu : lane == 1 ? 1.0 : sc[1]) / rho;
+      if (lane == 0) u.dz_src = x;
+      if (lane == 1) u.dz_z = x;
+      if (lane == 2) u.dz_qz = x;
+    } else if (w < 2) {
+      const int b = threadIdx.x;
+      if (b < nb) u.c2[b] = out[b] / rho;
+    } else if (w < 4) {
+      const int b = threadIdx.x - 64;
+      if (b < nb) u.c1[b] = out[nc + b] / rho;
     }
   }
 }
@@ -711,6 +820,7 @@ __global__ void __launch_bounds__(RSB_BLOCK) k_lz_d3(LzArgs<V> a, int j, double 
   __shared__ double sm[RSB_WARPS];
   __shared__ V ca[RSB_MAXC], cg[RSB_MAXC];
   __shared__ double out[1];
+  __shared__ double sp[RED_FEW_DOUBLES(1)];
   const Tile t = a.tiles[blockIdx.x];
   Unit& u = a.units[t.unit];
   if (u.status != U_ACTIVE || j >= u.msteps || j < u.j0) return;
@@ -800,7 +910,7 @@ __global__ void __launch_bounds__(RSB_BLOCK) k_lz_d3(LzArgs<V> a, int j, double 
   const double sum = block_total(acc, sm);
   if (threadIdx.x == 0) a.partials[blockIdx.x] = sum;
   if (last_cta(&u.cnt, u.ntile)) {
-    final_reduce(a.partials, a.stride, u.tile0, u.ntile, 1, out);
+    final_reduce_few(a.partials, a.stride, u.tile0, u.ntile, 1, out, sp);
     if (threadIdx.x == 0) {
       const double b = sqrt(out[0]);
       u.beta[j + 1] = b;
@@ -1125,7 +1235,7 @@ __device__ __forceinline__ void lz_ritz_t(const LzArgs<V>& a, int tix, V* Ys) {
 // vector only (no residual).
 template <typename V, bool CO>
 __device__ __forceinline__ void lz_resid_t(const LzArgs<V>& a, const V* y, int mode, int tix,
-                                           double* sm, double* out) {
+                                           double* sm, double* out, double* sp) {
   const Tile t = a.tiles[tix];
   Unit& u = a.units[t.unit];
   if (ldc<CO>(&u.status) != U_ACTIVE) return;
@@ -1156,7 +1266,7 @@ __device__ __forceinline__ void lz_resid_t(const LzArgs<V>& a, const V* y, int m
     if (threadIdx.x == 0) a.partials[(long long)c * a.stride + tix] = sum;
   }
   if (last_cta(&u.cnt, u.ntile)) {
-    final_reduce(a.partials, a.stride, u.tile0, u.ntile, nv, out);
+    final_reduce_few(a.partials, a.stride, u.tile0, u.ntile, nv, out, sp);
     if (threadIdx.x == 0) {
       u.ynorm2 = out[1];
       u.cp[0] = out[2] * u.isn;
@@ -1203,7 +1313,7 @@ __device__ __forceinline__ void lz_resid_t(const LzArgs<V>& a, const V* y, int m
 // converging): y -= B cp (in place); dots of the result against B -> c2.
 template <typename V, bool CO>
 __device__ __forceinline__ void proj2_t(const LzArgs<V>& a, V* y, int tix, double* sm,
-                                        double* out) {
+                                        double* out, double* sp) {
   const Tile t = a.tiles[tix];
   Unit& u = a.units[t.unit];
   if (ldc<CO>(&u.status) != U_ACTIVE || ldc<CO>(&u.j0) != 0) return;
@@ -1229,7 +1339,7 @@ __device__ __forceinline__ void proj2_t(const LzArgs<V>& a, V* y, int tix, doubl
     if (threadIdx.x == 0) a.partials[(long long)c * a.stride + tix] = sum;
   }
   if (last_cta(&u.cnt, u.ntile)) {
-    final_reduce(a.partials, a.stride, u.tile0, u.ntile, nv, out);
+    final_reduce_few(a.partials, a.stride, u.tile0, u.ntile, nv, out, sp);
     if (threadIdx.x == 0) {
       u.c2[0] = out[0] * u.isn;
       for (int l = 0; l < nd; ++l) u.c2[1 + l] = out[1 + l];
@@ -1240,7 +1350,7 @@ __device__ __forceinline__ void proj2_t(const LzArgs<V>& a, V* y, int tix, doubl
 // w0 = y - B c2 (second pass), beta0 = ||w0||; a cycle starts at step 0.
 template <typename V, bool CO>
 __device__ __forceinline__ void proj3_t(const LzArgs<V>& a, const V* y, int tix, double* sm,
-                                        double* out) {
+                                        double* out, double* sp) {
   const Tile t = a.tiles[tix];
   Unit& u = a.units[t.unit];
   if (ldc<CO>(&u.status) != U_ACTIVE || ldc<CO>(&u.j0) != 0) return;
@@ -1260,7 +1370,7 @@ __device__ __forceinline__ void proj3_t(const LzArgs<V>& a, const V* y, int tix,
   const double sum = block_sum(acc.get(), sm);
   if (threadIdx.x == 0) a.partials[tix] = sum;
   if (last_cta(&u.cnt, u.ntile)) {
-    final_reduce(a.partials, a.stride, u.tile0, u.ntile, 1, out);
+    final_reduce_few(a.partials, a.stride, u.tile0, u.ntile, 1, out, sp);
     if (threadIdx.x == 0) {
       u.beta0 = sqrt(out[0]);
       u.msteps = u.m;
@@ -1279,19 +1389,22 @@ __global__ void __launch_bounds__(RSB_BLOCK) k_lz_resid(LzArgs<V> a, const V* __
                                                         int mode) {
   __shared__ double sm[RSB_WARPS];
   __shared__ double out[3 + RSB_MAXD];
-  lz_resid_t<V, false>(a, y, mode, blockIdx.x, sm, out);
+  __shared__ double sp[RED_FEW_DOUBLES(3 + RSB_MAXD)];
+  lz_resid_t<V, false>(a, y, mode, blockIdx.x, sm, out, sp);
 }
 template <typename V>
 __global__ void __launch_bounds__(RSB_BLOCK) k_proj2(LzArgs<V> a, V* __restrict__ y) {
   __shared__ double sm[RSB_WARPS];
   __shared__ double out[1 + RSB_MAXD];
-  proj2_t<V, false>(a, y, blockIdx.x, sm, out);
+  __shared__ double sp[RED_FEW_DOUBLES(1 + RSB_MAXD)];
+  proj2_t<V, false>(a, y, blockIdx.x, sm, out, sp);
 }
 template <typename V>
 __global__ void __launch_bounds__(RSB_BLOCK) k_proj3(LzArgs<V> a, const V* __restrict__ y) {
   __shared__ double sm[RSB_WARPS];
   __shared__ double out[1];
-  proj3_t<V, false>(a, y, blockIdx.x, sm, out);
+  __shared__ double sp[RED_FEW_DOUBLES(1)];
+  proj3_t<V, false>(a, y, blockIdx.x, sm, out, sp);
 }
 
 // ----------------------------------------------------------------------------
@@ -1305,6 +1418,7 @@ template <typename V>
 union CycleShared {
   JacShared<V> J;
   double wsd[SUBROWS];
+  double red[RED_FEW_DOUBLES(RED_FEW)];
 };
 
 template <typename V>
@@ -1316,13 +1430,14 @@ __global__ void __launch_bounds__(RSB_BLOCK, 2)
   __shared__ double sm[RSB_WARPS];
   __shared__ V cv[RSB_MAXC];
   V* ws = reinterpret_cast<V*>(sh.wsd);
+  double* red = sh.red;
   const unsigned G = gridDim.x;
   for (int j = jstart; j < M; ++j) {
     for (int t = blockIdx.x; t < ntiles; t += G) lz_a_t<V, true>(a, j, t, ws, out);
     if (!grid_sync(gb, G)) return;
     for (int t = blockIdx.x; t < ntiles; t += G) lz_b_t<V, true>(a, j, t, ws, cv, out);
     if (!grid_sync(gb, G)) return;
-    for (int t = blockIdx.x; t < ntiles; t += G) lz_c_t<V, true>(a, j, breakdown, t, cv, sm, out);
+    for (int t = blockIdx.x; t < ntiles; t += G) lz_c_t<V, true>(a, j, breakdown, t, cv, sm, out, red);
     if (!grid_sync(gb, G)) return;
   }
   for (int u = blockIdx.x; u < nunits; u += G) lz_eig_u<V, true>(a.units[u], unit_S(a.S, u), sh.J);
@@ -1332,11 +1447,11 @@ __global__ void __launch_bounds__(RSB_BLOCK, 2)
     __syncthreads();
   }
   if (!grid_sync(gb, G)) return;
-  for (int t = blockIdx.x; t < ntiles; t += G) lz_resid_t<V, true>(a, a.Y, 0, t, sm, out);
+  for (int t = blockIdx.x; t < ntiles; t += G) lz_resid_t<V, true>(a, a.Y, 0, t, sm, out, red);
   if (!grid_sync(gb, G)) return;
-  for (int t = blockIdx.x; t < ntiles; t += G) proj2_t<V, true>(a, a.Y, t, sm, out);
+  for (int t = blockIdx.x; t < ntiles; t += G) proj2_t<V, true>(a, a.Y, t, sm, out, red);
   if (!grid_sync(gb, G)) return;
-  for (int t = blockIdx.x; t < ntiles; t += G) proj3_t<V, true>(a, a.Y, t, sm, out);
+  for (int t = blockIdx.x; t < ntiles; t += G) proj3_t<V, true>(a, a.Y, t, sm, out, red);
 }
 
 // ----------------------------------------------------------------------------
@@ -1644,8 +1759,14 @@ __global__ void __launch_bounds__(RSB_BLOCK, 2)
   __shared__ double out[2 * RSB_MAXC + 2];
   __shared__ double dsc[3], dsk[RSB_MAXM];
   __shared__ double sm[RSB_WARPS];
-  __shared__ double beta_sh;
+  __shared__ double beta_sh, inu_sh;
   __shared__ V scale_sh;
+  // the Jacobi workspace is free outside lz_eig_u: the copy of S during the steps,
+  // and the scratch of the residual's and the projections' reductions
+  static_assert(sizeof(JacShared<V>) >= sizeof(double) * RSB_MAXM * RSB_MAXM, "copy of S");
+  static_assert(sizeof(JacShared<V>) >= sizeof(double) * RED_FEW_DOUBLES(RED_FEW), "scratch");
+  double* Ssh = reinterpret_cast<double*>(res_sh);
+  double* red = Ssh;
   const unsigned G = gridDim.x;
   const int tix = blockIdx.x;
   const Tile t = a.tiles[tix];
@@ -1675,7 +1796,14 @@ __global__ void __launch_bounds__(RSB_BLOCK, 2)
     int msteps = __ldcg(&u.msteps);
     if (threadIdx.x == 0) {
       beta_sh = __ldcg(&u.beta0);
-      scale_sh = V(1.0 / beta_sh);
+      inu_sh = 1.0 / beta_sh;
+      scale_sh = V(inu_sh);
+    }
+    // every CTA of the unit keeps its own copy of S during the steps
+    if constexpr (sizeof(V) == 4) {
+      const double* Sm = unit_S(a.S, t.unit);
+      for (int idx = threadIdx.x; idx < RSB_MAXM * RSB_MAXM; idx += RSB_BLOCK)
+        Ssh[idx] = __ldcg(Sm + idx);
     }
     __syncthreads();
     int ph = 0;
@@ -1697,9 +1825,10 @@ __global__ void __launch_bounds__(RSB_BLOCK, 2)
           final_reduce(a.partials, a.stride, u.tile0, u.ntile, nc, out);
           final_reduce(a.partials + (long long)nc * a.stride, a.stride, u.tile0, u.ntile, nc,
                        out + nc);
-          const double inu = 1.0 / beta_sh;
-          d2_finish<true>(out, out + nc, nb, nd, j, inu, isn, unit_S(a.S, t.unit),
-                          tix == u.tile0, dsc, dsk);
+          const double inu = inu_sh;
+          d2_finish(out, out + nc, nb, nd, j, inu, isn, Ssh, dsc, dsk);
+          d2_store_S(Ssh, j, dsc, dsk);
+          if (tix == u.tile0) d2_store_S(unit_S(a.S, t.unit), j, dsc, dsk);
           const double rho = dsc[0];
           for (int k = threadIdx.x; k < nb; k += RSB_BLOCK) {
             const double ck = out[k] / rho, gk = out[nc + k] / rho;
@@ -1717,7 +1846,8 @@ __global__ void __launch_bounds__(RSB_BLOCK, 2)
           if (threadIdx.x == 0) {
             const double b = sqrt(out[0]);
             beta_sh = b;
-            scale_sh = V(1.0 / b);
+            inu_sh = 1.0 / b;
+            scale_sh = V(inu_sh);
             if (lead) u.beta[j + 1] = b;
             if (b <= breakdown * u.dmax && lead) {  // invariant subspace: the cycle ends here
               u.msteps = j + 1;
@@ -1773,11 +1903,11 @@ __global__ void __launch_bounds__(RSB_BLOCK, 2)
     if (!grid_sync(gb, G)) return;
     res_ritz<V>(a, t, u, Qs, trs, &J.Z[0][0]);
     if (!grid_sync(gb, G)) return;
-    lz_resid_t<V, true>(ac, a.Y, 0, tix, sm, out);
+    lz_resid_t<V, true>(ac, a.Y, 0, tix, sm, out, red);
     if (!grid_sync(gb, G)) return;
-    proj2_t<V, true>(a, a.Y, tix, sm, out);
+    proj2_t<V, true>(a, a.Y, tix, sm, out, red);
     if (!grid_sync(gb, G)) return;
-    proj3_t<V, true>(a, a.Y, tix, sm, out);
+    proj3_t<V, true>(a, a.Y, tix, sm, out, red);
     if (!grid_sync(gb, G)) return;
     if (__ldcg(a.n_active) == 0) break;
   }
@@ -1919,7 +2049,7 @@ static int lz_start(LzArgs<V>& a, int ntiles, uint64_t sd, const double* from64,
 
 template <typename V>
 static int lz_cycle(LzArgs<V>& a, int ntiles, int nunits, int M, double breakdown, GridBar* gb,
-                    int trmax, cudaStream_t s) {
+                    int trmax, int ntmax, int nd, cudaStream_t s) {
   // CTAs per tile of step A1
   const int nsub = std::max(1, (trmax + A1_RPT * RSB_BLOCK - 1) / (A1_RPT * RSB_BLOCK));
   for (int j = 0; j < M; ++j) {
@@ -1931,25 +2061,32 @@ static int lz_cycle(LzArgs<V>& a, int ntiles, int nunits, int M, double breakdow
       pi = prof_before(PROF_LZ_A2, s);
       k_lz_d2<V><<<ntiles, RSB_BLOCK, staged_smem<V>(j + 2), s>>>(a, j, gb);
       RSB_CKL("k_lz_d2");
+      const int G = close_ctas(ntmax, close_ncoef<CLOSE_D2>(nd, j));
+      k_lz_close<V, CLOSE_D2><<<nunits * G, RSB_BLOCK, 0, s>>>(a, j, G);
+      RSB_CKL("k_lz_close<D2>");
       prof_after(pi, s);
       pi = prof_before(PROF_LZ_B, s);
       k_lz_d3<V><<<ntiles, RSB_BLOCK, 0, s>>>(a, j, breakdown);
       RSB_CKL("k_lz_d3");
       prof_after(pi, s);
-      continue;
+    } else {  // FP64: bound by GB300's FP64 rate; register-streaming kernels, CGS2
+      const int G = close_ctas(ntmax, close_ncoef<CLOSE_A>(nd, j));
+      k_lz_a<V><<<ntiles, RSB_BLOCK, 0, s>>>(a, j);
+      RSB_CKL("k_lz_a");
+      k_lz_close<V, CLOSE_A><<<nunits * G, RSB_BLOCK, 0, s>>>(a, j, G);
+      RSB_CKL("k_lz_close<A>");
+      prof_after(pi, s);
+      pi = prof_before(PROF_LZ_B, s);
+      k_lz_b<V><<<ntiles, RSB_BLOCK, 0, s>>>(a, j);
+      RSB_CKL("k_lz_b");
+      k_lz_close<V, CLOSE_B><<<nunits * G, RSB_BLOCK, 0, s>>>(a, j, G);
+      RSB_CKL("k_lz_close<B>");
+      prof_after(pi, s);
+      pi = prof_before(PROF_LZ_C, s);
+      k_lz_c<V><<<ntiles, RSB_BLOCK, 0, s>>>(a, j, breakdown);
+      RSB_CKL("k_lz_c");
+      prof_after(pi, s);
     }
-    // FP64: bound by GB300's FP64 rate; register-streaming kernels, CGS2
-    k_lz_a<V><<<ntiles, RSB_BLOCK, 0, s>>>(a, j);
-    RSB_CKL("k_lz_a");
-    prof_after(pi, s);
-    pi = prof_before(PROF_LZ_B, s);
-    k_lz_b<V><<<ntiles, RSB_BLOCK, 0, s>>>(a, j);
-    RSB_CKL("k_lz_b");
-    prof_after(pi, s);
-    pi = prof_before(PROF_LZ_C, s);
-    k_lz_c<V><<<ntiles, RSB_BLOCK, 0, s>>>(a, j, breakdown);
-    RSB_CKL("k_lz_c");
-    prof_after(pi, s);
   }
   k_lz_eig<V><<<nunits, RSB_BLOCK, 0, s>>>(a.units, a.S, nunits);
   RSB_CKL("k_lz_eig");
@@ -1980,6 +2117,7 @@ static int lanczos_run(const LevelGraph& G, const Tile* tiles, int ntiles, Unit*
   rc = lz_start<V>(a, ntiles, sd, from64, from32, s);
   if (rc) return rc;
   const double breakdown = 1e-14;
+  const int nd = (B.D[0] ? 1 : 0) + (B.D[1] ? 1 : 0);  // deflation vectors of every active unit
   if (B.gb) {
     // a fresh barrier (count, generation, error word) for this solve; the
     // failure-path test hook starts the count where no CTA sees the last arrival
@@ -2061,7 +2199,7 @@ static int lanczos_run(const LevelGraph& G, const Tile* tiles, int ntiles, Unit*
     cudaGraph_t graph = nullptr;
     RSB_CK(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
     prof_capture_begin();
-    rc = lz_cycle<V>(a, ntiles, nunits, M, breakdown, B.gb, B.trmax, s);
+    rc = lz_cycle<V>(a, ntiles, nunits, M, breakdown, B.gb, B.trmax, B.ntmax, nd, s);
     cap_pairs = prof_capture_end();
     cudaGraph_t g2 = nullptr;
     cudaError_t e = cudaStreamEndCapture(s, &g2);
@@ -2081,14 +2219,14 @@ static int lanczos_run(const LevelGraph& G, const Tile* tiles, int ntiles, Unit*
   for (int cyc = 0; cyc < 100000; ++cyc) {
     if (exec) {
       cudaError_t e = cudaGraphLaunch(exec, s);
-      rsb_count_launch(3 * M + 5);  // the kernels of one cycle
+      rsb_count_launch((sizeof(V) == 4 ? 4 : 5) * M + 5);  // the kernels of one cycle
       if (e != cudaSuccess) {
         cudaGraphExecDestroy(exec);
         return rsb_set_cuda_error(e, "cudaGraphLaunch");
       }
       prof_replay(cap_pairs);
     } else {
-      rc = lz_cycle<V>(a, ntiles, nunits, M, breakdown, B.gb, B.trmax, s);
+      rc = lz_cycle<V>(a, ntiles, nunits, M, breakdown, B.gb, B.trmax, B.ntmax, nd, s);
       if (rc) return rc;
     }
     rc = read_active(B, s, &active);
