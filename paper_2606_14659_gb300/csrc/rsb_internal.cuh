@@ -87,6 +87,7 @@ struct Unit {
   int64_t inner_total;
   double theta, resid, ynorm2;
   double beta0;          // norm of the first new vector of the cycle (unnormalised)
+  double inu;            // 1 / norm of the newest vector (the next step's src)
   double th[RSB_MAXKEEP + 1];  // smallest Ritz values of the last cycle
   double alpha[RSB_MAXM];
   double beta[RSB_MAXM + 1];
@@ -268,8 +269,7 @@ template <> struct Acc<float> {
 // S, c1 + c2 - e), and only lane 0 converts to FP64: on GB300 an FP64
 // instruction costs a warp about 16 SM cycles, an FP32 one a fraction of one.
 __device__ __forceinline__ double warp_total(const Acc<double>& a) { return warp_sum(a.s); }
-__device__ __forceinline__ double warp_total(const Acc<float>& a) {
-  float s = a.s, c = a.c;
+__device__ __forceinline__ void warp_merge(float& s, float& c) {  // result in every lane
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
     const float s2 = __shfl_xor_sync(0xffffffffu, s, o);
@@ -280,6 +280,10 @@ __device__ __forceinline__ double warp_total(const Acc<float>& a) {
     c = __fsub_rn(__fadd_rn(c, c2), e);
     s = S;
   }
+}
+__device__ __forceinline__ double warp_total(const Acc<float>& a) {
+  float s = a.s, c = a.c;
+  warp_merge(s, c);
   return (threadIdx.x & 31) == 0 ? (double)s - (double)c : 0.0;
 }
 

@@ -263,11 +263,7 @@ __device__ __forceinline__ void lz_a_t(const LzArgs<V>& a, int j, int tix, V* ws
   const V* src = (j & 1) ? a.W1 : a.W0;
   V* dst = (j & 1) ? a.W0 : a.W1;
   V* qj = a.Q + (long long)j * a.N;
-  // 1 / beta once per CTA (an FP64 division per thread costs the SM's FP64 pipe)
-  if (threadIdx.x == 0)
-    out[0] = 1.0 / (j == ldc<CO>(&u.j0) ? ldc<CO>(&u.beta0) : ldc<CO>(&u.beta[j]));
-  __syncthreads();
-  const V s = V(out[0]);
+  const V s = V(ldc<CO>(&u.inu));
   const int nd = u.nd;
   const int nc = 2 + nd + j;
   Acc<V> acc[MAXCW];
@@ -396,6 +392,7 @@ __device__ __forceinline__ void lz_c_t(const LzArgs<V>& a, int j, double breakdo
     if (threadIdx.x == 0) {
       const double b = sqrt(out[0]);
       u.beta[j + 1] = b;
+      u.inu = 1.0 / b;
       if (b <= breakdown * u.dmax) {  // invariant subspace: the cycle ends here
         u.msteps = j + 1;
         u.broke = 1;
@@ -428,114 +425,62 @@ __global__ void __launch_bounds__(RSB_BLOCK) k_lz_c(LzArgs<V> a, int j, double b
   lz_c_t<V, false>(a, j, breakdown, blockIdx.x, cv, sm, out, sp);
 }
 
-// ----------------------------------------------------------------------------
-// Bulk-copy staging (launch modes 0 and 1, FP32 step D2).  The tile is walked
-// in chunks of ST_CH rows; for every chunk one thread issues 1-D bulk copies
-// (cp.async.bulk, completion counted in bytes on an mbarrier) of the chunk's
-// rows of the basis (and of the step's work vectors) into shared memory, one
-// chunk ahead of the one being computed.  Waits on the mbarrier are bounded
-// (2 s of the global timer): on timeout the CTA sets the grid error word, waits
-// (bounded) for its own copies still in flight and returns.
-// ----------------------------------------------------------------------------
-// The staged kernels walk a tile in chunks of ST_CH rows through ST_NB
-// buffers: while a chunk is being computed, the next ST_NB - 1 chunks are in
-// flight.  Thread 0 issues the copies of a chunk, one per basis vector.
-// (Measured slower on GB300: four buffers of 128 rows for the same shared
-// memory, twice the copies for the same bytes; the copies issued by the 32
-// lanes of a warp together; and an L2 bulk prefetch of the chunks two ahead of
-// the copies.)
-#define ST_CH 256
-#define ST_NB 2
-
-template <typename V>
-struct BulkRows {
-  static constexpr int AL = 16 / sizeof(V);        // rows per 16 bytes
-  static constexpr int CRB = ST_CH + AL;           // staged rows per vector and buffer
-};
-
-template <typename V>
-constexpr size_t staged_smem(int nq) {
-  return ST_NB * (size_t)nq * BulkRows<V>::CRB * sizeof(V);
-}
-
-// Wait for chunk ci (buffer ci % ST_NB); false (uniform) when the copies did
-// not complete in time, after flagging the grid error word and draining this
-// CTA's copies still in flight (chunks ci .. ci + ST_NB - 1).
-__device__ __forceinline__ bool staged_wait(uint64_t* bar, int ci, int nchunk, GridBar* gb) {
-  const bool ok = mbar_wait_bounded(&bar[ci % ST_NB], (ci / ST_NB) & 1, 2000000000ull);
-  if (!__syncthreads_or(!ok)) return true;
-  if (threadIdx.x == 0) {
-    atomicMax(&gb->err, 1);
-    bool drained = true;
-    for (int c = ci; c < min(nchunk, ci + ST_NB); ++c)
-      drained = mbar_wait_bounded(&bar[c % ST_NB], (c / ST_NB) & 1, 1000000000ull) && drained;
-    if (!drained) atomicMax(&gb->err, 2);
-  }
-  __syncthreads();
-  return false;
-}
-
-// Thread 0: rows [c0, c1) of q_0..q_{nq-1} (rounded out to 16 bytes) into
-// buffer b of Qb ([ST_NB][slots][CRB]), completing on bar[b].
-// (extra and extra2, when given, are N-vectors staged after q_{nq-1}; slots =
-// nq plus the extras given)
-template <typename V>
-__device__ __forceinline__ void bulk_issue_chunk(const LzArgs<V>& a, V* Qb, uint64_t* bar, int nq,
-                                                 int b, int c0, int c1,
-                                                 const V* extra = nullptr,
-                                                 const V* extra2 = nullptr) {
-  constexpr int AL = BulkRows<V>::AL, CRB = BulkRows<V>::CRB;
-  const int slots = nq + (extra ? 1 : 0) + (extra2 ? 1 : 0);
-  const int a0 = c0 & ~(AL - 1);
-  const int len = (c1 - a0 + AL - 1) / AL * AL;
-  const unsigned bytes = (unsigned)(len * sizeof(V));
-  V* dst = Qb + (size_t)b * slots * CRB;
-  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-  mbar_expect_tx(&bar[b], bytes * (unsigned)slots);
-  for (int k = 0; k < nq; ++k)
-    bulk_g2s(dst + (size_t)k * CRB, a.Q + (long long)k * a.N + a0, bytes, &bar[b]);
-  int k = nq;
-  if (extra) bulk_g2s(dst + (size_t)(k++) * CRB, extra + a0, bytes, &bar[b]);
-  if (extra2) bulk_g2s(dst + (size_t)k * CRB, extra2 + a0, bytes, &bar[b]);
-}
-
-// Thread 0 of a staged kernel: the copies of chunk c into its buffer.
-template <typename V>
-__device__ __forceinline__ void stage_chunk(const LzArgs<V>& a, V* Qb, uint64_t* bar, int nq,
-                                            const Tile& t, int c, const V* extra = nullptr,
-                                            const V* extra2 = nullptr) {
-  const int n0 = t.row0 + c * ST_CH;
-  bulk_issue_chunk(a, Qb, bar, nq, c % ST_NB, n0, min(t.row1, n0 + ST_CH), extra, extra2);
-}
-
 // Step D1 of the FP32 streaming path: z = L (src / nu_j) into the work vector
-// AP (src stays as it is: D2 and D3 read it).  A CTA takes A1_RPT * RSB_BLOCK consecutive rows of a tile (CTA b: tile
-// b / nsub, part b % nsub of it), A1_RPT rows per thread.
-#ifndef A1_RPT
-#define A1_RPT 4
-#endif
+// AP (src stays as it is: D2 and D3 read it).  A CTA takes A1_ROWS consecutive rows
+// of a tile (CTA b: tile b / nsub, part b % nsub of it).
+// Bound: the latency of entry load, then gather, at HBM's rate (the entries, 4 B
+// each, are read once; 9 of 10 gathers of src hit L1).  A thread has the 13 entries
+// of half an interior row of a 26-neighbour mesh in flight, then their gathers, at
+// 48 registers; the entries are loaded as streams (evicted first), which keeps src
+// in L1 and the basis that D2 reads next in L2.  At 3.7M rows 80 us, of which the
+// bytes take 61; eight entries at a time took 94, through L1 88.  (Also measured:
+// the next entries loaded before the current gathers 84 us; entries brought to
+// shared memory by bulk copies, which leaves L1 too small for src, 95 us.)
+#define A1_P 13
+#define A1_ROWS (4 * RSB_BLOCK)
 template <typename V>
-__global__ void __launch_bounds__(RSB_BLOCK) k_lz_a1(LzArgs<V> a, int j, int nsub) {
-  __shared__ double scale;
+__global__ void __launch_bounds__(RSB_BLOCK, 5) k_lz_a1(LzArgs<V> a, int j, int nsub) {
   const int tix = (int)(blockIdx.x / (unsigned)nsub);
   const Tile t = a.tiles[tix];
-  const long long p0 = (long long)t.row0 +
-                       (long long)(blockIdx.x - (unsigned)tix * nsub) * (A1_RPT * RSB_BLOCK);
+  const long long p0 =
+      (long long)t.row0 + (long long)(blockIdx.x - (unsigned)tix * nsub) * A1_ROWS;
   if (p0 >= t.row1) return;
-  const int p1 = (int)min((long long)t.row1, p0 + A1_RPT * RSB_BLOCK);
+  const int p1 = (int)min((long long)t.row1, p0 + A1_ROWS);
   const Unit& u = a.units[t.unit];
   if (u.status != U_ACTIVE || j >= u.msteps || j < u.j0) return;
-  if (threadIdx.x == 0) scale = 1.0 / (j == u.j0 ? u.beta0 : u.beta[j]);
-  __syncthreads();
-  const V s = V(scale);
-  const V* src = (j & 1) ? a.W1 : a.W0;
-  V* z = a.AP;
+  const V s = V(u.inu);
+  const V* __restrict__ src = (j & 1) ? a.W1 : a.W0;
   unsigned long long pbytes = 0;
-#pragma unroll 4
   for (int r = (int)p0 + threadIdx.x; r < p1; r += RSB_BLOCK) {
+    const int64_t base = a.slice_ptr[r >> 5];
+    const int width = (int)((a.slice_ptr[(r >> 5) + 1] - base) >> 5);
+    const uint32_t* e = a.ent + base + (r & 31);
     const V xr = src[r];
-    z[r] = s * spmv_row_ro<V>(a.slice_ptr, a.ent, src, r, xr);
-    if (a.pb_a) pbytes += 4ull * row_width(a.slice_ptr, r) + 2ull * sizeof(V);
+    V acc = V(0);
+    int k0 = 0;
+    for (; k0 + A1_P <= width; k0 += A1_P) {
+      uint32_t p[A1_P];
+      V xv[A1_P];
+#pragma unroll
+      for (int i = 0; i < A1_P; ++i) p[i] = __ldcs(e + 32 * (k0 + i));
+#pragma unroll
+      for (int i = 0; i < A1_P; ++i) xv[i] = __ldg(src + ent_col(p[i]));
+#pragma unroll
+      for (int i = 0; i < A1_P; ++i) acc += V(ent_w(p[i])) * (xr - xv[i]);
+    }
+    if (k0 < width) {
+      uint32_t p[A1_P];
+      V xv[A1_P];
+#pragma unroll
+      for (int i = 0; i < A1_P; ++i) p[i] = k0 + i < width ? __ldcs(e + 32 * (k0 + i)) : 0u;
+#pragma unroll
+      for (int i = 0; i < A1_P; ++i) xv[i] = k0 + i < width ? __ldg(src + ent_col(p[i])) : xr;
+#pragma unroll
+      for (int i = 0; i < A1_P; ++i)
+        if (k0 + i < width) acc += V(ent_w(p[i])) * (xr - xv[i]);
+    }
+    a.AP[r] = s * acc;
+    if (a.pb_a) pbytes += 4ull * width + 2ull * sizeof(V);
   }
   if (a.pb_a) prof_add(a.pb_a, pbytes);
 }
@@ -620,7 +565,7 @@ __device__ __forceinline__ void d2_store_S(double* Sm, int j, const double* sc, 
 // step, DCGS2: Swirydowicz, Langou, Ananthan, Yang and Thomas, "Low
 // synchronization Gram-Schmidt and GMRES algorithms", 2020).  v = src / nu_j
 // has been projected once against B = [u0, D, q_0..q_{j-1}]; z = L v (D1).
-// One staged pass over q_0..q_{j-1}, src and z takes a = B^T v, g = B^T z,
+// One pass over q_0..q_{j-1}, src and z takes a = B^T v, g = B^T z,
 // v.v and v.z; k_lz_close then forms
 //   rho = sqrt(v.v - a.a)                  q_j = (v - B a) / rho
 //   L q_j = (z - L B a) / rho, where L B a lies in span(B, q_j) up to
@@ -631,81 +576,117 @@ __device__ __forceinline__ void d2_store_S(double* Sm, int j, const double* sc, 
 // and the coefficients of D3.  Partials: [a_b (b < nb), v.v] then
 // [g_b (b < nb), v.z], nb = 1 + nd + j.
 // ----------------------------------------------------------------------------
+// A basis value is used by one coefficient only, so nothing is staged: a warp owns
+// up to D2_CPW coefficients (c = w + W i of the W warps the launch gives a tile) and
+// streams their vectors through registers, D2_RG rows a lane at a time, with no CTA
+// barrier anywhere; v and z, which every warp reads, come from L1.  A lane adds the
+// rows lane, lane + 32, ... of the tile in order, whatever W is.
+// Bound: HBM and L2 (es (j + 2) bytes a row), with the issue slots half busy (10 FP32
+// instructions per coefficient and row).  At 3.7M rows, mean over j, 74 us, of which
+// the bytes take 58; with chunks of the basis staged in shared memory by bulk copies
+// (four CTAs of 8 warps per SM, two barriers a chunk) 97 us; three coefficients a warp
+// 75 us, four 98 us.
+#define D2_CPW 2
+#define D2_RG 4
+#define D2_MAXTHREADS (32 * ((RSB_MAXC + D2_CPW - 1) / D2_CPW))
+static inline int d2_threads(int nc) { return 32 * ((nc + D2_CPW - 1) / D2_CPW); }
+
+// One warp's NC coefficients over the tile's rows (r0: the lane's first row).  SP:
+// some are u0 (kind 1) or FP64 deflation vectors (kind 2), not vectors in V.
+template <typename V, int NC, bool SP>
+__device__ __forceinline__ void d2_rows(const V* const (&q)[D2_CPW], const int (&kind)[D2_CPW],
+                                        const double* const (&d)[D2_CPW], const V* v, const V* z,
+                                        int r, int row1, Acc<V> (&av)[D2_CPW],
+                                        Acc<V> (&az)[D2_CPW]) {
+  // (r + 32 (D2_RG - 1) < row1 for every lane: the bound is the warp's first row)
+  const int lane = threadIdx.x & 31;
+  for (; r - lane + 32 * D2_RG <= row1; r += 32 * D2_RG) {
+    V vs[D2_RG], zs[D2_RG], qs[NC][D2_RG];
+#pragma unroll
+    for (int i = 0; i < NC; ++i) {
+      if (!SP || kind[i] == 3) {
+#pragma unroll
+        for (int g = 0; g < D2_RG; ++g) qs[i][g] = q[i][r + 32 * g];
+      } else if (kind[i] == 2) {
+#pragma unroll
+        for (int g = 0; g < D2_RG; ++g) qs[i][g] = V(d[i][r + 32 * g]);
+      } else {
+#pragma unroll
+        for (int g = 0; g < D2_RG; ++g) qs[i][g] = V(1);
+      }
+    }
+#pragma unroll
+    for (int g = 0; g < D2_RG; ++g) {
+      vs[g] = v[r + 32 * g];
+      zs[g] = z[r + 32 * g];
+    }
+#pragma unroll
+    for (int g = 0; g < D2_RG; ++g)
+#pragma unroll
+      for (int i = 0; i < NC; ++i) {
+        av[i].add(qs[i][g] * vs[g]);
+        az[i].add(qs[i][g] * zs[g]);
+      }
+  }
+  for (; r < row1; r += 32) {
+    const V vs = v[r], zs = z[r];
+#pragma unroll
+    for (int i = 0; i < NC; ++i) {
+      const V qs = !SP || kind[i] == 3 ? q[i][r] : kind[i] == 2 ? V(d[i][r]) : V(1);
+      av[i].add(qs * vs);
+      az[i].add(qs * zs);
+    }
+  }
+}
+
 template <typename V>
-__global__ void __launch_bounds__(RSB_BLOCK, 4) k_lz_d2(LzArgs<V> a, int j, GridBar* gb) {
-  extern __shared__ __align__(128) unsigned char d2_sh[];
-  constexpr int AL = BulkRows<V>::AL, CRB = BulkRows<V>::CRB;
-  __shared__ __align__(8) uint64_t bar[ST_NB];
+__global__ void __launch_bounds__(D2_MAXTHREADS, 2) k_lz_d2(LzArgs<V> a, int j) {
   const Tile t = a.tiles[blockIdx.x];
   const Unit& u = a.units[t.unit];
   if (u.status != U_ACTIVE || j >= u.msteps || j < u.j0) return;
-  V* Qb = reinterpret_cast<V*>(d2_sh);  // [ST_NB][j + 2][CRB]: q_0..q_{j-1}, src, z
   const int nd = u.nd;
   const int nb = 1 + nd + j;  // columns of B
   const int nc = nb + 1;      // plus v itself (v.v, v.z)
-  const int nq = j;
-  const int slots = nq + 2;
-  const V* src = (j & 1) ? a.W1 : a.W0;
-  const int nchunk = (t.row1 - t.row0 + ST_CH - 1) / ST_CH;
-  if (threadIdx.x == 0) {
-    for (int b = 0; b < ST_NB; ++b) mbar_init(&bar[b], 1);
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  }
-  __syncthreads();
-  if (threadIdx.x == 0)
-    for (int c = 0; c < min(nchunk, ST_NB - 1); ++c)
-      bulk_issue_chunk(a, Qb, bar, nq, c, t.row0 + c * ST_CH,
-                       min(t.row1, t.row0 + (c + 1) * ST_CH), src, (const V*)a.AP);
-  Acc<V> av[MAXCW], az[MAXCW];
-  unsigned long long pbytes = 0;
-  for (int ci = 0; ci < nchunk; ++ci) {
-    if (threadIdx.x == 0 && ci + ST_NB - 1 < nchunk)
-      stage_chunk(a, Qb, bar, nq, t, ci + ST_NB - 1, src, (const V*)a.AP);
-    if (!staged_wait(bar, ci, nchunk, gb)) return;
-    const int c0 = t.row0 + ci * ST_CH;
-    const int c1 = min(t.row1, c0 + ST_CH);
-    const V* Qc = Qb + (size_t)(ci % ST_NB) * slots * CRB + (c0 - (c0 & ~(AL - 1)));
-    const V* vs = Qc + (size_t)nq * CRB;
-    const V* zs = vs + CRB;
-    const int nr = c1 - c0;
-    if (a.pb_a2 && (int)threadIdx.x < nr)
-      pbytes += sizeof(V) * (unsigned long long)(2 + j) + 8ull * nd;
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, W = blockDim.x >> 5;
+  const V* v = (j & 1) ? a.W1 : a.W0;
+  const V* q[D2_CPW];
+  const double* d[D2_CPW];
+  int kind[D2_CPW];  // 1 ones (u0), 2 FP64 deflation vector, 3 vector
+  bool sp = false;
 #pragma unroll
-    for (int i = 0; i < MAXCW; ++i) {
-      const int c = w + RSB_WARPS * i;
-      if (c < nc) {
-        if (c == 0) {
-          for (int rl = lane; rl < nr; rl += 32) {
-            av[i].add(vs[rl]);
-            az[i].add(zs[rl]);
-          }
-        } else if (c <= nd) {
-          const double* d = c == 1 ? a.D0 : a.D1;
-          for (int rl = lane; rl < nr; rl += 32) {
-            const V dv = V(d[c0 + rl]);
-            av[i].add(dv * vs[rl]);
-            az[i].add(dv * zs[rl]);
-          }
-        } else {
-          const V* q = c < nb ? Qc + (size_t)(c - 1 - nd) * CRB : vs;
-          for (int rl = lane; rl < nr; rl += 32) {
-            const V qv = q[rl];
-            av[i].add(qv * vs[rl]);
-            az[i].add(qv * zs[rl]);
-          }
-        }
-      }
-    }
-    __syncthreads();
+  for (int i = 0; i < D2_CPW; ++i) {
+    const int c = w + W * i;
+    kind[i] = c == 0 ? 1 : c <= nd ? 2 : 3;
+    sp |= kind[i] != 3;
+    d[i] = c == 1 ? a.D0 : a.D1;
+    q[i] = c >= nb ? v : a.Q + (long long)max(c - 1 - nd, 0) * a.N;
   }
-  store_dots<V>(a, nc, av, blockIdx.x);
-  {
-    LzArgs<V> a2 = a;
-    a2.partials = a.partials + (long long)nc * a.stride;
-    store_dots<V>(a2, nc, az, blockIdx.x);
+  const int ncw = (nc - 1 - w) / W + 1;  // this warp's coefficients (W <= nc)
+  Acc<V> av[D2_CPW], az[D2_CPW];
+  const int r0 = t.row0 + lane;
+  if (ncw == 2) {
+    if (sp) d2_rows<V, 2, true>(q, kind, d, v, a.AP, r0, t.row1, av, az);
+    else d2_rows<V, 2, false>(q, kind, d, v, a.AP, r0, t.row1, av, az);
+  } else {
+    if (sp) d2_rows<V, 1, true>(q, kind, d, v, a.AP, r0, t.row1, av, az);
+    else d2_rows<V, 1, false>(q, kind, d, v, a.AP, r0, t.row1, av, az);
   }
-  if (a.pb_a2) prof_add(a.pb_a2, pbytes);
+  __syncwarp();
+  // the warp's sums, converted to FP64 together (lane 2 i: a, lane 2 i + 1: g)
+  V S = V(0), C = V(0);
+#pragma unroll
+  for (int i = 0; i < D2_CPW; ++i) {
+    warp_merge(av[i].s, av[i].c);
+    warp_merge(az[i].s, az[i].c);
+    if (lane == 2 * i) { S = av[i].s; C = av[i].c; }
+    if (lane == 2 * i + 1) { S = az[i].s; C = az[i].c; }
+  }
+  const double sum = (double)S - (double)C;
+  const int c = w + W * (lane >> 1);
+  if (lane < 2 * D2_CPW && c < nc)
+    a.partials[(long long)((lane & 1) ? nc + c : c) * a.stride + blockIdx.x] = sum;
+  if (a.pb_a2 && threadIdx.x == 0)
+    atomicAdd(a.pb_a2, (t.row1 - t.row0) * (sizeof(V) * (unsigned long long)(2 + j) + 8ull * nd));
 }
 
 // ----------------------------------------------------------------------------
@@ -749,10 +730,8 @@ __global__ void __launch_bounds__(RSB_BLOCK) k_lz_close(LzArgs<V> a, int j, int 
   const double* P = a.partials + (long long)c0 * a.stride;
   double* Sm = unit_S(a.S, ui);
   __shared__ double Ss[MODE == CLOSE_D2 ? RSB_MAXM * RSB_MAXM : 1];
-  __shared__ double inu_sh;
   if constexpr (MODE == CLOSE_D2) {
     for (int idx = threadIdx.x; idx < j * RSB_MAXM; idx += RSB_BLOCK) Ss[idx] = Sm[idx];
-    if (threadIdx.x == 0) inu_sh = 1.0 / (j == u.j0 ? u.beta0 : u.beta[j]);
   }
   if (per == 4) {
     final_reduce_few(P, a.stride, u.tile0, nt, n, out, sp);
@@ -788,7 +767,7 @@ __global__ void __launch_bounds__(RSB_BLOCK) k_lz_close(LzArgs<V> a, int j, int 
     }
     __shared__ double sc[3], sk[RSB_MAXM];
     __syncthreads();
-    const double inu = inu_sh;
+    const double inu = u.inu;
     d2_finish(out, out + nc, nb, nd, j, inu, u.isn, Ss, sc, sk);
     d2_store_S(Sm, j, sc, sk);
     const double rho = sc[0];
@@ -815,105 +794,106 @@ __global__ void __launch_bounds__(RSB_BLOCK) k_lz_close(LzArgs<V> a, int j, int 
 // w_{j+1} = z / rho - B g~ - (q_j.z / rho) q_j (a~ = a / rho, g~ = g / rho;
 // one pass over the basis, two updates per loaded value); q_j goes to the
 // basis, w_{j+1} to the other work vector, nu_{j+1} = ||w_{j+1}||.
+// Bound: HBM and L2 (es (j + 4) bytes a row).  32 registers, so that eight CTAs
+// (all 64 warps of an SM) hold loads in flight and 1216 tiles run at once: 81 us at
+// 3.7M rows in 973 tiles, mean over j, of which the bytes take 62; with 16 loads a
+// thread, 48 registers and five CTAs the last, nearly empty wave of tiles made it 106.
+// The tiles are taken in the opposite order of D2, which has just streamed the same
+// vectors: what it read last is still in L2 (4 % at 1M rows, nothing at 3.7M).
+#define D3_KB 4  // basis vectors a round
+#define D3_RR 2  // rows a thread
 template <typename V>
-__global__ void __launch_bounds__(RSB_BLOCK) k_lz_d3(LzArgs<V> a, int j, double breakdown) {
+__global__ void __launch_bounds__(RSB_BLOCK, 8) k_lz_d3(LzArgs<V> a, int j, double breakdown) {
   __shared__ double sm[RSB_WARPS];
-  __shared__ V ca[RSB_MAXC], cg[RSB_MAXC];
+  __shared__ __align__(16) V cc[RSB_MAXC][2];  // a~, g~
   __shared__ double out[1];
   __shared__ double sp[RED_FEW_DOUBLES(1)];
-  const Tile t = a.tiles[blockIdx.x];
+  const int tix = gridDim.x - 1 - blockIdx.x;
+  const Tile t = a.tiles[tix];
   Unit& u = a.units[t.unit];
   if (u.status != U_ACTIVE || j >= u.msteps || j < u.j0) return;
   const int nd = u.nd;
   const int nb = 1 + nd + j;
-  stage_coef<V, false>(u.c2, nb, u.isn, ca);
-  stage_coef<V, false>(u.c1, nb, u.isn, cg);
+  for (int k = threadIdx.x; k < nb; k += RSB_BLOCK) {
+    const double x = u.c2[k], y = u.c1[k];
+    cc[k][0] = k == 0 ? V(x * u.isn) : V(x);
+    cc[k][1] = k == 0 ? V(y * u.isn) : V(y);
+  }
+  __syncthreads();
   const V ssrc = V(u.dz_src), sz = V(u.dz_z), sqz = V(u.dz_qz);
   const V* src = (j & 1) ? a.W1 : a.W0;
   V* dst = (j & 1) ? a.W0 : a.W1;
-  const V* z = a.AP;
-  V* qj = a.Q + (long long)j * a.N;
   Acc<V> acc;
-  unsigned long long pbytes = 0;
-  for (int base = t.row0; base < t.row1; base += SUBROWS) {
-    const int end = min(t.row1, base + SUBROWS);
-    V q[RSB_SUBR], w[RSB_SUBR];
-    bool ok[RSB_SUBR];
+  for (int r0 = t.row0 + threadIdx.x; r0 < t.row1; r0 += D3_RR * RSB_BLOCK) {
+    V q[D3_RR], w[D3_RR];
+    bool ok[D3_RR];
 #pragma unroll
-    for (int rr = 0; rr < RSB_SUBR; ++rr) {
-      const int r = base + rr * RSB_BLOCK + threadIdx.x;
-      ok[rr] = r < end;
+    for (int rr = 0; rr < D3_RR; ++rr) {
+      const int r = r0 + rr * RSB_BLOCK;
+      ok[rr] = r < t.row1;
       q[rr] = ok[rr] ? ssrc * src[r] : V(0);
-      w[rr] = ok[rr] ? sz * z[r] : V(0);
+      w[rr] = ok[rr] ? sz * a.AP[r] : V(0);
       if (ok[rr] && unit_has(u, a.ckey, r)) {
-        q[rr] -= ca[0];
-        w[rr] -= cg[0];
+        q[rr] -= cc[0][0];
+        w[rr] -= cc[0][1];
       }
     }
     for (int l = 0; l < nd; ++l) {
-      const double* d = l == 0 ? a.D0 : a.D1;
+      const double* d = (l == 0 ? a.D0 : a.D1) + r0;
 #pragma unroll
-      for (int rr = 0; rr < RSB_SUBR; ++rr) {
-        const int r = base + rr * RSB_BLOCK + threadIdx.x;
+      for (int rr = 0; rr < D3_RR; ++rr)
         if (ok[rr]) {
-          const V dv = V(d[r]);
-          q[rr] -= ca[1 + l] * dv;
-          w[rr] -= cg[1 + l] * dv;
+          const V dv = V(d[rr * RSB_BLOCK]);
+          q[rr] -= cc[1 + l][0] * dv;
+          w[rr] -= cc[1 + l][1] * dv;
         }
-      }
     }
-    const V* cqa = ca + 1 + nd;
-    const V* cqg = cg + 1 + nd;
+    const V* qk = a.Q + r0;
+    const V(*ck)[2] = cc + 1 + nd;
     int k = 0;
-    for (; k + 4 <= j; k += 4) {  // four basis vectors per round
-      V qv[4][RSB_SUBR];
+    for (; k + D3_KB <= j; k += D3_KB, qk += D3_KB * a.N, ck += D3_KB) {
+      V qv[D3_KB][D3_RR];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const V* qk = a.Q + (long long)(k + i) * a.N + base + threadIdx.x;
+      for (int i = 0; i < D3_KB; ++i)
 #pragma unroll
-        for (int rr = 0; rr < RSB_SUBR; ++rr) qv[i][rr] = ok[rr] ? qk[rr * RSB_BLOCK] : V(0);
-      }
+        for (int rr = 0; rr < D3_RR; ++rr)
+          qv[i][rr] = ok[rr] ? qk[i * a.N + rr * RSB_BLOCK] : V(0);
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const V ka = cqa[k + i], kg = cqg[k + i];
+      for (int i = 0; i < D3_KB; ++i)
 #pragma unroll
-        for (int rr = 0; rr < RSB_SUBR; ++rr) {
-          q[rr] -= ka * qv[i][rr];
-          w[rr] -= kg * qv[i][rr];
+        for (int rr = 0; rr < D3_RR; ++rr) {
+          q[rr] -= ck[i][0] * qv[i][rr];
+          w[rr] -= ck[i][1] * qv[i][rr];
         }
-      }
     }
-    for (; k < j; ++k) {
-      const V ka = cqa[k], kg = cqg[k];
-      const V* qk = a.Q + (long long)k * a.N + base + threadIdx.x;
+    for (; k < j; ++k, qk += a.N, ++ck)
 #pragma unroll
-      for (int rr = 0; rr < RSB_SUBR; ++rr)
+      for (int rr = 0; rr < D3_RR; ++rr)
         if (ok[rr]) {
           const V b = qk[rr * RSB_BLOCK];
-          q[rr] -= ka * b;
-          w[rr] -= kg * b;
+          q[rr] -= ck[0][0] * b;
+          w[rr] -= ck[0][1] * b;
         }
-    }
 #pragma unroll
-    for (int rr = 0; rr < RSB_SUBR; ++rr) {
-      const int r = base + rr * RSB_BLOCK + threadIdx.x;
+    for (int rr = 0; rr < D3_RR; ++rr)
       if (ok[rr]) {
+        const int r = r0 + rr * RSB_BLOCK;
         w[rr] -= sqz * q[rr];
-        qj[r] = q[rr];
+        a.Q[(long long)j * a.N + r] = q[rr];
         dst[r] = w[rr];
         acc.add(w[rr] * w[rr]);
-        if (a.pb_b) pbytes += sizeof(V) * (unsigned long long)(4 + j) + 8ull * nd;
       }
-    }
   }
-  if (a.pb_b) prof_add(a.pb_b, pbytes);
+  if (a.pb_b && threadIdx.x == 0)
+    atomicAdd(a.pb_b, (t.row1 - t.row0) * (sizeof(V) * (unsigned long long)(4 + j) + 8ull * nd));
   const double sum = block_total(acc, sm);
-  if (threadIdx.x == 0) a.partials[blockIdx.x] = sum;
+  if (threadIdx.x == 0) a.partials[tix] = sum;
   if (last_cta(&u.cnt, u.ntile)) {
     final_reduce_few(a.partials, a.stride, u.tile0, u.ntile, 1, out, sp);
     if (threadIdx.x == 0) {
       const double b = sqrt(out[0]);
       u.beta[j + 1] = b;
+      u.inu = 1.0 / b;
       if (b <= breakdown * u.dmax) {  // invariant subspace: the cycle ends here
         u.msteps = j + 1;
         u.broke = 1;
@@ -1285,6 +1265,7 @@ __device__ __forceinline__ void lz_resid_t(const LzArgs<V>& a, const V* y, int m
           // thick restart: the kept Ritz vectors occupy q_0..q_{kk-1}; the next
           // cycle starts at step kk from the residual direction
           u.beta0 = u.beta[u.msteps];
+          u.inu = 1.0 / u.beta0;
           u.j0 = u.kk;
           u.msteps = u.m;
           atomicMin(a.jmin, u.kk);
@@ -1373,6 +1354,7 @@ __device__ __forceinline__ void proj3_t(const LzArgs<V>& a, const V* y, int tix,
     final_reduce_few(a.partials, a.stride, u.tile0, u.ntile, 1, out, sp);
     if (threadIdx.x == 0) {
       u.beta0 = sqrt(out[0]);
+      u.inu = 1.0 / u.beta0;
       u.msteps = u.m;
       u.broke = 0;
     }
@@ -1796,7 +1778,7 @@ __global__ void __launch_bounds__(RSB_BLOCK, 2)
     int msteps = __ldcg(&u.msteps);
     if (threadIdx.x == 0) {
       beta_sh = __ldcg(&u.beta0);
-      inu_sh = 1.0 / beta_sh;
+      inu_sh = __ldcg(&u.inu);
       scale_sh = V(inu_sh);
     }
     // every CTA of the unit keeps its own copy of S during the steps
@@ -2048,10 +2030,10 @@ static int lz_start(LzArgs<V>& a, int ntiles, uint64_t sd, const double* from64,
 }
 
 template <typename V>
-static int lz_cycle(LzArgs<V>& a, int ntiles, int nunits, int M, double breakdown, GridBar* gb,
-                    int trmax, int ntmax, int nd, cudaStream_t s) {
-  // CTAs per tile of step A1
-  const int nsub = std::max(1, (trmax + A1_RPT * RSB_BLOCK - 1) / (A1_RPT * RSB_BLOCK));
+static int lz_cycle(LzArgs<V>& a, int ntiles, int nunits, int M, double breakdown, int trmax,
+                    int ntmax, int nd, cudaStream_t s) {
+  // CTAs per tile of step D1
+  const int nsub = std::max(1, (trmax + A1_ROWS - 1) / A1_ROWS);
   for (int j = 0; j < M; ++j) {
     int pi = prof_before(PROF_LZ_A, s);
     if constexpr (sizeof(V) == 4) {  // FP32: bandwidth-bound; CGS2 with the second pass delayed
@@ -2059,7 +2041,7 @@ static int lz_cycle(LzArgs<V>& a, int ntiles, int nunits, int M, double breakdow
       RSB_CKL("k_lz_a1");
       prof_after(pi, s);
       pi = prof_before(PROF_LZ_A2, s);
-      k_lz_d2<V><<<ntiles, RSB_BLOCK, staged_smem<V>(j + 2), s>>>(a, j, gb);
+      k_lz_d2<V><<<ntiles, d2_threads(2 + nd + j), 0, s>>>(a, j);
       RSB_CKL("k_lz_d2");
       const int G = close_ctas(ntmax, close_ncoef<CLOSE_D2>(nd, j));
       k_lz_close<V, CLOSE_D2><<<nunits * G, RSB_BLOCK, 0, s>>>(a, j, G);
@@ -2109,7 +2091,7 @@ static int lanczos_run(const LevelGraph& G, const Tile* tiles, int ntiles, Unit*
                        const double* from64, const float* from32, int use_graph,
                        cudaStream_t s) {
   LzArgs<V> a = make_args<V>(G, tiles, ntiles, units, ckey, B);
-  // step A1 and the resident kernel size their launches by the largest tile
+  // step D1 and the resident kernel size their launches by the largest tile
   if (B.trmax <= 0) return rsb_set_error(RSB_EINVAL, "Lanczos solve without its largest tile size");
   int active = 0;
   int rc = read_active(B, s, &active);
@@ -2183,23 +2165,13 @@ static int lanczos_run(const LevelGraph& G, const Tile* tiles, int ntiles, Unit*
     }
     return rc;
   }
-  // the staged step D2 (FP32) needs up to 2 * (M + 1) * (RSB_BLOCK + 4) floats of
-  // dynamic shared memory (85 KB at M = 40)
-  if constexpr (sizeof(V) == 4) {
-    RSB_CK(cudaFuncSetAttribute(k_lz_d2<V>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)staged_smem<V>(M + 1)));
-    // the whole carveout as shared memory: D2 is bound by the CTAs per SM that
-    // its staged chunks leave room for (two at the default carveout)
-    RSB_CK(cudaFuncSetAttribute(k_lz_d2<V>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                cudaSharedmemCarveoutMaxShared));
-  }
   cudaGraphExec_t exec = nullptr;
   std::vector<int> cap_pairs;
   if (use_graph) {
     cudaGraph_t graph = nullptr;
     RSB_CK(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
     prof_capture_begin();
-    rc = lz_cycle<V>(a, ntiles, nunits, M, breakdown, B.gb, B.trmax, B.ntmax, nd, s);
+    rc = lz_cycle<V>(a, ntiles, nunits, M, breakdown, B.trmax, B.ntmax, nd, s);
     cap_pairs = prof_capture_end();
     cudaGraph_t g2 = nullptr;
     cudaError_t e = cudaStreamEndCapture(s, &g2);
@@ -2226,7 +2198,7 @@ static int lanczos_run(const LevelGraph& G, const Tile* tiles, int ntiles, Unit*
       }
       prof_replay(cap_pairs);
     } else {
-      rc = lz_cycle<V>(a, ntiles, nunits, M, breakdown, B.gb, B.trmax, B.ntmax, nd, s);
+      rc = lz_cycle<V>(a, ntiles, nunits, M, breakdown, B.trmax, B.ntmax, nd, s);
       if (rc) return rc;
     }
     rc = read_active(B, s, &active);
@@ -2653,7 +2625,7 @@ static int inverse_run(const LevelGraph& G, const Tile* tiles, int ntiles, Unit*
                        int use_graph, int64_t* inner_out, cudaStream_t s,
                        const std::vector<Unit>* amg_units) {
   LzArgs<V> a = make_args<V>(G, tiles, ntiles, units, ckey, B);
-  // step A1 and the resident kernel size their launches by the largest tile
+  // step D1 and the resident kernel size their launches by the largest tile
   if (B.trmax <= 0) return rsb_set_error(RSB_EINVAL, "Lanczos solve without its largest tile size");
   int active = 0;
   int rc = read_active(B, s, &active);
