@@ -115,6 +115,7 @@ struct Unit {
   int32_t best;
   int32_t ncand;
   unsigned int cnt;      // last-CTA counter of the segmented reductions
+  unsigned int gbar;     // arrivals at the unit's barrier (resident solve)
   int32_t axis;          // RCB: coordinate axis of the split
 };
 
@@ -281,6 +282,52 @@ __device__ __forceinline__ void warp_merge(float& s, float& c) {  // result in e
     s = S;
   }
 }
+// One butterfly step on the upper half of an array of 2 H accumulators: a lane keeps
+// the first or the second H by its bit o and merges them with its partner's, so that
+// the sums of 2 H accumulators cost 2 H - 1 merges a lane for the first steps.  Every
+// accumulator sees the merges of warp_merge in its order.
+template <int H>
+__device__ __forceinline__ void warp_merge_half(float* s, float* c, int o) {
+  const bool up = (threadIdx.x & o) != 0;
+#pragma unroll
+  for (int i = 0; i < H; ++i) {
+    const float s1 = up ? s[H + i] : s[i], c1 = up ? c[H + i] : c[i];
+    const float ss = up ? s[i] : s[H + i], cs = up ? c[i] : c[H + i];
+    const float s2 = __shfl_xor_sync(0xffffffffu, ss, o);
+    const float c2 = __shfl_xor_sync(0xffffffffu, cs, o);
+    const float S = __fadd_rn(s1, s2);
+    const float bb = __fsub_rn(S, s1);
+    const float e = __fadd_rn(__fsub_rn(s1, __fsub_rn(S, bb)), __fsub_rn(s2, bb));
+    c[i] = __fsub_rn(__fadd_rn(c1, c2), e);
+    s[i] = S;
+  }
+}
+// The warp's sums of 4 or 16 accumulators (s, c): accumulator k's total comes back in
+// the lane whose bits 16, 8 (, 4, 2), highest first, spell k (bits below: any).
+template <int N>
+__device__ __forceinline__ double warp_totals(float (&s)[N], float (&c)[N]) {
+  static_assert(N == 4 || N == 16, "");
+  if constexpr (N == 16) {
+    warp_merge_half<8>(s, c, 16);
+    warp_merge_half<4>(s, c, 8);
+    warp_merge_half<2>(s, c, 4);
+    warp_merge_half<1>(s, c, 2);
+  } else {
+    warp_merge_half<2>(s, c, 16);
+    warp_merge_half<1>(s, c, 8);
+  }
+#pragma unroll
+  for (int o = N == 16 ? 1 : 4; o > 0; o >>= 1) {
+    const float s2 = __shfl_xor_sync(0xffffffffu, s[0], o);
+    const float c2 = __shfl_xor_sync(0xffffffffu, c[0], o);
+    const float S = __fadd_rn(s[0], s2);
+    const float bb = __fsub_rn(S, s[0]);
+    const float e = __fadd_rn(__fsub_rn(s[0], __fsub_rn(S, bb)), __fsub_rn(s2, bb));
+    c[0] = __fsub_rn(__fadd_rn(c[0], c2), e);
+    s[0] = S;
+  }
+  return (double)s[0] - (double)c[0];
+}
 __device__ __forceinline__ double warp_total(const Acc<float>& a) {
   float s = a.s, c = a.c;
   warp_merge(s, c);
@@ -397,6 +444,58 @@ __device__ __forceinline__ bool grid_sync(GridBar* b, unsigned nblocks) {
   return s_ok != 0;
 }
 
+// Barrier of the CTAs of one unit inside a co-resident launch: thread 0 of each CTA
+// adds its arrival (release) to a counter that only grows and waits (acquire) until
+// the round's arrivals are complete, so a barrier costs one fire-and-forget addition
+// and the polls; a CTA that is alone takes the CTA barrier.  Units do not wait for one
+// another.  The wait is bounded as grid_sync's is.  base: the counter's start, zero
+// but for the failure-path test, which puts it out of reach.
+struct UnitBar {
+  unsigned* p;
+  unsigned n, target;
+  GridBar* gb;
+  bool alone;
+  __device__ __forceinline__ UnitBar(unsigned* counter, unsigned ntile, unsigned base, GridBar* g)
+      : p(counter), n(ntile), target(base), gb(g), alone(ntile == 1 && base == 0) {}
+  __device__ __forceinline__ void arrive() {
+    __syncthreads();
+    if (!alone && threadIdx.x == 0)
+      asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(1u) : "memory");
+  }
+  __device__ __forceinline__ bool wait() {
+    __shared__ int s_ok;
+    target += n;
+    if (!alone) {
+      if (threadIdx.x == 0) {
+        bool ok = true;
+        unsigned spins = 0;
+        unsigned long long t0 = 0;
+        while ((int)(ld_acquire(p) - target) < 0) {
+          if ((++spins & 255u) == 0) {
+            const unsigned long long now = global_ns();
+            if (t0 == 0) t0 = now;
+            if (*(volatile int*)&gb->err) ok = false;
+            else if (now - t0 > 4000000000ull) {
+              atomicExch(&gb->err, 1);
+              ok = false;
+            }
+            if (!ok) break;
+          }
+        }
+        s_ok = ok;
+      }
+      __syncthreads();
+      return s_ok != 0;
+    }
+    __syncthreads();
+    return true;
+  }
+  __device__ __forceinline__ bool sync() {
+    arrive();
+    return wait();
+  }
+};
+
 // Loads of data another CTA may have written earlier in the same launch go
 // through L2 (L1 is not coherent across SMs).
 template <bool CO, typename T>
@@ -494,6 +593,49 @@ __device__ __forceinline__ void final_reduce_few(const double* partials, long lo
     acc += __shfl_xor_sync(0xffffffffu, acc, 2);
     acc += __shfl_xor_sync(0xffffffffu, acc, 1);
     if (s == 0) out[c] = acc;
+  }
+  __syncthreads();
+}
+
+// final_reduce for a unit of at most RED_SMALL tiles, for any number of coefficients:
+// eight lanes of the CTA per coefficient, all of a lane's tiles loaded at once; the
+// same sums in the same order.
+#define RED_SMALL 96
+__device__ __forceinline__ void final_reduce_small(const double* partials, long long stride, int t0,
+                                                   int nt, int nc, double* out) {
+  const int s = threadIdx.x & 7;
+  const int nq = (nt + 31) >> 5;
+  for (int cb = 0; cb < nc; cb += RSB_BLOCK / 8) {
+    const int c = cb + (threadIdx.x >> 3);
+    if ((c & ~3) >= nc) break;  // no coefficient of this warp is left
+    const bool on = c < nc;
+    const double* p = partials + (long long)(on ? c : 0) * stride + t0;
+    double v[RED_SMALL / 8];
+#pragma unroll
+    for (int q = 0; q < RED_SMALL / 32; ++q)
+      if (q < nq) {
+#pragma unroll
+        for (int i = 4 * q; i < 4 * q + 4; ++i) v[i] = s + 8 * i < nt ? __ldcg(p + s + 8 * i) : 0.0;
+      }
+    double acc = v[0];
+    if (nt > 8) {
+#pragma unroll
+      for (int q = 0; q < RED_SMALL / 32; ++q)
+        if (q < nq) {
+          if (s + 32 * q + 24 < nt) {
+            const double x = (v[4 * q] + v[4 * q + 1]) + (v[4 * q + 2] + v[4 * q + 3]);
+            acc = q == 0 ? x : acc + x;
+          } else {
+#pragma unroll
+            for (int i = q == 0 ? 1 : 4 * q; i < 4 * q + 4; ++i)
+              if (s + 8 * i < nt) acc += v[i];
+          }
+        }
+    }
+    if (nt > 4) acc += __shfl_xor_sync(0xffffffffu, acc, 4);
+    acc += __shfl_xor_sync(0xffffffffu, acc, 2);
+    acc += __shfl_xor_sync(0xffffffffu, acc, 1);
+    if (on && s == 0) out[c] = acc;
   }
   __syncthreads();
 }

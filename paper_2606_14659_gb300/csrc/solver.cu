@@ -488,8 +488,8 @@ __global__ void __launch_bounds__(RSB_BLOCK, 5) k_lz_a1(LzArgs<V> a, int j, int 
 // Closing arithmetic of step D2 for one unit (every thread of the CTA takes
 // part), from the reduced totals av = [a_b (b < nb), v.v] and gz = [g_b
 // (b < nb), v.z] of src, scaled here in place to v = src / nu (inu = 1 / nu)
-// and u0 = 1/sqrt(n) on its entry; sc[0..2] = rho, q_j.z, alpha and
-// sk[0..j) = S_kj come back in shared memory.  Ss: columns < j of S (row k at
+// and u0 = 1/sqrt(n) on its entry; sc[0..1] = rho, q_j.z and sk[0..j) = S_kj come
+// back in shared memory (sk to be read after a CTA barrier, sc at once).  Ss: columns < j of S (row k at
 // k * RSB_MAXM; S is symmetric).  The streaming kernel and the resident kernel
 // both call this, so both modes produce the same numbers.
 // On GB300 an FP64 warp instruction holds its SM sub-partition for 64 cycles
@@ -539,24 +539,24 @@ __device__ __forceinline__ void d2_finish(double* av, double* gz, int nb, int nd
     if (k < j && part == 0) sk[k] = gz[1 + nd + k] - sa;
   }
   __syncthreads();
-  const double rho = sc[0];
-  if (tid < j) sk[tid] = sk[tid] / rho;
-  __syncthreads();
-  if (w == 7) {
-    double sig = 0.0;
-    for (int k = lane; k < j; k += 32) sig = fma(sk[k], aq[k], sig);
-    sig = warp_sum(sig);
-    if (lane == 0) sc[2] = (sc[1] - sig) / rho;
-  }
-  __syncthreads();
+  if (tid < j) sk[tid] = sk[tid] / sc[0];
 }
 
-// Column and row j of S from the finished step D2.
-__device__ __forceinline__ void d2_store_S(double* Sm, int j, const double* sc, const double* sk) {
-  for (int k = threadIdx.x; k <= j; k += RSB_BLOCK) {
-    const double v = k < j ? sk[k] : sc[2];
-    Sm[k * RSB_MAXM + j] = v;
-    Sm[j * RSB_MAXM + k] = v;
+// alpha = S_jj after d2_finish and a CTA barrier, by one warp (valid in every lane):
+// nothing of the step waits for it.
+__device__ __forceinline__ double d2_alpha(const double* av, int nd, int j, const double* sc,
+                                           const double* sk) {
+  const double* aq = av + 1 + nd;
+  double sig = 0.0;
+  for (int k = threadIdx.x & 31; k < j; k += 32) sig = fma(sk[k], aq[k], sig);
+  return (sc[1] - warp_sum(sig)) / sc[0];
+}
+
+// Entries k < j of column and row j of S from the finished step D2.
+__device__ __forceinline__ void d2_store_S(double* Sm, int j, const double* sk) {
+  for (int k = threadIdx.x; k < j; k += RSB_BLOCK) {
+    Sm[k * RSB_MAXM + j] = sk[k];
+    Sm[j * RSB_MAXM + k] = sk[k];
   }
 }
 
@@ -672,19 +672,12 @@ __global__ void __launch_bounds__(D2_MAXTHREADS, 2) k_lz_d2(LzArgs<V> a, int j) 
     else d2_rows<V, 1, false>(q, kind, d, v, a.AP, r0, t.row1, av, az);
   }
   __syncwarp();
-  // the warp's sums, converted to FP64 together (lane 2 i: a, lane 2 i + 1: g)
-  V S = V(0), C = V(0);
-#pragma unroll
-  for (int i = 0; i < D2_CPW; ++i) {
-    warp_merge(av[i].s, av[i].c);
-    warp_merge(az[i].s, az[i].c);
-    if (lane == 2 * i) { S = av[i].s; C = av[i].c; }
-    if (lane == 2 * i + 1) { S = az[i].s; C = az[i].c; }
-  }
-  const double sum = (double)S - (double)C;
-  const int c = w + W * (lane >> 1);
-  if (lane < 2 * D2_CPW && c < nc)
-    a.partials[(long long)((lane & 1) ? nc + c : c) * a.stride + blockIdx.x] = sum;
+  // the warp's sums, converted to FP64 together
+  float S[4] = {av[0].s, az[0].s, av[1].s, az[1].s}, C[4] = {av[0].c, az[0].c, av[1].c, az[1].c};
+  const double sum = warp_totals<4>(S, C);
+  const int k = lane >> 3, c = w + W * (k >> 1);
+  if ((lane & 7) == 0 && c < nc)
+    a.partials[(long long)((k & 1) ? nc + c : c) * a.stride + blockIdx.x] = sum;
   if (a.pb_a2 && threadIdx.x == 0)
     atomicAdd(a.pb_a2, (t.row1 - t.row0) * (sizeof(V) * (unsigned long long)(2 + j) + 8ull * nd));
 }
@@ -765,17 +758,15 @@ __global__ void __launch_bounds__(RSB_BLOCK) k_lz_close(LzArgs<V> a, int j, int 
       for (int c = threadIdx.x; c < ncoef; c += RSB_BLOCK)
         out[c] = __ldcg(c < nc ? u.c2 + c : u.c1 + (c - nc));
     }
-    __shared__ double sc[3], sk[RSB_MAXM];
+    __shared__ double sc[2], sk[RSB_MAXM];
     __syncthreads();
     const double inu = u.inu;
     d2_finish(out, out + nc, nb, nd, j, inu, u.isn, Ss, sc, sk);
-    d2_store_S(Sm, j, sc, sk);
     const double rho = sc[0];
     // D3: q_j = src / (nu rho) - sum_b (a_b / rho) b,
     //     w = z / rho - sum_b (g_b / rho) b - (q_j.z / rho) q_j
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (w == 4) {
-      if (lane == 0) u.alpha[j] = sc[2];
       const double x = (lane == 0 ? inu : lane == 1 ? 1.0 : sc[1]) / rho;
       if (lane == 0) u.dz_src = x;
       if (lane == 1) u.dz_z = x;
@@ -786,6 +777,15 @@ __global__ void __launch_bounds__(RSB_BLOCK) k_lz_close(LzArgs<V> a, int j, int 
     } else if (w < 4) {
       const int b = threadIdx.x - 64;
       if (b < nb) u.c1[b] = out[nc + b] / rho;
+    }
+    __syncthreads();
+    d2_store_S(Sm, j, sk);
+    if (w == 7) {
+      const double alpha = d2_alpha(out, nd, j, sc, sk);
+      if (lane == 0) {
+        u.alpha[j] = alpha;
+        Sm[j * RSB_MAXM + j] = alpha;
+      }
     }
   }
 }
@@ -1459,6 +1459,16 @@ __host__ __device__ constexpr size_t res_smem_bytes(int M, int trs) {
          res_align(sizeof(V) * RSB_MAXD * (size_t)trs) + sizeof(V) * (size_t)M * (size_t)trs;
 }
 
+// What bounds a step here is latency: a chain of L2 round trips (SpMV, partials, two
+// or three barriers) and of FP64 operations, each of which holds an SM sub-partition
+// for 64 cycles.  So units synchronise on their own barriers and run their cycles
+// independently of one another; FP64 work is done by whole warps, once (the closing
+// divisions of a step used to be done by every warp: 1.7 us); S_jj, which nothing
+// waits for, is computed while the norms travel; a unit of one tile exchanges nothing
+// through global memory but the SpMV operand.  FP32 step of the 512-row mesh 21.5 ->
+// about 11 us, the 131072-row box into 64 parts 167 -> 113 ms, the 512-row box into 8
+// parts 19.8 -> 13.7 ms.
+//
 // Dots of [1, D, q_0..] with the tile's w: the coefficient split across warps
 // and the per-lane row order of tile_dots.
 template <typename V>
@@ -1496,31 +1506,59 @@ __device__ __forceinline__ V res_upd_row(const V* cv, int nd, int nq, const V* Q
   return w;
 }
 
+// (out: where the dots of a unit of one tile go, else null)
 template <typename V>
 __device__ __forceinline__ void res_store_dots(double* P, long long stride, int nc,
-                                               Acc<V> (&acc)[MAXCW], int tix) {
+                                               Acc<V> (&acc)[MAXCW], int tix, double* out) {
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
 #pragma unroll
   for (int i = 0; i < MAXCW; ++i) {
     const int c = w + RSB_WARPS * i;
     if (c < nc) {
       const double s = warp_total(acc[i]);
-      if (lane == 0) P[(long long)c * stride + tix] = s;
+      if (lane == 0) {
+        if (out) out[c] = s;
+        else P[(long long)c * stride + tix] = s;
+      }
     }
   }
 }
 
-// The step phases write per-tile partials into P; after the grid barrier
-// every CTA of the unit reduces them itself (fixed order, so all CTAs hold
-// the same coefficients), which takes the last-CTA ticket and the staging of
-// the coefficients off the critical path.  Consecutive phases alternate
-// between two partial buffers: a buffer is rewritten only after a barrier
-// that follows every CTA's reduction of its previous contents.
+// The step phases write per-tile partials into P; after the unit's barrier every CTA
+// of the unit holds the same totals.  Consecutive phases alternate between partial
+// buffers: a buffer is rewritten only after a barrier that follows every CTA's
+// reduction of its previous contents.
 //
+// Totals of ncoef coefficients of the unit in out (shared memory).  One tile: the
+// dots are in out already.  Up to RED_SMALL tiles every CTA reduces them itself (at 96
+// tiles the additions take as long as a barrier); above, coefficient c is summed by
+// CTA c of the unit alone, and the totals (in tot, ncoef doubles of the unit) are
+// exchanged over one more barrier (256 tiles reduced by every CTA took 14.5 us).
+__device__ __forceinline__ bool res_totals(const double* P, long long stride, const Unit& u, int tix,
+                                           int ncoef, double* out, double* tot, double* scratch,
+                                           UnitBar& ub) {
+  const int nt = u.ntile;
+  if (nt == 1) return true;
+  if (nt <= RED_SMALL) {
+    final_reduce_small(P, stride, u.tile0, nt, ncoef, out);
+    return true;
+  }
+  // (nt > 96 >= ncoef: every CTA has at most one)
+  const int c = tix - u.tile0;
+  if (c < ncoef) {
+    final_reduce_few(P + (long long)c * stride, stride, u.tile0, nt, 1, out, scratch);
+    if (threadIdx.x == 0) tot[c] = out[0];
+  }
+  if (!ub.sync()) return false;
+  for (int k = threadIdx.x; k < ncoef; k += RSB_BLOCK) out[k] = __ldcg(tot + k);
+  __syncthreads();
+  return true;
+}
+
 // A(j): q_j = src * s into shared memory, w = L q_j, dots [1, D, q_0..q_j]^T w.
 template <typename V>
 __device__ void res_a(const LzArgs<V>& a, int j, V s, int tix, const Tile& t, const Unit& u,
-                      V* Qs, const V* Ds, int trs, V* ws, double* P) {
+                      V* Qs, const V* Ds, int trs, V* ws, double* P, double* out) {
   const int nr = t.row1 - t.row0;
   const V* src = (j & 1) ? a.W1 : a.W0;
   const int nd = u.nd;
@@ -1538,7 +1576,7 @@ __device__ void res_a(const LzArgs<V>& a, int j, V s, int tix, const Tile& t, co
   __syncthreads();
   Acc<V> acc[MAXCW];
   res_dots<V>(t, nd, nc, Qs, Ds, trs, ws, acc);
-  res_store_dots<V>(P, a.stride, nc, acc, tix);
+  res_store_dots<V>(P, a.stride, nc, acc, tix, out);
   if (a.pb_a) prof_add(a.pb_a, pbytes);
 }
 
@@ -1546,7 +1584,7 @@ __device__ void res_a(const LzArgs<V>& a, int j, V s, int tix, const Tile& t, co
 template <typename V>
 __device__ void res_b(const LzArgs<V>& a, int j, int tix, const Tile& t, int nd, bool masked,
                       uint64_t key, const V* Qs, const V* Ds, int trs, V* ws, const V* cv,
-                      double* P) {
+                      double* P, double* out) {
   const int nr = t.row1 - t.row0;
   const int nc = 2 + nd + j;
   unsigned long long pbytes = 0;
@@ -1558,15 +1596,15 @@ __device__ void res_b(const LzArgs<V>& a, int j, int tix, const Tile& t, int nd,
   __syncthreads();
   Acc<V> acc[MAXCW];
   res_dots<V>(t, nd, nc, Qs, Ds, trs, ws, acc);
-  res_store_dots<V>(P, a.stride, nc, acc, tix);
+  res_store_dots<V>(P, a.stride, nc, acc, tix, out);
   if (a.pb_b) prof_add(a.pb_b, pbytes);
 }
 
 // C(j): w -= basis c2 into W[(j + 1) & 1] (the next SpMV operand), ||w||^2.
 template <typename V>
-__device__ void res_c(const LzArgs<V>& a, int j, int tix, const Tile& t, int nd, bool masked,
-                      uint64_t key, const V* Qs, const V* Ds, int trs, const V* ws,
-                      const V* cv, double* sm, double* P) {
+__device__ double res_c(const LzArgs<V>& a, int j, const Tile& t, int nd, bool masked,
+                        uint64_t key, const V* Qs, const V* Ds, int trs, const V* ws,
+                        const V* cv, double* sm) {
   const int nr = t.row1 - t.row0;
   V* dst = (j & 1) ? a.W0 : a.W1;
   Acc<V> acc;
@@ -1579,110 +1617,192 @@ __device__ void res_c(const LzArgs<V>& a, int j, int tix, const Tile& t, int nd,
     if (a.pb_c) pbytes += sizeof(V) * (unsigned long long)(3 + j) + 8ull * nd;
   }
   if (a.pb_c) prof_add(a.pb_c, pbytes);
-  const double sum = block_total(acc, sm);
-  if (threadIdx.x == 0) P[tix] = sum;
+  return block_total(acc, sm);
 }
 
 // FP32 steps with the delayed second pass (D1-D3 of the streaming kernels,
-// in their order).  D1(j): v = src rows into vs, z = L (src / nu) into ws.
+// in their order).  D1(j): v = src rows into vs, z = L (src / nu) into ws; two rows
+// of a thread at once, eight entries of each in flight.  own: the unit is this tile,
+// so every gather is served from vs.
 template <typename V>
-__device__ void res_d1(const LzArgs<V>& a, int j, V s, const Tile& t, V* vs, V* ws) {
+__device__ void res_d1(const LzArgs<V>& a, int j, V s, const Tile& t, V* vs, V* ws, bool own) {
   const int nr = t.row1 - t.row0;
   const V* src = (j & 1) ? a.W1 : a.W0;
+  for (int rl = threadIdx.x; rl < nr; rl += RSB_BLOCK) vs[rl] = __ldcg(src + t.row0 + rl);
+  if (own) __syncthreads();
   unsigned long long pbytes = 0;
-  for (int rl = threadIdx.x; rl < nr; rl += RSB_BLOCK) {
-    const int r = t.row0 + rl;
-    const V xr = __ldcg(src + r);
-    vs[rl] = xr;
-    ws[rl] = s * spmv_row<V, true>(a.slice_ptr, a.ent, src, r, xr);
-    if (a.pb_a) pbytes += 4ull * row_width(a.slice_ptr, r) + 2ull * sizeof(V);
+  for (int rl = threadIdx.x; rl < nr; rl += 2 * RSB_BLOCK) {
+    int width[2];
+    const uint32_t* e[2];
+    V xr[2], acc[2];
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      const int r = t.row0 + rl + i * RSB_BLOCK;
+      width[i] = 0;
+      e[i] = a.ent;
+      xr[i] = acc[i] = V(0);
+      if (r < t.row1) {
+        const int64_t base = a.slice_ptr[r >> 5];
+        width[i] = (int)((a.slice_ptr[(r >> 5) + 1] - base) >> 5);
+        e[i] = a.ent + base + (r & 31);
+        xr[i] = vs[rl + i * RSB_BLOCK];
+        if (a.pb_a) pbytes += 4ull * width[i] + 2ull * sizeof(V);
+      }
+    }
+    const int wmax = max(width[0], width[1]);
+    for (int k0 = 0; k0 < wmax; k0 += 8) {
+      uint32_t p[2][8];
+      V xv[2][8];
+#pragma unroll
+      for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+          p[i][k] = k0 + k < width[i] ? __ldg(e[i] + 32 * (k0 + k)) : 0u;
+#pragma unroll
+      for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          xv[i][k] = xr[i];
+          if (k0 + k < width[i])
+            xv[i][k] = own ? vs[(int)ent_col(p[i][k]) - t.row0] : __ldcg(src + ent_col(p[i][k]));
+        }
+#pragma unroll
+      for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+          if (k0 + k < width[i]) acc[i] += V(ent_w(p[i][k])) * (xr[i] - xv[i][k]);
+    }
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+      if (rl + i * RSB_BLOCK < nr) ws[rl + i * RSB_BLOCK] = s * acc[i];
   }
   if (a.pb_a) prof_add(a.pb_a, pbytes);
   __syncthreads();
 }
 
 // D2(j): dots of v (vs) and z (ws) with [1, D, q_0..q_{j-1}] and with v, in the
-// per-lane order of k_lz_d2 (partials [a_b, v.v] then [g_b, v.z]).
+// per-lane order of k_lz_d2 (partials [a_b, v.v] then [g_b, v.z]; out: as in
+// res_store_dots).  A warp takes its coefficients two at a time.
 template <typename V>
 __device__ void res_d2(const LzArgs<V>& a, int j, int tix, const Tile& t, int nd, const V* Qs,
-                       const V* Ds, int trs, const V* vs, const V* ws, double* P) {
+                       const V* Ds, int trs, const V* vs, const V* ws, double* P, double* out) {
   const int nr = t.row1 - t.row0;
   const int nb = 1 + nd + j;
   const int nc = nb + 1;
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  Acc<V> av[MAXCW], az[MAXCW];
+  float S[16], C[16];
 #pragma unroll
-  for (int i = 0; i < MAXCW; ++i) {
-    const int c = w + RSB_WARPS * i;
-    if (c < nc) {
-      if (c == 0) {
-        for (int rl = lane; rl < nr; rl += 32) {
-          av[i].add(vs[rl]);
-          az[i].add(ws[rl]);
-        }
-      } else if (c <= nd) {
-        const V* d = Ds + (size_t)(c - 1) * trs;
-        for (int rl = lane; rl < nr; rl += 32) {
-          av[i].add(d[rl] * vs[rl]);
-          az[i].add(d[rl] * ws[rl]);
-        }
-      } else {
-        const V* q = c < nb ? Qs + (size_t)(c - 1 - nd) * trs : vs;
-        for (int rl = lane; rl < nr; rl += 32) {
-          const V qv = q[rl];
-          av[i].add(qv * vs[rl]);
-          az[i].add(qv * ws[rl]);
-        }
+  for (int i = 0; i < 16; ++i) S[i] = C[i] = 0.f;
+#pragma unroll
+  for (int i = 0; i < MAXCW; i += 2) {
+    const int c0 = w + RSB_WARPS * i, c1 = c0 + RSB_WARPS;
+    if (c0 >= nc) break;
+    // basis vector, FP64 deflation vector in the vector type, v itself; u0 (ones)
+    // takes the place of a vector by its value
+    auto vec = [&](int c) {
+      return c >= nb ? vs : c > nd ? Qs + (size_t)(c - 1 - nd) * trs : Ds + (size_t)max(c - 1, 0) * trs;
+    };
+    const V* q0 = vec(c0);
+    const V* q1 = vec(c1);
+    Acc<V> a0, z0, a1, z1;
+    if (c0 == 0) {
+      for (int rl = lane; rl < nr; rl += 32) {
+        const V x = vs[rl], z = ws[rl], y = q1[rl];
+        a0.add(x);
+        z0.add(z);
+        a1.add(y * x);
+        z1.add(y * z);
+      }
+    } else if (c1 < nc) {
+#pragma unroll 4
+      for (int rl = lane; rl < nr; rl += 32) {
+        const V x = vs[rl], z = ws[rl], y0 = q0[rl], y1 = q1[rl];
+        a0.add(y0 * x);
+        z0.add(y0 * z);
+        a1.add(y1 * x);
+        z1.add(y1 * z);
+      }
+    } else {
+#pragma unroll 4
+      for (int rl = lane; rl < nr; rl += 32) {
+        const V y0 = q0[rl];
+        a0.add(y0 * vs[rl]);
+        z0.add(y0 * ws[rl]);
       }
     }
+    S[2 * i] = a0.s;
+    C[2 * i] = a0.c;
+    S[2 * i + 1] = z0.s;
+    C[2 * i + 1] = z0.c;
+    S[2 * i + 2] = a1.s;
+    C[2 * i + 2] = a1.c;
+    S[2 * i + 3] = z1.s;
+    C[2 * i + 3] = z1.c;
   }
-  res_store_dots<V>(P, a.stride, nc, av, tix);
-  res_store_dots<V>(P + (long long)nc * a.stride, a.stride, nc, az, tix);
-  if (a.pb_a2) {
-    unsigned long long pbytes = 0;
-    for (int rl = threadIdx.x; rl < nr; rl += RSB_BLOCK)
-      pbytes += sizeof(V) * (unsigned long long)(2 + j) + 8ull * nd;
-    prof_add(a.pb_a2, pbytes);
+  const double sum = warp_totals<16>(S, C);
+  const int k = lane >> 1, c = w + RSB_WARPS * (k >> 1);
+  if ((lane & 1) == 0 && c < nc) {
+    const int cc = (k & 1) ? nc + c : c;
+    if (out) out[cc] = sum;
+    else P[(long long)cc * a.stride + tix] = sum;
   }
+  if (a.pb_a2 && threadIdx.x == 0)
+    atomicAdd(a.pb_a2, nr * (sizeof(V) * (unsigned long long)(2 + j) + 8ull * nd));
 }
 
 // D3(j): q_j = ssrc v - B ca into Qs, w = sz z - B cg - sqz q_j into
-// W[(j + 1) & 1], ||w||^2 (the per-row order of k_lz_d3).
+// W[(j + 1) & 1], ||w||^2 (the per-row order of k_lz_d3; cc: the pairs ca, cg; dz:
+// ssrc, sz, sqz).  Returns the tile's sum in thread 0.
 template <typename V>
-__device__ void res_d3(const LzArgs<V>& a, int j, int tix, const Tile& t, int nd, bool masked,
-                       uint64_t key, V* Qs, const V* Ds, int trs, const V* vs, const V* ws,
-                       const V* ca, const V* cg, V ssrc, V sz, V sqz, double* sm, double* P) {
+__device__ double res_d3(const LzArgs<V>& a, int j, const Tile& t, int nd, bool masked, uint64_t key,
+                         V* Qs, const V* Ds, int trs, const V* vs, const V* ws, const V (*cc)[2],
+                         const V* dz, double* sm) {
   const int nr = t.row1 - t.row0;
   V* dst = (j & 1) ? a.W0 : a.W1;
+  const V ssrc = dz[0], sz = dz[1], sqz = dz[2];
   Acc<V> acc;
-  unsigned long long pbytes = 0;
-  for (int rl = threadIdx.x; rl < nr; rl += RSB_BLOCK) {
-    const bool in_unit = !masked || a.ckey[t.row0 + rl] == key;
-    V q = ssrc * vs[rl];
-    V w = sz * ws[rl];
-    if (in_unit) {
-      q -= ca[0];
-      w -= cg[0];
-    }
+  for (int rl = threadIdx.x; rl < nr; rl += 2 * RSB_BLOCK) {
+    const bool two = rl + RSB_BLOCK < nr;
+    const int r2 = two ? rl + RSB_BLOCK : rl;  // (a lone row is computed twice, kept once)
+    V q[2] = {ssrc * vs[rl], ssrc * vs[r2]};
+    V w[2] = {sz * ws[rl], sz * ws[r2]};
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+      if (!masked || a.ckey[t.row0 + (i ? r2 : rl)] == key) {
+        q[i] -= cc[0][0];
+        w[i] -= cc[0][1];
+      }
     for (int l = 0; l < nd; ++l) {
-      const V dv = Ds[(size_t)l * trs + rl];
-      q -= ca[1 + l] * dv;
-      w -= cg[1 + l] * dv;
+      const V d0 = Ds[(size_t)l * trs + rl], d1 = Ds[(size_t)l * trs + r2];
+      q[0] -= cc[1 + l][0] * d0;
+      w[0] -= cc[1 + l][1] * d0;
+      q[1] -= cc[1 + l][0] * d1;
+      w[1] -= cc[1 + l][1] * d1;
     }
+    const V(*ck)[2] = cc + 1 + nd;
+#pragma unroll 8
     for (int k = 0; k < j; ++k) {
-      const V b = Qs[(size_t)k * trs + rl];
-      q -= ca[1 + nd + k] * b;
-      w -= cg[1 + nd + k] * b;
+      const V b0 = Qs[(size_t)k * trs + rl], b1 = Qs[(size_t)k * trs + r2];
+      const V ka = ck[k][0], kg = ck[k][1];
+      q[0] -= ka * b0;
+      w[0] -= kg * b0;
+      q[1] -= ka * b1;
+      w[1] -= kg * b1;
     }
-    w -= sqz * q;
-    Qs[(size_t)j * trs + rl] = q;
-    dst[t.row0 + rl] = w;
-    acc.add(w * w);
-    if (a.pb_b) pbytes += sizeof(V) * (unsigned long long)(4 + j) + 8ull * nd;
+    w[0] -= sqz * q[0];
+    Qs[(size_t)j * trs + rl] = q[0];
+    dst[t.row0 + rl] = w[0];
+    acc.add(w[0] * w[0]);
+    if (two) {
+      w[1] -= sqz * q[1];
+      Qs[(size_t)j * trs + r2] = q[1];
+      dst[t.row0 + r2] = w[1];
+      acc.add(w[1] * w[1]);
+    }
   }
-  if (a.pb_b) prof_add(a.pb_b, pbytes);
-  const double sum = block_total(acc, sm);
-  if (threadIdx.x == 0) P[tix] = sum;
+  if (a.pb_b && threadIdx.x == 0)
+    atomicAdd(a.pb_b, nr * (sizeof(V) * (unsigned long long)(4 + j) + 8ull * nd));
+  return block_total(acc, sm);
 }
 
 // coefficients of a finished reduction: c[0] carries the 1/sqrt(n) of u0 (as
@@ -1719,17 +1839,44 @@ __device__ void res_ritz(const LzArgs<V>& a, const Tile& t, const Unit& u, V* Qs
     atomicAdd(a.pb_a, (unsigned long long)nr * sizeof(V) * (K + kk + 1));
 }
 
+// The norm of the new vector from the tiles' sums (mine: this tile's, thread 0's):
+// beta_{j+1}, 1 / beta_{j+1} and the vector-type scale in shared memory; the unit's
+// first CTA records it and the end of the cycle on an invariant subspace.  Returns
+// true when the cycle ends here.
+template <typename V>
+__device__ __forceinline__ bool res_norm(const LzArgs<V>& a, Unit& u, int j, int tix, double breakdown,
+                                         double mine, const double* Pn, double* out,
+                                         double* scratch, double* beta, double* inu, V* scale) {
+  if (u.ntile > 1)
+    final_reduce_few(Pn, a.stride, u.tile0, u.ntile, 1, out, scratch);
+  if (threadIdx.x == 0) {
+    const double b = sqrt(u.ntile > 1 ? out[0] : mine);
+    *beta = b;
+    *inu = 1.0 / b;
+    *scale = V(*inu);
+    if (tix == u.tile0) {
+      u.beta[j + 1] = b;
+      if (b <= breakdown * u.dmax) {  // invariant subspace: the cycle ends here
+        u.msteps = j + 1;
+        u.broke = 1;
+      }
+    }
+  }
+  __syncthreads();
+  return *beta <= breakdown * u.dmax;
+}
+
 template <typename V>
 __global__ void __launch_bounds__(RSB_BLOCK, 2)
-    k_lz_res(LzArgs<V> a, int M, int trs, double breakdown, int nunits, int maxcyc, GridBar* gb) {
+    k_lz_res(LzArgs<V> a, int M, int trs, double breakdown, int maxcyc, GridBar* gb) {
   extern __shared__ __align__(16) unsigned char res_sh[];
   JacShared<V>& J = *reinterpret_cast<JacShared<V>*>(res_sh);
   size_t off = res_align(sizeof(JacShared<V>));
   double* c1 = reinterpret_cast<double*>(res_sh + off);
   double* c2 = c1 + RSB_MAXC;
   off += res_align(2 * sizeof(double) * RSB_MAXC);
-  V* cv1 = reinterpret_cast<V*>(res_sh + off);
-  V* cv2 = cv1 + RSB_MAXC;
+  V* cv = reinterpret_cast<V*>(res_sh + off);  // two coefficient sets (FP32: pairs)
+  V(*cc)[2] = reinterpret_cast<V(*)[2]>(cv);
   off += res_align(2 * sizeof(V) * RSB_MAXC);
   V* ws = reinterpret_cast<V*>(res_sh + off);
   off += res_align(sizeof(V) * (size_t)trs);
@@ -1739,43 +1886,45 @@ __global__ void __launch_bounds__(RSB_BLOCK, 2)
   off += res_align(sizeof(V) * RSB_MAXD * (size_t)trs);
   V* Qs = reinterpret_cast<V*>(res_sh + off);
   __shared__ double out[2 * RSB_MAXC + 2];
-  __shared__ double dsc[3], dsk[RSB_MAXM];
+  __shared__ double dsc[2], dsk[RSB_MAXM];
   __shared__ double sm[RSB_WARPS];
   __shared__ double beta_sh, inu_sh;
-  __shared__ V scale_sh;
-  // the Jacobi workspace is free outside lz_eig_u: the copy of S during the steps,
-  // and the scratch of the residual's and the projections' reductions
+  __shared__ V scale_sh, dz[3];
+  // the Jacobi workspace is free outside lz_eig_u: the copy of S during the steps and
+  // the scratch of the reductions between them
   static_assert(sizeof(JacShared<V>) >= sizeof(double) * RSB_MAXM * RSB_MAXM, "copy of S");
   static_assert(sizeof(JacShared<V>) >= sizeof(double) * RED_FEW_DOUBLES(RED_FEW), "scratch");
   double* Ssh = reinterpret_cast<double*>(res_sh);
   double* red = Ssh;
-  const unsigned G = gridDim.x;
+  // (the steps' own reductions must leave Ssh alone)
+  __shared__ double red1[RED_FEW_DOUBLES(1)];
   const int tix = blockIdx.x;
   const Tile t = a.tiles[tix];
   Unit& u = a.units[t.unit];
+  if (__ldcg(&u.status) != U_ACTIVE) return;
   const int nr = t.row1 - t.row0;
   const int nd = u.nd;
   const bool masked = u.masked;
   const uint64_t key = u.key;
   const double isn = u.isn;
-  const bool lead = tix == u.tile0 && threadIdx.x == 0;
+  const bool first = tix == u.tile0;
+  UnitBar ub(&u.gbar, u.ntile, __ldcg(&gb->count), gb);
+  double* const direct = u.ntile == 1 ? out : nullptr;
+  // partial buffers: FP32 dots in the first two, FP64 dots in each in turn, the norms
+  // apart, so that no CTA rewrites rows another CTA may still reduce
   double* const Pb[2] = {a.partials, a.partials + (long long)RSB_MAXC * a.stride};
+  double* const Pn = a.partials + (long long)(2 * RSB_MAXC) * a.stride;
+  // exchanged totals of a unit of more than RED_SMALL tiles (RSB_MAXC a tile)
+  double* const tot = a.partials + (3 * a.stride + u.tile0) * (long long)RSB_MAXC;
   // the tile's deflation vectors in the vector type, once per solve
   for (int l = 0; l < nd; ++l) {
     const double* d = l == 0 ? a.D0 : a.D1;
     for (int rl = threadIdx.x; rl < nr; rl += RSB_BLOCK) Ds[(size_t)l * trs + rl] = V(d[t.row0 + rl]);
   }
-  __syncthreads();
-  int* jm = a.jmin;  // two slots: read one at a cycle's start, refill the other
   for (int cyc = 0; cyc < maxcyc; ++cyc) {
-    const int jstart = cyc == 0 ? 0 : min(max(__ldcg(jm + (cyc & 1)), 0), M);
-    if (tix == 0 && threadIdx.x == 0) jm[(cyc + 1) & 1] = 0x7FFFFFFF;
-    LzArgs<V> ac = a;
-    ac.jmin = jm + ((cyc + 1) & 1);
     // the unit's step state, tracked identically by all of its CTAs
-    const bool on = __ldcg(&u.status) == U_ACTIVE;
     const int j0 = __ldcg(&u.j0);
-    int msteps = __ldcg(&u.msteps);
+    int msteps = min(__ldcg(&u.msteps), M);
     if (threadIdx.x == 0) {
       beta_sh = __ldcg(&u.beta0);
       inu_sh = __ldcg(&u.inu);
@@ -1788,72 +1937,60 @@ __global__ void __launch_bounds__(RSB_BLOCK, 2)
         Ssh[idx] = __ldcg(Sm + idx);
     }
     __syncthreads();
-    int ph = 0;
-    for (int j = jstart; j < M; ++j) {
-      const bool st = on && j < msteps && j >= j0;
+    for (int j = j0; j < msteps; ++j) {
+      double mine;
       if constexpr (sizeof(V) == 4) {
-        // FP32: the streaming kernels' steps D1-D3 (second pass delayed);
-        // partials: D2 in rows [0, 2 nc), the norm in row 2 RSB_MAXC, so that
-        // no CTA rewrites rows another CTA of the unit may still reduce
+        // FP32: the streaming kernels' steps D1-D3 (second pass delayed)
         const int nb = 1 + nd + j;
         const int nc = nb + 1;
-        double* Pn = a.partials + (long long)(2 * RSB_MAXC) * a.stride;
-        if (st) {
-          res_d1<V>(a, j, scale_sh, t, vs, ws);
-          res_d2<V>(a, j, tix, t, nd, Qs, Ds, trs, vs, ws, a.partials);
-        }
-        if (!grid_sync(gb, G)) return;
-        if (st) {
-          final_reduce(a.partials, a.stride, u.tile0, u.ntile, nc, out);
-          final_reduce(a.partials + (long long)nc * a.stride, a.stride, u.tile0, u.ntile, nc,
-                       out + nc);
-          const double inu = inu_sh;
-          d2_finish(out, out + nc, nb, nd, j, inu, isn, Ssh, dsc, dsk);
-          d2_store_S(Ssh, j, dsc, dsk);
-          if (tix == u.tile0) d2_store_S(unit_S(a.S, t.unit), j, dsc, dsk);
-          const double rho = dsc[0];
-          for (int k = threadIdx.x; k < nb; k += RSB_BLOCK) {
-            const double ck = out[k] / rho, gk = out[nc + k] / rho;
-            cv2[k] = k == 0 ? V(ck * isn) : V(ck);
-            cv1[k] = k == 0 ? V(gk * isn) : V(gk);
+        res_d1<V>(a, j, scale_sh, t, vs, ws, direct != nullptr);
+        res_d2<V>(a, j, tix, t, nd, Qs, Ds, trs, vs, ws, a.partials, direct);
+        if (!ub.sync()) return;
+        if (!res_totals(a.partials, a.stride, u, tix, 2 * nc, out, tot, red1, ub)) return;
+        const double inu = inu_sh;
+        d2_finish(out, out + nc, nb, nd, j, inu, isn, Ssh, dsc, dsk);
+        const double rho = dsc[0];
+        const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+        if (w < 4) {
+          const int k = threadIdx.x & 63, h = threadIdx.x >> 6;
+          if (k < nb) {
+            const double x = out[h * nc + k] / rho;
+            cc[k][h] = k == 0 ? V(x * isn) : V(x);
           }
-          if (lead) u.alpha[j] = dsc[2];
-          __syncthreads();
-          res_d3<V>(a, j, tix, t, nd, masked, key, Qs, Ds, trs, vs, ws, cv2, cv1, V(inu / rho),
-                    V(1.0 / rho), V(dsc[1] / rho), sm, Pn);
+        } else if (w == 4 && lane < 3) {
+          dz[lane] = V((lane == 0 ? inu : lane == 1 ? 1.0 : dsc[1]) / rho);
         }
-        if (!grid_sync(gb, G)) return;
-        if (st) {
-          final_reduce(Pn, a.stride, u.tile0, u.ntile, 1, out);
-          if (threadIdx.x == 0) {
-            const double b = sqrt(out[0]);
-            beta_sh = b;
-            inu_sh = 1.0 / b;
-            scale_sh = V(inu_sh);
-            if (lead) u.beta[j + 1] = b;
-            if (b <= breakdown * u.dmax && lead) {  // invariant subspace: the cycle ends here
-              u.msteps = j + 1;
-              u.broke = 1;
+        __syncthreads();
+        mine = res_d3<V>(a, j, t, nd, masked, key, Qs, Ds, trs, vs, ws, cc, dz, sm);
+        if (threadIdx.x == 0) Pn[tix] = mine;
+        ub.arrive();
+        // while the norms travel: column j of S
+        d2_store_S(Ssh, j, dsk);
+        if (first) d2_store_S(unit_S(a.S, t.unit), j, dsk);
+        if (w == 7) {
+          const double alpha = d2_alpha(out, nd, j, dsc, dsk);
+          if (lane == 0) {
+            Ssh[j * RSB_MAXM + j] = alpha;
+            if (first) {
+              unit_S(a.S, t.unit)[j * RSB_MAXM + j] = alpha;
+              u.alpha[j] = alpha;
             }
           }
-          __syncthreads();
-          if (beta_sh <= breakdown * u.dmax) msteps = j + 1;
         }
-        continue;
-      }
-      const int nc = 2 + nd + j;
-      if (st) res_a<V>(a, j, scale_sh, tix, t, u, Qs, Ds, trs, ws, Pb[ph & 1]);
-      if (!grid_sync(gb, G)) return;
-      if (st) {
-        final_reduce(Pb[ph & 1], a.stride, u.tile0, u.ntile, nc, out);
-        res_coef<V>(out, nc, isn, c1, cv1);
-        res_b<V>(a, j, tix, t, nd, masked, key, Qs, Ds, trs, ws, cv1, Pb[(ph + 1) & 1]);
-      }
-      if (!grid_sync(gb, G)) return;
-      if (st) {
-        final_reduce(Pb[(ph + 1) & 1], a.stride, u.tile0, u.ntile, nc, out);
-        res_coef<V>(out, nc, isn, c2, cv2);
-        if (tix == u.tile0) {  // column j of S = Q^T L Q
+        if (!ub.wait()) return;
+        if (res_norm<V>(a, u, j, tix, breakdown, mine, Pn, out, red1, &beta_sh, &inu_sh, &scale_sh))
+          msteps = j + 1;
+      } else {
+        const int nc = 2 + nd + j;
+        res_a<V>(a, j, scale_sh, tix, t, u, Qs, Ds, trs, ws, Pb[0], direct);
+        if (!ub.sync()) return;
+        if (!res_totals(Pb[0], a.stride, u, tix, nc, out, tot, red1, ub)) return;
+        res_coef<V>(out, nc, isn, c1, cv);
+        res_b<V>(a, j, tix, t, nd, masked, key, Qs, Ds, trs, ws, cv, Pb[1], direct);
+        if (!ub.sync()) return;
+        if (!res_totals(Pb[1], a.stride, u, tix, nc, out, tot + RSB_MAXC, red1, ub)) return;
+        res_coef<V>(out, nc, isn, c2, cv + RSB_MAXC);
+        if (first) {  // column j of S = Q^T L Q
           double* Sm = unit_S(a.S, t.unit);
           for (int k = threadIdx.x; k <= j; k += RSB_BLOCK) {
             const double v = c1[1 + nd + k] + c2[1 + nd + k];
@@ -1861,37 +1998,26 @@ __global__ void __launch_bounds__(RSB_BLOCK, 2)
             Sm[j * RSB_MAXM + k] = v;
           }
         }
-        res_c<V>(a, j, tix, t, nd, masked, key, Qs, Ds, trs, ws, cv2, sm, Pb[ph & 1]);
+        mine = res_c<V>(a, j, t, nd, masked, key, Qs, Ds, trs, ws, cv + RSB_MAXC, sm);
+        if (threadIdx.x == 0) Pn[tix] = mine;
+        if (!ub.sync()) return;
+        if (res_norm<V>(a, u, j, tix, breakdown, mine, Pn, out, red1, &beta_sh, &inu_sh, &scale_sh))
+          msteps = j + 1;
       }
-      if (!grid_sync(gb, G)) return;
-      if (st) {
-        final_reduce(Pb[ph & 1], a.stride, u.tile0, u.ntile, 1, out);
-        if (threadIdx.x == 0) {
-          const double b = sqrt(out[0]);
-          beta_sh = b;
-          scale_sh = V(1.0 / b);
-          if (lead) u.beta[j + 1] = b;
-          if (b <= breakdown * u.dmax && lead) {  // invariant subspace: the cycle ends here
-            u.msteps = j + 1;
-            u.broke = 1;
-          }
-        }
-        __syncthreads();
-        if (beta_sh <= breakdown * u.dmax) msteps = j + 1;
-      }
-      ++ph;
     }
-    for (int uu = blockIdx.x; uu < nunits; uu += G) lz_eig_u<V, true>(a.units[uu], unit_S(a.S, uu), J);
-    if (!grid_sync(gb, G)) return;
+    if (first) lz_eig_u<V, true>(u, unit_S(a.S, t.unit), J);
+    if (!ub.sync()) return;
     res_ritz<V>(a, t, u, Qs, trs, &J.Z[0][0]);
-    if (!grid_sync(gb, G)) return;
-    lz_resid_t<V, true>(ac, a.Y, 0, tix, sm, out, red);
-    if (!grid_sync(gb, G)) return;
-    proj2_t<V, true>(a, a.Y, tix, sm, out, red);
-    if (!grid_sync(gb, G)) return;
-    proj3_t<V, true>(a, a.Y, tix, sm, out, red);
-    if (!grid_sync(gb, G)) return;
-    if (__ldcg(a.n_active) == 0) break;
+    if (!ub.sync()) return;
+    lz_resid_t<V, true>(a, a.Y, 0, tix, sm, out, red);
+    if (!ub.sync()) return;
+    if (__ldcg(&u.status) != U_ACTIVE) return;
+    if (__ldcg(&u.j0) == 0) {  // explicit restart from y
+      proj2_t<V, true>(a, a.Y, tix, sm, out, red);
+      if (!ub.sync()) return;
+      proj3_t<V, true>(a, a.Y, tix, sm, out, red);
+      if (!ub.sync()) return;
+    }
   }
 }
 
@@ -1946,6 +2072,7 @@ __global__ void k_solve_init(Unit* units, int nunits, int nd, int krylov, int ma
   u.inner = 0;
   u.inner_total = 0;
   u.cg_done = 0;
+  u.gbar = 0;
   u.status = U_ACTIVE;
   atomicAdd(n_active, 1);
 }
@@ -2116,7 +2243,7 @@ static int lanczos_run(const LevelGraph& G, const Tile* tiles, int ntiles, Unit*
     RSB_CK(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
     int trs = B.trmax;
     const size_t smem = res_smem_bytes<V>(M, trs);
-    if (smem + 1024 <= (size_t)optin) {  // room for the kernel's static shared memory
+    if (smem + 4096 <= (size_t)optin) {  // room for the kernel's static shared memory
       RSB_CK(cudaFuncSetAttribute(k_lz_res<V>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   (int)smem));
       RSB_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_lz_res<V>, RSB_BLOCK, smem));
@@ -2126,8 +2253,7 @@ static int lanczos_run(const LevelGraph& G, const Tile* tiles, int ntiles, Unit*
         GridBar* gb = B.gb;
         LzArgs<V> ar = a;  // the persistent kernel's phases count into one family
         ar.pb_a = ar.pb_a2 = ar.pb_b = ar.pb_c = prof_bytes(PROF_CYCLE);
-        void* args[] = {(void*)&ar, (void*)&M, (void*)&trs, (void*)&bd, (void*)&nunits,
-                        (void*)&maxcyc, (void*)&gb};
+        void* args[] = {(void*)&ar, (void*)&M, (void*)&trs, (void*)&bd, (void*)&maxcyc, (void*)&gb};
         const int pi = prof_before(PROF_CYCLE, s);
         cudaError_t e = cudaLaunchCooperativeKernel((const void*)k_lz_res<V>, ntiles, RSB_BLOCK,
                                                     args, smem, s);
