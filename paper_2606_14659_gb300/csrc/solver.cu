@@ -913,8 +913,9 @@ template <typename T>
 struct JacShared {
   T A[RSB_MAXM][RSB_MAXM + 1];
   T Z[RSB_MAXM][RSB_MAXM + 1];
-  T c[RSB_MAXM / 2], s[RSB_MAXM / 2];
-  int p[RSB_MAXM / 2], q[RSB_MAXM / 2];
+  // rotations (c, s) and index pairs (p | q << 8) of a round, and of the next one
+  __align__(16) T cs[2][RSB_MAXM / 2][2];
+  int pq[2][RSB_MAXM / 2];
   double red[RSB_WARPS];
   int rank[RSB_MAXM];
 };
@@ -956,13 +957,50 @@ __device__ __forceinline__ void jac_rotation(double app, double aqq, double apq,
   s = t * r;
 }
 
-// tasks per thread and round: np*np + np*n2 <= 20*20 + 20*40 over RSB_BLOCK threads
-#define EIG_TASKS ((RSB_MAXM * RSB_MAXM * 3 / 4 + RSB_BLOCK - 1) / RSB_BLOCK)
+// The rotations of round rnd into buffer b, by lanes < n2 / 2 of one warp
+// (round-robin pairing: slot 0 holds index 0, the others rotate).
+template <typename T>
+__device__ __forceinline__ void jac_pairs(JacShared<T>& J, int b, int rnd, int n2, int K) {
+  const int i = threadIdx.x & 31;
+  if (i >= n2 / 2) return;
+  int ia = i + rnd - 1, ib = n2 - 2 - i + rnd;
+  if (ia >= n2 - 1) ia -= n2 - 1;
+  if (ib >= n2 - 1) ib -= n2 - 1;
+  int pa = i == 0 ? 0 : ia + 1;
+  int pb = ib + 1;
+  if (pa > pb) { const int tt = pa; pa = pb; pb = tt; }
+  T cc = T(1), ss = T(0);
+  const T apq = J.A[pa][pb];
+  if (pb < K && apq != T(0)) jac_rotation(J.A[pa][pa], J.A[pb][pb], apq, cc, ss);
+  J.pq[b][i] = pa | (pb << 8);
+  J.cs[b][i][0] = cc;
+  J.cs[b][i][1] = ss;
+}
 
+// The 2x2 block (rows of pair 1, columns of pair 2): the column rotation, then the
+// row rotation.
+template <typename T>
+__device__ __forceinline__ void jac_block(T& a11, T& a12, T& a21, T& a22, T c1, T s1, T c2, T s2) {
+  const T b11 = c2 * a11 - s2 * a12, b12 = s2 * a11 + c2 * a12;
+  const T b21 = c2 * a21 - s2 * a22, b22 = s2 * a21 + c2 * a22;
+  a11 = c1 * b11 - s1 * b21;
+  a21 = s1 * b11 + c1 * b21;
+  a12 = c1 * b12 - s1 * b22;
+  a22 = s1 * b12 + c1 * b22;
+}
+
+// Bound: the latency of a round (some 300 of them), in FP64 its arithmetic as well.
+// A round is two phases: every thread updates its 2x2 blocks of A (all of its loads
+// before its stores: the blocks are disjoint); then one warp computes the next round's
+// rotations from the new A while the others apply this round's to Z, which the
+// rotations do not need.  In FP32 every block is updated (both triangles, each with its
+// own rounding), in FP64 the upper ones, which are mirrored.  With the rotations alone
+// in a phase of their own and the updates one after the other, 40 x 40 took 200 us in
+// FP32 and 1240 us in FP64.
 template <typename T, bool CO>
-__device__ void lz_eig_u(Unit& u, double* Sm, JacShared<T>& J) {
+__device__ __noinline__ void lz_eig_u(Unit& u, double* Sm, JacShared<T>& J) {
   if (ldc<CO>(&u.status) != U_ACTIVE) return;
-  const int tid = threadIdx.x;
+  const int tid = threadIdx.x, w = tid >> 5;
   const int K = ldc<CO>(&u.msteps);
   const int n2 = K + (K & 1);
   for (int idx = tid; idx < n2 * n2; idx += RSB_BLOCK) {
@@ -983,80 +1021,134 @@ __device__ void lz_eig_u(Unit& u, double* Sm, JacShared<T>& J) {
   __syncthreads();
   const double eps2 = sizeof(T) == 8 ? 1e-30 : 1e-14;
   const double thr = fro * eps2;
-  // this thread's tasks of every round: np*np blocks of A (pair i1 x pair i2),
-  // then np*n2 (pair, row) updates of Z; fixed for the whole solve
   const int np = n2 / 2;
-  int ta[EIG_TASKS], tb[EIG_TASKS];
+  // this thread's blocks of A (pair i1 x pair i2; FP32: two, FP64: one with i1 <= i2)
+  // and (pair, row) updates of Z (warps 1..7); fixed for the whole solve
+  constexpr int NB = sizeof(T) == 8 ? 1 : 2;
+  constexpr int NZ = (RSB_MAXM * RSB_MAXM / 2 + RSB_BLOCK - 33) / (RSB_BLOCK - 32);
+  int i1[NB], i2[NB], zi[NZ], zr[NZ];
 #pragma unroll
-  for (int k = 0; k < EIG_TASKS; ++k) {
+  for (int k = 0; k < NB; ++k) {
     const int task = tid + k * RSB_BLOCK;
-    ta[k] = -1;
-    tb[k] = 0;
-    if (task < np * np) {
-      ta[k] = task / np;
-      tb[k] = task - ta[k] * np;
-    } else if (task < np * np + np * n2) {
-      const int zt = task - np * np;
-      ta[k] = -2;
-      tb[k] = ((zt / n2) << 8) | (zt % n2);
+    i1[k] = -1;
+    i2[k] = 0;
+    if constexpr (sizeof(T) == 8) {
+      int row = 0, left = task;  // row-major upper triangle
+      while (row < np && left >= np - row) left -= np - row++;
+      if (row < np) {
+        i1[k] = row;
+        i2[k] = row + left;
+      }
+    } else if (task < np * np) {
+      i1[k] = task / np;
+      i2[k] = task - i1[k] * np;
     }
   }
-  for (int sweep = 0; sweep < 20; ++sweep) {
-    double off = 0.0;
-    for (int idx = tid; idx < K * K; idx += RSB_BLOCK) {
-      const int i = idx / K, k = idx % K;
-      if (i < k) off += (double)J.A[i][k] * (double)J.A[i][k];
-    }
-    off = block_sum(off, J.red);
-    if (tid == 0) J.red[0] = off;
-    __syncthreads();
-    off = J.red[0];
-    __syncthreads();
-    if (off <= thr) break;
-    for (int rnd = 0; rnd < n2 - 1; ++rnd) {
-      if (tid < np) {
-        // round-robin pairing: slot 0 holds index 0, the others rotate
-        int ia = tid + rnd - 1, ib = n2 - 2 - tid + rnd;
-        if (ia >= n2 - 1) ia -= n2 - 1;
-        if (ib >= n2 - 1) ib -= n2 - 1;
-        int pa = tid == 0 ? 0 : ia + 1;
-        int pb = ib + 1;
-        if (pa > pb) { const int tt = pa; pa = pb; pb = tt; }
-        T cc = T(1), ss = T(0);
-        const T apq = J.A[pa][pb];
-        if (pb < K && apq != T(0)) jac_rotation(J.A[pa][pa], J.A[pb][pb], apq, cc, ss);
-        J.p[tid] = pa;
-        J.q[tid] = pb;
-        J.c[tid] = cc;
-        J.s[tid] = ss;
-      }
-      __syncthreads();
-      // the round's rotations act on disjoint index pairs, so every 2x2 block
-      // (pair i1 rows, pair i2 columns) is updated in place by one thread:
-      // the column rotation, then the row rotation; Z takes the column one
 #pragma unroll
-      for (int k = 0; k < EIG_TASKS; ++k) {
-        if (ta[k] >= 0) {
-          const int i1 = ta[k], i2 = tb[k];
-          const int p1 = J.p[i1], q1 = J.q[i1], p2 = J.p[i2], q2 = J.q[i2];
-          const T c1 = J.c[i1], s1 = J.s[i1], c2 = J.c[i2], s2 = J.s[i2];
-          const T a11 = J.A[p1][p2], a12 = J.A[p1][q2], a21 = J.A[q1][p2], a22 = J.A[q1][q2];
-          const T b11 = c2 * a11 - s2 * a12, b12 = s2 * a11 + c2 * a12;
-          const T b21 = c2 * a21 - s2 * a22, b22 = s2 * a21 + c2 * a22;
-          J.A[p1][p2] = c1 * b11 - s1 * b21;
-          J.A[q1][p2] = s1 * b11 + c1 * b21;
-          J.A[p1][q2] = c1 * b12 - s1 * b22;
-          J.A[q1][q2] = s1 * b12 + c1 * b22;
-        } else if (ta[k] == -2) {
-          const int i = tb[k] >> 8, r = tb[k] & 255;
-          const int pa = J.p[i], pb = J.q[i];
-          const T cc = J.c[i], ss = J.s[i];
-          const T zx = J.Z[r][pa], zy = J.Z[r][pb];
-          J.Z[r][pa] = cc * zx - ss * zy;
-          J.Z[r][pb] = ss * zx + cc * zy;
+  for (int k = 0; k < NZ; ++k) {
+    const int zt = tid - 32 + k * (RSB_BLOCK - 32);
+    zi[k] = -1;
+    zr[k] = 0;
+    if (w > 0 && zt < np * n2) {
+      zi[k] = zt / n2;
+      zr[k] = zt - zi[k] * n2;
+    }
+  }
+  int buf = 0;
+  if (w == 0) jac_pairs(J, 0, 0, n2, K);
+  for (int sweep = 0; sweep < 20; ++sweep) {
+    // off-diagonal mass against thr: a quick FP32 sum decides unless it lies within
+    // 0.1 % of thr (its own error is below 1e-5), then the FP64 sum does
+    float q = 0.f;
+    for (int i = tid >> 3; i < K; i += RSB_BLOCK / 8)
+      for (int k = i + 1 + (tid & 7); k < K; k += 8) {
+        const float x = (float)J.A[i][k];
+        q = fmaf(x, x, q);
+      }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
+    if ((tid & 31) == 0) J.red[w] = (double)q;
+    __syncthreads();
+    float qs = 0.f;
+#pragma unroll
+    for (int i = 0; i < RSB_WARPS; ++i) qs += (float)J.red[i];
+    const float thrf = (float)thr;
+    __syncthreads();
+    if (!(qs > 1.001f * thrf)) {
+      bool stop = qs < 0.999f * thrf;
+      if (!stop || sizeof(T) == 8) {  // (FP64: thr may be below FP32's range)
+        double off = 0.0;
+        for (int idx = tid; idx < K * K; idx += RSB_BLOCK) {
+          const int i = idx / K, k = idx % K;
+          if (i < k) off += (double)J.A[i][k] * (double)J.A[i][k];
         }
+        off = block_sum(off, J.red);
+        if (tid == 0) J.red[0] = off;
+        __syncthreads();
+        off = J.red[0];
+        __syncthreads();
+        stop = off <= thr;
+      }
+      if (stop) break;
+    }
+    for (int rnd = 0; rnd < n2 - 1; ++rnd) {
+      T a11[NB], a12[NB], a21[NB], a22[NB];
+      int p1[NB], q1[NB], p2[NB], q2[NB];
+#pragma unroll
+      for (int k = 0; k < NB; ++k)
+        if (i1[k] >= 0) {
+          const int x = J.pq[buf][i1[k]], y = J.pq[buf][i2[k]];
+          p1[k] = x & 255;
+          q1[k] = x >> 8;
+          p2[k] = y & 255;
+          q2[k] = y >> 8;
+          a11[k] = J.A[p1[k]][p2[k]];
+          a12[k] = J.A[p1[k]][q2[k]];
+          a21[k] = J.A[q1[k]][p2[k]];
+          a22[k] = J.A[q1[k]][q2[k]];
+        }
+#pragma unroll
+      for (int k = 0; k < NB; ++k)
+        if (i1[k] >= 0) {
+          jac_block(a11[k], a12[k], a21[k], a22[k], J.cs[buf][i1[k]][0], J.cs[buf][i1[k]][1],
+                    J.cs[buf][i2[k]][0], J.cs[buf][i2[k]][1]);
+          J.A[p1[k]][p2[k]] = a11[k];
+          J.A[q1[k]][p2[k]] = a21[k];
+          J.A[p1[k]][q2[k]] = a12[k];
+          J.A[q1[k]][q2[k]] = a22[k];
+          if (sizeof(T) == 8 && i1[k] != i2[k]) {
+            J.A[p2[k]][p1[k]] = a11[k];
+            J.A[p2[k]][q1[k]] = a21[k];
+            J.A[q2[k]][p1[k]] = a12[k];
+            J.A[q2[k]][q1[k]] = a22[k];
+          }
+        }
+      __syncthreads();
+      if (w == 0) {
+        jac_pairs(J, buf ^ 1, rnd + 1 < n2 - 1 ? rnd + 1 : 0, n2, K);
+      } else {
+        T zx[NZ], zy[NZ], c[NZ], sn[NZ];
+        int pa[NZ], pb[NZ];
+#pragma unroll
+        for (int k = 0; k < NZ; ++k)
+          if (zi[k] >= 0) {
+            const int x = J.pq[buf][zi[k]];
+            pa[k] = x & 255;
+            pb[k] = x >> 8;
+            c[k] = J.cs[buf][zi[k]][0];
+            sn[k] = J.cs[buf][zi[k]][1];
+            zx[k] = J.Z[zr[k]][pa[k]];
+            zy[k] = J.Z[zr[k]][pb[k]];
+          }
+#pragma unroll
+        for (int k = 0; k < NZ; ++k)
+          if (zi[k] >= 0) {
+            J.Z[zr[k]][pa[k]] = c[k] * zx[k] - sn[k] * zy[k];
+            J.Z[zr[k]][pb[k]] = sn[k] * zx[k] + c[k] * zy[k];
+          }
       }
       __syncthreads();
+      buf ^= 1;
     }
   }
   // ascending order (ties by index)
