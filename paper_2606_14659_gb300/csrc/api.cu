@@ -428,6 +428,16 @@ struct MeshIn {
   int64_t nnz;
 };
 
+static int invalid_graph(int f) {
+  std::string why = "invalid graph:";
+  if (f & 1) why += " row_ptr";
+  if (f & 2) why += " column out of range";
+  if (f & 4) why += " self loop";
+  if (f & 8) why += " weight outside 1..7";
+  if (f & 16) why += " asymmetric";
+  return rsb_set_error(RSB_EINVAL, why);
+}
+
 // perm / iperm (optional, meshes concatenated, indices local to each mesh): row
 // i of mesh m in the level-0 graph is the caller's row perm[off_m + i], and the
 // caller's row j becomes row iperm[off_m + j]
@@ -456,14 +466,7 @@ static int build_level0(Ctx& c, const std::vector<MeshIn>& meshes, int validate,
   RSB_CK(cudaMemcpyAsync(c.h_pinned, flag, sizeof(int), cudaMemcpyDeviceToHost, c.s));
   RSB_CK(cudaStreamSynchronize(c.s));
   if (c.h_pinned[0]) {
-    const int f = c.h_pinned[0];
-    std::string why = "invalid graph:";
-    if (f & 1) why += " row_ptr";
-    if (f & 2) why += " column out of range";
-    if (f & 4) why += " self loop";
-    if (f & 8) why += " weight outside 1..7";
-    if (f & 16) why += " asymmetric";
-    return rsb_set_error(RSB_EINVAL, why);
+    return invalid_graph(c.h_pinned[0]);
   }
   if ((rc = launch_slice_widths(dptr<int32_t>(c.len), N, dptr<int64_t>(c.slice_sz), c.s))) return rc;
   RSB_CK(cudaMemsetAsync(dptr<int64_t>(c.slice_sz) + nsl, 0, sizeof(int64_t), c.s));
@@ -1496,8 +1499,61 @@ extern "C" int rsb_fiedler(const rsb_csr* g, const rsb_options* opt, double* lam
 // ----------------------------------------------------------------------------
 // Laplacian action and its bandwidth benchmark
 // ----------------------------------------------------------------------------
-static int lap_common(const rsb_csr* g, const void* x, void* y, int f32, int reps, double* ms,
-                      double* bytes, void* stream) {
+// One application: the entries are read once, so no sliced-ELL copy is made.
+static int lap_apply(const rsb_csr* g, const void* x, void* y, int f32, void* stream) {
+  if (!g || g->n < 1) return rsb_set_error(RSB_EINVAL, "graph");
+  if (g->n >= RSB_MAXN) return rsb_set_error(RSB_EINVAL, "n out of range");
+  if (!g->row_ptr) return rsb_set_error(RSB_EINVAL, "NULL row_ptr");
+  Ctx* pc = nullptr;
+  int rc = begin_call(&pc, stream);
+  if (rc) return rc;
+  Ctx& c = *pc;
+  MeshIn m = {g->n, g->row_ptr, g->col, g->weight, nullptr, nullptr, 0};
+  if (!g->col || !is_device_ptr(g->row_ptr) || !is_device_ptr(g->col) ||
+      (g->weight && !is_device_ptr(g->weight))) {
+    rsb_csr host = *g;  // (the action needs neither ids nor coordinates)
+    host.gid = nullptr;
+    host.coords = nullptr;
+    if ((rc = mesh_from(c, &host, m))) return end_call(c, stream, rc);
+  }
+  const int64_t N = g->n;
+  const size_t es = f32 ? 4 : 8;
+  const void* xd = x;
+  void* yd = y;
+  DevBuf tx, ty;
+  if (!is_device_ptr(x)) {
+    if ((rc = devbuf_reserve(tx, es * N))) return end_call(c, stream, rc);
+    RSB_CK(cudaMemcpyAsync(tx.p, x, es * N, cudaMemcpyHostToDevice, c.s));
+    xd = tx.p;
+  }
+  const bool yh = !is_device_ptr(y);
+  if (yh) {
+    if ((rc = devbuf_reserve(ty, es * N))) {
+      rc = end_call(c, stream, rc);
+      free_buf(tx);
+      return rc;
+    }
+    yd = ty.p;
+  }
+  // faults are reported into pinned host words that the call reads after its only
+  // synchronisation
+  int* err = c.h_pinned + 8;
+  for (int i = 0; i < 5; ++i) err[i] = 0;
+  rc = launch_csr_apply(m.row_ptr, m.col, m.wt, N, f32, xd, yd, err, c.s);
+  if (!rc && yh) {
+    cudaError_t e = cudaMemcpyAsync(y, yd, es * N, cudaMemcpyDeviceToHost, c.s);
+    if (e != cudaSuccess) rc = rsb_set_cuda_error(e, "copy y");
+  }
+  rc = end_call(c, stream, rc);
+  free_buf(tx);
+  free_buf(ty);
+  int f = 0;
+  for (int i = 0; i < 5; ++i) f |= err[i] ? 1 << i : 0;
+  if (!rc && f) return invalid_graph(f);
+  return rc;
+}
+
+static int lap_bench(const rsb_csr* g, int f32, int reps, double* ms, double* bytes, void* stream) {
   if (!g || g->n < 1) return rsb_set_error(RSB_EINVAL, "graph");
   Ctx* pc = nullptr;
   int rc = begin_call(&pc, stream);
@@ -1511,56 +1567,28 @@ static int lap_common(const rsb_csr* g, const void* x, void* y, int f32, int rep
   if (rc) return end_call(c, stream, rc);
   const int64_t N = G.n;
   const size_t es = f32 ? 4 : 8;
-  const void* xd = x;
-  void* yd = y;
   DevBuf tx, ty;
-  const bool xh = x && !is_device_ptr(x), yh = y && !is_device_ptr(y);
-  if (reps > 0) {
-    if ((rc = devbuf_reserve(tx, es * N)) || (rc = devbuf_reserve(ty, es * N)))
-      return end_call(c, stream, rc);
-    RSB_CK(cudaMemsetAsync(tx.p, 0, es * N, c.s));
-    xd = tx.p;
-    yd = ty.p;
-  } else {
-    if (xh) {
-      if ((rc = devbuf_reserve(tx, es * N))) return end_call(c, stream, rc);
-      RSB_CK(cudaMemcpyAsync(tx.p, x, es * N, cudaMemcpyHostToDevice, c.s));
-      xd = tx.p;
-    }
-    if (yh) {
-      if ((rc = devbuf_reserve(ty, es * N))) return end_call(c, stream, rc);
-      yd = ty.p;
-    }
-  }
+  if ((rc = devbuf_reserve(tx, es * N)) || (rc = devbuf_reserve(ty, es * N)))
+    return end_call(c, stream, rc);
+  RSB_CK(cudaMemsetAsync(tx.p, 0, es * N, c.s));
   auto apply = [&]() -> int {
-    return f32 ? launch_spmv_f32(G, (const float*)xd, (float*)yd, c.s)
-               : launch_spmv_f64(G, (const double*)xd, (double*)yd, c.s);
+    return f32 ? launch_spmv_f32(G, (const float*)tx.p, (float*)ty.p, c.s)
+               : launch_spmv_f64(G, (const double*)tx.p, (double*)ty.p, c.s);
   };
-  if (reps <= 0) {
-    rc = apply();
-    if (!rc && yh) {
-      cudaError_t e = cudaMemcpyAsync(y, yd, es * N, cudaMemcpyDeviceToHost, c.s);
-      if (e != cudaSuccess) rc = rsb_set_cuda_error(e, "copy y");
-    }
-  } else {
-    cudaEvent_t e0, e1;
-    cudaEventCreate(&e0);
-    cudaEventCreate(&e1);
-    for (int w = 0; w < 3 && !rc; ++w) rc = apply();
-    cudaEventRecord(e0, c.s);
-    for (int i = 0; i < reps && !rc; ++i) rc = apply();
-    cudaEventRecord(e1, c.s);
-    cudaEventSynchronize(e1);
-    float t = 0;
-    cudaEventElapsedTime(&t, e0, e1);
-    cudaEventDestroy(e0);
-    cudaEventDestroy(e1);
-    if (ms) *ms = (double)t / reps;
-    if (bytes) {
-      int64_t nnz = meshes[0].nnz;
-      *bytes = 4.0 * (double)nnz + 2.0 * (double)es * (double)N;
-    }
-  }
+  cudaEvent_t e0, e1;
+  cudaEventCreate(&e0);
+  cudaEventCreate(&e1);
+  for (int w = 0; w < 3 && !rc; ++w) rc = apply();
+  cudaEventRecord(e0, c.s);
+  for (int i = 0; i < reps && !rc; ++i) rc = apply();
+  cudaEventRecord(e1, c.s);
+  cudaEventSynchronize(e1);
+  float t = 0;
+  cudaEventElapsedTime(&t, e0, e1);
+  cudaEventDestroy(e0);
+  cudaEventDestroy(e1);
+  if (ms) *ms = (double)t / reps;
+  if (bytes) *bytes = 4.0 * (double)meshes[0].nnz + 2.0 * (double)es * (double)N;
   rc = end_call(c, stream, rc);
   free_buf(tx);
   free_buf(ty);
@@ -1569,16 +1597,16 @@ static int lap_common(const rsb_csr* g, const void* x, void* y, int f32, int rep
 
 extern "C" int rsb_laplacian_apply(const rsb_csr* g, const double* x, double* y, void* stream) {
   if (!x || !y) return rsb_set_error(RSB_EINVAL, "NULL vector");
-  return lap_common(g, x, y, 0, 0, nullptr, nullptr, stream);
+  return lap_apply(g, x, y, 0, stream);
 }
 extern "C" int rsb_laplacian_apply_f32(const rsb_csr* g, const float* x, float* y, void* stream) {
   if (!x || !y) return rsb_set_error(RSB_EINVAL, "NULL vector");
-  return lap_common(g, x, y, 1, 0, nullptr, nullptr, stream);
+  return lap_apply(g, x, y, 1, stream);
 }
 extern "C" int rsb_laplacian_bench(const rsb_csr* g, int f32, int reps, double* ms_per_apply,
                                    double* useful_bytes, void* stream) {
   if (reps < 1) return rsb_set_error(RSB_EINVAL, "reps");
-  return lap_common(g, nullptr, nullptr, f32 ? 1 : 0, reps, ms_per_apply, useful_bytes, stream);
+  return lap_bench(g, f32 ? 1 : 0, reps, ms_per_apply, useful_bytes, stream);
 }
 
 extern "C" void rsb_test_poison_barrier(int on) { g_rsb_poison_barrier = on ? 1 : 0; }

@@ -253,6 +253,117 @@ int launch_spmv_f32(const LevelGraph& G, const float* x, float* y, cudaStream_t 
 }
 
 // ----------------------------------------------------------------------------
+// Laplacian action straight from CSR, for a graph that is applied once: the
+// validation of k_validate (without the symmetry check) and the action in one pass
+// over the entries, instead of building the sliced-ELL copy first.
+// Bound: HBM in FP32 (8 B an entry, read once), the FP64 rate in FP64 (one FMA an
+// entry).  The entries of a warp's 32 rows are contiguous, so the warp brings them to
+// shared memory packed as in the sliced form, coalesced and up to CSR_CAP at a time,
+// and every lane sums its row from there in entry order: the rows of spmv_row_ro bit
+// for bit.  192 x 128 x 96, 10 % deleted (54M entries): FP64 call 603 us with the
+// sliced copy (read and checked, lengths, scan, written, read again).
+// err: five words the host sees (zero before the launch); a fault in the graph sets
+// the word of its kind, and y is then not to be used.  Reads stay inside
+// [0, row_ptr[n]) of col and wt and [0, n) of x whatever the graph holds.
+// ----------------------------------------------------------------------------
+#define CSR_CAP 1024
+template <typename V>
+__global__ void __launch_bounds__(RSB_BLOCK) k_csr_apply(const int64_t* __restrict__ row_ptr,
+                                                         const int32_t* __restrict__ col,
+                                                         const int32_t* __restrict__ wt, int32_t n,
+                                                         const V* __restrict__ x, V* __restrict__ y,
+                                                         volatile int* err) {
+  __shared__ uint32_t sh[RSB_WARPS][CSR_CAP];
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int64_t r0 = (int64_t)blockIdx.x * RSB_BLOCK + 32 * w;
+  if (r0 >= n) return;
+  const int rows = (int)min((int64_t)32, n - r0);
+  const int64_t r = r0 + lane;
+  const int64_t nnz = row_ptr[n];
+  int64_t b = 0, e = 0;
+  if (lane < rows) {
+    b = row_ptr[r];
+    e = row_ptr[r + 1];
+  }
+  // the warp's entries; rows that do not follow one another inside [0, nnz) are faults
+  const int64_t w0 = __shfl_sync(0xffffffffu, b, 0);
+  const int64_t w1 = __shfl_sync(0xffffffffu, e, rows - 1);
+  int f = 0;
+  if (lane < rows && (e < b || (r == 0 && b != 0) || b < w0 || e > w1 || b < 0 || e > nnz)) f = 1;
+  if (__any_sync(0xffffffffu, f)) {
+    if (f) err[0] = 1;
+    return;
+  }
+  uint32_t* ws = sh[w];
+  const V xr = lane < rows ? x[r] : V(0);
+  V acc = V(0);
+  uint32_t dsum = 0;
+  for (int64_t base = w0; base < w1; base += CSR_CAP) {
+    const int m = (int)min((int64_t)CSR_CAP, w1 - base);
+    for (int i0 = lane; i0 < m; i0 += 8 * 32) {
+      int32_t c[8], g[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) c[i] = i0 + 32 * i < m ? __ldcs(col + base + i0 + 32 * i) : 0;
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+        g[i] = wt && i0 + 32 * i < m ? __ldcs(wt + base + i0 + 32 * i) : 1;
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+        if (i0 + 32 * i < m) {
+          if ((uint32_t)c[i] >= (uint32_t)n) {
+            f |= 2;
+            c[i] = 0;
+          }
+          if (g[i] < 1 || g[i] > 7) f |= 8;
+          ws[i0 + 32 * i] = ((uint32_t)g[i] << RSB_COLBITS) | (uint32_t)c[i];
+        }
+    }
+    __syncwarp();
+    const int k1 = (int)(min(e, base + m) - base);
+    for (int k0 = (int)(max(b, base) - base); k0 < k1; k0 += 8) {
+      uint32_t p[8];
+      V xv[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) p[i] = k0 + i < k1 ? ws[k0 + i] : 0u;
+#pragma unroll
+      for (int i = 0; i < 8; ++i) xv[i] = k0 + i < k1 ? __ldg(x + ent_col(p[i])) : xr;
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+        if (k0 + i < k1) {
+          if (ent_col(p[i]) == (uint32_t)r) f |= 4;
+          if constexpr (sizeof(V) == 8) {
+            acc = fma(weight_f64(ent_w(p[i])), xv[i], acc);
+            dsum += ent_w(p[i]);
+          } else {
+            acc += V(ent_w(p[i])) * (xr - xv[i]);
+          }
+        }
+    }
+    __syncwarp();
+  }
+  if constexpr (sizeof(V) == 8) acc = fma((double)dsum, xr, -acc);
+  if (lane < rows) y[r] = acc;
+  if (f & 2) err[1] = 1;
+  if (f & 4) err[2] = 1;
+  if (f & 8) err[3] = 1;
+}
+
+int launch_csr_apply(const int64_t* row_ptr, const int32_t* col, const int32_t* wt, int64_t n,
+                     int f32, const void* x, void* y, int* err, cudaStream_t s) {
+  const unsigned nb = (unsigned)((n + RSB_BLOCK - 1) / RSB_BLOCK);
+  const int pi = prof_before(PROF_SPMV, s);
+  if (f32)
+    k_csr_apply<float><<<nb, RSB_BLOCK, 0, s>>>(row_ptr, col, wt, (int32_t)n, (const float*)x,
+                                                (float*)y, err);
+  else
+    k_csr_apply<double><<<nb, RSB_BLOCK, 0, s>>>(row_ptr, col, wt, (int32_t)n, (const double*)x,
+                                                 (double*)y, err);
+  RSB_CKL("k_csr_apply");
+  prof_after(pi, s);
+  return RSB_OK;
+}
+
+// ----------------------------------------------------------------------------
 // connected components: lock-free union-find (hook larger root under smaller)
 // ----------------------------------------------------------------------------
 // parent[x] <= x always holds, so every find() walk is finite; the hook retry

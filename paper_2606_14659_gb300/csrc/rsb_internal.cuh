@@ -788,6 +788,8 @@ int launch_scan_i64(const int64_t* in, int64_t* out_excl, int64_t n, void* tmp, 
 size_t scan_tmp_bytes(int64_t n);
 int launch_spmv_f64(const LevelGraph& G, const double* x, double* y, cudaStream_t s);
 int launch_spmv_f32(const LevelGraph& G, const float* x, float* y, cudaStream_t s);
+int launch_csr_apply(const int64_t* row_ptr, const int32_t* col, const int32_t* wt, int64_t n,
+                     int f32, const void* x, void* y, int* err, cudaStream_t s);
 int launch_cc(const LevelGraph& G, int32_t* parent, uint64_t* ckey, int* flag, cudaStream_t s);
 int launch_comp_count(const LevelGraph& G, const int32_t* parent, int32_t* seg_ncomp,
                       cudaStream_t s);
