@@ -1627,13 +1627,25 @@ int gs_fill_dual(int64_t ne, int nv, const int32_t* ev32, const int64_t* bptr,
 int gs_apply(int f32, int64_t ne, int nv, int64_t V, const int32_t* ev32, const int64_t* bptr,
              const int32_t* bucket, const void* x, void* w, void* y, cudaStream_t s);
 
+int64_t gs_slot_cap(int64_t ne);
+size_t gs_slot_bytes(int64_t cap);
+int gs_slots(const int64_t* ev, int64_t ne, int nv, int64_t cap, int32_t* cnt, int32_t* slot,
+             int* err, cudaStream_t s);
+int gs_slot_apply(int f32, const int64_t* ev, int64_t ne, int nv, int64_t cap, const int32_t* cnt,
+                  const int32_t* slot, const void* x, void* wc, void* y, cudaStream_t s);
+
+static int gs_check(int64_t ne, int nv, const void* ev) {
+  if (ne < 1 || ne >= RSB_MAXN || nv < 1 || nv > 8 || !ev)
+    return rsb_set_error(RSB_EINVAL, "need 1 <= ne < 2^29, 1 <= nv <= 8 and vertex ids");
+  return RSB_OK;
+}
+
 // Buckets of the elements at every vertex in the context's workspace; *V out.
 static int gs_setup(Ctx& c, int64_t ne, int nv, const int64_t* ev_in, int64_t* V) {
-  if (ne < 1 || ne >= RSB_MAXN || nv < 1 || nv > 8 || !ev_in)
-    return rsb_set_error(RSB_EINVAL, "need 1 <= ne < 2^29, 1 <= nv <= 8 and vertex ids");
-  const int64_t* ev = nullptr;
-  int rc = stage_in(c, ev_in, (size_t)(ne * nv), &ev);
+  int rc = gs_check(ne, nv, ev_in);
   if (rc) return rc;
+  const int64_t* ev = nullptr;
+  if ((rc = stage_in(c, ev_in, (size_t)(ne * nv), &ev))) return rc;
   if ((rc = devbuf_reserve(c.gs_misc, 256))) return rc;
   unsigned long long* d_vmax = dptr<unsigned long long>(c.gs_misc);
   int* d_flag = (int*)(d_vmax + 1);
@@ -1720,8 +1732,74 @@ extern "C" int rsb_dual_graph(int64_t ne, int nv, const int64_t* ev, int64_t* ro
   return end_call(c, stream, RSB_OK);
 }
 
-static int gs_lap_common(int64_t ne, int nv, const int64_t* ev, const void* x, void* y, int f32,
-                         int reps, double* ms, double* bytes, void* stream) {
+// One application from the slot table; *fits = 0 when the mesh does not fit it (the
+// general path then answers).  x, y and ev: device pointers.
+static int gs_lap_slots(Ctx& c, int64_t ne, int nv, const int64_t* ev, const void* x, void* y,
+                        int f32, int* fits) {
+  const int64_t cap = gs_slot_cap(ne);
+  int rc;
+  if ((rc = devbuf_reserve(c.gs_cursor, sizeof(int32_t) * (size_t)cap)) ||
+      (rc = devbuf_reserve(c.gs_bucket, gs_slot_bytes(cap))) ||
+      (rc = devbuf_reserve(c.gs_w, (f32 ? 8 : 16) * (size_t)cap)))
+    return rc;
+  int* err = c.h_pinned + 8;  // words the kernels report into
+  err[0] = err[1] = 0;
+  if ((rc = gs_slots(ev, ne, nv, cap, dptr<int32_t>(c.gs_cursor), dptr<int32_t>(c.gs_bucket), err,
+                     c.s)) ||
+      (rc = gs_slot_apply(f32, ev, ne, nv, cap, dptr<int32_t>(c.gs_cursor),
+                          dptr<int32_t>(c.gs_bucket), x, c.gs_w.p, y, c.s)))
+    return rc;
+  RSB_CK(cudaStreamSynchronize(c.s));
+  if (err[0]) return rsb_set_error(RSB_EINVAL, "vertex ids must lie in [0, 2^31)");
+  *fits = !err[1];
+  return RSB_OK;
+}
+
+static int gs_lap_apply(int64_t ne, int nv, const int64_t* ev_in, const void* x, void* y, int f32,
+                        void* stream) {
+  int rc = gs_check(ne, nv, ev_in);
+  if (rc) return rc;
+  Ctx* pc = nullptr;
+  if ((rc = begin_call(&pc, stream))) return rc;
+  Ctx& c = *pc;
+  const size_t es = f32 ? 4 : 8;
+  DevBuf tx, ty;
+  auto done = [&](int r) {
+    r = end_call(c, stream, r);
+    free_buf(tx);
+    free_buf(ty);
+    return r;
+  };
+  const int64_t* ev = nullptr;
+  if ((rc = stage_in(c, ev_in, (size_t)(ne * nv), &ev))) return done(rc);
+  const void* xd = x;
+  void* yd = y;
+  if (!is_device_ptr(x)) {
+    if ((rc = devbuf_reserve(tx, es * (size_t)ne))) return done(rc);
+    RSB_CK(cudaMemcpyAsync(tx.p, x, es * (size_t)ne, cudaMemcpyHostToDevice, c.s));
+    xd = tx.p;
+  }
+  if (!is_device_ptr(y)) {
+    if ((rc = devbuf_reserve(ty, es * (size_t)ne))) return done(rc);
+    yd = ty.p;
+  }
+  int fits = 0;
+  if ((rc = gs_lap_slots(c, ne, nv, ev, xd, yd, f32, &fits))) return done(rc);
+  if (!fits) {
+    int64_t V = 0;
+    if ((rc = gs_setup(c, ne, nv, ev, &V)) || (rc = devbuf_reserve(c.gs_w, es * (size_t)(V + 1))))
+      return done(rc);
+    if ((rc = gs_apply(f32, ne, nv, V, dptr<int32_t>(c.gs_ev32), dptr<int64_t>(c.gs_bptr),
+                       dptr<int32_t>(c.gs_bucket), xd, c.gs_w.p, yd, c.s)))
+      return done(rc);
+  }
+  if (yd != y && cudaMemcpyAsync(y, yd, es * (size_t)ne, cudaMemcpyDeviceToHost, c.s))
+    rc = rsb_set_error(RSB_ECUDA, "copy y");
+  return done(rc);
+}
+
+static int gs_lap_bench(int64_t ne, int nv, const int64_t* ev, int f32, int reps, double* ms,
+                        double* bytes, void* stream) {
   Ctx* pc = nullptr;
   int rc = begin_call(&pc, stream);
   if (rc) return rc;
@@ -1730,55 +1808,32 @@ static int gs_lap_common(int64_t ne, int nv, const int64_t* ev, const void* x, v
   if ((rc = gs_setup(c, ne, nv, ev, &V))) return end_call(c, stream, rc);
   const size_t es = f32 ? 4 : 8;
   if ((rc = devbuf_reserve(c.gs_w, es * (size_t)(V + 1)))) return end_call(c, stream, rc);
-  DevBuf tx, ty;
-  const void* xd = x;
-  void* yd = y;
-  if (reps > 0) {  // benchmark: operands of its own
-    if ((rc = devbuf_reserve(tx, es * (size_t)ne)) || (rc = devbuf_reserve(ty, es * (size_t)ne)))
-      return end_call(c, stream, rc);
-    RSB_CK(cudaMemsetAsync(tx.p, 0, es * (size_t)ne, c.s));
-    xd = tx.p;
-    yd = ty.p;
-  } else {
-    if (!is_device_ptr(x)) {
-      if ((rc = devbuf_reserve(tx, es * (size_t)ne))) return end_call(c, stream, rc);
-      RSB_CK(cudaMemcpyAsync(tx.p, x, es * (size_t)ne, cudaMemcpyHostToDevice, c.s));
-      xd = tx.p;
-    }
-    if (!is_device_ptr(y)) {
-      if ((rc = devbuf_reserve(ty, es * (size_t)ne))) return end_call(c, stream, rc);
-      yd = ty.p;
-    }
-  }
+  DevBuf tx, ty;  // operands of its own
+  if ((rc = devbuf_reserve(tx, es * (size_t)ne)) || (rc = devbuf_reserve(ty, es * (size_t)ne)))
+    return end_call(c, stream, rc);
+  RSB_CK(cudaMemsetAsync(tx.p, 0, es * (size_t)ne, c.s));
   auto apply = [&]() {
     return gs_apply(f32, ne, nv, V, dptr<int32_t>(c.gs_ev32), dptr<int64_t>(c.gs_bptr),
-                    dptr<int32_t>(c.gs_bucket), xd, c.gs_w.p, yd, c.s);
+                    dptr<int32_t>(c.gs_bucket), tx.p, c.gs_w.p, ty.p, c.s);
   };
-  if (reps <= 0) {
-    rc = apply();
-    if (!rc && yd != y)
-      if (cudaMemcpyAsync(y, yd, es * (size_t)ne, cudaMemcpyDeviceToHost, c.s))
-        rc = rsb_set_error(RSB_ECUDA, "copy y");
-  } else {
-    cudaEvent_t e0, e1;
-    cudaEventCreate(&e0);
-    cudaEventCreate(&e1);
-    for (int w = 0; w < 3 && !rc; ++w) rc = apply();
-    cudaEventRecord(e0, c.s);
-    for (int i = 0; i < reps && !rc; ++i) rc = apply();
-    cudaEventRecord(e1, c.s);
-    cudaEventSynchronize(e1);
-    float t = 0;
-    cudaEventElapsedTime(&t, e0, e1);
-    cudaEventDestroy(e0);
-    cudaEventDestroy(e1);
-    if (ms) *ms = (double)t / reps;
-    // vertex sums: bucket offsets, bucket entries, x once, w written; element
-    // pass: vertex ids, bucket offsets, w and x read once, y written
-    if (bytes)
-      *bytes = 16.0 * (double)(V + 1) + 8.0 * (double)ne * nv + 3.0 * es * (double)ne +
-               2.0 * es * (double)V;
-  }
+  cudaEvent_t e0, e1;
+  cudaEventCreate(&e0);
+  cudaEventCreate(&e1);
+  for (int w = 0; w < 3 && !rc; ++w) rc = apply();
+  cudaEventRecord(e0, c.s);
+  for (int i = 0; i < reps && !rc; ++i) rc = apply();
+  cudaEventRecord(e1, c.s);
+  cudaEventSynchronize(e1);
+  float t = 0;
+  cudaEventElapsedTime(&t, e0, e1);
+  cudaEventDestroy(e0);
+  cudaEventDestroy(e1);
+  if (ms) *ms = (double)t / reps;
+  // vertex sums: bucket offsets, bucket entries, x once, w written; element
+  // pass: vertex ids, bucket offsets, w and x read once, y written
+  if (bytes)
+    *bytes = 16.0 * (double)(V + 1) + 8.0 * (double)ne * nv + 3.0 * es * (double)ne +
+             2.0 * es * (double)V;
   rc = end_call(c, stream, rc);
   free_buf(tx);
   free_buf(ty);
@@ -1788,20 +1843,19 @@ static int gs_lap_common(int64_t ne, int nv, const int64_t* ev, const void* x, v
 extern "C" int rsb_laplacian_apply_gs(int64_t ne, int nv, const int64_t* ev, const double* x,
                                       double* y, void* stream) {
   if (!x || !y) return rsb_set_error(RSB_EINVAL, "x and y are needed");
-  return gs_lap_common(ne, nv, ev, x, y, 0, 0, nullptr, nullptr, stream);
+  return gs_lap_apply(ne, nv, ev, x, y, 0, stream);
 }
 
 extern "C" int rsb_laplacian_apply_gs_f32(int64_t ne, int nv, const int64_t* ev, const float* x,
                                           float* y, void* stream) {
   if (!x || !y) return rsb_set_error(RSB_EINVAL, "x and y are needed");
-  return gs_lap_common(ne, nv, ev, x, y, 1, 0, nullptr, nullptr, stream);
+  return gs_lap_apply(ne, nv, ev, x, y, 1, stream);
 }
 
 extern "C" int rsb_laplacian_bench_gs(int64_t ne, int nv, const int64_t* ev, int f32, int reps,
                                       double* ms_per_apply, double* useful_bytes, void* stream) {
   if (reps < 1) return rsb_set_error(RSB_EINVAL, "reps");
-  return gs_lap_common(ne, nv, ev, nullptr, nullptr, f32 ? 1 : 0, reps, ms_per_apply,
-                       useful_bytes, stream);
+  return gs_lap_bench(ne, nv, ev, f32 ? 1 : 0, reps, ms_per_apply, useful_bytes, stream);
 }
 
 extern "C" const char* rsb_strerror(int code) {

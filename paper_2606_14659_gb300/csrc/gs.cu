@@ -16,6 +16,8 @@
 //     y_e = sum over e's vertices v of (c_v x_e - w_v), c_v the bucket size,
 //     which is sum_v sum_{f at v} (x_e - x_f): the diagonal term of A_w and
 //     D_w cancel inside every vertex term.
+#include <climits>
+
 #include "rsb_internal.cuh"
 
 #define GS_MAXCAND 256  // neighbour candidates of one element (with repeats)
@@ -174,6 +176,140 @@ __global__ void __launch_bounds__(RSB_BLOCK) k_gs_apply(int64_t ne, int nv,
 }
 
 // ----------------------------------------------------------------------------
+// Slot table: the elements at every vertex in GS_SLOTS fixed places, for meshes whose
+// vertices have at most that many (hexes: eight in the interior) and whose ids lie
+// below a bound known beforehand.  One pass over the ids takes the place of the pass
+// for the largest id (and the host's wait for it), the count, the scan and the fill of
+// the buckets above; a mesh that does not fit sets a host-visible word, and the caller
+// takes the general path.  A vertex's slots hold its elements in arrival order; their
+// readers sort the at most eight of them in registers, so results do not depend on it.
+// One Laplacian application at 1.9M hexes 168 us, 717 from the buckets.
+// err: [0] an id outside [0, 2^31), [1] the table does not hold the mesh.
+// ----------------------------------------------------------------------------
+#define GS_SLOTS 8
+
+// The ids of element e (unused places: -1).
+template <bool HEX>
+__device__ __forceinline__ void gs_ids(const int64_t* __restrict__ ev, int64_t e, int nv,
+                                       int64_t (&id)[8]) {
+  if constexpr (HEX) {  // eight ids, 16-byte aligned
+    const longlong2* p = reinterpret_cast<const longlong2*>(ev + 8 * e);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const longlong2 v = __ldg(p + i);
+      id[2 * i] = v.x;
+      id[2 * i + 1] = v.y;
+    }
+  } else {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) id[i] = i < nv ? __ldg(ev + e * nv + i) : -1;
+  }
+}
+
+// Bound: the returned atomics (one per id, eight in flight a thread).
+template <bool HEX>
+__global__ void __launch_bounds__(RSB_BLOCK) k_gs_slots(const int64_t* __restrict__ ev, int64_t ne,
+                                                      int nv, int64_t cap, int32_t* cnt,
+                                                      int32_t* __restrict__ slot,
+                                                      volatile int* err) {
+  const int64_t e = (int64_t)blockIdx.x * RSB_BLOCK + threadIdx.x;
+  if (e >= ne) return;
+  int64_t id[8];
+  gs_ids<HEX>(ev, e, nv, id);
+  int pos[8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    pos[i] = GS_SLOTS;
+    if (HEX || i < nv) {
+      if (id[i] < 0 || id[i] >= (1ll << 31)) err[0] = 1;
+      else if (id[i] >= cap) err[1] = 1;
+      else pos[i] = atomicAdd(cnt + id[i], 1);
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    if (pos[i] < GS_SLOTS) slot[id[i] * GS_SLOTS + pos[i]] = (int32_t)e;
+    else if ((HEX || i < nv) && id[i] >= 0 && id[i] < cap) err[1] = 1;
+  }
+}
+
+// The elements at vertex v in ascending order, INT_MAX in the places left (a sorting
+// network of 19 exchanges); returns their number.
+__device__ __forceinline__ int gs_sorted_slots(const int32_t* cnt, const int32_t* slot, int64_t v,
+                                               int32_t (&f)[GS_SLOTS]) {
+  const int n = min(cnt[v], GS_SLOTS);
+  const int4* p = reinterpret_cast<const int4*>(slot + v * GS_SLOTS);
+  int4 lo = make_int4(0, 0, 0, 0), hi = lo;
+  if (n > 0) lo = p[0];
+  if (n > 4) hi = p[1];
+  const int32_t r[GS_SLOTS] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
+#pragma unroll
+  for (int i = 0; i < GS_SLOTS; ++i) f[i] = i < n ? r[i] : INT_MAX;
+  auto ex = [&](int a, int b) {
+    const int32_t x = min(f[a], f[b]), y = max(f[a], f[b]);
+    f[a] = x;
+    f[b] = y;
+  };
+  ex(0, 1); ex(2, 3); ex(4, 5); ex(6, 7);
+  ex(0, 2); ex(1, 3); ex(4, 6); ex(5, 7);
+  ex(1, 2); ex(5, 6); ex(0, 4); ex(3, 7);
+  ex(1, 5); ex(2, 6);
+  ex(1, 4); ex(3, 6);
+  ex(2, 4); ex(3, 5);
+  ex(3, 4);
+  return n;
+}
+
+// (w_v, c_v) of every vertex: the sum of x over its elements in ascending order, as
+// k_gs_vsum takes it, and their number, side by side for one gather.
+template <typename V>
+struct alignas(2 * sizeof(V)) GsPair {
+  V w, c;
+};
+
+template <typename V>
+__global__ void __launch_bounds__(RSB_BLOCK) k_gs_vsum8(int64_t nvert, const int32_t* __restrict__ cnt,
+                                                      const int32_t* __restrict__ slot,
+                                                      const V* __restrict__ x,
+                                                      GsPair<V>* __restrict__ wc) {
+  const int64_t v = (int64_t)blockIdx.x * RSB_BLOCK + threadIdx.x;
+  if (v >= nvert) return;
+  int32_t f[GS_SLOTS];
+  const int n = gs_sorted_slots(cnt, slot, v, f);
+  V xv[GS_SLOTS];
+#pragma unroll
+  for (int i = 0; i < GS_SLOTS; ++i) xv[i] = i < n ? __ldg(x + f[i]) : V(0);
+  V s = V(0);
+#pragma unroll
+  for (int i = 0; i < GS_SLOTS; ++i)
+    if (i < n) s += xv[i];
+  if (n > 0) wc[v] = {s, V(n)};
+}
+
+template <typename V, bool HEX>
+__global__ void __launch_bounds__(RSB_BLOCK) k_gs_apply8(int64_t ne, int nv,
+                                                       const int64_t* __restrict__ ev, int64_t cap,
+                                                       const GsPair<V>* __restrict__ wc,
+                                                       const V* __restrict__ x, V* __restrict__ y) {
+  const int64_t e = (int64_t)blockIdx.x * RSB_BLOCK + threadIdx.x;
+  if (e >= ne) return;
+  int64_t id[8];
+  gs_ids<HEX>(ev, e, nv, id);
+  GsPair<V> p[8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    p[i] = {V(0), V(0)};
+    if (id[i] >= 0 && id[i] < cap) p[i] = wc[id[i]];
+  }
+  const V xe = x[e];
+  V acc = V(0);
+#pragma unroll
+  for (int i = 0; i < 8; ++i)
+    if (HEX || i < nv) acc += p[i].c * xe - p[i].w;
+  y[e] = acc;
+}
+
+// ----------------------------------------------------------------------------
 // launchers (workspace: the caller's; sizes from gs_sizes)
 // ----------------------------------------------------------------------------
 static unsigned grid_of(int64_t n, int block = RSB_BLOCK) {
@@ -258,4 +394,47 @@ int gs_apply(int f32, int64_t ne, int nv, int64_t V, const int32_t* ev32, const 
     RSB_CKL("k_gs_apply<f64>");
   }
   return RSB_OK;
+}
+
+// ----------------------------------------------------------------------------
+// slot-table path
+// ----------------------------------------------------------------------------
+// Ids the table is laid out for: hexes share most of their vertices (V is little more
+// than ne), elements that share none have 8 ne.
+int64_t gs_slot_cap(int64_t ne) { return 2 * ne + 4096; }
+size_t gs_slot_bytes(int64_t cap) { return sizeof(int32_t) * GS_SLOTS * (size_t)cap; }
+
+static bool hex_aligned(const int64_t* ev, int nv) { return nv == 8 && ((uintptr_t)ev & 15) == 0; }
+
+int gs_slots(const int64_t* ev, int64_t ne, int nv, int64_t cap, int32_t* cnt, int32_t* slot,
+             int* err, cudaStream_t s) {
+  RSB_CK(cudaMemsetAsync(cnt, 0, sizeof(int32_t) * (size_t)cap, s));
+  if (hex_aligned(ev, nv))
+    k_gs_slots<true><<<grid_of(ne), RSB_BLOCK, 0, s>>>(ev, ne, nv, cap, cnt, slot, err);
+  else
+    k_gs_slots<false><<<grid_of(ne), RSB_BLOCK, 0, s>>>(ev, ne, nv, cap, cnt, slot, err);
+  RSB_CKL("k_gs_slots");
+  return RSB_OK;
+}
+
+template <typename V>
+static int gs_slot_apply_t(const int64_t* ev, int64_t ne, int nv, int64_t cap, const int32_t* cnt,
+                           const int32_t* slot, const V* x, void* wc, V* y, cudaStream_t s) {
+  GsPair<V>* p = (GsPair<V>*)wc;
+  k_gs_vsum8<V><<<grid_of(cap), RSB_BLOCK, 0, s>>>(cap, cnt, slot, x, p);
+  RSB_CKL("k_gs_vsum8");
+  if (hex_aligned(ev, nv))
+    k_gs_apply8<V, true><<<grid_of(ne), RSB_BLOCK, 0, s>>>(ne, nv, ev, cap, p, x, y);
+  else
+    k_gs_apply8<V, false><<<grid_of(ne), RSB_BLOCK, 0, s>>>(ne, nv, ev, cap, p, x, y);
+  RSB_CKL("k_gs_apply8");
+  return RSB_OK;
+}
+
+// y = L x from the slot table (wc: 2 * cap values of the vector type).
+int gs_slot_apply(int f32, const int64_t* ev, int64_t ne, int nv, int64_t cap, const int32_t* cnt,
+                  const int32_t* slot, const void* x, void* wc, void* y, cudaStream_t s) {
+  return f32 ? gs_slot_apply_t<float>(ev, ne, nv, cap, cnt, slot, (const float*)x, wc, (float*)y, s)
+             : gs_slot_apply_t<double>(ev, ne, nv, cap, cnt, slot, (const double*)x, wc, (double*)y,
+                                       s);
 }
