@@ -281,7 +281,7 @@ struct Ctx {
   DevBuf coords_cat;            // RCB: (x, y, z) per element, caller order, meshes concatenated
   DevBuf perm, iperm, rcb_home;  // RCB reordering: new row -> caller row and back
   // gather-scatter (element -> vertex ids): buckets of elements per vertex
-  DevBuf gs_count, gs_cursor, gs_bptr, gs_bucket, gs_ev32, gs_len, gs_rowptr, gs_w, gs_misc;
+  DevBuf gs_count, gs_cursor, gs_bptr, gs_bucket, gs_ev32, gs_len, gs_rowptr, gs_w, gs_misc, gs_rows;
   DevBuf part_concat;
   int trmax = 0;    // largest tile of the level being solved, rows
   int ntmax = 0;    // most tiles of one of its units
@@ -1634,6 +1634,12 @@ int gs_slots(const int64_t* ev, int64_t ne, int nv, int64_t cap, int32_t* cnt, i
 int gs_slot_apply(int f32, const int64_t* ev, int64_t ne, int nv, int64_t cap, const int32_t* cnt,
                   const int32_t* slot, const void* x, void* wc, void* y, cudaStream_t s);
 
+size_t gs_rows_bytes(int64_t ne);
+int gs_slot_rows(const int64_t* ev, int64_t ne, int nv, int64_t cap, const int32_t* cnt,
+                 int32_t* slot, uint32_t* ent, int64_t* len, int* err, cudaStream_t s);
+int gs_slot_write(int64_t ne, const uint32_t* ent, const int64_t* row_ptr, int32_t* col,
+                  int32_t* wt, cudaStream_t s);
+
 static int gs_check(int64_t ne, int nv, const void* ev) {
   if (ne < 1 || ne >= RSB_MAXN || nv < 1 || nv > 8 || !ev)
     return rsb_set_error(RSB_EINVAL, "need 1 <= ne < 2^29, 1 <= nv <= 8 and vertex ids");
@@ -1664,7 +1670,59 @@ static int gs_setup(Ctx& c, int64_t ne, int nv, const int64_t* ev_in, int64_t* V
                     dptr<int32_t>(c.gs_ev32), c.scan_tmp.p, c.scan_tmp.cap, c.s);
 }
 
-extern "C" int rsb_dual_graph(int64_t ne, int nv, const int64_t* ev, int64_t* row_ptr,
+// Row lengths and offsets of the dual graph in c.gs_rowptr, their total in *total: from
+// the slot table (with want_rows, the rows in c.gs_rows as well) when the mesh fits it
+// (*slots = 1), else from the buckets.
+static int dual_rows(Ctx& c, int64_t ne, int nv, const int64_t* ev, bool want_rows, int64_t* total,
+                     int* slots) {
+  int rc;
+  const int64_t cap = gs_slot_cap(ne);
+  if ((rc = devbuf_reserve(c.gs_cursor, sizeof(int32_t) * (size_t)cap)) ||
+      (rc = devbuf_reserve(c.gs_bucket, gs_slot_bytes(cap))) ||
+      (rc = devbuf_reserve(c.gs_len, sizeof(int64_t) * (size_t)(ne + 2))) ||
+      (rc = devbuf_reserve(c.gs_rowptr, sizeof(int64_t) * (size_t)(ne + 2))) ||
+      (rc = devbuf_reserve(c.scan_tmp, scan_tmp_bytes(ne + 2))) ||
+      (want_rows && (rc = devbuf_reserve(c.gs_rows, gs_rows_bytes(ne)))))
+    return rc;
+  int64_t* len = dptr<int64_t>(c.gs_len);
+  int64_t* rp = dptr<int64_t>(c.gs_rowptr);
+  int* err = c.h_pinned + 8;
+  err[0] = err[1] = err[2] = 0;
+  if ((rc = gs_slots(ev, ne, nv, cap, dptr<int32_t>(c.gs_cursor), dptr<int32_t>(c.gs_bucket), err,
+                     c.s)) ||
+      (rc = gs_slot_rows(ev, ne, nv, cap, dptr<int32_t>(c.gs_cursor), dptr<int32_t>(c.gs_bucket),
+                         want_rows ? dptr<uint32_t>(c.gs_rows) : nullptr, len, err, c.s)))
+    return rc;
+  RSB_CK(cudaMemsetAsync(len + ne, 0, sizeof(int64_t), c.s));
+  if ((rc = launch_scan_i64(len, rp, ne + 1, c.scan_tmp.p, c.scan_tmp.cap, c.s))) return rc;
+  RSB_CK(cudaMemcpyAsync(total, rp + ne, sizeof(int64_t), cudaMemcpyDeviceToHost, c.s));
+  RSB_CK(cudaStreamSynchronize(c.s));
+  if (err[0]) return rsb_set_error(RSB_EINVAL, "vertex ids must lie in [0, 2^31)");
+  int flag = err[2] ? 4 : 0;
+  *slots = !err[1];
+  if (!*slots) {
+    int64_t V = 0;
+    if ((rc = gs_setup(c, ne, nv, ev, &V))) return rc;
+    int* d_flag = (int*)(dptr<unsigned long long>(c.gs_misc) + 1);
+    if ((rc = gs_row_lengths(ne, nv, dptr<int32_t>(c.gs_ev32), dptr<int64_t>(c.gs_bptr),
+                             dptr<int32_t>(c.gs_bucket), len, d_flag, c.s)))
+      return rc;
+    RSB_CK(cudaMemsetAsync(len + ne, 0, sizeof(int64_t), c.s));
+    if ((rc = launch_scan_i64(len, rp, ne + 1, c.scan_tmp.p, c.scan_tmp.cap, c.s))) return rc;
+    RSB_CK(cudaMemcpyAsync(total, rp + ne, sizeof(int64_t), cudaMemcpyDeviceToHost, c.s));
+    RSB_CK(cudaMemcpyAsync(&flag, d_flag, sizeof(int), cudaMemcpyDeviceToHost, c.s));
+    RSB_CK(cudaStreamSynchronize(c.s));
+  }
+  if (flag & 2)
+    return rsb_set_error(RSB_EINVAL, "an element meets more than 256 other elements at its "
+                                     "vertices");
+  if (flag & 4)
+    return rsb_set_error(RSB_EINVAL, "two elements share more than 7 vertices (duplicate "
+                                     "elements)");
+  return RSB_OK;
+}
+
+extern "C" int rsb_dual_graph(int64_t ne, int nv, const int64_t* ev_in, int64_t* row_ptr,
                               int32_t* col, int32_t* weight, int64_t cap, int64_t* nnz,
                               void* stream) {
   if (!row_ptr || !nnz) return rsb_set_error(RSB_EINVAL, "row_ptr and nnz are needed");
@@ -1672,33 +1730,14 @@ extern "C" int rsb_dual_graph(int64_t ne, int nv, const int64_t* ev, int64_t* ro
   int rc = begin_call(&pc, stream);
   if (rc) return rc;
   Ctx& c = *pc;
-  int64_t V = 0;
-  if ((rc = gs_setup(c, ne, nv, ev, &V))) return end_call(c, stream, rc);
-  int* d_flag = (int*)(dptr<unsigned long long>(c.gs_misc) + 1);
-  if ((rc = devbuf_reserve(c.gs_len, sizeof(int64_t) * (size_t)(ne + 2))) ||
-      (rc = devbuf_reserve(c.gs_rowptr, sizeof(int64_t) * (size_t)(ne + 2))))
-    return end_call(c, stream, rc);
-  int64_t* len = dptr<int64_t>(c.gs_len);
-  int64_t* rp = dptr<int64_t>(c.gs_rowptr);
-  const int32_t* ev32 = dptr<int32_t>(c.gs_ev32);
-  const int64_t* bptr = dptr<int64_t>(c.gs_bptr);
-  const int32_t* bucket = dptr<int32_t>(c.gs_bucket);
-  if ((rc = gs_row_lengths(ne, nv, ev32, bptr, bucket, len, d_flag, c.s)))
-    return end_call(c, stream, rc);
-  RSB_CK(cudaMemsetAsync(len + ne, 0, sizeof(int64_t), c.s));
-  if ((rc = launch_scan_i64(len, rp, ne + 1, c.scan_tmp.p, c.scan_tmp.cap, c.s)))
+  const int64_t* ev = nullptr;
+  if ((rc = gs_check(ne, nv, ev_in)) || (rc = stage_in(c, ev_in, (size_t)(ne * nv), &ev)))
     return end_call(c, stream, rc);
   int64_t total = 0;
-  int flag = 0;
-  RSB_CK(cudaMemcpyAsync(&total, rp + ne, sizeof(int64_t), cudaMemcpyDeviceToHost, c.s));
-  RSB_CK(cudaMemcpyAsync(&flag, d_flag, sizeof(int), cudaMemcpyDeviceToHost, c.s));
-  RSB_CK(cudaStreamSynchronize(c.s));
-  if (flag & 2)
-    return end_call(c, stream, rsb_set_error(RSB_EINVAL, "an element meets more than 256 "
-                                                         "other elements at its vertices"));
-  if (flag & 4)
-    return end_call(c, stream, rsb_set_error(RSB_EINVAL, "two elements share more than 7 "
-                                                         "vertices (duplicate elements)"));
+  int slots = 0;
+  if ((rc = dual_rows(c, ne, nv, ev, col && weight, &total, &slots)))
+    return end_call(c, stream, rc);
+  const int64_t* rp = dptr<int64_t>(c.gs_rowptr);
   *nnz = total;
   RSB_CK(cudaMemcpyAsync(row_ptr, rp, sizeof(int64_t) * (size_t)(ne + 1), cudaMemcpyDefault, c.s));
   if (col || weight) {
@@ -1717,7 +1756,9 @@ extern "C" int rsb_dual_graph(int64_t ne, int nv, const int64_t* ev, int64_t* ro
     }
     if (!cd) colp = (int32_t*)tc.p;
     if (!wd) wtp = (int32_t*)tw.p;
-    rc = gs_fill_dual(ne, nv, ev32, bptr, bucket, rp, colp, wtp, c.s);
+    rc = slots ? gs_slot_write(ne, dptr<uint32_t>(c.gs_rows), rp, colp, wtp, c.s)
+               : gs_fill_dual(ne, nv, dptr<int32_t>(c.gs_ev32), dptr<int64_t>(c.gs_bptr),
+                              dptr<int32_t>(c.gs_bucket), rp, colp, wtp, c.s);
     if (!rc && !cd)
       if (cudaMemcpyAsync(col, colp, sizeof(int32_t) * total, cudaMemcpyDeviceToHost, c.s))
         rc = rsb_set_error(RSB_ECUDA, "copy col");
@@ -1891,7 +1932,7 @@ extern "C" void rsb_release(void) {
                      &c->seg_ncomp, &c->counters, &c->part_concat, &c->blk, &c->coords_cat,
                      &c->perm, &c->iperm, &c->rcb_home, &c->gs_count, &c->gs_cursor,
                      &c->gs_bptr, &c->gs_bucket, &c->gs_ev32, &c->gs_len, &c->gs_rowptr,
-                     &c->gs_w, &c->gs_misc};
+                     &c->gs_w, &c->gs_misc, &c->gs_rows};
     for (DevBuf* b : all) free_buf(*b);
     for (int k = 0; k < 2; ++k) {
       PrecBufs& p = c->pb[k];

@@ -364,13 +364,22 @@ def rsb_dual_graph(ev, device: str = "cuda", stream=None):
     rp = torch.empty(ne + 1, dtype=torch.int64, device=dev)
     nnz = C.c_int64(0)
     st = _stream(stream)
-    _check(lib.rsb_dual_graph(ne, nv, _ptr(evt), _ptr(rp), None, None, 0, C.byref(nnz), st),
-           "rsb_dual_graph")
-    col = torch.empty(max(nnz.value, 1), dtype=torch.int32, device=dev)
-    w = torch.empty(max(nnz.value, 1), dtype=torch.int32, device=dev)
-    _check(lib.rsb_dual_graph(ne, nv, _ptr(evt), _ptr(rp), _ptr(col), _ptr(w), nnz.value,
-                              C.byref(nnz), st), "rsb_dual_graph")
-    return ne, rp, col[:nnz.value], w[:nnz.value]
+    # one call with room for 26 neighbours an element (the interior of a hex mesh; the
+    # call says when that is too little), a second with the exact room otherwise
+    cap = 26 * ne
+    for _ in range(2):
+        col = torch.empty(max(cap, 1), dtype=torch.int32, device=dev)
+        w = torch.empty(max(cap, 1), dtype=torch.int32, device=dev)
+        code = lib.rsb_dual_graph(ne, nv, _ptr(evt), _ptr(rp), _ptr(col), _ptr(w), cap,
+                                  C.byref(nnz), st)
+        if code != RSB_EINVAL or nnz.value <= cap:
+            break
+        cap = nnz.value
+    _check(code, "rsb_dual_graph")
+    col, w = col[:nnz.value], w[:nnz.value]
+    if nnz.value < cap // 2:  # do not hold on to room that is mostly unused
+        col, w = col.clone(), w.clone()
+    return ne, rp, col, w
 
 
 def rsb_laplacian_apply_gs(ev, x, y=None, stream=None):
