@@ -2452,6 +2452,7 @@ template <typename V>
 __global__ void __launch_bounds__(RSB_BLOCK) k_cg_init(LzArgs<V> a) {
   __shared__ double sm[RSB_WARPS];
   __shared__ double out[1];
+  __shared__ double sp[RED_FEW_DOUBLES(1)];
   const Tile t = a.tiles[blockIdx.x];
   Unit& u = a.units[t.unit];
   if (u.status != U_ACTIVE) return;
@@ -2467,12 +2468,13 @@ __global__ void __launch_bounds__(RSB_BLOCK) k_cg_init(LzArgs<V> a) {
   const double sum = block_sum(acc.get(), sm);
   if (threadIdx.x == 0) a.partials[blockIdx.x] = sum;
   if (last_cta(&u.cnt, u.ntile)) {
-    final_reduce(a.partials, a.stride, u.tile0, u.ntile, 1, out);
+    final_reduce_few(a.partials, a.stride, u.tile0, u.ntile, 1, out, sp);
     if (threadIdx.x == 0) {
       u.rr = out[0];
       u.bnorm = sqrt(out[0]);
       u.inner = 0;
       u.cg_done = 0;
+      u.gbar = 0;
     }
   }
 }
@@ -2482,6 +2484,7 @@ template <typename V>
 __global__ void __launch_bounds__(RSB_BLOCK) k_cg_ap(LzArgs<V> a) {
   __shared__ double sm[RSB_WARPS];
   __shared__ double out[1];
+  __shared__ double sp[RED_FEW_DOUBLES(1)];
   const Tile t = a.tiles[blockIdx.x];
   Unit& u = a.units[t.unit];
   if (u.status != U_ACTIVE || u.cg_done) return;
@@ -2498,7 +2501,7 @@ __global__ void __launch_bounds__(RSB_BLOCK) k_cg_ap(LzArgs<V> a) {
   const double sum = block_sum(acc.get(), sm);
   if (threadIdx.x == 0) a.partials[blockIdx.x] = sum;
   if (last_cta(&u.cnt, u.ntile)) {
-    final_reduce(a.partials, a.stride, u.tile0, u.ntile, 1, out);
+    final_reduce_few(a.partials, a.stride, u.tile0, u.ntile, 1, out, sp);
     if (threadIdx.x == 0) u.cg_alpha = u.rr / out[0];
   }
 }
@@ -2509,6 +2512,7 @@ __global__ void __launch_bounds__(RSB_BLOCK) k_cg_xr(LzArgs<V> a, double cg_tol,
                                                      int* n_cg) {
   __shared__ double sm[RSB_WARPS];
   __shared__ double out[2 + RSB_MAXD];
+  __shared__ double sp[RED_FEW_DOUBLES(2 + RSB_MAXD)];
   const Tile t = a.tiles[blockIdx.x];
   Unit& u = a.units[t.unit];
   if (u.status != U_ACTIVE || u.cg_done) return;
@@ -2531,7 +2535,7 @@ __global__ void __launch_bounds__(RSB_BLOCK) k_cg_xr(LzArgs<V> a, double cg_tol,
     if (threadIdx.x == 0) a.partials[(long long)c * a.stride + blockIdx.x] = sum;
   }
   if (last_cta(&u.cnt, u.ntile)) {
-    final_reduce(a.partials, a.stride, u.tile0, u.ntile, nv, out);
+    final_reduce_few(a.partials, a.stride, u.tile0, u.ntile, nv, out, sp);
     if (threadIdx.x == 0) {
       double cp2 = 0.0;
       u.cp[0] = out[1] * u.isn;
@@ -2584,6 +2588,7 @@ __global__ void __launch_bounds__(RSB_BLOCK) k_fcg_xr(LzArgs<V> a, double cg_tol
                                                       int* n_cg) {
   __shared__ double sm[RSB_WARPS];
   __shared__ double out[2 + RSB_MAXD];
+  __shared__ double sp[RED_FEW_DOUBLES(2 + RSB_MAXD)];
   const Tile t = a.tiles[blockIdx.x];
   Unit& u = a.units[t.unit];
   if (u.status != U_ACTIVE || u.cg_done) return;
@@ -2608,7 +2613,7 @@ __global__ void __launch_bounds__(RSB_BLOCK) k_fcg_xr(LzArgs<V> a, double cg_tol
     if (threadIdx.x == 0) a.partials[(long long)c * a.stride + blockIdx.x] = sum;
   }
   if (last_cta(&u.cnt, u.ntile)) {
-    final_reduce(a.partials, a.stride, u.tile0, u.ntile, nv, out);
+    final_reduce_few(a.partials, a.stride, u.tile0, u.ntile, nv, out, sp);
     if (threadIdx.x == 0) {
       double cp2 = 0.0;
       u.cp[0] = out[1] * u.isn;
@@ -2649,6 +2654,7 @@ template <typename V>
 __global__ void __launch_bounds__(RSB_BLOCK) k_fcg_z(LzArgs<V> a) {
   __shared__ double sm[RSB_WARPS];
   __shared__ double out[3 + RSB_MAXD];
+  __shared__ double sp[RED_FEW_DOUBLES(3 + RSB_MAXD)];
   const Tile t = a.tiles[blockIdx.x];
   Unit& u = a.units[t.unit];
   if (u.status != U_ACTIVE || u.cg_done) return;
@@ -2673,7 +2679,7 @@ __global__ void __launch_bounds__(RSB_BLOCK) k_fcg_z(LzArgs<V> a) {
     if (threadIdx.x == 0) a.partials[(long long)c * a.stride + blockIdx.x] = sum;
   }
   if (last_cta(&u.cnt, u.ntile)) {
-    final_reduce(a.partials, a.stride, u.tile0, u.ntile, nv, out);
+    final_reduce_few(a.partials, a.stride, u.tile0, u.ntile, nv, out, sp);
     if (threadIdx.x == 0) {
       u.fz_rz = out[0];
       u.fz_ro = out[1];
@@ -2717,6 +2723,7 @@ template <typename V>
 __global__ void __launch_bounds__(RSB_BLOCK) k_inv_rq(LzArgs<V> a) {
   __shared__ double sm[RSB_WARPS];
   __shared__ double out[2];
+  __shared__ double sp[RED_FEW_DOUBLES(2)];
   const Tile t = a.tiles[blockIdx.x];
   Unit& u = a.units[t.unit];
   if (u.status != U_ACTIVE) return;
@@ -2734,7 +2741,7 @@ __global__ void __launch_bounds__(RSB_BLOCK) k_inv_rq(LzArgs<V> a) {
     if (threadIdx.x == 0) a.partials[(long long)c * a.stride + blockIdx.x] = sum;
   }
   if (last_cta(&u.cnt, u.ntile)) {
-    final_reduce(a.partials, a.stride, u.tile0, u.ntile, 2, out);
+    final_reduce_few(a.partials, a.stride, u.tile0, u.ntile, 2, out, sp);
     if (threadIdx.x == 0) {
       u.theta = out[0] / out[1];
       u.ynorm2 = out[1];
@@ -2748,6 +2755,7 @@ template <typename V>
 __global__ void __launch_bounds__(RSB_BLOCK) k_inv_res(LzArgs<V> a, int max_outer, int refine) {
   __shared__ double sm[RSB_WARPS];
   __shared__ double out[2 + RSB_MAXD];
+  __shared__ double sp[RED_FEW_DOUBLES(2 + RSB_MAXD)];
   const Tile t = a.tiles[blockIdx.x];
   Unit& u = a.units[t.unit];
   if (u.status != U_ACTIVE) return;
@@ -2769,7 +2777,7 @@ __global__ void __launch_bounds__(RSB_BLOCK) k_inv_res(LzArgs<V> a, int max_oute
     if (threadIdx.x == 0) a.partials[(long long)c * a.stride + blockIdx.x] = sum;
   }
   if (last_cta(&u.cnt, u.ntile)) {
-    final_reduce(a.partials, a.stride, u.tile0, u.ntile, nv, out);
+    final_reduce_few(a.partials, a.stride, u.tile0, u.ntile, nv, out, sp);
     if (threadIdx.x == 0) {
       u.resid = sqrt(out[0] / u.ynorm2);
       u.cp[0] = out[1] * u.isn;
@@ -2790,6 +2798,174 @@ __global__ void __launch_bounds__(RSB_BLOCK) k_inv_res(LzArgs<V> a, int max_oute
       }
     }
   }
+}
+
+// ----------------------------------------------------------------------------
+// Resident CG (launch mode 3): one cooperative launch runs the CG solve of every unit
+// when every tile gets a co-resident CTA.  x, r, p and L p of a tile's rows stay in
+// shared memory; global memory carries p (the SpMV's operand), the partials and the
+// unit's barrier.  Units iterate independently.  Rows, sums and their order are those
+// of k_cg_ap, k_cg_xr and k_cg_p, so both modes give the same numbers.
+// Bound: latency, three barriers and two reductions an iteration.  Three launches, each
+// with the chain of a last CTA's reduction, took 55 us an iteration at 256k rows (500
+// tiles).
+// ----------------------------------------------------------------------------
+template <typename V>
+constexpr size_t cg_res_smem(int trs) {
+  return 4 * res_align(sizeof(V) * (size_t)trs);
+}
+
+template <typename V>
+__global__ void __launch_bounds__(RSB_BLOCK, 4)
+    k_cg_res(LzArgs<V> a, int trs, double cg_tol, int cg_maxit, GridBar* gb) {
+  extern __shared__ __align__(16) unsigned char cg_sh[];
+  const size_t vb = res_align(sizeof(V) * (size_t)trs);
+  V* X = reinterpret_cast<V*>(cg_sh);
+  V* R = reinterpret_cast<V*>(cg_sh + vb);
+  V* P = reinterpret_cast<V*>(cg_sh + 2 * vb);
+  V* AP = reinterpret_cast<V*>(cg_sh + 3 * vb);
+  __shared__ double sm[RSB_WARPS];
+  __shared__ double out[2 + RSB_MAXD];
+  __shared__ double sp[RED_FEW_DOUBLES(2 + RSB_MAXD)];
+  __shared__ double rr_sh;
+  __shared__ V al_sh, be_sh, cp_sh[1 + RSB_MAXD];
+  __shared__ int done_sh;
+  const int tix = blockIdx.x;
+  const Tile t = a.tiles[tix];
+  Unit& u = a.units[t.unit];
+  if (__ldcg(&u.status) != U_ACTIVE) return;
+  const int nr = t.row1 - t.row0;
+  const int nd = u.nd, nv = 2 + nd, nt = u.ntile;
+  const bool first = tix == u.tile0;
+  const double bnorm = u.bnorm, isn = u.isn;
+  UnitBar ub(&u.gbar, nt, __ldcg(&gb->count), gb);
+  double* const P1 = a.partials;                       // p.Lp
+  double* const P2 = a.partials + a.stride;            // ||r||^2 and the projection of r
+  const V* Pg = a.P;
+  for (int rl = threadIdx.x; rl < nr; rl += RSB_BLOCK) {
+    X[rl] = V(0);
+    R[rl] = a.R[t.row0 + rl];
+    P[rl] = a.P[t.row0 + rl];
+  }
+  if (threadIdx.x == 0) {
+    rr_sh = u.rr;
+    done_sh = 0;
+  }
+  __syncthreads();
+  unsigned long long pbytes = 0;
+  int it = 0;
+  while (true) {
+    // AP = L P, p.Lp -> alpha
+    Acc<V> acc;
+    for (int rl = threadIdx.x; rl < nr; rl += RSB_BLOCK) {
+      const int r = t.row0 + rl;
+      const int64_t base = a.slice_ptr[r >> 5];
+      const int width = (int)((a.slice_ptr[(r >> 5) + 1] - base) >> 5);
+      const uint32_t* e = a.ent + base + (r & 31);
+      const V pr = P[rl];
+      V ap = V(0);
+      uint32_t dsum = 0;
+      for (int k0 = 0; k0 < width; k0 += 13) {
+        uint32_t p[13];
+        V xv[13];
+#pragma unroll
+        for (int i = 0; i < 13; ++i) p[i] = k0 + i < width ? __ldg(e + 32 * (k0 + i)) : 0u;
+#pragma unroll
+        for (int i = 0; i < 13; ++i) xv[i] = k0 + i < width ? __ldcg(Pg + ent_col(p[i])) : pr;
+#pragma unroll
+        for (int i = 0; i < 13; ++i)
+          if (k0 + i < width) {
+            if constexpr (sizeof(V) == 8) {
+              ap = fma(weight_f64(ent_w(p[i])), xv[i], ap);
+              dsum += ent_w(p[i]);
+            } else {
+              ap += V(ent_w(p[i])) * (pr - xv[i]);
+            }
+          }
+      }
+      if constexpr (sizeof(V) == 8) ap = fma((double)dsum, pr, -ap);
+      AP[rl] = ap;
+      acc.add(pr * ap);
+      if (a.pb_cg) pbytes += 4ull * width + 2ull * sizeof(V);
+    }
+    double sum = block_sum(acc.get(), sm);
+    if (nt > 1) {
+      if (threadIdx.x == 0) P1[tix] = sum;
+      if (!ub.sync()) return;
+      final_reduce_few(P1, a.stride, u.tile0, nt, 1, out, sp);
+      sum = out[0];
+    }
+    if (threadIdx.x == 0) al_sh = V(rr_sh / sum);
+    __syncthreads();
+    // x += alpha p, r -= alpha Ap; ||r||^2 and the projection of r
+    const V al = al_sh;
+    Acc<V> r2, rs, d0, d1;
+    for (int rl = threadIdx.x; rl < nr; rl += RSB_BLOCK) {
+      X[rl] += al * P[rl];
+      const V rn = R[rl] - al * AP[rl];
+      R[rl] = rn;
+      r2.add(rn * rn);
+      rs.add(rn);
+      if (nd > 0) d0.add(V(a.D0[t.row0 + rl]) * rn);
+      if (nd > 1) d1.add(V(a.D1[t.row0 + rl]) * rn);
+    }
+    const double v[2 + RSB_MAXD] = {r2.get(), rs.get(), d0.get(), d1.get()};
+#pragma unroll
+    for (int c = 0; c < 2 + RSB_MAXD; ++c)
+      if (c < nv) {
+        const double x = block_sum(v[c], sm);
+        if (threadIdx.x == 0) {
+          if (nt > 1) P2[(long long)c * a.stride + tix] = x;
+          else out[c] = x;
+        }
+      }
+    if (nt > 1) {
+      if (!ub.sync()) return;
+      final_reduce_few(P2, a.stride, u.tile0, nt, nv, out, sp);
+    }
+    ++it;
+    if (threadIdx.x == 0) {
+      double cp2 = 0.0, cp[1 + RSB_MAXD];
+      cp[0] = out[1] * isn;
+      cp2 += cp[0] * cp[0];
+      for (int l = 0; l < nd; ++l) {
+        cp[1 + l] = out[2 + l];
+        cp2 += cp[1 + l] * cp[1 + l];
+      }
+      const double rrn = fmax(out[0] - cp2, 0.0);
+      if (sqrt(rrn) <= cg_tol * bnorm || it >= cg_maxit) {
+        done_sh = 1;
+      } else {
+        be_sh = V(rrn / rr_sh);
+        rr_sh = rrn;
+        cp_sh[0] = V(cp[0] * isn);
+        for (int l = 0; l < nd; ++l) cp_sh[1 + l] = V(cp[1 + l]);
+      }
+    }
+    __syncthreads();
+    if (done_sh) break;
+    // r -= B cp, p = r + beta p
+    const V be = be_sh;
+    for (int rl = threadIdx.x; rl < nr; rl += RSB_BLOCK) {
+      const int r = t.row0 + rl;
+      V x = R[rl];
+      if (unit_has(u, a.ckey, r)) x -= cp_sh[0];
+      if (nd > 0) x -= cp_sh[1] * V(a.D0[r]);
+      if (nd > 1) x -= cp_sh[2] * V(a.D1[r]);
+      R[rl] = x;
+      const V pn = x + be * P[rl];
+      P[rl] = pn;
+      a.P[r] = pn;
+    }
+    if (!ub.sync()) return;
+  }
+  for (int rl = threadIdx.x; rl < nr; rl += RSB_BLOCK) a.X[t.row0 + rl] = X[rl];
+  if (first && threadIdx.x == 0) {
+    u.inner = it;
+    u.inner_total += it;
+    u.cg_done = 1;
+  }
+  if (a.pb_cg) prof_add(a.pb_cg, pbytes);
 }
 
 __global__ void k_count_cg(Unit* units, int nunits, int* n_cg) {
@@ -2855,10 +3031,26 @@ static int inverse_run(const LevelGraph& G, const Tile* tiles, int ntiles, Unit*
     if ((rc = amg_setup(sizeof(V) == 4, G, tiles, ntiles, units, *amg_units, s))) return rc;
     amgG = &G;
   }
+  // one cooperative launch per CG solve when every tile gets a co-resident CTA
+  bool res = false;
+  const size_t cg_smem = cg_res_smem<V>(B.trmax);
+  if (use_graph == 3 && !amgG && B.gb) {
+    int dev = 0, nsm = 0, optin = 0, occ = 0;
+    RSB_CK(cudaGetDevice(&dev));
+    RSB_CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+    RSB_CK(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+    if (cg_smem + 12288 <= (size_t)optin) {  // room for the kernel's static shared memory
+      RSB_CK(cudaFuncSetAttribute(k_cg_res<V>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)cg_smem));
+      RSB_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_cg_res<V>, RSB_BLOCK, cg_smem));
+      res = (long long)occ * nsm >= ntiles;
+    }
+    RSB_CK(cudaMemsetAsync(B.gb, 0, sizeof(GridBar), s));
+  }
   const int CGK = 8;
   cudaGraphExec_t exec = nullptr;
   std::vector<int> cap_pairs;
-  if (use_graph) {
+  if (use_graph && !res) {
     cudaGraph_t graph = nullptr;
     RSB_CK(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
     prof_capture_begin();
@@ -2877,10 +3069,23 @@ static int inverse_run(const LevelGraph& G, const Tile* tiles, int ntiles, Unit*
   for (int outer = 0; outer < max_outer + 1 && active > 0; ++outer) {
     k_cg_init<V><<<ntiles, RSB_BLOCK, 0, s>>>(a);
     RSB_CKL("k_cg_init");
-    RSB_CK(cudaMemsetAsync(B.n_cg, 0, sizeof(int), s));
-    k_count_cg<<<(nunits + 127) / 128, 128, 0, s>>>(units, nunits, B.n_cg);
-    RSB_CKL("k_count_cg");
-    for (int blk = 0; blk < cg_maxit / CGK + 2; ++blk) {
+    if (!res) {
+      RSB_CK(cudaMemsetAsync(B.n_cg, 0, sizeof(int), s));
+      k_count_cg<<<(nunits + 127) / 128, 128, 0, s>>>(units, nunits, B.n_cg);
+      RSB_CKL("k_count_cg");
+    }
+    if (res) {
+      int trs = B.trmax;
+      GridBar* gb = B.gb;
+      void* args[] = {(void*)&a, (void*)&trs, (void*)&cg_tol, (void*)&cg_maxit, (void*)&gb};
+      const int pi = prof_before(PROF_CG_AP, s);
+      cudaError_t e = cudaLaunchCooperativeKernel((const void*)k_cg_res<V>, ntiles, RSB_BLOCK, args,
+                                                  cg_smem, s);
+      rsb_count_launch(1);
+      if (e != cudaSuccess) return rsb_set_cuda_error(e, "cudaLaunchCooperativeKernel(k_cg_res)");
+      prof_after(pi, s);
+    }
+    for (int blk = 0; !res && blk < cg_maxit / CGK + 2; ++blk) {
       if (exec) {
         cudaError_t e = cudaGraphLaunch(exec, s);
         rsb_count_launch((amgG ? 7 + 13 * 20 : 3) * CGK);
