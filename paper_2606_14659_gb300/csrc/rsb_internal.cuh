@@ -334,6 +334,45 @@ __device__ __forceinline__ double warp_total(const Acc<float>& a) {
   return (threadIdx.x & 31) == 0 ? (double)s - (double)c : 0.0;
 }
 
+// The warp of a CTA that should take its serial FP64 work (0..3).  CTAs that share an
+// SM otherwise put it all on the sub-partition of their warps 0, where an FP64
+// instruction waits 64 cycles for each of the others; resident CTAs are dealt to the
+// SMs in turn, so the turn picks the warp.
+__device__ __forceinline__ int fp64_warp() {
+  unsigned nsm;
+  asm("mov.u32 %0, %%nsmid;" : "=r"(nsm));
+  return (int)(blockIdx.x / nsm) & 3;
+}
+
+// block_sum of NV values per thread, in the same order, with half its FP64
+// instructions: sixteen lanes take a warp's 32 values.  Total c comes back in lane c of
+// warp fw.  vals: NV * RSB_BLOCK doubles, sm: NV * RSB_WARPS doubles of shared memory.
+template <int NV>
+__device__ __forceinline__ double block_sums(const double (&v)[NV], int nv, double* vals, double* sm,
+                                             int fw) {
+#pragma unroll
+  for (int c = 0; c < NV; ++c)
+    if (c < nv) vals[c * RSB_BLOCK + threadIdx.x] = v[c];
+  __syncthreads();
+  for (int g = threadIdx.x >> 4; g < nv * RSB_WARPS; g += RSB_BLOCK / 16) {
+    const double* p = vals + 32 * g + (threadIdx.x & 15);
+    double x = p[0] + p[16];
+    const unsigned mask = (g | 1) < nv * RSB_WARPS ? 0xffffffffu : 0xffffu << (threadIdx.x & 16);
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) x += __shfl_xor_sync(mask, x, o);
+    if ((threadIdx.x & 15) == 0) sm[g] = x;
+  }
+  __syncthreads();
+  double s = 0.0;
+  if ((int)(threadIdx.x >> 5) == fw && (int)(threadIdx.x & 31) < nv) {
+    const double* p = sm + RSB_WARPS * (threadIdx.x & 31);
+    s = p[0];
+#pragma unroll
+    for (int i = 1; i < RSB_WARPS; ++i) s += p[i];
+  }
+  return s;
+}
+
 // Block total of per-thread accumulators (warp_total per warp, then the warps
 // in order in FP64); result valid in thread 0.
 template <typename V>
@@ -554,11 +593,13 @@ __device__ __forceinline__ void final_reduce(const double* partials, long long s
 // eight lanes (15 us for 973 tiles); here every thread of the CTA forms the
 // four-tile sums of some (tile block, lane) at once, so that one round of loads
 // and nt / 32 additions are left on the chain.  sp: shared scratch of
-// RED_FEW_DOUBLES(nc) doubles.
+// RED_FEW_DOUBLES(nc) doubles.  rot: the warp that takes the chain of coefficient 0
+// (see fp64_warp).
 #define RED_FEW 5
 #define RED_FEW_DOUBLES(nc) ((nc) * (RSB_MAXTILES_PER_UNIT / 32) * 8)
 __device__ __forceinline__ void final_reduce_few(const double* partials, long long stride, int t0,
-                                                 int nt, int nc, double* out, double* sp) {
+                                                 int nt, int nc, double* out, double* sp,
+                                                 int rot = 0) {
   const int nq = nt > 24 ? (nt - 25) / 32 + 1 : 0;  // 32-tile blocks with a full lane
   for (int idx = threadIdx.x; idx < nc * nq * 8; idx += RSB_BLOCK) {
     const int s = idx & 7, cq = idx >> 3;
@@ -570,7 +611,7 @@ __device__ __forceinline__ void final_reduce_few(const double* partials, long lo
       sp[idx] = (a0 + a1) + (a2 + a3);
     }
   }
-  const int c = threadIdx.x >> 5, s = threadIdx.x & 31;
+  const int c = ((threadIdx.x >> 5) - rot) & (RSB_WARPS - 1), s = threadIdx.x & 31;
   const bool on = c < nc && s < 8;
   const int fb = on && nt > 24 + s ? (nt - 25 - s) / 32 + 1 : 0;  // full blocks of this lane
   double r[4] = {0.0, 0.0, 0.0, 0.0};

@@ -105,6 +105,39 @@ __device__ __forceinline__ V spmv_row(const int64_t* __restrict__ slice_ptr,
   return acc;
 }
 
+// The same for x that other CTAs of the launch wrote before a barrier: plain loads
+// (L1 may serve them), eight in flight.
+template <typename V>
+__device__ __forceinline__ V spmv_row_batched(const int64_t* __restrict__ slice_ptr,
+                                              const uint32_t* __restrict__ ent, const V* x, int r,
+                                              V xr) {
+  const int64_t base = slice_ptr[r >> 5];
+  const int width = (int)((slice_ptr[(r >> 5) + 1] - base) >> 5);
+  const uint32_t* e = ent + base + (r & 31);
+  V acc = V(0);
+  uint32_t dsum = 0;
+  for (int k0 = 0; k0 < width; k0 += 8) {
+    uint32_t p[8];
+    V xv[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) p[i] = k0 + i < width ? __ldg(e + 32 * (k0 + i)) : 0u;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) xv[i] = k0 + i < width ? x[ent_col(p[i])] : xr;
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+      if (k0 + i < width) {
+        if constexpr (sizeof(V) == 8) {
+          acc = fma(weight_f64(ent_w(p[i])), xv[i], acc);
+          dsum += ent_w(p[i]);
+        } else {
+          acc += V(ent_w(p[i])) * (xr - xv[i]);
+        }
+      }
+  }
+  if constexpr (sizeof(V) == 8) return fma((double)dsum, xr, -acc);
+  return acc;
+}
+
 // ----------------------------------------------------------------------------
 // Gram-Schmidt building blocks.  The basis is [u0, D_0.., q_0..q_j] with
 // u0 = 1/sqrt(n) on unit rows (its dot is taken as a plain sum and scaled by
@@ -1628,7 +1661,7 @@ __device__ __forceinline__ void res_store_dots(double* P, long long stride, int 
 // exchanged over one more barrier (256 tiles reduced by every CTA took 14.5 us).
 __device__ __forceinline__ bool res_totals(const double* P, long long stride, const Unit& u, int tix,
                                            int ncoef, double* out, double* tot, double* scratch,
-                                           UnitBar& ub) {
+                                           UnitBar& ub, int fw) {
   const int nt = u.ntile;
   if (nt == 1) return true;
   if (nt <= RED_SMALL) {
@@ -1638,7 +1671,7 @@ __device__ __forceinline__ bool res_totals(const double* P, long long stride, co
   // (nt > 96 >= ncoef: every CTA has at most one)
   const int c = tix - u.tile0;
   if (c < ncoef) {
-    final_reduce_few(P + (long long)c * stride, stride, u.tile0, nt, 1, out, scratch);
+    final_reduce_few(P + (long long)c * stride, stride, u.tile0, nt, 1, out, scratch, fw);
     if (threadIdx.x == 0) tot[c] = out[0];
   }
   if (!ub.sync()) return false;
@@ -1658,8 +1691,8 @@ __device__ void res_a(const LzArgs<V>& a, int j, V s, int tix, const Tile& t, co
   unsigned long long pbytes = 0;
   for (int rl = threadIdx.x; rl < nr; rl += RSB_BLOCK) {
     const int r = t.row0 + rl;
-    const V xr = __ldcg(src + r);
-    ws[rl] = s * spmv_row<V, true>(a.slice_ptr, a.ent, src, r, xr);
+    const V xr = src[r];
+    ws[rl] = s * spmv_row_batched<V>(a.slice_ptr, a.ent, src, r, xr);
     Qs[(size_t)j * trs + rl] = s * xr;
     if (a.pb_a)
       pbytes += 4ull * row_width(a.slice_ptr, r) + sizeof(V) * (unsigned long long)(4 + j) +
@@ -1756,7 +1789,7 @@ __device__ void res_d1(const LzArgs<V>& a, int j, V s, const Tile& t, V* vs, V* 
         for (int k = 0; k < 8; ++k) {
           xv[i][k] = xr[i];
           if (k0 + k < width[i])
-            xv[i][k] = own ? vs[(int)ent_col(p[i][k]) - t.row0] : __ldcg(src + ent_col(p[i][k]));
+            xv[i][k] = own ? vs[(int)ent_col(p[i][k]) - t.row0] : src[ent_col(p[i][k])];
         }
 #pragma unroll
       for (int i = 0; i < 2; ++i)
@@ -1938,11 +1971,16 @@ __device__ void res_ritz(const LzArgs<V>& a, const Tile& t, const Unit& u, V* Qs
 template <typename V>
 __device__ __forceinline__ bool res_norm(const LzArgs<V>& a, Unit& u, int j, int tix, double breakdown,
                                          double mine, const double* Pn, double* out,
-                                         double* scratch, double* beta, double* inu, V* scale) {
-  if (u.ntile > 1)
-    final_reduce_few(Pn, a.stride, u.tile0, u.ntile, 1, out, scratch);
-  if (threadIdx.x == 0) {
-    const double b = sqrt(u.ntile > 1 ? out[0] : mine);
+                                         double* scratch, double* beta, double* inu, V* scale,
+                                         int fw) {
+  if (u.ntile > 1) {
+    final_reduce_few(Pn, a.stride, u.tile0, u.ntile, 1, out, scratch, fw);
+  } else {
+    if (threadIdx.x == 0) out[0] = mine;
+    __syncthreads();
+  }
+  if ((int)threadIdx.x == 32 * fw) {
+    const double b = sqrt(out[0]);
     *beta = b;
     *inu = 1.0 / b;
     *scale = V(*inu);
@@ -2000,6 +2038,7 @@ __global__ void __launch_bounds__(RSB_BLOCK, 2)
   const uint64_t key = u.key;
   const double isn = u.isn;
   const bool first = tix == u.tile0;
+  const int fw = fp64_warp();
   UnitBar ub(&u.gbar, u.ntile, __ldcg(&gb->count), gb);
   double* const direct = u.ntile == 1 ? out : nullptr;
   // partial buffers: FP32 dots in the first two, FP64 dots in each in turn, the norms
@@ -2038,7 +2077,7 @@ __global__ void __launch_bounds__(RSB_BLOCK, 2)
         res_d1<V>(a, j, scale_sh, t, vs, ws, direct != nullptr);
         res_d2<V>(a, j, tix, t, nd, Qs, Ds, trs, vs, ws, a.partials, direct);
         if (!ub.sync()) return;
-        if (!res_totals(a.partials, a.stride, u, tix, 2 * nc, out, tot, red1, ub)) return;
+        if (!res_totals(a.partials, a.stride, u, tix, 2 * nc, out, tot, red1, ub, fw)) return;
         const double inu = inu_sh;
         d2_finish(out, out + nc, nb, nd, j, inu, isn, Ssh, dsc, dsk);
         const double rho = dsc[0];
@@ -2070,17 +2109,17 @@ __global__ void __launch_bounds__(RSB_BLOCK, 2)
           }
         }
         if (!ub.wait()) return;
-        if (res_norm<V>(a, u, j, tix, breakdown, mine, Pn, out, red1, &beta_sh, &inu_sh, &scale_sh))
+        if (res_norm<V>(a, u, j, tix, breakdown, mine, Pn, out, red1, &beta_sh, &inu_sh, &scale_sh, fw))
           msteps = j + 1;
       } else {
         const int nc = 2 + nd + j;
         res_a<V>(a, j, scale_sh, tix, t, u, Qs, Ds, trs, ws, Pb[0], direct);
         if (!ub.sync()) return;
-        if (!res_totals(Pb[0], a.stride, u, tix, nc, out, tot, red1, ub)) return;
+        if (!res_totals(Pb[0], a.stride, u, tix, nc, out, tot, red1, ub, fw)) return;
         res_coef<V>(out, nc, isn, c1, cv);
         res_b<V>(a, j, tix, t, nd, masked, key, Qs, Ds, trs, ws, cv, Pb[1], direct);
         if (!ub.sync()) return;
-        if (!res_totals(Pb[1], a.stride, u, tix, nc, out, tot + RSB_MAXC, red1, ub)) return;
+        if (!res_totals(Pb[1], a.stride, u, tix, nc, out, tot + RSB_MAXC, red1, ub, fw)) return;
         res_coef<V>(out, nc, isn, c2, cv + RSB_MAXC);
         if (first) {  // column j of S = Q^T L Q
           double* Sm = unit_S(a.S, t.unit);
@@ -2093,7 +2132,7 @@ __global__ void __launch_bounds__(RSB_BLOCK, 2)
         mine = res_c<V>(a, j, t, nd, masked, key, Qs, Ds, trs, ws, cv + RSB_MAXC, sm);
         if (threadIdx.x == 0) Pn[tix] = mine;
         if (!ub.sync()) return;
-        if (res_norm<V>(a, u, j, tix, breakdown, mine, Pn, out, red1, &beta_sh, &inu_sh, &scale_sh))
+        if (res_norm<V>(a, u, j, tix, breakdown, mine, Pn, out, red1, &beta_sh, &inu_sh, &scale_sh, fw))
           msteps = j + 1;
       }
     }
@@ -2806,9 +2845,13 @@ __global__ void __launch_bounds__(RSB_BLOCK) k_inv_res(LzArgs<V> a, int max_oute
 // shared memory; global memory carries p (the SpMV's operand), the partials and the
 // unit's barrier.  Units iterate independently.  Rows, sums and their order are those
 // of k_cg_ap, k_cg_xr and k_cg_p, so both modes give the same numbers.
-// Bound: latency, three barriers and two reductions an iteration.  Three launches, each
-// with the chain of a last CTA's reduction, took 55 us an iteration at 256k rows (500
+// Bound: latency, three barriers and two reductions an iteration; the FP64 work of
+// the up to four CTAs of an SM is dealt to its sub-partitions.  Three launches, each
+// with the chain of a last CTA's reduction, took 45 us an iteration at 256k rows (500
 // tiles).
+// The SpMV gathers p with plain loads: the barrier orders them after the other CTAs'
+// stores (their release, thread 0's acquire, the CTA barrier), so L1 may serve the
+// gathers that share lines.
 // ----------------------------------------------------------------------------
 template <typename V>
 constexpr size_t cg_res_smem(int trs) {
@@ -2824,9 +2867,11 @@ __global__ void __launch_bounds__(RSB_BLOCK, 4)
   V* R = reinterpret_cast<V*>(cg_sh + vb);
   V* P = reinterpret_cast<V*>(cg_sh + 2 * vb);
   V* AP = reinterpret_cast<V*>(cg_sh + 3 * vb);
-  __shared__ double sm[RSB_WARPS];
+  __shared__ double sm[RSB_WARPS * (2 + RSB_MAXD)];
   __shared__ double out[2 + RSB_MAXD];
+  // scratch of the reductions over the tiles and, at other times, over the threads
   __shared__ double sp[RED_FEW_DOUBLES(2 + RSB_MAXD)];
+  static_assert(RED_FEW_DOUBLES(2 + RSB_MAXD) >= (2 + RSB_MAXD) * RSB_BLOCK, "scratch");
   __shared__ double rr_sh;
   __shared__ V al_sh, be_sh, cp_sh[1 + RSB_MAXD];
   __shared__ int done_sh;
@@ -2837,6 +2882,8 @@ __global__ void __launch_bounds__(RSB_BLOCK, 4)
   const int nr = t.row1 - t.row0;
   const int nd = u.nd, nv = 2 + nd, nt = u.ntile;
   const bool first = tix == u.tile0;
+  const int fw = fp64_warp(), lane = threadIdx.x & 31;
+  const bool fpw = (int)(threadIdx.x >> 5) == fw;
   const double bnorm = u.bnorm, isn = u.isn;
   UnitBar ub(&u.gbar, nt, __ldcg(&gb->count), gb);
   double* const P1 = a.partials;                       // p.Lp
@@ -2871,7 +2918,7 @@ __global__ void __launch_bounds__(RSB_BLOCK, 4)
 #pragma unroll
         for (int i = 0; i < 13; ++i) p[i] = k0 + i < width ? __ldg(e + 32 * (k0 + i)) : 0u;
 #pragma unroll
-        for (int i = 0; i < 13; ++i) xv[i] = k0 + i < width ? __ldcg(Pg + ent_col(p[i])) : pr;
+        for (int i = 0; i < 13; ++i) xv[i] = k0 + i < width ? Pg[ent_col(p[i])] : pr;
 #pragma unroll
         for (int i = 0; i < 13; ++i)
           if (k0 + i < width) {
@@ -2888,14 +2935,15 @@ __global__ void __launch_bounds__(RSB_BLOCK, 4)
       acc.add(pr * ap);
       if (a.pb_cg) pbytes += 4ull * width + 2ull * sizeof(V);
     }
-    double sum = block_sum(acc.get(), sm);
+    const double v1[1] = {acc.get()};
+    double sum = block_sums<1>(v1, 1, sp, sm, fw);
     if (nt > 1) {
-      if (threadIdx.x == 0) P1[tix] = sum;
+      if (fpw && lane == 0) P1[tix] = sum;
       if (!ub.sync()) return;
-      final_reduce_few(P1, a.stride, u.tile0, nt, 1, out, sp);
+      final_reduce_few(P1, a.stride, u.tile0, nt, 1, out, sp, fw);
       sum = out[0];
     }
-    if (threadIdx.x == 0) al_sh = V(rr_sh / sum);
+    if (fpw && lane == 0) al_sh = V(rr_sh / sum);
     __syncthreads();
     // x += alpha p, r -= alpha Ap; ||r||^2 and the projection of r
     const V al = al_sh;
@@ -2910,21 +2958,19 @@ __global__ void __launch_bounds__(RSB_BLOCK, 4)
       if (nd > 1) d1.add(V(a.D1[t.row0 + rl]) * rn);
     }
     const double v[2 + RSB_MAXD] = {r2.get(), rs.get(), d0.get(), d1.get()};
-#pragma unroll
-    for (int c = 0; c < 2 + RSB_MAXD; ++c)
-      if (c < nv) {
-        const double x = block_sum(v[c], sm);
-        if (threadIdx.x == 0) {
-          if (nt > 1) P2[(long long)c * a.stride + tix] = x;
-          else out[c] = x;
-        }
-      }
+    const double x = block_sums<2 + RSB_MAXD>(v, nv, sp, sm, fw);
+    if (fpw && lane < nv) {
+      if (nt > 1) P2[(long long)lane * a.stride + tix] = x;
+      else out[lane] = x;
+    }
     if (nt > 1) {
       if (!ub.sync()) return;
-      final_reduce_few(P2, a.stride, u.tile0, nt, nv, out, sp);
+      final_reduce_few(P2, a.stride, u.tile0, nt, nv, out, sp, fw);
+    } else {
+      __syncthreads();
     }
     ++it;
-    if (threadIdx.x == 0) {
+    if (fpw && lane == 0) {
       double cp2 = 0.0, cp[1 + RSB_MAXD];
       cp[0] = out[1] * isn;
       cp2 += cp[0] * cp[0];
