@@ -37,6 +37,10 @@ int launch_select(const LevelGraph& G, const Tile* tiles, int ntiles, Unit* unit
 int launch_split_below(const LevelGraph& G, const Tile* tiles, int ntiles, Unit* units,
                        const uint64_t* ckey, const double* v, int cand, double* partials,
                        cudaStream_t s);
+size_t split_scratch_bytes(int nunits);
+int launch_split(const LevelGraph& G, const Tile* tiles, int ntiles, Unit* units, int nunits,
+                 const uint64_t* ckey, const double* v, int cand, double tie_rel, int fixed_sign,
+                 uint8_t* side, void* scratch, GridBar* gb, cudaStream_t s, int* done);
 int launch_choose(const LevelGraph& G, const Tile* tiles, int ntiles, Unit* units,
                   const uint64_t* ckey, const uint8_t* side, int cb, double* partials,
                   cudaStream_t s);
@@ -273,7 +277,7 @@ struct Ctx {
   DevBuf len, slice_sz, scan_tmp, tmp64, newpos;
   DevBuf parent, cmin, ckey, side;
   DevBuf units, tiles, sunits, stiles;
-  DevBuf hist, partials, mom, sbuf, blk;
+  DevBuf hist, partials, mom, sbuf, blk, split;
   DevBuf cand[3];
   PrecBufs pb[2];  // 0: FP64, 1: FP32
   DevBuf seg_row0, seg_nleft, seg_child0, seg_p0, seg_split, seg_keystar, seg_unit, seg_ncomp;
@@ -324,6 +328,7 @@ struct Counters {
   GridBar gb;
   int jmin[2];
   long long inner;  // CG iterations of the inverse-iteration solves
+  GridBar gb_split; // error word of the splits (kept for the whole call)
 };
 
 // ----------------------------------------------------------------------------
@@ -744,6 +749,26 @@ static int solve_candidate(Ctx& c, const LevelGraph& G, const Tile* tiles, int n
   return RSB_OK;
 }
 
+// Orientation and split of every unit by one candidate's vector.
+static int split_candidate(Ctx& c, const LevelGraph& G, const Tile* tiles, int ntiles, Unit* units,
+                           int nunits, const uint64_t* ckey, const double* v, int cand,
+                           double tie_rel, int fixed_sign, double* partials, uint8_t* side,
+                           int* hist) {
+  int rc, done = 0;
+  if ((rc = devbuf_reserve(c.split, split_scratch_bytes(nunits))) ||
+      (rc = launch_split(G, tiles, ntiles, units, nunits, ckey, v, cand, tie_rel, fixed_sign, side,
+                         c.split.p, &dptr<Counters>(c.counters)->gb_split, c.s, &done)) ||
+      done)
+    return rc;
+  if ((rc = launch_orient(G, tiles, ntiles, units, ckey, v, cand, tie_rel, partials, c.s,
+                          fixed_sign)) ||
+      (rc = launch_select(G, tiles, ntiles, units, nunits, ckey, v, 0, cand, hist, c.s)) ||
+      (rc = launch_split_below(G, tiles, ntiles, units, ckey, v, cand, partials, c.s)) ||
+      (rc = launch_select(G, tiles, ntiles, units, nunits, ckey, v, 1, cand, hist, c.s)))
+    return rc;
+  return launch_split_assign(G, tiles, ntiles, units, ckey, v, side, cand, c.s);
+}
+
 // All candidates, rotation, orientation, split and choice for the level's units.
 static int split_units(Ctx& c, const LevelGraph& G, std::vector<Unit>& hunits,
                        const std::vector<Tile>& htiles, const rsb_options& o, RunStats& rs) {
@@ -777,14 +802,10 @@ static int split_units(Ctx& c, const LevelGraph& G, std::vector<Unit>& hunits,
     uint8_t* side = dptr<uint8_t>(c.side);
     int* hist = dptr<int>(c.hist);
     if ((rc = launch_rcb_vector(G, tiles, ntiles, units, dptr<double>(c.coords_cat), v0, partials,
-                                c.s)) ||
-        (rc = launch_orient(G, tiles, ntiles, units, ckey, v0, 0, o.tie_rel, partials, c.s, 1)) ||
-        (rc = launch_select(G, tiles, ntiles, units, nunits, ckey, v0, 0, 0, hist, c.s)) ||
-        (rc = launch_split_below(G, tiles, ntiles, units, ckey, v0, 0, partials, c.s)) ||
-        (rc = launch_select(G, tiles, ntiles, units, nunits, ckey, v0, 1, 0, hist, c.s)) ||
-        (rc = launch_split_assign(G, tiles, ntiles, units, ckey, v0, side, 0, c.s)))
+                                c.s)))
       return rc;
-    return RSB_OK;
+    return split_candidate(c, G, tiles, ntiles, units, nunits, ckey, v0, 0, o.tie_rel, 1, partials,
+                           side, hist);
   }
   if ((rc = launch_degree_max(G, tiles, ntiles, units, ckey, partials, c.s))) return rc;
   const int ncmax = o.degenerate_policy == RSB_DEGEN_RESOLVE ? 3 : 1;
@@ -804,15 +825,8 @@ static int split_units(Ctx& c, const LevelGraph& G, std::vector<Unit>& hunits,
   int* hist = dptr<int>(c.hist);
   double* vs[3] = {v0, v1, v2};
   for (int cand = 0; cand < ncmax; ++cand) {
-    if ((rc = launch_orient(G, tiles, ntiles, units, ckey, vs[cand], cand, o.tie_rel, partials, c.s)))
-      return rc;
-    if ((rc = launch_select(G, tiles, ntiles, units, nunits, ckey, vs[cand], 0, cand, hist, c.s)))
-      return rc;
-    if ((rc = launch_split_below(G, tiles, ntiles, units, ckey, vs[cand], cand, partials, c.s)))
-      return rc;
-    if ((rc = launch_select(G, tiles, ntiles, units, nunits, ckey, vs[cand], 1, cand, hist, c.s)))
-      return rc;
-    if ((rc = launch_split_assign(G, tiles, ntiles, units, ckey, vs[cand], side, cand, c.s)))
+    if ((rc = split_candidate(c, G, tiles, ntiles, units, nunits, ckey, vs[cand], cand, o.tie_rel, 0,
+                              partials, side, hist)))
       return rc;
   }
   if (ncmax > 1) {
@@ -1090,8 +1104,10 @@ static int run_rsb(Ctx& c, const std::vector<MeshIn>& meshes, const std::vector<
                            cudaMemcpyDeviceToDevice, c.s));
   // CC error flag (a bound that can never be reached in a correct run)
   RSB_CK(cudaMemcpyAsync(c.h_pinned, &cn->flag, sizeof(int), cudaMemcpyDeviceToHost, c.s));
+  RSB_CK(cudaMemcpyAsync(c.h_pinned + 1, &cn->gb_split.err, sizeof(int), cudaMemcpyDeviceToHost, c.s));
   RSB_CK(cudaStreamSynchronize(c.s));
   if (c.h_pinned[0] & 32) return rsb_set_error(RSB_ETIMEOUT, "union-find bound reached");
+  if (c.h_pinned[1]) return rsb_set_error(RSB_ETIMEOUT, "a bounded device wait gave up");
   if (st) {
     st->levels = levels;
     st->nonconverged = rs.nonconv;
@@ -1929,7 +1945,7 @@ extern "C" void rsb_release(void) {
                      &c->tiles, &c->sunits, &c->stiles, &c->hist, &c->partials, &c->mom, &c->sbuf,
                      &c->cand[0], &c->cand[1], &c->cand[2], &c->seg_row0, &c->seg_nleft,
                      &c->seg_child0, &c->seg_p0, &c->seg_split, &c->seg_keystar, &c->seg_unit,
-                     &c->seg_ncomp, &c->counters, &c->part_concat, &c->blk, &c->coords_cat,
+                     &c->seg_ncomp, &c->counters, &c->part_concat, &c->blk, &c->split, &c->coords_cat,
                      &c->perm, &c->iperm, &c->rcb_home, &c->gs_count, &c->gs_cursor,
                      &c->gs_bptr, &c->gs_bucket, &c->gs_ev32, &c->gs_len, &c->gs_rowptr,
                      &c->gs_w, &c->gs_misc, &c->gs_rows};

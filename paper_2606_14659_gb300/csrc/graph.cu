@@ -681,11 +681,13 @@ __global__ void __launch_bounds__(RSB_BLOCK)
     partials[(long long)threadIdx.x * stride + blockIdx.x] = b;
   }
   if (last_cta(&u.cnt, u.ntile)) {
-    if (threadIdx.x < 6) {
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (w < 6) {
       double b = -1e300;
-      for (int i = 0; i < u.ntile; ++i)
-        b = fmax(b, __ldcg(partials + threadIdx.x * stride + u.tile0 + i));
-      out[threadIdx.x] = b;
+      for (int i = lane; i < u.ntile; i += 32)
+        b = fmax(b, __ldcg(partials + w * stride + u.tile0 + i));
+      b = warp_max(b);
+      if (lane == 0) out[w] = b;
     }
     __syncthreads();
     if (threadIdx.x == 0) {

@@ -10,6 +10,8 @@
 //   * the gid rule comparing two candidate splits of a repeated eigenvalue
 //     (reading R5), and the final side of every row including whole
 //     components placed by reading R8.
+#include <algorithm>
+
 #include "rsb_internal.cuh"
 
 // ----------------------------------------------------------------------------
@@ -150,12 +152,20 @@ __global__ void __launch_bounds__(RSB_BLOCK)
     partials[stride + blockIdx.x] = gv;
   }
   if (last_cta(&u.cnt, u.ntile)) {
-    if (threadIdx.x == 0) {
+    if (threadIdx.x < 32) {
       double bg = 1e300, bv = 0.0;
-      for (int i = 0; i < u.ntile; ++i) {
+      for (int i = threadIdx.x; i < u.ntile; i += 32) {
         const double pg = __ldcg(partials + u.tile0 + i);
-        if (pg < bg) { bg = pg; bv = __ldcg(partials + stride + u.tile0 + i); }
+        const double pv = __ldcg(partials + stride + u.tile0 + i);
+        if (pg < bg) { bg = pg; bv = pv; }
       }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        const double og = __shfl_xor_sync(0xffffffffu, bg, o);
+        const double ov = __shfl_xor_sync(0xffffffffu, bv, o);
+        if (og < bg) { bg = og; bv = ov; }
+      }
+      if (threadIdx.x != 0) return;
       u.gstar = (int64_t)bg;
       u.gstar_v = bv;
       u.sign = fixed_sign ? 1.0 : (bv > 0.0 ? -1.0 : 1.0);
@@ -344,6 +354,341 @@ int launch_split_assign(const LevelGraph& G, const Tile* tiles, int ntiles, Unit
 }
 
 // ----------------------------------------------------------------------------
+// The whole split of one candidate in one cooperative launch: orientation (R4), the
+// k-th value, the tie window and the tie gid (R7), and the side bit of every row - the
+// steps of k_orient_*, k_sel_*, k_split_below and k_split_assign above, which take 36
+// launches and remain for levels of more tiles than SPLIT_MAXL a co-resident CTA.
+// Bound: the 12 to 20 grid barriers (about 2 us each) and, on large levels, one read of
+// v from L2 for each radix pass.  A CTA walks its tiles in every phase and keeps their
+// units' selection state; digits that all keys of a unit share (known from its smallest
+// and largest key) take no pass.  Values are compared as their integer keys, because an
+// FP64 comparison holds an SM sub-partition for 64 cycles; only rows near the tie
+// window take its FP64 test.  The split of a level of 512 rows 0.55 -> 0.12-0.26 ms (two
+// or three candidates), of 2.1M rows by coordinates 0.5-0.9 -> 0.27-0.3 ms.
+// ----------------------------------------------------------------------------
+#define SPLIT_MAXL 32  // tiles of a CTA
+#define SPLIT_BINS 256
+
+// Per-unit scratch: zeroed (Z) and set to all ones (O) before the launch.
+struct SplitZ {
+  int hist[3][SPLIT_BINS];   // three buffers in turn: one filled, one read, one cleared
+  unsigned long long kmax, tmax;
+  unsigned long long below;
+  unsigned long long sgn;    // 1: v[g*] <= 0, 2: v[g*] > 0
+};
+struct SplitO {
+  unsigned long long kmin, tmin, gmin;
+};
+
+__device__ __forceinline__ uint64_t split_key(double x, bool neg) {
+  uint64_t b = (uint64_t)__double_as_longlong(x);
+  if (neg) b ^= 0x8000000000000000ull;
+  if (b == 0x8000000000000000ull) b = 0;  // -0 and +0 are one value
+  return (b >> 63) ? ~b : (b | 0x8000000000000000ull);
+}
+__device__ __forceinline__ unsigned long long warp_max_u64(unsigned long long x) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const unsigned long long y = __shfl_xor_sync(0xffffffffu, x, o);
+    x = y > x ? y : x;
+  }
+  return x;
+}
+__device__ __forceinline__ unsigned long long warp_min_u64(unsigned long long x) {
+  return ~warp_max_u64(~x);
+}
+// first byte (0 = most significant) in which two keys differ; 8 when none does
+__device__ __forceinline__ int first_byte(uint64_t a, uint64_t b) {
+  return a == b ? 8 : __clzll((long long)(a ^ b)) >> 3;
+}
+__device__ __forceinline__ uint64_t top_bytes(uint64_t k, int n) {
+  return n == 0 ? 0ull : n >= 8 ? k : k & ~(~0ull >> (8 * n));
+}
+
+__global__ void __launch_bounds__(RSB_BLOCK, 4)
+    k_split(const int64_t* __restrict__ gid, const Tile* __restrict__ tiles, int ntiles, Unit* units,
+            const uint64_t* __restrict__ ckey, const double* __restrict__ v, int cand, double tie_rel,
+            int fixed_sign, uint8_t* side, SplitZ* Z, SplitO* O, unsigned* counter, GridBar* gb) {
+  __shared__ int sh[SPLIT_BINS];
+  __shared__ int wtot[RSB_WARPS];
+  __shared__ uint64_t prefix[SPLIT_MAXL];
+  __shared__ long long rank[SPLIT_MAXL];
+  __shared__ int first[SPLIT_MAXL];       // passes before this one are decided; 8: none left
+  __shared__ uint8_t neg[SPLIT_MAXL], on[SPLIT_MAXL];
+  __shared__ uint64_t klim[SPLIT_MAXL], klo[SPLIT_MAXL], khi[SPLIT_MAXL];
+  __shared__ double vk[SPLIT_MAXL], tau[SPLIT_MAXL];
+  __shared__ unsigned long long red[2][RSB_WARPS];
+  const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
+  const int G = gridDim.x;
+  UnitBar bar(counter, G, 0u, gb);
+  // tiles blockIdx, blockIdx + G, ... of this CTA
+  const int nl = (ntiles - (int)blockIdx.x + G - 1) / G;
+  for (int l = tid; l < nl; l += RSB_BLOCK) {
+    const Unit& u = units[tiles[blockIdx.x + l * G].unit];
+    on[l] = u.valid && cand < u.ncand;
+    neg[l] = 0;
+  }
+  __syncthreads();
+  // smallest and largest key of every unit
+  for (int l = 0; l < nl; ++l) {
+    if (!on[l]) continue;
+    const Tile t = tiles[blockIdx.x + l * G];
+    const Unit& u = units[t.unit];
+    unsigned long long hi = 0, lo = ~0ull;
+    for (int r = t.row0 + tid; r < t.row1; r += RSB_BLOCK) {
+      if (!unit_has(u, ckey, r)) continue;
+      const uint64_t k = split_key(v[r], false);
+      hi = k > hi ? k : hi;
+      lo = k < lo ? k : lo;
+    }
+    hi = warp_max_u64(hi);
+    lo = warp_min_u64(lo);
+    if (lane == 0) {
+      red[0][w] = hi;
+      red[1][w] = lo;
+    }
+    __syncthreads();
+    if (w == 0) {
+      hi = warp_max_u64(lane < RSB_WARPS ? red[0][lane] : 0ull);
+      lo = warp_min_u64(lane < RSB_WARPS ? red[1][lane] : ~0ull);
+      if (lane == 0 && lo <= hi) {
+        atomicMax(&Z[t.unit].kmax, hi);
+        atomicMin(&O[t.unit].kmin, lo);
+      }
+    }
+    __syncthreads();
+  }
+  if (!bar.sync()) return;
+  if (!fixed_sign) {
+    // g*: the smallest gid with |v| >= max|v| / 2
+    for (int l = 0; l < nl; ++l) {
+      if (!on[l]) continue;
+      const Tile t = tiles[blockIdx.x + l * G];
+      const Unit& u = units[t.unit];
+      const double amax = fmax(fabs(dkey_inv(__ldcg(&Z[t.unit].kmax))),
+                               fabs(dkey_inv(__ldcg(&O[t.unit].kmin))));
+      const uint64_t thr = split_key(0.5 * amax, false);
+      unsigned long long g = ~0ull;
+      for (int r = t.row0 + tid; r < t.row1; r += RSB_BLOCK) {
+        if (!unit_has(u, ckey, r)) continue;
+        if (split_key(fabs(v[r]), false) >= thr) {
+          const unsigned long long x = (unsigned long long)gid[r] ^ 0x8000000000000000ull;
+          g = x < g ? x : g;
+        }
+      }
+      g = warp_min_u64(g);
+      if (lane == 0 && g != ~0ull) atomicMin(&O[t.unit].gmin, g);
+    }
+    if (!bar.sync()) return;
+    for (int l = 0; l < nl; ++l) {  // the sign of v there (gids of a graph are distinct)
+      if (!on[l]) continue;
+      const Tile t = tiles[blockIdx.x + l * G];
+      const Unit& u = units[t.unit];
+      const int64_t g = (int64_t)(__ldcg(&O[t.unit].gmin) ^ 0x8000000000000000ull);
+      for (int r = t.row0 + tid; r < t.row1; r += RSB_BLOCK)
+        if (gid[r] == g && unit_has(u, ckey, r)) Z[t.unit].sgn = v[r] > 0.0 ? 2 : 1;
+    }
+    if (!bar.sync()) return;
+  }
+  // the k-th value, then among its ties the gid, a byte a pass
+  for (int l = tid; l < nl; l += RSB_BLOCK) {
+    first[l] = 8;
+    if (!on[l]) continue;
+    const int ui = tiles[blockIdx.x + l * G].unit;
+    const bool ng = !fixed_sign && __ldcg(&Z[ui].sgn) == 2;
+    uint64_t hi = __ldcg(&Z[ui].kmax), lo = __ldcg(&O[ui].kmin);
+    if (ng) {  // keys of the negated values
+      const uint64_t x = ~lo;
+      lo = ~hi;
+      hi = x;
+      if (lo == 0x7FFFFFFFFFFFFFFFull) lo = 0x8000000000000000ull;
+      if (hi == 0x7FFFFFFFFFFFFFFFull) hi = 0x8000000000000000ull;
+    }
+    neg[l] = ng;
+    rank[l] = units[ui].k;
+    first[l] = first_byte(lo, hi);
+    prefix[l] = top_bytes(lo, first[l]);
+  }
+  __syncthreads();
+  for (int stage = 0; stage < 2; ++stage) {
+    for (int p = 0; p < 8; ++p) {
+      const int shift = 56 - 8 * p;
+      const int buf = (stage * 8 + p) % 3, nxt = (buf + 1) % 3;
+      const uint64_t himask = p == 0 ? 0ull : ~0ull << (shift + 8);
+      for (int l = 0; l < nl; ++l) {
+        if (!on[l]) continue;
+        const Tile t = tiles[blockIdx.x + l * G];
+        const Unit& u = units[t.unit];
+        if (t.row0 == u.row0) Z[t.unit].hist[nxt][tid] = 0;  // read two passes ago
+        if (p < first[l]) continue;
+        sh[tid] = 0;
+        __syncthreads();
+        const uint64_t want = prefix[l] & himask;
+        const bool ng = neg[l];
+        for (int r = t.row0 + tid; r < t.row1; r += RSB_BLOCK) {
+          if (!unit_has(u, ckey, r)) continue;
+          uint64_t key = split_key(v[r], ng);
+          if (stage == 1) {
+            if (key < klo[l] || key > khi[l]) continue;
+            const double x = ng ? -v[r] : v[r];
+            if (!(fabs(x - vk[l]) <= tau[l])) continue;
+            key = (uint64_t)gid[r];
+          }
+          if ((key & himask) == want) atomicAdd(&sh[(key >> shift) & 255u], 1);
+        }
+        __syncthreads();
+        const int c = sh[tid];
+        if (c) atomicAdd(&Z[t.unit].hist[buf][tid], c);
+        __syncthreads();
+      }
+      if (!bar.sync()) return;
+      for (int l = 0; l < nl; ++l) {
+        if (!on[l] || p < first[l]) continue;
+        const int ui = tiles[blockIdx.x + l * G].unit;
+        const int c = __ldcg(&Z[ui].hist[buf][tid]);
+        int x = c;  // inclusive sums over the bins
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const int y = __shfl_up_sync(0xffffffffu, x, o);
+          if (lane >= o) x += y;
+        }
+        if (lane == 31) wtot[w] = x;
+        const long long k = rank[l];
+        __syncthreads();
+        for (int i = 0; i < w; ++i) x += wtot[i];
+        if (c > 0 && x - c < k && k <= x) {
+          rank[l] = k - (x - c);
+          prefix[l] |= (uint64_t)tid << shift;
+        }
+        __syncthreads();
+      }
+    }
+    if (stage == 1) break;
+    // v_k, the rows below its tie window, the range of the ties' gids
+    for (int l = tid; l < nl; l += RSB_BLOCK)
+      if (on[l]) {
+        const int ui = tiles[blockIdx.x + l * G].unit;
+        const double hi = dkey_inv(__ldcg(&Z[ui].kmax)), lo = dkey_inv(__ldcg(&O[ui].kmin));
+        vk[l] = dkey_inv(prefix[l]);
+        tau[l] = tie_rel * (hi - lo);
+        klim[l] = split_key(vk[l] - tau[l], false);
+        klo[l] = split_key(vk[l] - 1.5 * tau[l], false);
+        khi[l] = split_key(vk[l] + 1.5 * tau[l], false);
+      }
+    __syncthreads();
+    for (int l = 0; l < nl; ++l) {
+      if (!on[l]) continue;
+      const Tile t = tiles[blockIdx.x + l * G];
+      const Unit& u = units[t.unit];
+      const bool ng = neg[l];
+      int below = 0;
+      unsigned long long hi = 0, lo = ~0ull;
+      for (int r = t.row0 + tid; r < t.row1; r += RSB_BLOCK) {
+        if (!unit_has(u, ckey, r)) continue;
+        const uint64_t key = split_key(v[r], ng);
+        below += key < klim[l];
+        if (key >= klo[l] && key <= khi[l]) {
+          const double x = ng ? -v[r] : v[r];
+          if (fabs(x - vk[l]) <= tau[l]) {
+            const unsigned long long g = (unsigned long long)gid[r];
+            hi = g > hi ? g : hi;
+            lo = g < lo ? g : lo;
+          }
+        }
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) below += __shfl_xor_sync(0xffffffffu, below, o);
+      hi = warp_max_u64(hi);
+      lo = warp_min_u64(lo);
+      if (lane == 0) {
+        if (below) atomicAdd(&Z[t.unit].below, (unsigned long long)below);
+        if (lo <= hi) {
+          atomicMax(&Z[t.unit].tmax, hi);
+          atomicMin(&O[t.unit].tmin, lo);
+        }
+      }
+    }
+    if (!bar.sync()) return;
+    for (int l = tid; l < nl; l += RSB_BLOCK)
+      if (on[l]) {
+        const Tile t = tiles[blockIdx.x + l * G];
+        Unit& u = units[t.unit];
+        const long long below = (long long)__ldcg(&Z[t.unit].below);
+        const uint64_t hi = __ldcg(&Z[t.unit].tmax), lo = __ldcg(&O[t.unit].tmin);
+        rank[l] = u.k - below;
+        // (no tie goes left: nothing to select)
+        first[l] = rank[l] <= 0 || lo > hi ? 8 : first_byte(lo, hi);
+        prefix[l] = rank[l] <= 0 || lo > hi ? 0ull : top_bytes(lo, first[l]);
+        if (t.row0 == u.row0) {
+          u.sign = neg[l] ? -1.0 : 1.0;
+          u.vk = vk[l];
+          u.tau = tau[l];
+          u.below = below;
+        }
+      }
+    __syncthreads();
+  }
+  // side bits
+  for (int l = 0; l < nl; ++l) {
+    if (!on[l]) continue;
+    const Tile t = tiles[blockIdx.x + l * G];
+    const Unit& u = units[t.unit];
+    const bool ng = neg[l];
+    // rank is 1-based among the ties until it is used up; a unit without a tie to its
+    // left was given no passes and prefix 0
+    const bool none = (long long)u.k - (long long)__ldcg(&Z[t.unit].below) <= 0;
+    const uint64_t gthr = prefix[l];
+    const uint8_t bit = (uint8_t)(1u << cand);
+    for (int r = t.row0 + tid; r < t.row1; r += RSB_BLOCK) {
+      if (!unit_has(u, ckey, r)) continue;
+      const uint64_t key = split_key(v[r], ng);
+      bool left = key < klim[l];
+      if (!left && !none && key >= klo[l] && key <= khi[l]) {
+        const double x = ng ? -v[r] : v[r];
+        if (fabs(x - vk[l]) <= tau[l]) left = (uint64_t)gid[r] <= gthr;
+      }
+      side[r] = left ? (uint8_t)(side[r] & ~bit) : (uint8_t)(side[r] | bit);
+    }
+  }
+}
+
+size_t split_scratch_bytes(int nunits) {
+  return (sizeof(SplitZ) + sizeof(SplitO)) * (size_t)nunits + 256;
+}
+
+// scratch: split_scratch_bytes.  *done = 0 when the level has too many tiles for one
+// co-resident launch (the caller then takes the steps one by one).
+int launch_split(const LevelGraph& G, const Tile* tiles, int ntiles, Unit* units, int nunits,
+                 const uint64_t* ckey, const double* v, int cand, double tie_rel, int fixed_sign,
+                 uint8_t* side, void* scratch, GridBar* gb, cudaStream_t s, int* done) {
+  *done = 0;
+  if (ntiles <= 0 || nunits <= 0) {
+    *done = 1;
+    return RSB_OK;
+  }
+  int dev = 0, nsm = 0, occ = 0;
+  RSB_CK(cudaGetDevice(&dev));
+  RSB_CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+  RSB_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_split, RSB_BLOCK, 0));
+  const int grid = std::min(ntiles, std::min(occ, 4) * nsm);  // (more only makes the barriers longer)
+  if (grid <= 0 || (long long)grid * SPLIT_MAXL < ntiles) return RSB_OK;
+  unsigned* counter = (unsigned*)scratch;
+  SplitZ* Z = (SplitZ*)((char*)scratch + 256);
+  SplitO* O = (SplitO*)(Z + nunits);
+  RSB_CK(cudaMemsetAsync(scratch, 0, 256 + sizeof(SplitZ) * (size_t)nunits, s));
+  RSB_CK(cudaMemsetAsync(O, 0xFF, sizeof(SplitO) * (size_t)nunits, s));
+  const int64_t* gid = G.gid;
+  void* args[] = {(void*)&gid, (void*)&tiles, (void*)&ntiles, (void*)&units, (void*)&ckey, (void*)&v,
+                  (void*)&cand, (void*)&tie_rel, (void*)&fixed_sign, (void*)&side, (void*)&Z,
+                  (void*)&O, (void*)&counter, (void*)&gb};
+  cudaError_t e = cudaLaunchCooperativeKernel((const void*)k_split, grid, RSB_BLOCK, args, 0, s);
+  rsb_count_launch();
+  if (e != cudaSuccess) return rsb_set_cuda_error(e, "cudaLaunchCooperativeKernel(k_split)");
+  *done = 1;
+  return RSB_OK;
+}
+
+// ----------------------------------------------------------------------------
 // R5 gid rule: smallest gid where candidates a and b disagree, and whether a
 // has it on the left.  Result: u.best updated (a wins -> a, else b) among
 // candidates of equal cut; the caller runs it after comparing cuts.
@@ -386,13 +731,21 @@ __global__ void __launch_bounds__(RSB_BLOCK)
     partials[stride + blockIdx.x] = (double)aleft;
   }
   if (last_cta(&u.cnt, u.ntile)) {
-    if (threadIdx.x == 0) {
+    if (threadIdx.x < 32) {
       double bg = 1e300;
       int al = 1;
-      for (int i = 0; i < u.ntile; ++i) {
+      for (int i = threadIdx.x; i < u.ntile; i += 32) {
         const double pg = __ldcg(partials + u.tile0 + i);
-        if (pg < bg) { bg = pg; al = (int)__ldcg(partials + stride + u.tile0 + i); }
+        const int pl = (int)__ldcg(partials + stride + u.tile0 + i);
+        if (pg < bg) { bg = pg; al = pl; }
       }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        const double og = __shfl_xor_sync(0xffffffffu, bg, o);
+        const int ol = __shfl_xor_sync(0xffffffffu, al, o);
+        if (og < bg) { bg = og; al = ol; }
+      }
+      if (threadIdx.x != 0) return;
       const int64_t cut_a = u.cut[ca], cut_b = u.cut[cb];
       bool b_wins;
       if (cut_b != cut_a) b_wins = cut_b < cut_a;
