@@ -446,8 +446,10 @@ static int invalid_graph(int f) {
 // perm / iperm (optional, meshes concatenated, indices local to each mesh): row
 // i of mesh m in the level-0 graph is the caller's row perm[off_m + i], and the
 // caller's row j becomes row iperm[off_m + j]
+// rows_only: the checked per-row arrays without the graph (coordinate bisection)
 static int build_level0(Ctx& c, const std::vector<MeshIn>& meshes, int validate, LevelGraph& G,
-                        const int64_t* perm = nullptr, const int32_t* iperm = nullptr) {
+                        const int64_t* perm = nullptr, const int32_t* iperm = nullptr,
+                        bool rows_only = false) {
   int64_t N = 0;
   for (auto& m : meshes) N += m.n;
   if (N >= RSB_MAXN) return rsb_set_error(RSB_EINVAL, "too many rows (limit 2^29)");
@@ -463,8 +465,8 @@ static int build_level0(Ctx& c, const std::vector<MeshIn>& meshes, int validate,
   int64_t off = 0;
   for (auto& m : meshes) {
     if ((rc = launch_validate(m.row_ptr, m.col, m.wt, m.n, validate, flag, c.s))) return rc;
-    if ((rc = launch_row_lengths(m.row_ptr, m.n, dptr<int32_t>(c.len) + off, c.s,
-                                 perm ? perm + off : nullptr)))
+    if (!rows_only && (rc = launch_row_lengths(m.row_ptr, m.n, dptr<int32_t>(c.len) + off, c.s,
+                                               perm ? perm + off : nullptr)))
       return rc;
     off += m.n;
   }
@@ -472,6 +474,26 @@ static int build_level0(Ctx& c, const std::vector<MeshIn>& meshes, int validate,
   RSB_CK(cudaStreamSynchronize(c.s));
   if (c.h_pinned[0]) {
     return invalid_graph(c.h_pinned[0]);
+  }
+  for (int k = 0; k < 2; ++k) {
+    if ((rc = devbuf_reserve(c.gid[k], sizeof(int64_t) * (N + 32)))) return rc;
+    if ((rc = devbuf_reserve(c.home[k], sizeof(int64_t) * (N + 32)))) return rc;
+    if ((rc = devbuf_reserve(c.row_seg[k], sizeof(int32_t) * (N + 32)))) return rc;
+  }
+  G.n = (int32_t)N;
+  G.nslices = nsl;
+  G.gid = dptr<int64_t>(c.gid[0]);
+  G.home = dptr<int64_t>(c.home[0]);
+  G.row_seg = dptr<int32_t>(c.row_seg[0]);
+  if (rows_only) {
+    off = 0;
+    for (size_t i = 0; i < meshes.size(); ++i) {
+      if ((rc = launch_fill_rows(meshes[i].gid, meshes[i].n, off, off, (int32_t)i, G.gid, G.home,
+                                 G.row_seg, c.s)))
+        return rc;
+      off += meshes[i].n;
+    }
+    return RSB_OK;
   }
   if ((rc = launch_slice_widths(dptr<int32_t>(c.len), N, dptr<int64_t>(c.slice_sz), c.s))) return rc;
   RSB_CK(cudaMemsetAsync(dptr<int64_t>(c.slice_sz) + nsl, 0, sizeof(int64_t), c.s));
@@ -483,21 +505,12 @@ static int build_level0(Ctx& c, const std::vector<MeshIn>& meshes, int validate,
                          cudaMemcpyDeviceToHost, c.s));
   RSB_CK(cudaStreamSynchronize(c.s));
   if ((rc = devbuf_reserve(c.ent[0], sizeof(uint32_t) * (size_t)std::max<int64_t>(total, 1)))) return rc;
-  for (int k = 0; k < 2; ++k) {
+  for (int k = 0; k < 2; ++k)
     if ((rc = devbuf_reserve(c.deg[k], sizeof(int32_t) * (N + 32)))) return rc;
-    if ((rc = devbuf_reserve(c.gid[k], sizeof(int64_t) * (N + 32)))) return rc;
-    if ((rc = devbuf_reserve(c.home[k], sizeof(int64_t) * (N + 32)))) return rc;
-    if ((rc = devbuf_reserve(c.row_seg[k], sizeof(int32_t) * (N + 32)))) return rc;
-  }
   if ((rc = devbuf_reserve(c.slice_ptr[1], sizeof(int64_t) * (nsl + 2)))) return rc;
-  G.n = (int32_t)N;
-  G.nslices = nsl;
   G.slice_ptr = dptr<int64_t>(c.slice_ptr[0]);
   G.ent = dptr<uint32_t>(c.ent[0]);
   G.deg = dptr<int32_t>(c.deg[0]);
-  G.gid = dptr<int64_t>(c.gid[0]);
-  G.home = dptr<int64_t>(c.home[0]);
-  G.row_seg = dptr<int32_t>(c.row_seg[0]);
   G.nent = total;
   off = 0;
   for (size_t i = 0; i < meshes.size(); ++i) {
@@ -856,9 +869,9 @@ static int run_rsb(Ctx& c, const std::vector<MeshIn>& meshes, const std::vector<
                    int64_t* home_out = nullptr) {
   LevelGraph G;
   trace_mark(c.s, "call start");
-  int rc = build_level0(c, meshes, o.validate, G, perm, iperm);
-  if (rc) return rc;
   const bool rcb = o.method == RSB_RCB;
+  int rc = build_level0(c, meshes, o.validate, G, perm, iperm, rcb);
+  if (rc) return rc;
   if (rcb) {
     int64_t nall = 0;
     for (auto& m : meshes) nall += m.n;
@@ -933,10 +946,7 @@ static int run_rsb(Ctx& c, const std::vector<MeshIn>& meshes, const std::vector<
     // components of every segment
     if ((rc = devbuf_reserve(c.seg_ncomp, sizeof(int32_t) * nseg))) return rc;
     std::vector<int32_t> ncomp(nseg, 1);
-    if (rcb) {
-      // geometric splits ignore connectivity: every segment is one piece
-      RSB_CK(cudaMemsetAsync(c.ckey.p, 0, sizeof(uint64_t) * (size_t)G.n, c.s));
-    } else {
+    if (!rcb) {  // (geometric splits ignore connectivity: every segment is one piece)
       RSB_CK(cudaMemsetAsync(c.seg_ncomp.p, 0, sizeof(int32_t) * nseg, c.s));
       if ((rc = launch_cc(G, dptr<int32_t>(c.parent), dptr<uint64_t>(c.cmin), &cn->flag, c.s)))
         return rc;
@@ -1045,11 +1055,10 @@ static int run_rsb(Ctx& c, const std::vector<MeshIn>& meshes, const std::vector<
     if ((rc = devbuf_reserve(c.seg_split, sizeof(uint8_t) * nseg))) return rc;
     if ((rc = devbuf_reserve(c.seg_keystar, sizeof(uint64_t) * nseg))) return rc;
     if ((rc = devbuf_reserve(c.seg_unit, sizeof(int32_t) * nseg))) return rc;
-    // connected segments: every row has the same key, use the unit's side
     std::vector<uint64_t> ks(nseg);
     std::vector<uint8_t> spl(nseg);
     for (int i = 0; i < nseg; ++i) {
-      spl[i] = split[i] ? 1 : 0;
+      spl[i] = split[i];
       ks[i] = split[i] == 2 ? keystar[i] : 0;
     }
     RSB_CK(cudaMemcpyAsync(c.seg_row0.p, h_row0.data(), sizeof(int64_t) * nseg,
@@ -1061,14 +1070,8 @@ static int run_rsb(Ctx& c, const std::vector<MeshIn>& meshes, const std::vector<
     RSB_CK(cudaMemcpyAsync(c.seg_split.p, spl.data(), nseg, cudaMemcpyHostToDevice, c.s));
     RSB_CK(cudaMemcpyAsync(c.seg_unit.p, seg_unit.data(), sizeof(int32_t) * nseg,
                            cudaMemcpyHostToDevice, c.s));
-    // for connected segments the comparison key must equal every row's key:
-    // give them the key of the segment's first row
     RSB_CK(cudaMemcpyAsync(c.seg_keystar.p, ks.data(), sizeof(uint64_t) * nseg,
                            cudaMemcpyHostToDevice, c.s));
-    for (int i = 0; i < nseg; ++i)
-      if (split[i] == 1)
-        RSB_CK(cudaMemcpyAsync(dptr<uint64_t>(c.seg_keystar) + i, dptr<uint64_t>(c.ckey) + segs[i].row0,
-                               sizeof(uint64_t), cudaMemcpyDeviceToDevice, c.s));
     if ((rc = launch_finalize_side(G, dptr<uint8_t>(c.seg_split), dptr<uint64_t>(c.seg_keystar),
                                    dptr<int32_t>(c.seg_unit), dptr<Unit>(c.units),
                                    dptr<uint64_t>(c.ckey), dptr<uint8_t>(c.side), c.s)))

@@ -758,7 +758,7 @@ struct LevelGraph {
   int32_t n = 0;
   int64_t nslices = 0;
   int64_t* slice_ptr = nullptr;  // nslices + 1
-  uint32_t* ent = nullptr;       // packed entries
+  uint32_t* ent = nullptr;       // packed entries (null: rows only, coordinate bisection)
   int32_t* deg = nullptr;        // weighted degree per row
   int64_t* gid = nullptr;
   int64_t* home = nullptr;       // index into the caller's (concatenated) output
@@ -829,6 +829,8 @@ int launch_scan_i64(const int64_t* in, int64_t* out_excl, int64_t n, void* tmp, 
 size_t scan_tmp_bytes(int64_t n);
 int launch_spmv_f64(const LevelGraph& G, const double* x, double* y, cudaStream_t s);
 int launch_spmv_f32(const LevelGraph& G, const float* x, float* y, cudaStream_t s);
+int launch_fill_rows(const int64_t* gid_in, int64_t n, int64_t row_off, int64_t home_off, int32_t seg,
+                     int64_t* gid, int64_t* home, int32_t* row_seg, cudaStream_t s);
 int launch_csr_apply(const int64_t* row_ptr, const int32_t* col, const int32_t* wt, int64_t n,
                      int f32, const void* x, void* y, int* err, cudaStream_t s);
 int launch_cc(const LevelGraph& G, int32_t* parent, uint64_t* ckey, int* flag, cudaStream_t s);

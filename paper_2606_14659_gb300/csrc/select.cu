@@ -768,8 +768,10 @@ int launch_choose(const LevelGraph& G, const Tile* tiles, int ntiles, Unit* unit
 // ----------------------------------------------------------------------------
 // final side of every row of the level (0 left, 1 right)
 // ----------------------------------------------------------------------------
-// seg_split[s]: 1 when segment s is bisected at this level.
-// seg_keystar[s]: component key of the straddling (or last fitting) component.
+// seg_split[s]: 1 when segment s is bisected at this level and connected, 2 when it
+// is bisected and fell apart.
+// seg_keystar[s]: component key of the straddling (or last fitting) component of a
+// segment that fell apart.
 // seg_unit[s]: unit solving the straddler, or -1 when components fit exactly.
 __global__ void k_finalize_side(const int32_t* __restrict__ row_seg, int32_t n,
                                 const uint8_t* __restrict__ seg_split,
@@ -781,7 +783,7 @@ __global__ void k_finalize_side(const int32_t* __restrict__ row_seg, int32_t n,
   const int s = row_seg[r];
   uint8_t out = 0;
   if (seg_split[s]) {
-    const uint64_t k = ckey[r], ks = seg_keystar[s];
+    const uint64_t k = seg_split[s] == 2 ? ckey[r] : 0, ks = seg_split[s] == 2 ? seg_keystar[s] : 0;
     if (k < ks) out = 0;
     else if (k > ks) out = 1;
     else {
