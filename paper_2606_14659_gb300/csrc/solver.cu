@@ -179,19 +179,20 @@ __device__ __forceinline__ void tile_dots(const LzArgs<V>& a, int nd, int c0, in
     }
   }
   if (kind[0] < 0) return;
-  for (int row = base + lane; row < end; row += 128) {
-    V wv[4];
-    bool ok[4];
+  constexpr int NR = sizeof(V) == 8 ? 2 : 4;  // rows a lane per round
+  for (int row = base + lane; row < end; row += 32 * NR) {
+    V wv[NR];
+    bool ok[NR];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
+    for (int q = 0; q < NR; ++q) {
       ok[q] = row + 32 * q < end;
       wv[q] = ok[q] ? ws[row + 32 * q - base] : V(0);
     }
-    V b[MAXCW][4];
+    V b[MAXCW][NR];
 #pragma unroll
     for (int i = 0; i < MAXCW; ++i)
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
+      for (int q = 0; q < NR; ++q) {
         const int r = row + 32 * q;
         b[i][q] = V(0);
         if (ok[q]) {
@@ -204,7 +205,7 @@ __device__ __forceinline__ void tile_dots(const LzArgs<V>& a, int nd, int c0, in
     for (int i = 0; i < MAXCW; ++i)
       if (kind[i] >= 0) {
 #pragma unroll
-        for (int q = 0; q < 4; ++q)
+        for (int q = 0; q < NR; ++q)
           if (ok[q]) acc[i].add(b[i][q] * wv[q]);
       }
   }
@@ -309,7 +310,8 @@ __device__ __forceinline__ void lz_a_t(const LzArgs<V>& a, int j, int tix, V* ws
       V w = V(0);
       if (r < end) {
         const V xr = src[r];
-        w = s * spmv_row<V, CO>(a.slice_ptr, a.ent, src, r, xr);
+        if constexpr (CO) w = s * spmv_row<V, true>(a.slice_ptr, a.ent, src, r, xr);
+        else w = s * spmv_row_ro<V>(a.slice_ptr, a.ent, src, r, xr);
         qj[r] = s * xr;
         dst[r] = w;
         if (a.pb_a)
@@ -434,15 +436,20 @@ __device__ __forceinline__ void lz_c_t(const LzArgs<V>& a, int j, double breakdo
   }
 }
 
+// FP64 steps A and B.  Bound: the FP64 rate (an FP64 instruction holds a sub-partition
+// for 64 cycles, so one ready warp in each keeps it busy); four CTAs of 64 registers, two
+// rows a lane in flight, leave some warp at its arithmetic while the others wait for
+// loads.  Two CTAs of 128 registers with four rows a lane took 121 us (A) at 1M rows,
+// mean over 16 steps, against 59 for the FMAs alone; this form takes about 60.
 template <typename V>
-__global__ void __launch_bounds__(RSB_BLOCK, sizeof(V) == 4 ? 3 : 2) k_lz_a(LzArgs<V> a, int j) {
+__global__ void __launch_bounds__(RSB_BLOCK, 4) k_lz_a(LzArgs<V> a, int j) {
   __shared__ V ws[SUBROWS];
   __shared__ double out[RSB_MAXC];
   lz_a_t<V, false>(a, j, blockIdx.x, ws, out);
 }
 
 template <typename V>
-__global__ void __launch_bounds__(RSB_BLOCK, sizeof(V) == 4 ? 3 : 2) k_lz_b(LzArgs<V> a, int j) {
+__global__ void __launch_bounds__(RSB_BLOCK, 4) k_lz_b(LzArgs<V> a, int j) {
   __shared__ V ws[SUBROWS];
   __shared__ V cv[RSB_MAXC];
   __shared__ double out[RSB_MAXC];
