@@ -1029,6 +1029,8 @@ __device__ __forceinline__ void jac_block(T& a11, T& a12, T& a21, T& a22, T c1, 
   a22 = s1 * b12 + c1 * b22;
 }
 
+// Sweeps of rotations of J.A (K x K, padded to n2) with J.Z <- J.Z R, until the
+// off-diagonal mass is at most thr.
 // Bound: the latency of a round (some 300 of them), in FP64 its arithmetic as well.
 // A round is two phases: every thread updates its 2x2 blocks of A (all of its loads
 // before its stores: the blocks are disjoint); then one warp computes the next round's
@@ -1037,30 +1039,9 @@ __device__ __forceinline__ void jac_block(T& a11, T& a12, T& a21, T& a22, T c1, 
 // own rounding), in FP64 the upper ones, which are mirrored.  With the rotations alone
 // in a phase of their own and the updates one after the other, 40 x 40 took 200 us in
 // FP32 and 1240 us in FP64.
-template <typename T, bool CO>
-__device__ __noinline__ void lz_eig_u(Unit& u, double* Sm, JacShared<T>& J) {
-  if (ldc<CO>(&u.status) != U_ACTIVE) return;
+template <typename T>
+__device__ void jac_sweeps(JacShared<T>& J, int K, int n2, double thr) {
   const int tid = threadIdx.x, w = tid >> 5;
-  const int K = ldc<CO>(&u.msteps);
-  const int n2 = K + (K & 1);
-  for (int idx = tid; idx < n2 * n2; idx += RSB_BLOCK) {
-    const int i = idx / n2, k = idx % n2;
-    J.A[i][k] = (i < K && k < K) ? T(ldc<CO>(Sm + i * RSB_MAXM + k)) : T(0);
-    J.Z[i][k] = i == k ? T(1) : T(0);
-  }
-  __syncthreads();
-  double fro = 0.0;
-  for (int idx = tid; idx < K * K; idx += RSB_BLOCK) {
-    const double x = (double)J.A[idx / K][idx % K];
-    fro += x * x;
-  }
-  fro = block_sum(fro, J.red);
-  if (tid == 0) J.red[0] = fro;
-  __syncthreads();
-  fro = J.red[0];
-  __syncthreads();
-  const double eps2 = sizeof(T) == 8 ? 1e-30 : 1e-14;
-  const double thr = fro * eps2;
   const int np = n2 / 2;
   // this thread's blocks of A (pair i1 x pair i2; FP32: two, FP64: one with i1 <= i2)
   // and (pair, row) updates of Z (warps 1..7); fixed for the whole solve
@@ -1191,6 +1172,178 @@ __device__ __noinline__ void lz_eig_u(Unit& u, double* Sm, JacShared<T>& J) {
       buf ^= 1;
     }
   }
+}
+
+// J.A <- S (columns and rows < K, else 0), J.Z <- I; returns sum S_ij^2 to every thread.
+template <typename T, bool CO>
+__device__ double jac_load(const double* Sm, JacShared<T>& J, int K, int n2) {
+  const int tid = threadIdx.x;
+  for (int idx = tid; idx < n2 * n2; idx += RSB_BLOCK) {
+    const int i = idx / n2, k = idx % n2;
+    J.A[i][k] = (i < K && k < K) ? T(ldc<CO>(Sm + i * RSB_MAXM + k)) : T(0);
+    J.Z[i][k] = i == k ? T(1) : T(0);
+  }
+  __syncthreads();
+  double fro = 0.0;
+  for (int idx = tid; idx < K * K; idx += RSB_BLOCK) {
+    const double x = (double)J.A[idx / K][idx % K];
+    fro += x * x;
+  }
+  fro = block_sum(fro, J.red);
+  if (tid == 0) J.red[0] = fro;
+  __syncthreads();
+  fro = J.red[0];
+  __syncthreads();
+  return fro;
+}
+
+// FP64 eigenpairs of S from the FP32 ones: the iteration of Ogita and Aishima
+// ("Iterative refinement for symmetric eigenvalue decomposition", 2018).  With
+// R = I - X^T X and B = X^T S X, lambda_i = B_ii / (1 - R_ii), the correction
+// X <- X + X E, E_ij = (B_ij + lambda_j R_ij) / (lambda_j - lambda_i), E_ii = R_ii / 2,
+// squares the error; it ends when |E| is small enough that the square is below FP64's
+// rounding.  False (uniform) when a correction is not small (eigenvalues too close for
+// their FP32 vectors): the caller then takes the FP64 rotations.  On return J.Z holds
+// the vectors and the diagonal of J.A the values.
+// Bound: the FP64 rate, three to four K^3 products an iteration, two iterations as a
+// rule, where the rotations take five to eight sweeps (816 us for 40 x 40, 183 for 16 x
+// 16): 512-row box into 8 parts (14 polish cycles of 16) 12.4 -> 10.8 ms, FP64 Fiedler
+// pair of 28k rows (7 cycles of 40) 15.0 -> 13.8 ms.
+template <bool CO>
+__device__ bool eig_refine(const double* Sm, JacShared<double>& J, int K, int n2) {
+  constexpr int NE = (RSB_MAXM * RSB_MAXM + RSB_BLOCK - 1) / RSB_BLOCK;
+  const int tid = threadIdx.x;
+  double* lam = &J.cs[0][0][0];  // K values
+  // X from the FP32 vectors (which lie in J.Z's place)
+  {
+    const JacShared<float>& F = *reinterpret_cast<const JacShared<float>*>(&J.Z[0][0]);
+    float z[NE];
+#pragma unroll
+    for (int m = 0; m < NE; ++m) {
+      const int idx = tid + m * RSB_BLOCK;
+      z[m] = idx < K * K ? F.Z[idx / K][idx % K] : 0.f;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int m = 0; m < NE; ++m) {
+      const int idx = tid + m * RSB_BLOCK;
+      if (idx < K * K) J.Z[idx / K][idx % K] = (double)z[m];
+    }
+    __syncthreads();
+  }
+  for (int it = 0; it < 6; ++it) {
+    // J.A <- S X (S symmetric: read by rows l, coalesced over i)
+    for (int idx = tid; idx < K * K; idx += RSB_BLOCK) {
+      const int k = idx / K, i = idx % K;
+      double x = 0.0;
+#pragma unroll 4
+      for (int l = 0; l < K; ++l) x = fma(ldc<CO>(Sm + l * RSB_MAXM + i), J.Z[l][k], x);
+      J.A[i][k] = x;
+    }
+    __syncthreads();
+    // B and R, entry (i, k) with i <= k in one thread
+    double bij[NE], rij[NE];
+#pragma unroll
+    for (int m = 0; m < NE; ++m) {
+      const int idx = tid + m * RSB_BLOCK;
+      const int i = idx / K, k = idx % K;
+      bij[m] = rij[m] = 0.0;
+      if (idx < K * K && i <= k) {
+        double x = 0.0, y = i == k ? 1.0 : 0.0;
+        for (int l = 0; l < K; ++l) {
+          const double z = J.Z[l][i];
+          x = fma(z, J.A[l][k], x);
+          y = fma(-z, J.Z[l][k], y);
+        }
+        bij[m] = x;
+        rij[m] = y;
+        if (i == k) lam[i] = x / (1.0 - y);
+      }
+    }
+    __syncthreads();
+    // E into J.A
+    float emax = 0.f;
+#pragma unroll
+    for (int m = 0; m < NE; ++m) {
+      const int idx = tid + m * RSB_BLOCK;
+      const int i = idx / K, k = idx % K;
+      if (idx < K * K && i <= k) {
+        if (i == k) {
+          J.A[i][i] = 0.5 * rij[m];
+          const float e = fabsf((float)rij[m]);
+          emax = e <= emax ? emax : e;  // (a NaN is kept)
+        } else {
+          // E_ik and E_ki; FP32 is accurate enough for a correction
+          const float d = (float)(lam[k] - lam[i]);
+          const float nik = (float)fma(lam[k], rij[m], bij[m]);
+          const float nki = (float)fma(lam[i], rij[m], bij[m]);
+          const bool zero = nik == 0.f && nki == 0.f;
+          const float eik = zero ? 0.f : nik / d, eki = zero ? 0.f : -nki / d;
+          J.A[i][k] = (double)eik;
+          J.A[k][i] = (double)eki;
+          const float e = fabsf(eik) + fabsf(eki);
+          emax = e <= emax ? emax : e;
+        }
+      }
+    }
+    const bool bad = !(emax <= 1e-2f);
+    const bool more = !(emax <= 2e-9f);
+    const int any_bad = __syncthreads_or(bad);
+    const int any_more = __syncthreads_or(more);
+    if (any_bad) return false;
+    // X <- X + X E
+    double x[NE];
+#pragma unroll
+    for (int m = 0; m < NE; ++m) {
+      const int idx = tid + m * RSB_BLOCK;
+      const int i = idx / K, k = idx % K;
+      x[m] = 0.0;
+      if (idx < K * K) {
+        double y = J.Z[i][k];
+#pragma unroll 4
+        for (int l = 0; l < K; ++l) y = fma(J.Z[i][l], J.A[l][k], y);
+        x[m] = y;
+      }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int m = 0; m < NE; ++m) {
+      const int idx = tid + m * RSB_BLOCK;
+      if (idx < K * K) J.Z[idx / K][idx % K] = x[m];
+    }
+    __syncthreads();
+    if (!any_more) {
+      if (tid < K) J.A[tid][tid] = lam[tid];
+      __syncthreads();
+      return true;
+    }
+  }
+  return false;
+}
+
+// Ritz pairs of one unit: FP32 by rotations; FP64 by FP32 rotations and their
+// refinement, or by FP64 rotations where that does not converge.
+template <typename T, bool CO>
+__device__ __noinline__ void lz_eig_u(Unit& u, double* Sm, JacShared<T>& J) {
+  if (ldc<CO>(&u.status) != U_ACTIVE) return;
+  const int tid = threadIdx.x;
+  const int K = ldc<CO>(&u.msteps);
+  const int n2 = K + (K & 1);
+  if constexpr (sizeof(T) == 4) {
+    const double fro = jac_load<T, CO>(Sm, J, K, n2);
+    jac_sweeps(J, K, n2, fro * 1e-14);
+  } else {
+    static_assert(sizeof(J) - sizeof(J.A) >= sizeof(JacShared<float>), "FP32 workspace");
+    JacShared<float>& F = *reinterpret_cast<JacShared<float>*>(&J.Z[0][0]);
+    const double fro = jac_load<float, CO>(Sm, F, K, n2);
+    jac_sweeps(F, K, n2, fro * 1e-14);
+    __syncthreads();
+    if (!eig_refine<CO>(Sm, J, K, n2)) {
+      const double f = jac_load<T, CO>(Sm, J, K, n2);
+      jac_sweeps(J, K, n2, f * 1e-30);
+    }
+  }
+  __syncthreads();
   // ascending order (ties by index)
   if (tid < K) {
     const T e = J.A[tid][tid];
