@@ -541,8 +541,15 @@ static int max_unit_tiles(const std::vector<Unit>& units) {
 
 // mesh_rows[i]: the element count of the mesh unit i belongs to (empty: the
 // units are parts of one mesh, whose rows they cover)
+// fp64_small: FP64 solves by default tiles.  A small mesh then has tiles of one row a
+// thread, because an FP64 row takes 64 cycles of a sub-partition an operation and twice
+// the tiles put twice the SMs to work: 28k rows, 40 FP64 steps 37 -> 27 us each.  Up to
+// RSB_SMALL_FP64 rows the tiles (with one more for every unit's remainder) still fit the
+// 152 SMs one each, so that the solve stays resident; a unit of two tiles or fewer of two
+// rows would pay more for barriers than it gains.
+#define RSB_SMALL_FP64 31000
 static void make_tiles(std::vector<Unit>& units, std::vector<Tile>& tiles, int rmin = RSB_MINR,
-                       const std::vector<int64_t>& mesh_rows = {}) {
+                       const std::vector<int64_t>& mesh_rows = {}, bool fp64_small = false) {
   tiles.clear();
   // rows per thread of a tile: at least rmin (memory-level parallelism), more
   // in a mesh so large that one of its levels would exceed about
@@ -559,7 +566,8 @@ static void make_tiles(std::vector<Unit>& units, std::vector<Tile>& tiles, int r
                           ((int64_t)RSB_BLOCK * RSB_TARGET_TILES);
     int64_t R = (nr + (int64_t)RSB_BLOCK * RSB_MAXTILES_PER_UNIT - 1) /
                 ((int64_t)RSB_BLOCK * RSB_MAXTILES_PER_UNIT);
-    if (R < rmin) R = rmin;
+    const bool one = fp64_small && nmesh <= RSB_SMALL_FP64 && nr > 2 * 2 * RSB_BLOCK;
+    if (R < rmin && !one) R = rmin;
     if (R < rmesh) R = rmesh;
     const int64_t tr = R * RSB_BLOCK;
     u.tile0 = (int32_t)tiles.size();
@@ -1038,7 +1046,8 @@ static int run_rsb(Ctx& c, const std::vector<MeshIn>& meshes, const std::vector<
     std::vector<Tile> htiles;
     std::vector<int64_t> hmesh;
     for (const Unit& u : hunits) hmesh.push_back(meshes[segs[u.seg].mesh].n);
-    make_tiles(hunits, htiles, o.tile_rows > 0 ? o.tile_rows : RSB_MINR, hmesh);
+    make_tiles(hunits, htiles, o.tile_rows > 0 ? o.tile_rows : RSB_MINR, hmesh,
+               o.precision == RSB_FP64 && o.tile_rows == 0);
     trace_mark(c.s, "level %d components and units", level);
     if ((rc = split_units(c, G, hunits, htiles, o, rs))) return rc;
     trace_mark(c.s, "level %d split (%d units)", level, (int)hunits.size());
@@ -1471,7 +1480,8 @@ extern "C" int rsb_fiedler(const rsb_csr* g, const rsb_options* opt, double* lam
   u.k = N / 2;
   u.isn = 1.0 / std::sqrt((double)N);
   std::vector<Tile> htiles;
-  make_tiles(hunits, htiles, o.tile_rows > 0 ? o.tile_rows : RSB_MINR);
+  make_tiles(hunits, htiles, o.tile_rows > 0 ? o.tile_rows : RSB_MINR, {},
+             o.precision == RSB_FP64 && o.tile_rows == 0);
   c.trmax = max_tile_rows(htiles);
   c.ntmax = max_unit_tiles(hunits);
   const int ntiles = (int)htiles.size();
