@@ -97,7 +97,8 @@ struct Unit {
   // CG scalars (§7): FP64 recurrences in both precisions
   double rr, cg_alpha, cg_beta, bnorm;
   double fz_rz, fz_ro;          // flexible CG: z.r and z.r_old of the new z
-  double dz_src, dz_z, dz_qz;   // delayed second pass: scales of src, z and q_j in step D3
+  float dz[3];                  // step D3 (FP32): scales of src, z and q_j, and the pairs
+  alignas(8) float cf[RSB_MAXC][2];  // a~, g~ of every basis column
   double cz[1 + RSB_MAXD];      // flexible CG: projection coefficients of z
   double rq, lnorm2;
   // select / split
@@ -375,19 +376,37 @@ __device__ __forceinline__ double block_sums(const double (&v)[NV], int nv, doub
 
 // Block total of per-thread accumulators (warp_total per warp, then the warps
 // in order in FP64); result valid in thread 0.
-template <typename V>
-__device__ __forceinline__ double block_total(const Acc<V>& a, double* sm) {
-  const double v = warp_total(a);
-  const int w = threadIdx.x >> 5;
-  if ((threadIdx.x & 31) == 0) sm[w] = v;
-  __syncthreads();
-  double s = 0.0;
-  if (threadIdx.x == 0) {
+__device__ __forceinline__ double block_total(const Acc<double>& a, double* sm) {
+  return block_sum(a.s, sm);
+}
+// FP32: the warps' states are converted to FP64 together by eight lanes.  NA
+// accumulators a thread stand for NA * blockDim / 32 warps' worth of rows: warp w of
+// accumulator i is warp w + i * blockDim / 32 of the order.
+template <int NA>
+__device__ __forceinline__ double block_total_n(const Acc<float> (&a)[NA], double* sm) {
+  float2* st = reinterpret_cast<float2*>(sm);
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
 #pragma unroll
-    for (int i = 0; i < RSB_WARPS; ++i) s += sm[i];
+  for (int i = 0; i < NA; ++i) {
+    float s = a[i].s, c = a[i].c;
+    warp_merge(s, c);
+    if (lane == 0) st[w + i * (RSB_WARPS / NA)] = make_float2(s, c);
   }
   __syncthreads();
-  return s;
+  double t = 0.0;
+  if (w == 0) {
+    const float2 p = lane < RSB_WARPS ? st[lane] : make_float2(0.f, 0.f);
+    const double v = (double)p.x - (double)p.y;
+    t = v;
+#pragma unroll
+    for (int i = 1; i < RSB_WARPS; ++i) t += __shfl_sync(0xffffffffu, v, i);
+  }
+  __syncthreads();
+  return t;
+}
+__device__ __forceinline__ double block_total(const Acc<float>& a, double* sm) {
+  const Acc<float> x[1] = {a};
+  return block_total_n<1>(x, sm);
 }
 
 // Gram-Schmidt coefficients in the vector type, converted once per CTA:
@@ -601,7 +620,7 @@ __device__ __forceinline__ void final_reduce_few(const double* partials, long lo
                                                  int nt, int nc, double* out, double* sp,
                                                  int rot = 0) {
   const int nq = nt > 24 ? (nt - 25) / 32 + 1 : 0;  // 32-tile blocks with a full lane
-  for (int idx = threadIdx.x; idx < nc * nq * 8; idx += RSB_BLOCK) {
+  for (int idx = threadIdx.x; idx < nc * nq * 8; idx += blockDim.x) {
     const int s = idx & 7, cq = idx >> 3;
     const int c = cq / nq, q = cq - c * nq;
     const int t = 32 * q + s;

@@ -807,16 +807,13 @@ __global__ void __launch_bounds__(RSB_BLOCK) k_lz_close(LzArgs<V> a, int j, int 
     //     w = z / rho - sum_b (g_b / rho) b - (q_j.z / rho) q_j
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (w == 4) {
-      const double x = (lane == 0 ? inu : lane == 1 ? 1.0 : sc[1]) / rho;
-      if (lane == 0) u.dz_src = x;
-      if (lane == 1) u.dz_z = x;
-      if (lane == 2) u.dz_qz = x;
-    } else if (w < 2) {
-      const int b = threadIdx.x;
-      if (b < nb) u.c2[b] = out[b] / rho;
+      if (lane < 3) u.dz[lane] = (float)((lane == 0 ? inu : lane == 1 ? 1.0 : sc[1]) / rho);
     } else if (w < 4) {
-      const int b = threadIdx.x - 64;
-      if (b < nb) u.c1[b] = out[nc + b] / rho;
+      const int b = threadIdx.x & 63, h = threadIdx.x >> 6;
+      if (b < nb) {
+        const double x = out[h * nc + b] / rho;
+        u.cf[b][h] = (float)(b == 0 ? x * u.isn : x);
+      }
     }
     __syncthreads();
     d2_store_S(Sm, j, sk);
@@ -840,10 +837,15 @@ __global__ void __launch_bounds__(RSB_BLOCK) k_lz_close(LzArgs<V> a, int j, int 
 // thread, 48 registers and five CTAs the last, nearly empty wave of tiles made it 106.
 // The tiles are taken in the opposite order of D2, which has just streamed the same
 // vectors: what it read last is still in L2 (4 % at 1M rows, nothing at 3.7M).
+// T = 256 threads, or 128 where the tiles are more than the chip holds CTAs of 256: the
+// CTAs of short tiles live for a chain of loads and a reduction whatever their rows, so
+// one wave of sixteen a SM beats two of eight (batch of 1800 tiles 260 -> 255 ms,
+// with the scales and coefficients converted once by the closing kernel).  A thread of 128 keeps the sums of rows
+// t and t + 128 of every 256 apart, which are merged in the order of 256 threads.
 #define D3_KB 4  // basis vectors a round
 #define D3_RR 2  // rows a thread
-template <typename V>
-__global__ void __launch_bounds__(RSB_BLOCK, 8) k_lz_d3(LzArgs<V> a, int j, double breakdown) {
+template <typename V, int T>
+__global__ void __launch_bounds__(T, 2048 / T) k_lz_d3(LzArgs<V> a, int j, double breakdown) {
   __shared__ double sm[RSB_WARPS];
   __shared__ __align__(16) V cc[RSB_MAXC][2];  // a~, g~
   __shared__ double out[1];
@@ -854,22 +856,22 @@ __global__ void __launch_bounds__(RSB_BLOCK, 8) k_lz_d3(LzArgs<V> a, int j, doub
   if (u.status != U_ACTIVE || j >= u.msteps || j < u.j0) return;
   const int nd = u.nd;
   const int nb = 1 + nd + j;
-  for (int k = threadIdx.x; k < nb; k += RSB_BLOCK) {
-    const double x = u.c2[k], y = u.c1[k];
-    cc[k][0] = k == 0 ? V(x * u.isn) : V(x);
-    cc[k][1] = k == 0 ? V(y * u.isn) : V(y);
+  for (int k = threadIdx.x; k < nb; k += T) {
+    const float2 x = *reinterpret_cast<const float2*>(u.cf[k]);
+    cc[k][0] = x.x;
+    cc[k][1] = x.y;
   }
   __syncthreads();
-  const V ssrc = V(u.dz_src), sz = V(u.dz_z), sqz = V(u.dz_qz);
+  const V ssrc = u.dz[0], sz = u.dz[1], sqz = u.dz[2];
   const V* src = (j & 1) ? a.W1 : a.W0;
   V* dst = (j & 1) ? a.W0 : a.W1;
-  Acc<V> acc;
-  for (int r0 = t.row0 + threadIdx.x; r0 < t.row1; r0 += D3_RR * RSB_BLOCK) {
+  Acc<V> acc[RSB_BLOCK / T];
+  for (int r0 = t.row0 + threadIdx.x; r0 < t.row1; r0 += D3_RR * T) {
     V q[D3_RR], w[D3_RR];
     bool ok[D3_RR];
 #pragma unroll
     for (int rr = 0; rr < D3_RR; ++rr) {
-      const int r = r0 + rr * RSB_BLOCK;
+      const int r = r0 + rr * T;
       ok[rr] = r < t.row1;
       q[rr] = ok[rr] ? ssrc * src[r] : V(0);
       w[rr] = ok[rr] ? sz * a.AP[r] : V(0);
@@ -883,7 +885,7 @@ __global__ void __launch_bounds__(RSB_BLOCK, 8) k_lz_d3(LzArgs<V> a, int j, doub
 #pragma unroll
       for (int rr = 0; rr < D3_RR; ++rr)
         if (ok[rr]) {
-          const V dv = V(d[rr * RSB_BLOCK]);
+          const V dv = V(d[rr * T]);
           q[rr] -= cc[1 + l][0] * dv;
           w[rr] -= cc[1 + l][1] * dv;
         }
@@ -897,7 +899,7 @@ __global__ void __launch_bounds__(RSB_BLOCK, 8) k_lz_d3(LzArgs<V> a, int j, doub
       for (int i = 0; i < D3_KB; ++i)
 #pragma unroll
         for (int rr = 0; rr < D3_RR; ++rr)
-          qv[i][rr] = ok[rr] ? qk[i * a.N + rr * RSB_BLOCK] : V(0);
+          qv[i][rr] = ok[rr] ? qk[i * a.N + rr * T] : V(0);
 #pragma unroll
       for (int i = 0; i < D3_KB; ++i)
 #pragma unroll
@@ -910,23 +912,23 @@ __global__ void __launch_bounds__(RSB_BLOCK, 8) k_lz_d3(LzArgs<V> a, int j, doub
 #pragma unroll
       for (int rr = 0; rr < D3_RR; ++rr)
         if (ok[rr]) {
-          const V b = qk[rr * RSB_BLOCK];
+          const V b = qk[rr * T];
           q[rr] -= ck[0][0] * b;
           w[rr] -= ck[0][1] * b;
         }
 #pragma unroll
     for (int rr = 0; rr < D3_RR; ++rr)
       if (ok[rr]) {
-        const int r = r0 + rr * RSB_BLOCK;
+        const int r = r0 + rr * T;
         w[rr] -= sqz * q[rr];
         a.Q[(long long)j * a.N + r] = q[rr];
         dst[r] = w[rr];
-        acc.add(w[rr] * w[rr]);
+        acc[rr % (RSB_BLOCK / T)].add(w[rr] * w[rr]);
       }
   }
   if (a.pb_b && threadIdx.x == 0)
     atomicAdd(a.pb_b, (t.row1 - t.row0) * (sizeof(V) * (unsigned long long)(4 + j) + 8ull * nd));
-  const double sum = block_total(acc, sm);
+  const double sum = block_total_n<RSB_BLOCK / T>(acc, sm);
   if (threadIdx.x == 0) a.partials[tix] = sum;
   if (last_cta(&u.cnt, u.ntile)) {
     final_reduce_few(a.partials, a.stride, u.tile0, u.ntile, 1, out, sp);
@@ -2450,6 +2452,7 @@ static int lz_start(LzArgs<V>& a, int ntiles, uint64_t sd, const double* from64,
 template <typename V>
 static int lz_cycle(LzArgs<V>& a, int ntiles, int nunits, int M, double breakdown, int trmax,
                     int ntmax, int nd, cudaStream_t s) {
+  constexpr int d3_one_wave = 8 * 152;  // CTAs of 256 threads at once
   // CTAs per tile of step D1
   const int nsub = std::max(1, (trmax + A1_ROWS - 1) / A1_ROWS);
   for (int j = 0; j < M; ++j) {
@@ -2466,7 +2469,8 @@ static int lz_cycle(LzArgs<V>& a, int ntiles, int nunits, int M, double breakdow
       RSB_CKL("k_lz_close<D2>");
       prof_after(pi, s);
       pi = prof_before(PROF_LZ_B, s);
-      k_lz_d3<V><<<ntiles, RSB_BLOCK, 0, s>>>(a, j, breakdown);
+      if (ntiles > d3_one_wave) k_lz_d3<V, 128><<<ntiles, 128, 0, s>>>(a, j, breakdown);
+      else k_lz_d3<V, 256><<<ntiles, 256, 0, s>>>(a, j, breakdown);
       RSB_CKL("k_lz_d3");
       prof_after(pi, s);
     } else {  // FP64: bound by GB300's FP64 rate; register-streaming kernels, CGS2
