@@ -541,12 +541,13 @@ static int max_unit_tiles(const std::vector<Unit>& units) {
 
 // mesh_rows[i]: the element count of the mesh unit i belongs to (empty: the
 // units are parts of one mesh, whose rows they cover)
-// fp64_small: FP64 solves by default tiles.  A small mesh then has tiles of one row a
-// thread, because an FP64 row takes 64 cycles of a sub-partition an operation and twice
-// the tiles put twice the SMs to work: 28k rows, 40 FP64 steps 37 -> 27 us each.  Up to
-// RSB_SMALL_FP64 rows the tiles (with one more for every unit's remainder) still fit the
-// 152 SMs one each, so that the solve stays resident; a unit of two tiles or fewer of two
-// rows would pay more for barriers than it gains.
+// fp64_small: the one FP64 solve of rsb_fiedler by default tiles.  A small mesh then has
+// tiles of one row a thread, because an FP64 row takes 64 cycles of a sub-partition an
+// operation and twice the tiles put twice the SMs to work: Fiedler pair of 28k rows 13.8
+// -> 11.3 ms.  Up to RSB_SMALL_FP64 rows the tiles still fit the 152 SMs one each, so that
+// the solve stays resident; a unit of two tiles or fewer of two rows would pay more for
+// barriers than it gains.  Partitions keep two rows: they tile a mesh alike alone and in
+// a batch, whose other meshes use those SMs (eight of 28k rows: 96 ms so, 88 before).
 #define RSB_SMALL_FP64 31000
 static void make_tiles(std::vector<Unit>& units, std::vector<Tile>& tiles, int rmin = RSB_MINR,
                        const std::vector<int64_t>& mesh_rows = {}, bool fp64_small = false) {
@@ -1046,8 +1047,7 @@ static int run_rsb(Ctx& c, const std::vector<MeshIn>& meshes, const std::vector<
     std::vector<Tile> htiles;
     std::vector<int64_t> hmesh;
     for (const Unit& u : hunits) hmesh.push_back(meshes[segs[u.seg].mesh].n);
-    make_tiles(hunits, htiles, o.tile_rows > 0 ? o.tile_rows : RSB_MINR, hmesh,
-               o.precision == RSB_FP64 && o.tile_rows == 0);
+    make_tiles(hunits, htiles, o.tile_rows > 0 ? o.tile_rows : RSB_MINR, hmesh);
     trace_mark(c.s, "level %d components and units", level);
     if ((rc = split_units(c, G, hunits, htiles, o, rs))) return rc;
     trace_mark(c.s, "level %d split (%d units)", level, (int)hunits.size());

@@ -60,3 +60,30 @@ def test_deflated_steps_streaming_equals_resident(rows):
     parts = [R.rsb_partition(G, 8, R.options(precision="mixed", use_graph=mode,
                                              tile_rows=rows))[0] for mode in (0, 1, 3)]
     assert torch.equal(parts[0], parts[1]) and torch.equal(parts[0], parts[2])
+
+
+def test_many_short_tiles_equal_the_mesh_alone():
+    """Step D3 runs CTAs of 128 threads once a level has more than 1216 tiles: 1300
+    one-tile units of 4 to 88 rows, each bit-equal to its mesh solved alone."""
+    meshes = [box_graph(2 + i % 3, 2, 1 + i % 11) for i in range(1300)]
+    o = R.options(precision="mixed", use_graph=1, krylov_dim=12, keep=4, max_restarts=6)
+    parts, _, _ = R.rsb_partition_batch([R.graph(g) for g in meshes], [4] * len(meshes), o)
+    for i in list(range(0, 33)) + [1299]:
+        alone, _, _ = R.rsb_partition(R.graph(meshes[i]), 4, o)
+        assert torch.equal(torch.as_tensor(parts[i]), torch.as_tensor(alone)), i
+
+
+# FP64 tiles have one row a thread in units above 1024 rows of meshes up to 31000
+FP64 = [box_graph(16, 16, 4), box_graph(41, 5, 5), box_graph(31, 25, 40), box_graph(52, 71, 9)]
+
+
+@pytest.mark.parametrize("g", FP64, ids=lambda g: str(g.n))
+def test_fp64_tiles_at_the_edges_of_their_rule(g):
+    G = R.graph(g)
+    got = [R.rsb_fiedler(G, R.options(precision="fp64", use_graph=m)) for m in (0, 1, 3)]
+    for lam, v, _, code in got[1:]:
+        assert lam == got[0][0] and code == got[0][3] and torch.equal(v, got[0][1])
+    assert got[0][3] == 0
+    lam, v = got[0][0], got[0][1].cpu().numpy()
+    dmax = O.degree(g).max()
+    assert np.linalg.norm(O.laplacian_apply(g, v) - lam * v) <= (1e-10 + 1e-13) * dmax
