@@ -1564,22 +1564,27 @@ static int lap_apply(const rsb_csr* g, const void* x, void* y, int f32, void* st
     }
     yd = ty.p;
   }
-  // faults are reported into pinned host words that the call reads after its only
-  // synchronisation
+  // faults are reported into pinned host words that the call reads once the kernel is
+  // done; a host y is left alone then
   int* err = c.h_pinned + 8;
   for (int i = 0; i < 5; ++i) err[i] = 0;
   rc = launch_csr_apply(m.row_ptr, m.col, m.wt, N, f32, xd, yd, err, c.s);
+  auto faults = [&] {
+    int f = 0;
+    for (int i = 0; i < 5; ++i) f |= err[i] ? 1 << i : 0;
+    return f;
+  };
   if (!rc && yh) {
-    cudaError_t e = cudaMemcpyAsync(y, yd, es * N, cudaMemcpyDeviceToHost, c.s);
+    cudaError_t e = cudaStreamSynchronize(c.s);
+    if (e == cudaSuccess && !faults())
+      e = cudaMemcpyAsync(y, yd, es * N, cudaMemcpyDeviceToHost, c.s);
     if (e != cudaSuccess) rc = rsb_set_cuda_error(e, "copy y");
   }
   rc = end_call(c, stream, rc);
   free_buf(tx);
   free_buf(ty);
-  int f = 0;
-  for (int i = 0; i < 5; ++i) f |= err[i] ? 1 << i : 0;
-  if (!rc && f) return invalid_graph(f);
-  return rc;
+  const int f = faults();
+  return !rc && f ? invalid_graph(f) : rc;
 }
 
 static int lap_bench(const rsb_csr* g, int f32, int reps, double* ms, double* bytes, void* stream) {

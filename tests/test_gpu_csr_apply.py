@@ -92,3 +92,13 @@ def test_malformed_graphs_are_refused(what):
         assert err.value.code == R.rsb.RSB_EINVAL
     ok = R.graph(box_graph(17, 5, 3))  # the next call is clean
     assert torch.isfinite(R.rsb_laplacian_apply(ok, x)).all()
+
+
+def test_refused_graph_leaves_a_host_vector():
+    g = box_graph(17, 5, 3)
+    G = R.graph(g, device="host")
+    G.weight[100] = 0
+    y = np.full(g.n, 3.5)
+    with pytest.raises(R.RSBError):
+        R.rsb_laplacian_apply(G, np.ones(g.n), y)
+    assert np.all(y == 3.5)
