@@ -103,7 +103,9 @@ typedef struct rsb_options {
                             kernel per cycle, 3 one persistent cooperative kernel per
                             solve whose CTAs keep their tile's basis rows in shared
                             memory when every tile gets a co-resident CTA (else 1);
-                            CG blocks use a CUDA graph for 1, 2 and 3                */
+                            CG: 3 one cooperative launch per CG solve when every tile
+                            gets a co-resident CTA, else (and for 1 and 2) blocks of
+                            iterations as a CUDA graph                            */
   int validate;          /* 1: also check symmetry of the input on the device      */
   int polish_cycles;     /* MIXED: at most this many FP64 Lanczos cycles of polish_dim
                             steps after the FP32 stage, stopping early at tol (0: only
@@ -217,8 +219,8 @@ int rsb_fiedler(const rsb_csr *g, const rsb_options *o, double *lambda2, double 
  * y = L x with L = D - A of graph g (§4 weighted Laplacian, §5 action), in FP64
  * (x, y double[n]) or FP32 (x, y float[n]): a building block exposed for testing.
  * Rows are summed in entry order, as the solvers sum the library's sliced-ELL
- * form.  The graph is checked on the way; when it is malformed (RSB_EINVAL), y is
- * undefined.
+ * form.  The graph is checked on the way; when it is malformed (RSB_EINVAL), a
+ * device y is undefined.
  */
 int rsb_laplacian_apply(const rsb_csr *g, const double *x, double *y, void *stream);
 int rsb_laplacian_apply_f32(const rsb_csr *g, const float *x, float *y, void *stream);
@@ -263,7 +265,8 @@ int rsb_dual_graph(int64_t ne, int nv, const int64_t *ev, int64_t *row_ptr, int3
  * (c_v x_e - w_v), c_v the number of elements at v and w_v their sum: the
  * weighted Laplacian of the dual graph above.  ne, nv, ev as in
  * rsb_dual_graph; x, y double[ne] (or float[ne] for the _f32 form), device or
- * host.  The vertex buckets are rebuilt by every call.
+ * host; y may be x.  The elements at every vertex are gathered anew by every call.
+ * When ids are refused (RSB_EINVAL), a device y other than x is undefined.
  */
 int rsb_laplacian_apply_gs(int64_t ne, int nv, const int64_t *ev, const double *x, double *y,
                            void *stream);

@@ -1704,6 +1704,15 @@ static int gs_setup(Ctx& c, int64_t ne, int nv, const int64_t* ev_in, int64_t* V
                     dptr<int32_t>(c.gs_ev32), c.scan_tmp.p, c.scan_tmp.cap, c.s);
 }
 
+// gs_setup after the slot table was tried: its room is larger than the buckets', so it
+// is given back when the buckets find none.
+static int gs_setup_after_slots(Ctx& c, int64_t ne, int nv, const int64_t* ev, int64_t* V) {
+  int rc = gs_setup(c, ne, nv, ev, V);
+  if (rc != RSB_ENOMEM) return rc;
+  for (DevBuf* b : {&c.gs_cursor, &c.gs_bucket, &c.gs_w, &c.gs_rows}) free_buf(*b);
+  return gs_setup(c, ne, nv, ev, V);
+}
+
 // Row lengths and offsets of the dual graph in c.gs_rowptr, their total in *total: from
 // the slot table (with want_rows, the rows in c.gs_rows as well) when the mesh fits it
 // (*slots = 1), else from the buckets.
@@ -1711,32 +1720,36 @@ static int dual_rows(Ctx& c, int64_t ne, int nv, const int64_t* ev, bool want_ro
                      int* slots) {
   int rc;
   const int64_t cap = gs_slot_cap(ne);
-  if ((rc = devbuf_reserve(c.gs_cursor, sizeof(int32_t) * (size_t)cap)) ||
-      (rc = devbuf_reserve(c.gs_bucket, gs_slot_bytes(cap))) ||
-      (rc = devbuf_reserve(c.gs_len, sizeof(int64_t) * (size_t)(ne + 2))) ||
+  if ((rc = devbuf_reserve(c.gs_len, sizeof(int64_t) * (size_t)(ne + 2))) ||
       (rc = devbuf_reserve(c.gs_rowptr, sizeof(int64_t) * (size_t)(ne + 2))) ||
-      (rc = devbuf_reserve(c.scan_tmp, scan_tmp_bytes(ne + 2))) ||
-      (want_rows && (rc = devbuf_reserve(c.gs_rows, gs_rows_bytes(ne)))))
+      (rc = devbuf_reserve(c.scan_tmp, scan_tmp_bytes(ne + 2))))
     return rc;
   int64_t* len = dptr<int64_t>(c.gs_len);
   int64_t* rp = dptr<int64_t>(c.gs_rowptr);
   int* err = c.h_pinned + 8;
   err[0] = err[1] = err[2] = 0;
-  if ((rc = gs_slots(ev, ne, nv, cap, dptr<int32_t>(c.gs_cursor), dptr<int32_t>(c.gs_bucket), err,
-                     c.s)) ||
-      (rc = gs_slot_rows(ev, ne, nv, cap, dptr<int32_t>(c.gs_cursor), dptr<int32_t>(c.gs_bucket),
-                         want_rows ? dptr<uint32_t>(c.gs_rows) : nullptr, len, err, c.s)))
-    return rc;
-  RSB_CK(cudaMemsetAsync(len + ne, 0, sizeof(int64_t), c.s));
-  if ((rc = launch_scan_i64(len, rp, ne + 1, c.scan_tmp.p, c.scan_tmp.cap, c.s))) return rc;
-  RSB_CK(cudaMemcpyAsync(total, rp + ne, sizeof(int64_t), cudaMemcpyDeviceToHost, c.s));
-  RSB_CK(cudaStreamSynchronize(c.s));
+  if ((rc = devbuf_reserve(c.gs_cursor, sizeof(int32_t) * (size_t)cap)) ||
+      (rc = devbuf_reserve(c.gs_bucket, gs_slot_bytes(cap))) ||
+      (want_rows && (rc = devbuf_reserve(c.gs_rows, gs_rows_bytes(ne))))) {
+    if (rc != RSB_ENOMEM) return rc;
+    err[1] = 1;  // no room for the table: the buckets take less
+  } else {
+    if ((rc = gs_slots(ev, ne, nv, cap, dptr<int32_t>(c.gs_cursor), dptr<int32_t>(c.gs_bucket),
+                       err, c.s)) ||
+        (rc = gs_slot_rows(ev, ne, nv, cap, dptr<int32_t>(c.gs_cursor), dptr<int32_t>(c.gs_bucket),
+                           want_rows ? dptr<uint32_t>(c.gs_rows) : nullptr, len, err, c.s)))
+      return rc;
+    RSB_CK(cudaMemsetAsync(len + ne, 0, sizeof(int64_t), c.s));
+    if ((rc = launch_scan_i64(len, rp, ne + 1, c.scan_tmp.p, c.scan_tmp.cap, c.s))) return rc;
+    RSB_CK(cudaMemcpyAsync(total, rp + ne, sizeof(int64_t), cudaMemcpyDeviceToHost, c.s));
+    RSB_CK(cudaStreamSynchronize(c.s));
+  }
   if (err[0]) return rsb_set_error(RSB_EINVAL, "vertex ids must lie in [0, 2^31)");
   int flag = err[2] ? 4 : 0;
   *slots = !err[1];
   if (!*slots) {
     int64_t V = 0;
-    if ((rc = gs_setup(c, ne, nv, ev, &V))) return rc;
+    if ((rc = gs_setup_after_slots(c, ne, nv, ev, &V))) return rc;
     int* d_flag = (int*)(dptr<unsigned long long>(c.gs_misc) + 1);
     if ((rc = gs_row_lengths(ne, nv, dptr<int32_t>(c.gs_ev32), dptr<int64_t>(c.gs_bptr),
                              dptr<int32_t>(c.gs_bucket), len, d_flag, c.s)))
@@ -1808,23 +1821,31 @@ extern "C" int rsb_dual_graph(int64_t ne, int nv, const int64_t* ev_in, int64_t*
 }
 
 // One application from the slot table; *fits = 0 when the mesh does not fit it (the
-// general path then answers).  x, y and ev: device pointers.
+// general path then answers).  x, y and ev: device pointers.  y may be x: it is then
+// written only once the table is known to hold the mesh.
 static int gs_lap_slots(Ctx& c, int64_t ne, int nv, const int64_t* ev, const void* x, void* y,
                         int f32, int* fits) {
   const int64_t cap = gs_slot_cap(ne);
   int rc;
+  *fits = 0;
   if ((rc = devbuf_reserve(c.gs_cursor, sizeof(int32_t) * (size_t)cap)) ||
       (rc = devbuf_reserve(c.gs_bucket, gs_slot_bytes(cap))) ||
       (rc = devbuf_reserve(c.gs_w, (f32 ? 8 : 16) * (size_t)cap)))
-    return rc;
+    return rc == RSB_ENOMEM ? RSB_OK : rc;  // (the buckets take less)
   int* err = c.h_pinned + 8;  // words the kernels report into
   err[0] = err[1] = 0;
   if ((rc = gs_slots(ev, ne, nv, cap, dptr<int32_t>(c.gs_cursor), dptr<int32_t>(c.gs_bucket), err,
-                     c.s)) ||
-      (rc = gs_slot_apply(f32, ev, ne, nv, cap, dptr<int32_t>(c.gs_cursor),
-                          dptr<int32_t>(c.gs_bucket), x, c.gs_w.p, y, c.s)))
+                     c.s)))
     return rc;
-  RSB_CK(cudaStreamSynchronize(c.s));
+  const size_t bytes = (f32 ? 4 : 8) * (size_t)ne;
+  const bool overlap = (uintptr_t)x < (uintptr_t)y + bytes && (uintptr_t)y < (uintptr_t)x + bytes;
+  if (overlap) RSB_CK(cudaStreamSynchronize(c.s));
+  if (!overlap || !(err[0] | err[1])) {
+    if ((rc = gs_slot_apply(f32, ev, ne, nv, cap, dptr<int32_t>(c.gs_cursor),
+                            dptr<int32_t>(c.gs_bucket), x, c.gs_w.p, y, c.s)))
+      return rc;
+    RSB_CK(cudaStreamSynchronize(c.s));
+  }
   if (err[0]) return rsb_set_error(RSB_EINVAL, "vertex ids must lie in [0, 2^31)");
   *fits = !err[1];
   return RSB_OK;
@@ -1862,7 +1883,8 @@ static int gs_lap_apply(int64_t ne, int nv, const int64_t* ev_in, const void* x,
   if ((rc = gs_lap_slots(c, ne, nv, ev, xd, yd, f32, &fits))) return done(rc);
   if (!fits) {
     int64_t V = 0;
-    if ((rc = gs_setup(c, ne, nv, ev, &V)) || (rc = devbuf_reserve(c.gs_w, es * (size_t)(V + 1))))
+    if ((rc = gs_setup_after_slots(c, ne, nv, ev, &V)) ||
+        (rc = devbuf_reserve(c.gs_w, es * (size_t)(V + 1))))
       return done(rc);
     if ((rc = gs_apply(f32, ne, nv, V, dptr<int32_t>(c.gs_ev32), dptr<int64_t>(c.gs_bptr),
                        dptr<int32_t>(c.gs_bucket), xd, c.gs_w.p, yd, c.s)))

@@ -4,7 +4,8 @@
 // Input: ne elements, nv global vertex ids each (8 for hexes), ids in
 // [0, V).  Set-up: the elements at every global vertex ("buckets": a
 // counting sort by vertex id, then every bucket sorted by element id, so the
-// result does not depend on the order of the atomics).  Q^T of §5 is then a
+// result does not depend on the order of the atomics; a mesh of at most eight
+// elements a vertex keeps them in fixed slots instead, below).  Q^T of §5 is then a
 // sum over a bucket, Q a read of the vertex's sum.
 //   * dual graph: element e's neighbours are the other elements in the buckets
 //     of its vertices; the weight of neighbour f is how many of e's vertices f

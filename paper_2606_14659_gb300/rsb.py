@@ -364,17 +364,27 @@ def rsb_dual_graph(ev, device: str = "cuda", stream=None):
     rp = torch.empty(ne + 1, dtype=torch.int64, device=dev)
     nnz = C.c_int64(0)
     st = _stream(stream)
-    # one call with room for 26 neighbours an element (the interior of a hex mesh; the
-    # call says when that is too little), a second with the exact room otherwise
-    cap = 26 * ne
-    for _ in range(2):
+
+    def ask(cap):
         col = torch.empty(max(cap, 1), dtype=torch.int32, device=dev)
         w = torch.empty(max(cap, 1), dtype=torch.int32, device=dev)
-        code = lib.rsb_dual_graph(ne, nv, _ptr(evt), _ptr(rp), _ptr(col), _ptr(w), cap,
-                                  C.byref(nnz), st)
-        if code != RSB_EINVAL or nnz.value <= cap:
-            break
+        return lib.rsb_dual_graph(ne, nv, _ptr(evt), _ptr(rp), _ptr(col), _ptr(w), cap,
+                                  C.byref(nnz), st), col, w
+
+    # one call with room for 26 neighbours an element (the interior of a hex mesh; the
+    # call says when that is too little); the exact room when that does not do
+    cap = 26 * ne
+    try:
+        code, col, w = ask(cap)
+    except torch.OutOfMemoryError:
+        code = RSB_ENOMEM
+    if code == RSB_ENOMEM:
+        col = w = None
+        _check(lib.rsb_dual_graph(ne, nv, _ptr(evt), _ptr(rp), None, None, 0, C.byref(nnz), st),
+               "rsb_dual_graph")
+    if code == RSB_ENOMEM or (code == RSB_EINVAL and nnz.value > cap):
         cap = nnz.value
+        code, col, w = ask(cap)
     _check(code, "rsb_dual_graph")
     col, w = col[:nnz.value], w[:nnz.value]
     if nnz.value < cap // 2:  # do not hold on to room that is mostly unused

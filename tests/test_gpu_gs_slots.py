@@ -111,3 +111,47 @@ def test_bad_ids_are_refused_by_both_paths():
             with pytest.raises(R.RSBError) as err:
                 call()
             assert err.value.code == R.rsb.RSB_EINVAL
+
+
+@pytest.mark.parametrize("name", ["hex", "fan9", "many"])  # fits; nine at a vertex; many neighbours
+@pytest.mark.parametrize("shift", [0, 1 << 20])
+def test_laplacian_in_place(name, shift):
+    ev = torch.from_numpy(MESHES[name] + shift).cuda()
+    x = torch.linspace(-1, 1, len(ev), dtype=torch.float64, device="cuda")
+    y = R.rsb.rsb_laplacian_apply_gs(ev, x)
+    z = x.clone()
+    R.rsb.rsb_laplacian_apply_gs(ev, z, z)
+    assert torch.equal(z, y)
+    ev[0, 0] = -1  # refused: the vector stays
+    z = x.clone()
+    with pytest.raises(R.RSBError):
+        R.rsb.rsb_laplacian_apply_gs(ev, z, z)
+    assert torch.equal(z, x)
+
+
+@pytest.mark.parametrize("who", ["torch", "library"])
+def test_dual_graph_without_the_large_room(who, monkeypatch):
+    """Room for 26 neighbours an element refused: the exact room is taken."""
+    ev = MESHES["quads"]
+    want = R.rsb.rsb_dual_graph(ev)
+    if who == "torch":
+        empty = torch.empty
+
+        def small(n, **kw):
+            if n >= 26 * len(ev):
+                raise torch.OutOfMemoryError("no room")
+            return empty(n, **kw)
+
+        monkeypatch.setattr(torch, "empty", small)
+    else:
+        class Lib:
+            calls = 0
+
+            def rsb_dual_graph(self, *a):
+                Lib.calls += 1
+                return R.rsb.RSB_ENOMEM if Lib.calls == 1 else lib.rsb_dual_graph(*a)
+
+        lib = R.rsb.load()
+        monkeypatch.setattr(R.rsb, "load", lambda: Lib())
+    got = R.rsb.rsb_dual_graph(ev)
+    assert got[0] == want[0] and all(torch.equal(a, b) for a, b in zip(got[1:], want[1:]))
