@@ -266,7 +266,6 @@ int rsb_dual_graph(int64_t ne, int nv, const int64_t *ev, int64_t *row_ptr, int3
  * weighted Laplacian of the dual graph above.  ne, nv, ev as in
  * rsb_dual_graph; x, y double[ne] (or float[ne] for the _f32 form), device or
  * host; y may be x.  The elements at every vertex are gathered anew by every call.
- * When ids are refused (RSB_EINVAL), a device y other than x is undefined.
  */
 int rsb_laplacian_apply_gs(int64_t ne, int nv, const int64_t *ev, const double *x, double *y,
                            void *stream);

@@ -285,7 +285,7 @@ struct Ctx {
   DevBuf coords_cat;            // RCB: (x, y, z) per element, caller order, meshes concatenated
   DevBuf perm, iperm, rcb_home;  // RCB reordering: new row -> caller row and back
   // gather-scatter (element -> vertex ids): buckets of elements per vertex
-  DevBuf gs_count, gs_cursor, gs_bptr, gs_bucket, gs_ev32, gs_len, gs_rowptr, gs_w, gs_misc, gs_rows;
+  DevBuf gs_count, gs_cnt, gs_bptr, gs_bucket, gs_ev32, gs_len, gs_rowptr, gs_w, gs_misc, gs_rows;
   DevBuf part_concat;
   int trmax = 0;    // largest tile of the level being solved, rows
   int ntmax = 0;    // most tiles of one of its units
@@ -1648,11 +1648,10 @@ extern "C" void rsb_test_poison_barrier(int on) { g_rsb_poison_barrier = on ? 1 
 // ----------------------------------------------------------------------------
 // element -> vertex ids: the dual graph and the matrix-free Laplacian (§5)
 // ----------------------------------------------------------------------------
-int gs_vertex_count(const int64_t* ev, int64_t cnt, unsigned long long* d_vmax, int* d_flag,
-                    int64_t* V, cudaStream_t s);
-int gs_buckets(const int64_t* ev, int64_t ne, int nv, int64_t V, int64_t* count, int64_t* cursor,
-               int64_t* bptr, int32_t* bucket, int32_t* ev32, void* scan_tmp, size_t scan_bytes,
-               cudaStream_t s);
+int gs_vertex_count(const int64_t* ev, int64_t cnt, unsigned long long* d_max,
+                    unsigned long long* h_max, int64_t* V, cudaStream_t s);
+int gs_buckets(const int64_t* ev, int64_t ne, int nv, int64_t V, int64_t* count, int64_t* bptr,
+               int32_t* bucket, int32_t* ev32, void* scan_tmp, size_t scan_bytes, cudaStream_t s);
 int gs_row_lengths(int64_t ne, int nv, const int32_t* ev32, const int64_t* bptr,
                    const int32_t* bucket, int64_t* len, int* d_flag, cudaStream_t s);
 int gs_fill_dual(int64_t ne, int nv, const int32_t* ev32, const int64_t* bptr,
@@ -1663,14 +1662,14 @@ int gs_apply(int f32, int64_t ne, int nv, int64_t V, const int32_t* ev32, const 
 
 int64_t gs_slot_cap(int64_t ne);
 size_t gs_slot_bytes(int64_t cap);
+size_t gs_cnt_bytes(int64_t cap);
 int gs_slots(const int64_t* ev, int64_t ne, int nv, int64_t cap, int32_t* cnt, int32_t* slot,
-             int* err, cudaStream_t s);
+             cudaStream_t s);
 int gs_slot_apply(int f32, const int64_t* ev, int64_t ne, int nv, int64_t cap, const int32_t* cnt,
-                  const int32_t* slot, const void* x, void* wc, void* y, cudaStream_t s);
-
+                  const int32_t* slot, const void* x, void* wc, void* y, int* err, cudaStream_t s);
 size_t gs_rows_bytes(int64_t ne);
-int gs_slot_rows(const int64_t* ev, int64_t ne, int nv, int64_t cap, const int32_t* cnt,
-                 int32_t* slot, uint32_t* ent, int64_t* len, int* err, cudaStream_t s);
+int gs_slot_rows(const int64_t* ev, int64_t ne, int nv, int64_t cap, int32_t* cnt, int32_t* slot,
+                 uint32_t* ent, int64_t* len, int* err, cudaStream_t s);
 int gs_slot_write(int64_t ne, const uint32_t* ent, const int64_t* row_ptr, int32_t* col,
                   int32_t* wt, cudaStream_t s);
 
@@ -1687,21 +1686,19 @@ static int gs_setup(Ctx& c, int64_t ne, int nv, const int64_t* ev_in, int64_t* V
   const int64_t* ev = nullptr;
   if ((rc = stage_in(c, ev_in, (size_t)(ne * nv), &ev))) return rc;
   if ((rc = devbuf_reserve(c.gs_misc, 256))) return rc;
-  unsigned long long* d_vmax = dptr<unsigned long long>(c.gs_misc);
-  int* d_flag = (int*)(d_vmax + 1);
-  if ((rc = gs_vertex_count(ev, ne * nv, d_vmax, d_flag, V, c.s))) return rc;
+  if ((rc = gs_vertex_count(ev, ne * nv, dptr<unsigned long long>(c.gs_misc),
+                            (unsigned long long*)(c.h_pinned + 12), V, c.s)))
+    return rc;
   const int64_t nV = *V;
   const size_t scan_bytes = scan_tmp_bytes(std::max<int64_t>(nV, ne) + 2);
   if ((rc = devbuf_reserve(c.gs_count, sizeof(int64_t) * (size_t)(nV + 2))) ||
-      (rc = devbuf_reserve(c.gs_cursor, sizeof(int64_t) * (size_t)(nV + 2))) ||
       (rc = devbuf_reserve(c.gs_bptr, sizeof(int64_t) * (size_t)(nV + 2))) ||
       (rc = devbuf_reserve(c.gs_bucket, sizeof(int32_t) * (size_t)(ne * nv))) ||
       (rc = devbuf_reserve(c.gs_ev32, sizeof(int32_t) * (size_t)(ne * nv))) ||
       (rc = devbuf_reserve(c.scan_tmp, scan_bytes)))
     return rc;
-  return gs_buckets(ev, ne, nv, nV, dptr<int64_t>(c.gs_count), dptr<int64_t>(c.gs_cursor),
-                    dptr<int64_t>(c.gs_bptr), dptr<int32_t>(c.gs_bucket),
-                    dptr<int32_t>(c.gs_ev32), c.scan_tmp.p, c.scan_tmp.cap, c.s);
+  return gs_buckets(ev, ne, nv, nV, dptr<int64_t>(c.gs_count), dptr<int64_t>(c.gs_bptr),
+                    dptr<int32_t>(c.gs_bucket), dptr<int32_t>(c.gs_ev32), c.scan_tmp.p, c.scan_tmp.cap, c.s);
 }
 
 // gs_setup after the slot table was tried: its room is larger than the buckets', so it
@@ -1709,7 +1706,7 @@ static int gs_setup(Ctx& c, int64_t ne, int nv, const int64_t* ev_in, int64_t* V
 static int gs_setup_after_slots(Ctx& c, int64_t ne, int nv, const int64_t* ev, int64_t* V) {
   int rc = gs_setup(c, ne, nv, ev, V);
   if (rc != RSB_ENOMEM) return rc;
-  for (DevBuf* b : {&c.gs_cursor, &c.gs_bucket, &c.gs_w, &c.gs_rows}) free_buf(*b);
+  for (DevBuf* b : {&c.gs_cnt, &c.gs_bucket, &c.gs_w, &c.gs_rows}) free_buf(*b);
   return gs_setup(c, ne, nv, ev, V);
 }
 
@@ -1728,15 +1725,15 @@ static int dual_rows(Ctx& c, int64_t ne, int nv, const int64_t* ev, bool want_ro
   int64_t* rp = dptr<int64_t>(c.gs_rowptr);
   int* err = c.h_pinned + 8;
   err[0] = err[1] = err[2] = 0;
-  if ((rc = devbuf_reserve(c.gs_cursor, sizeof(int32_t) * (size_t)cap)) ||
+  if ((rc = devbuf_reserve(c.gs_cnt, gs_cnt_bytes(cap))) ||
       (rc = devbuf_reserve(c.gs_bucket, gs_slot_bytes(cap))) ||
       (want_rows && (rc = devbuf_reserve(c.gs_rows, gs_rows_bytes(ne))))) {
     if (rc != RSB_ENOMEM) return rc;
     err[1] = 1;  // no room for the table: the buckets take less
   } else {
-    if ((rc = gs_slots(ev, ne, nv, cap, dptr<int32_t>(c.gs_cursor), dptr<int32_t>(c.gs_bucket),
-                       err, c.s)) ||
-        (rc = gs_slot_rows(ev, ne, nv, cap, dptr<int32_t>(c.gs_cursor), dptr<int32_t>(c.gs_bucket),
+    if ((rc = gs_slots(ev, ne, nv, cap, dptr<int32_t>(c.gs_cnt), dptr<int32_t>(c.gs_bucket),
+                       c.s)) ||
+        (rc = gs_slot_rows(ev, ne, nv, cap, dptr<int32_t>(c.gs_cnt), dptr<int32_t>(c.gs_bucket),
                            want_rows ? dptr<uint32_t>(c.gs_rows) : nullptr, len, err, c.s)))
       return rc;
     RSB_CK(cudaMemsetAsync(len + ne, 0, sizeof(int64_t), c.s));
@@ -1821,31 +1818,24 @@ extern "C" int rsb_dual_graph(int64_t ne, int nv, const int64_t* ev_in, int64_t*
 }
 
 // One application from the slot table; *fits = 0 when the mesh does not fit it (the
-// general path then answers).  x, y and ev: device pointers.  y may be x: it is then
-// written only once the table is known to hold the mesh.
+// general path then answers) and y is as it was.  x, y and ev: device pointers.
 static int gs_lap_slots(Ctx& c, int64_t ne, int nv, const int64_t* ev, const void* x, void* y,
                         int f32, int* fits) {
   const int64_t cap = gs_slot_cap(ne);
   int rc;
   *fits = 0;
-  if ((rc = devbuf_reserve(c.gs_cursor, sizeof(int32_t) * (size_t)cap)) ||
+  if ((rc = devbuf_reserve(c.gs_cnt, gs_cnt_bytes(cap))) ||
       (rc = devbuf_reserve(c.gs_bucket, gs_slot_bytes(cap))) ||
       (rc = devbuf_reserve(c.gs_w, (f32 ? 8 : 16) * (size_t)cap)))
     return rc == RSB_ENOMEM ? RSB_OK : rc;  // (the buckets take less)
   int* err = c.h_pinned + 8;  // words the kernels report into
   err[0] = err[1] = 0;
-  if ((rc = gs_slots(ev, ne, nv, cap, dptr<int32_t>(c.gs_cursor), dptr<int32_t>(c.gs_bucket), err,
-                     c.s)))
+  if ((rc = gs_slots(ev, ne, nv, cap, dptr<int32_t>(c.gs_cnt), dptr<int32_t>(c.gs_bucket),
+                     c.s)) ||
+      (rc = gs_slot_apply(f32, ev, ne, nv, cap, dptr<int32_t>(c.gs_cnt),
+                          dptr<int32_t>(c.gs_bucket), x, c.gs_w.p, y, err, c.s)))
     return rc;
-  const size_t bytes = (f32 ? 4 : 8) * (size_t)ne;
-  const bool overlap = (uintptr_t)x < (uintptr_t)y + bytes && (uintptr_t)y < (uintptr_t)x + bytes;
-  if (overlap) RSB_CK(cudaStreamSynchronize(c.s));
-  if (!overlap || !(err[0] | err[1])) {
-    if ((rc = gs_slot_apply(f32, ev, ne, nv, cap, dptr<int32_t>(c.gs_cursor),
-                            dptr<int32_t>(c.gs_bucket), x, c.gs_w.p, y, c.s)))
-      return rc;
-    RSB_CK(cudaStreamSynchronize(c.s));
-  }
+  RSB_CK(cudaStreamSynchronize(c.s));
   if (err[0]) return rsb_set_error(RSB_EINVAL, "vertex ids must lie in [0, 2^31)");
   *fits = !err[1];
   return RSB_OK;
@@ -1986,7 +1976,7 @@ extern "C" void rsb_release(void) {
                      &c->cand[0], &c->cand[1], &c->cand[2], &c->seg_row0, &c->seg_nleft,
                      &c->seg_child0, &c->seg_p0, &c->seg_split, &c->seg_keystar, &c->seg_unit,
                      &c->seg_ncomp, &c->counters, &c->part_concat, &c->blk, &c->split, &c->coords_cat,
-                     &c->perm, &c->iperm, &c->rcb_home, &c->gs_count, &c->gs_cursor,
+                     &c->perm, &c->iperm, &c->rcb_home, &c->gs_count, &c->gs_cnt,
                      &c->gs_bptr, &c->gs_bucket, &c->gs_ev32, &c->gs_len, &c->gs_rowptr,
                      &c->gs_w, &c->gs_misc, &c->gs_rows};
     for (DevBuf* b : all) free_buf(*b);

@@ -17,26 +17,35 @@
 //     y_e = sum over e's vertices v of (c_v x_e - w_v), c_v the bucket size,
 //     which is sum_v sum_{f at v} (x_e - x_f): the diagonal term of A_w and
 //     D_w cancel inside every vertex term.
+#include <algorithm>
 #include <climits>
 
 #include "rsb_internal.cuh"
 
 #define GS_MAXCAND 256  // neighbour candidates of one element (with repeats)
 
-__global__ void k_gs_maxid(const int64_t* __restrict__ ev, int64_t cnt, unsigned long long* vmax,
-                           int* flag) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+// Bound: the read of the ids; one atomic a CTA (an atomic a warp on the one address took
+// longer than the read).
+__global__ void __launch_bounds__(RSB_BLOCK) k_gs_maxid(const int64_t* __restrict__ ev, int64_t cnt,
+                                                      unsigned long long* vmax, int* flag) {
+  __shared__ long long wm[RSB_WARPS];
   long long m = -1;
-  if (i < cnt) {
-    m = ev[i];
-    if (m < 0 || m >= (1ll << 31)) {
-      atomicOr(flag, 1);
-      m = -1;
-    }
+  bool bad = false;
+  for (int64_t i = (int64_t)blockIdx.x * RSB_BLOCK + threadIdx.x; i < cnt;
+       i += (int64_t)gridDim.x * RSB_BLOCK) {
+    const long long v = ev[i];
+    if (v < 0 || v >= (1ll << 31)) bad = true;
+    else m = max(m, v);
   }
+  if (bad) atomicOr(flag, 1);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
-  if ((threadIdx.x & 31) == 0 && m >= 0) atomicMax(vmax, (unsigned long long)m);
+  if ((threadIdx.x & 31) == 0) wm[threadIdx.x >> 5] = m;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < RSB_WARPS; ++w) m = max(m, wm[w]);
+    if (m >= 0) atomicMax(vmax, (unsigned long long)m);
+  }
 }
 
 __global__ void k_gs_count(const int64_t* __restrict__ ev, int64_t cnt, int64_t* count) {
@@ -45,15 +54,15 @@ __global__ void k_gs_count(const int64_t* __restrict__ ev, int64_t cnt, int64_t*
 }
 
 // bucket fill (element ids; within a bucket in arrival order) and the slot
-// table ev32 (vertex ids as int32)
+// table ev32 (vertex ids as int32); the counts run down to zero
 __global__ void k_gs_fill(const int64_t* __restrict__ ev, int64_t cnt, int nv,
-                          const int64_t* __restrict__ bptr, int64_t* cursor, int32_t* bucket,
+                          const int64_t* __restrict__ bptr, int64_t* count, int32_t* bucket,
                           int32_t* ev32) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= cnt) return;
   const int64_t v = ev[i];
-  const unsigned long long pos = atomicAdd((unsigned long long*)(cursor + v), 1ull);
-  bucket[bptr[v] + (int64_t)pos] = (int32_t)(i / nv);
+  const int64_t left = (int64_t)atomicAdd((unsigned long long*)(count + v), ~0ull);
+  bucket[bptr[v + 1] - left] = (int32_t)(i / nv);  // in arrival order, nearly sorted
   ev32[i] = (int32_t)v;
 }
 
@@ -181,13 +190,16 @@ __global__ void __launch_bounds__(RSB_BLOCK) k_gs_apply(int64_t ne, int nv,
 // vertices have at most that many (hexes: eight in the interior) and whose ids lie
 // below a bound known beforehand.  One pass over the ids takes the place of the pass
 // for the largest id (and the host's wait for it), the count, the scan and the fill of
-// the buckets above; a mesh that does not fit sets a host-visible word, and the caller
-// takes the general path.  A vertex's slots hold its elements in arrival order; their
+// the buckets above; a mesh that does not fit sets a word, the kernels that follow return
+// at once, and the caller takes the general path.  A vertex's slots hold its elements in
+// arrival order; their
 // readers sort the at most eight of them in registers, so results do not depend on it.
 // One Laplacian application at 1.9M hexes 168 us, 717 from the buckets.
-// err: [0] an id outside [0, 2^31), [1] the table does not hold the mesh.
+// Words behind the counts, cleared with them: [0] an id outside [0, 2^31), [1] the table
+// does not hold the mesh, [2] two elements share more than 7 vertices.
 // ----------------------------------------------------------------------------
 #define GS_SLOTS 8
+#define GS_WORDS 4
 
 // The ids of element e (unused places: -1).
 template <bool HEX>
@@ -211,34 +223,45 @@ __device__ __forceinline__ void gs_ids(const int64_t* __restrict__ ev, int64_t e
 template <bool HEX>
 __global__ void __launch_bounds__(RSB_BLOCK) k_gs_slots(const int64_t* __restrict__ ev, int64_t ne,
                                                       int nv, int64_t cap, int32_t* cnt,
-                                                      int32_t* __restrict__ slot,
-                                                      volatile int* err) {
+                                                      int32_t* __restrict__ slot) {
   const int64_t e = (int64_t)blockIdx.x * RSB_BLOCK + threadIdx.x;
   if (e >= ne) return;
+  volatile int32_t* err = cnt + cap;
   int64_t id[8];
   gs_ids<HEX>(ev, e, nv, id);
+  bool out = false, full = false;
   int pos[8];
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
     pos[i] = GS_SLOTS;
     if (HEX || i < nv) {
-      if (id[i] < 0 || id[i] >= (1ll << 31)) err[0] = 1;
-      else if (id[i] >= cap) err[1] = 1;
+      if (id[i] < 0 || id[i] >= (1ll << 31)) out = true;
+      else if (id[i] >= cap) full = true;
       else pos[i] = atomicAdd(cnt + id[i], 1);
     }
   }
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
     if (pos[i] < GS_SLOTS) slot[id[i] * GS_SLOTS + pos[i]] = (int32_t)e;
-    else if ((HEX || i < nv) && id[i] >= 0 && id[i] < cap) err[1] = 1;
+    else if ((HEX || i < nv) && id[i] >= 0 && id[i] < cap) full = true;
   }
+  if (out && !err[0]) err[0] = 1;
+  if (full && !err[1]) err[1] = 1;
+}
+
+// Not zero: the table does not hold the mesh.  (Its readers load it beside their first
+// operands: as a load and a branch of its own it costs them 2 %.)
+__device__ __forceinline__ int gs_unfit(const int32_t* cnt, int64_t cap) {
+  return cnt[cap] | cnt[cap + 1];
 }
 
 // The elements at vertex v in ascending order, INT_MAX in the places left (a sorting
-// network of 19 exchanges); returns their number.
-__device__ __forceinline__ int gs_sorted_slots(const int32_t* cnt, const int32_t* slot, int64_t v,
-                                               int32_t (&f)[GS_SLOTS]) {
-  const int n = min(cnt[v], GS_SLOTS);
+// network of 19 exchanges); returns their number (0 when the mesh does
+// not fit).
+__device__ __forceinline__ int gs_sorted_slots(const int32_t* cnt, int64_t cap, const int32_t* slot,
+                                               int64_t v, int32_t (&f)[GS_SLOTS]) {
+  const int here = cnt[v], unfit = gs_unfit(cnt, cap);
+  const int n = unfit ? 0 : min(here, GS_SLOTS);
   const int4* p = reinterpret_cast<const int4*>(slot + v * GS_SLOTS);
   int4 lo = make_int4(0, 0, 0, 0), hi = lo;
   if (n > 0) lo = p[0];
@@ -276,7 +299,7 @@ __global__ void __launch_bounds__(RSB_BLOCK) k_gs_vsum8(int64_t nvert, const int
   const int64_t v = (int64_t)blockIdx.x * RSB_BLOCK + threadIdx.x;
   if (v >= nvert) return;
   int32_t f[GS_SLOTS];
-  const int n = gs_sorted_slots(cnt, slot, v, f);
+  const int n = gs_sorted_slots(cnt, nvert, slot, v, f);
   V xv[GS_SLOTS];
 #pragma unroll
   for (int i = 0; i < GS_SLOTS; ++i) xv[i] = i < n ? __ldg(x + f[i]) : V(0);
@@ -291,11 +314,18 @@ template <typename V, bool HEX>
 __global__ void __launch_bounds__(RSB_BLOCK) k_gs_apply8(int64_t ne, int nv,
                                                        const int64_t* __restrict__ ev, int64_t cap,
                                                        const GsPair<V>* __restrict__ wc,
-                                                       const V* __restrict__ x, V* __restrict__ y) {
+                                                       const int32_t* __restrict__ cnt,
+                                                       const V* __restrict__ x, V* __restrict__ y,
+                                                       volatile int* err) {
   const int64_t e = (int64_t)blockIdx.x * RSB_BLOCK + threadIdx.x;
   if (e >= ne) return;
+  const int unfit = gs_unfit(cnt, cap);
   int64_t id[8];
   gs_ids<HEX>(ev, e, nv, id);
+  if (unfit) {  // told to the host, which then takes the buckets
+    if (e == 0) err[0] = cnt[cap], err[1] = cnt[cap + 1];
+    return;
+  }
   GsPair<V> p[8];
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
@@ -316,7 +346,7 @@ __global__ void __launch_bounds__(RSB_BLOCK) k_gs_sort8(int64_t nvert, const int
   const int64_t v = (int64_t)blockIdx.x * RSB_BLOCK + threadIdx.x;
   if (v >= nvert) return;
   int32_t f[GS_SLOTS];
-  if (gs_sorted_slots(cnt, slot, v, f) == 0) return;
+  if (gs_sorted_slots(cnt, nvert, slot, v, f) == 0) return;
   int4* p = reinterpret_cast<int4*>(slot + v * GS_SLOTS);
   p[0] = make_int4(f[0], f[1], f[2], f[3]);
   p[1] = make_int4(f[4], f[5], f[6], f[7]);
@@ -325,8 +355,8 @@ __global__ void __launch_bounds__(RSB_BLOCK) k_gs_sort8(int64_t nvert, const int
 // Distinct neighbours of element e with their shared-vertex counts, ascending: a merge
 // of the sorted slots of its vertices, the heads in registers.  A neighbour's entry
 // (packed as in the sliced form) goes to ent[(32-row group * GS_ROW + k) * 32 + lane],
-// their number to len[e]; err[1]: more than GS_ROW neighbours, err[2]: more than 7
-// shared vertices.
+// their number to len[e].  More than GS_ROW neighbours set word 1, which stops the CTAs
+// that start later.
 // Bound: the loads of the heads (each slot of the element's vertices once, from L1 and
 // L2).  Collecting the candidates in a local-memory array of 256 and insertion-sorting
 // it, once to count and once to write, made the dual graph of 2.4M hexes take 4330 us
@@ -337,12 +367,16 @@ __global__ void __launch_bounds__(RSB_BLOCK) k_gs_merge(int64_t ne, int nv,
                                                       const int64_t* __restrict__ ev, int64_t cap,
                                                       const int32_t* __restrict__ slot,
                                                       uint32_t* __restrict__ ent,
-                                                      int64_t* __restrict__ len,
-                                                      volatile int* err) {
+                                                      int64_t* __restrict__ len, int32_t* cnt) {
   const int64_t e = (int64_t)blockIdx.x * RSB_BLOCK + threadIdx.x;
   if (e >= ne) return;
+  const int unfit = gs_unfit(cnt, cap);
   int64_t id[8];
   gs_ids<HEX>(ev, e, nv, id);
+  if (unfit) {
+    len[e] = 0;
+    return;
+  }
   const int32_t* p[8];
   int32_t h[8];
 #pragma unroll
@@ -377,8 +411,9 @@ __global__ void __launch_bounds__(RSB_BLOCK) k_gs_merge(int64_t ne, int nv,
       }
   }
   len[e] = d;
-  if (d > GS_ROW) err[1] = 1;
-  if (most > 7) err[2] = 1;
+  volatile int32_t* err = cnt + cap;
+  if (d > GS_ROW && !err[1]) err[1] = 1;
+  if (most > 7 && !err[2]) err[2] = 1;
 }
 
 // The merged rows into CSR: a warp's 32 rows are contiguous there, so they pass through
@@ -424,32 +459,29 @@ static unsigned grid_of(int64_t n, int block = RSB_BLOCK) {
 }
 
 // Largest vertex id + 1 (V) of the table, or an error for ids outside [0, 2^31).
-int gs_vertex_count(const int64_t* ev, int64_t cnt, unsigned long long* d_vmax, int* d_flag,
-                    int64_t* V, cudaStream_t s) {
-  RSB_CK(cudaMemsetAsync(d_vmax, 0, sizeof(unsigned long long), s));
-  RSB_CK(cudaMemsetAsync(d_flag, 0, sizeof(int), s));
+// d_max: two device words (the largest id, a flag), h_max: two pinned host words.
+int gs_vertex_count(const int64_t* ev, int64_t cnt, unsigned long long* d_max,
+                    unsigned long long* h_max, int64_t* V, cudaStream_t s) {
+  RSB_CK(cudaMemsetAsync(d_max, 0, 2 * sizeof(unsigned long long), s));
   if (cnt > 0) {
-    k_gs_maxid<<<grid_of(cnt), RSB_BLOCK, 0, s>>>(ev, cnt, d_vmax, d_flag);
+    k_gs_maxid<<<std::min(grid_of(cnt), 8u * 152u), RSB_BLOCK, 0, s>>>(ev, cnt, d_max,
+                                                                      (int*)(d_max + 1));
     RSB_CKL("k_gs_maxid");
   }
-  unsigned long long vm = 0;
-  int fl = 0;
-  RSB_CK(cudaMemcpyAsync(&vm, d_vmax, sizeof(vm), cudaMemcpyDeviceToHost, s));
-  RSB_CK(cudaMemcpyAsync(&fl, d_flag, sizeof(int), cudaMemcpyDeviceToHost, s));
+  RSB_CK(cudaMemcpyAsync(h_max, d_max, 2 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, s));
   RSB_CK(cudaStreamSynchronize(s));
-  if (fl) return rsb_set_error(RSB_EINVAL, "vertex ids must lie in [0, 2^31)");
-  *V = cnt > 0 ? (int64_t)vm + 1 : 0;
+  if (h_max[1]) return rsb_set_error(RSB_EINVAL, "vertex ids must lie in [0, 2^31)");
+  *V = cnt > 0 ? (int64_t)h_max[0] + 1 : 0;
   return RSB_OK;
 }
 
-// Buckets: bptr[V + 1], bucket[ne * nv], ev32[ne * nv]; count and cursor are
-// int64[V + 1] scratch.
-int gs_buckets(const int64_t* ev, int64_t ne, int nv, int64_t V, int64_t* count, int64_t* cursor,
-               int64_t* bptr, int32_t* bucket, int32_t* ev32, void* scan_tmp, size_t scan_bytes,
+// Buckets: bptr[V + 1], bucket[ne * nv], ev32[ne * nv]; count is int64[V + 1]
+// scratch.
+int gs_buckets(const int64_t* ev, int64_t ne, int nv, int64_t V, int64_t* count, int64_t* bptr,
+               int32_t* bucket, int32_t* ev32, void* scan_tmp, size_t scan_bytes,
                cudaStream_t s) {
   const int64_t cnt = ne * nv;
   RSB_CK(cudaMemsetAsync(count, 0, sizeof(int64_t) * (size_t)(V + 1), s));
-  RSB_CK(cudaMemsetAsync(cursor, 0, sizeof(int64_t) * (size_t)(V + 1), s));
   if (cnt > 0) {
     k_gs_count<<<grid_of(cnt), RSB_BLOCK, 0, s>>>(ev, cnt, count);
     RSB_CKL("k_gs_count");
@@ -457,7 +489,7 @@ int gs_buckets(const int64_t* ev, int64_t ne, int nv, int64_t V, int64_t* count,
   int rc = launch_scan_i64(count, bptr, V + 1, scan_tmp, scan_bytes, s);
   if (rc) return rc;
   if (cnt > 0) {
-    k_gs_fill<<<grid_of(cnt), RSB_BLOCK, 0, s>>>(ev, cnt, nv, bptr, cursor, bucket, ev32);
+    k_gs_fill<<<grid_of(cnt), RSB_BLOCK, 0, s>>>(ev, cnt, nv, bptr, count, bucket, ev32);
     RSB_CKL("k_gs_fill");
     k_gs_sort<<<grid_of(V), RSB_BLOCK, 0, s>>>(bptr, V, bucket);
     RSB_CKL("k_gs_sort");
@@ -513,56 +545,63 @@ size_t gs_slot_bytes(int64_t cap) { return sizeof(int32_t) * GS_SLOTS * (size_t)
 
 static bool hex_aligned(const int64_t* ev, int nv) { return nv == 8 && ((uintptr_t)ev & 15) == 0; }
 
+size_t gs_cnt_bytes(int64_t cap) { return sizeof(int32_t) * (size_t)(cap + GS_WORDS); }
+
 int gs_slots(const int64_t* ev, int64_t ne, int nv, int64_t cap, int32_t* cnt, int32_t* slot,
-             int* err, cudaStream_t s) {
-  RSB_CK(cudaMemsetAsync(cnt, 0, sizeof(int32_t) * (size_t)cap, s));
+             cudaStream_t s) {
+  RSB_CK(cudaMemsetAsync(cnt, 0, gs_cnt_bytes(cap), s));
   if (hex_aligned(ev, nv))
-    k_gs_slots<true><<<grid_of(ne), RSB_BLOCK, 0, s>>>(ev, ne, nv, cap, cnt, slot, err);
+    k_gs_slots<true><<<grid_of(ne), RSB_BLOCK, 0, s>>>(ev, ne, nv, cap, cnt, slot);
   else
-    k_gs_slots<false><<<grid_of(ne), RSB_BLOCK, 0, s>>>(ev, ne, nv, cap, cnt, slot, err);
+    k_gs_slots<false><<<grid_of(ne), RSB_BLOCK, 0, s>>>(ev, ne, nv, cap, cnt, slot);
   RSB_CKL("k_gs_slots");
   return RSB_OK;
 }
 
 template <typename V>
 static int gs_slot_apply_t(const int64_t* ev, int64_t ne, int nv, int64_t cap, const int32_t* cnt,
-                           const int32_t* slot, const V* x, void* wc, V* y, cudaStream_t s) {
+                           const int32_t* slot, const V* x, void* wc, V* y, int* err,
+                           cudaStream_t s) {
   GsPair<V>* p = (GsPair<V>*)wc;
   k_gs_vsum8<V><<<grid_of(cap), RSB_BLOCK, 0, s>>>(cap, cnt, slot, x, p);
   RSB_CKL("k_gs_vsum8");
   if (hex_aligned(ev, nv))
-    k_gs_apply8<V, true><<<grid_of(ne), RSB_BLOCK, 0, s>>>(ne, nv, ev, cap, p, x, y);
+    k_gs_apply8<V, true><<<grid_of(ne), RSB_BLOCK, 0, s>>>(ne, nv, ev, cap, p, cnt, x, y, err);
   else
-    k_gs_apply8<V, false><<<grid_of(ne), RSB_BLOCK, 0, s>>>(ne, nv, ev, cap, p, x, y);
+    k_gs_apply8<V, false><<<grid_of(ne), RSB_BLOCK, 0, s>>>(ne, nv, ev, cap, p, cnt, x, y, err);
   RSB_CKL("k_gs_apply8");
   return RSB_OK;
 }
 
-// y = L x from the slot table (wc: 2 * cap values of the vector type).
+// y = L x from the slot table (wc: 2 * cap values of the vector type); a mesh that does
+// not fit leaves y as it is and sets err[0] or err[1] (pinned host words).
 int gs_slot_apply(int f32, const int64_t* ev, int64_t ne, int nv, int64_t cap, const int32_t* cnt,
-                  const int32_t* slot, const void* x, void* wc, void* y, cudaStream_t s) {
-  return f32 ? gs_slot_apply_t<float>(ev, ne, nv, cap, cnt, slot, (const float*)x, wc, (float*)y, s)
+                  const int32_t* slot, const void* x, void* wc, void* y, int* err, cudaStream_t s) {
+  return f32 ? gs_slot_apply_t<float>(ev, ne, nv, cap, cnt, slot, (const float*)x, wc, (float*)y,
+                                      err, s)
              : gs_slot_apply_t<double>(ev, ne, nv, cap, cnt, slot, (const double*)x, wc, (double*)y,
-                                       s);
+                                       err, s);
 }
 
 // Row lengths of the dual graph from the slot table and, with ent, the rows
 // themselves for gs_slot_write (ent: gs_rows_bytes).
 size_t gs_rows_bytes(int64_t ne) { return sizeof(uint32_t) * GS_ROW * 32 * (size_t)((ne + 31) / 32); }
 
-int gs_slot_rows(const int64_t* ev, int64_t ne, int nv, int64_t cap, const int32_t* cnt,
-                 int32_t* slot, uint32_t* ent, int64_t* len, int* err, cudaStream_t s) {
+// err: pinned host words 0 to 2, valid once the stream is done.
+int gs_slot_rows(const int64_t* ev, int64_t ne, int nv, int64_t cap, int32_t* cnt, int32_t* slot,
+                 uint32_t* ent, int64_t* len, int* err, cudaStream_t s) {
   k_gs_sort8<<<grid_of(cap), RSB_BLOCK, 0, s>>>(cap, cnt, slot);
   RSB_CKL("k_gs_sort8");
   const unsigned nb = grid_of(ne);
   if (hex_aligned(ev, nv)) {
-    if (ent) k_gs_merge<true, true><<<nb, RSB_BLOCK, 0, s>>>(ne, nv, ev, cap, slot, ent, len, err);
-    else k_gs_merge<true, false><<<nb, RSB_BLOCK, 0, s>>>(ne, nv, ev, cap, slot, ent, len, err);
+    if (ent) k_gs_merge<true, true><<<nb, RSB_BLOCK, 0, s>>>(ne, nv, ev, cap, slot, ent, len, cnt);
+    else k_gs_merge<true, false><<<nb, RSB_BLOCK, 0, s>>>(ne, nv, ev, cap, slot, ent, len, cnt);
   } else {
-    if (ent) k_gs_merge<false, true><<<nb, RSB_BLOCK, 0, s>>>(ne, nv, ev, cap, slot, ent, len, err);
-    else k_gs_merge<false, false><<<nb, RSB_BLOCK, 0, s>>>(ne, nv, ev, cap, slot, ent, len, err);
+    if (ent) k_gs_merge<false, true><<<nb, RSB_BLOCK, 0, s>>>(ne, nv, ev, cap, slot, ent, len, cnt);
+    else k_gs_merge<false, false><<<nb, RSB_BLOCK, 0, s>>>(ne, nv, ev, cap, slot, ent, len, cnt);
   }
   RSB_CKL("k_gs_merge");
+  RSB_CK(cudaMemcpyAsync(err, cnt + cap, 3 * sizeof(int), cudaMemcpyDeviceToHost, s));
   return RSB_OK;
 }
 
