@@ -287,6 +287,7 @@ struct Ctx {
   // gather-scatter (element -> vertex ids): buckets of elements per vertex
   DevBuf gs_count, gs_cnt, gs_bptr, gs_bucket, gs_ev32, gs_len, gs_rowptr, gs_w, gs_misc, gs_rows;
   DevBuf part_concat;
+  DevBuf lap_x, lap_y;  // device copies of a Laplacian action's host vectors
   int trmax = 0;    // largest tile of the level being solved, rows
   int ntmax = 0;    // most tiles of one of its units
   std::vector<DevBuf> stage;  // staged host inputs
@@ -1549,20 +1550,15 @@ static int lap_apply(const rsb_csr* g, const void* x, void* y, int f32, void* st
   const size_t es = f32 ? 4 : 8;
   const void* xd = x;
   void* yd = y;
-  DevBuf tx, ty;
   if (!is_device_ptr(x)) {
-    if ((rc = devbuf_reserve(tx, es * N))) return end_call(c, stream, rc);
-    RSB_CK(cudaMemcpyAsync(tx.p, x, es * N, cudaMemcpyHostToDevice, c.s));
-    xd = tx.p;
+    if ((rc = devbuf_reserve(c.lap_x, es * N))) return end_call(c, stream, rc);
+    RSB_CK(cudaMemcpyAsync(c.lap_x.p, x, es * N, cudaMemcpyHostToDevice, c.s));
+    xd = c.lap_x.p;
   }
   const bool yh = !is_device_ptr(y);
   if (yh) {
-    if ((rc = devbuf_reserve(ty, es * N))) {
-      rc = end_call(c, stream, rc);
-      free_buf(tx);
-      return rc;
-    }
-    yd = ty.p;
+    if ((rc = devbuf_reserve(c.lap_y, es * N))) return end_call(c, stream, rc);
+    yd = c.lap_y.p;
   }
   // faults are reported into pinned host words that the call reads once the kernel is
   // done; a host y is left alone then
@@ -1581,8 +1577,6 @@ static int lap_apply(const rsb_csr* g, const void* x, void* y, int f32, void* st
     if (e != cudaSuccess) rc = rsb_set_cuda_error(e, "copy y");
   }
   rc = end_call(c, stream, rc);
-  free_buf(tx);
-  free_buf(ty);
   const int f = faults();
   return !rc && f ? invalid_graph(f) : rc;
 }
@@ -1978,7 +1972,7 @@ extern "C" void rsb_release(void) {
                      &c->seg_ncomp, &c->counters, &c->part_concat, &c->blk, &c->split, &c->coords_cat,
                      &c->perm, &c->iperm, &c->rcb_home, &c->gs_count, &c->gs_cnt,
                      &c->gs_bptr, &c->gs_bucket, &c->gs_ev32, &c->gs_len, &c->gs_rowptr,
-                     &c->gs_w, &c->gs_misc, &c->gs_rows};
+                     &c->gs_w, &c->gs_misc, &c->gs_rows, &c->lap_x, &c->lap_y};
     for (DevBuf* b : all) free_buf(*b);
     for (int k = 0; k < 2; ++k) {
       PrecBufs& p = c->pb[k];
