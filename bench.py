@@ -287,8 +287,8 @@ def aggregate(total_ms: float, units: float, dist=None, device=None):
 LAUNCH_NAMES = ["kernels", "cuda_graph", "persistent_cycle", "persistent_resident"]
 FAMILIES = {
     "lz_a": "k_lz_a1 (FP32 Lanczos step D1: SpMV z = L v_j of the sliced-ELL graph, v_j = w_j / nu_j)",
-    "lz_a2": ("k_lz_d2 (FP32 Lanczos step D2: dots of v_j and z with the basis in one pass, the "
-              "basis, v_j and z staged in shared memory by bulk copies)"),
+    "lz_a2": ("k_lz_d2 (FP32 Lanczos step D2: dots of v_j and z with the basis in one pass, two "
+              "coefficients a warp, the basis streamed through registers)"),
     "lz_b": ("k_lz_d3 (FP32 Lanczos step D3: q_j = (v_j - B a) / rho and w_{j+1} = (z - B g - "
              "(q_j.z) q_j) / rho in one pass over the basis, ||w_{j+1}||)"),
     "lz_c": "k_lz_c (FP64 Lanczos step C: w -= Q c2 and ||w||)",

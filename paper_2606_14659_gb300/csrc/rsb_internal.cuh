@@ -41,8 +41,8 @@
 #define RSB_MAXTILES_PER_UNIT 1024
 #define RSB_MINR 2    // minimum rows per thread of a tile
 // Tiles of a large level: rows per thread grow until the level has about this
-// many tiles (eight waves of two CTAs on each of 152 SMs), so that a streaming
-// kernel's tile spans many bulk-copy chunks and its pipeline fills
+// many tiles (eight waves of two CTAs on each of 152 SMs), so that a tile's
+// reductions are few beside its rows
 #define RSB_TARGET_TILES 2432
 #define RSB_SUBR 4    // rows per thread handled between two CTA barriers
 #define RSB_COLBITS 29
@@ -144,12 +144,6 @@ __device__ __forceinline__ double warp_max(double v) {
   for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
   return v;
 }
-__device__ __forceinline__ long long warp_sum_ll(long long v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-
 // Block sum of one double per thread, deterministic; result valid in thread 0.
 __device__ __forceinline__ double block_sum(double v, double* sm) {
   v = warp_sum(v);

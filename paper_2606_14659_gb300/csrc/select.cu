@@ -9,7 +9,8 @@
 //     value are ties and go left in ascending gid),
 //   * the gid rule comparing two candidate splits of a repeated eigenvalue
 //     (reading R5), and the final side of every row including whole
-//     components placed by reading R8.
+//     components placed by reading R8;
+// in one cooperative launch per candidate where a level allows it.
 #include <algorithm>
 
 #include "rsb_internal.cuh"

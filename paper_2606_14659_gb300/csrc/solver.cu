@@ -2427,10 +2427,6 @@ static int read_active(SolveBufs& B, cudaStream_t s, int* out) {
   RSB_CK(cudaStreamSynchronize(s));
   prof_collect();
   *out = *B.h_active;
-  if (B.gb && B.h_active[1] == 2)
-    return rsb_set_error(RSB_ETIMEOUT,
-                         "a bounded device wait gave up and a CTA's bulk copies in flight did "
-                         "not drain before it exited");
   if (B.gb && B.h_active[1]) return rsb_set_error(RSB_ETIMEOUT, "a bounded device wait gave up");
   return RSB_OK;
 }
