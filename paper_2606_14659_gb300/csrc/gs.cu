@@ -250,7 +250,7 @@ __global__ void __launch_bounds__(RSB_BLOCK) k_gs_slots(const int64_t* __restric
 }
 
 // Not zero: the table does not hold the mesh.  (Its readers load it beside their first
-// operands: as a load and a branch of its own it costs them 2 %.)
+// operands: as a load and a branch of its own it costs them 1 %.)
 __device__ __forceinline__ int gs_unfit(const int32_t* cnt, int64_t cap) {
   return cnt[cap] | cnt[cap + 1];
 }
@@ -360,7 +360,7 @@ __global__ void __launch_bounds__(RSB_BLOCK) k_gs_sort8(int64_t nvert, const int
 // Bound: the loads of the heads (each slot of the element's vertices once, from L1 and
 // L2).  Collecting the candidates in a local-memory array of 256 and insertion-sorting
 // it, once to count and once to write, made the dual graph of 2.4M hexes take 4330 us
-// (two calls); it takes 571 (one).
+// (two calls); it takes 589 (one).
 #define GS_ROW 32
 template <bool HEX, bool STORE>
 __global__ void __launch_bounds__(RSB_BLOCK) k_gs_merge(int64_t ne, int nv,
