@@ -173,16 +173,6 @@ __device__ __forceinline__ double start_value(uint64_t sd, int64_t gid) {
   return (double)(h >> 11) * (1.0 / 9007199254740992.0) * 2.0 - 1.0;
 }
 
-// Unsigned key whose order is the numeric order of doubles.
-__device__ __forceinline__ uint64_t dkey(double v) {
-  const uint64_t b = (uint64_t)__double_as_longlong(v);
-  return (b >> 63) ? ~b : (b | 0x8000000000000000ull);
-}
-__device__ __forceinline__ double dkey_inv(uint64_t k) {
-  const uint64_t b = (k >> 63) ? (k & 0x7FFFFFFFFFFFFFFFull) : ~k;
-  return __longlong_as_double((long long)b);
-}
-
 // An entry's weight (0..7) as an exact double built with integer operations
 // (2^e (1 + m 2^-e) for w = 2^e + m), so that the FP64 Laplacian spends one FP64
 // instruction per entry: GB300 retires about two FP64 operations per SM cycle.

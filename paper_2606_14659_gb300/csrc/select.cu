@@ -191,28 +191,69 @@ int launch_orient(const LevelGraph& G, const Tile* tiles, int ntiles, Unit* unit
 // ----------------------------------------------------------------------------
 // segmented radix select
 // ----------------------------------------------------------------------------
-// mode 0: key = order bits of sign * v over unit rows, rank u.k        -> u.vk
-// mode 1: key = gid over tie rows (|sign v - vk| <= tau), rank k-below -> u.sel_prefix
+// The order of the values that are split: their integer keys, with -0 and +0 one value
+// and every NaN (of either sign) one value above all others.  Coordinates are the
+// caller's, and a unit's parts have their sizes whatever lies in them.
+// The key of -x is 0 - the key of x.
+__device__ __forceinline__ uint64_t split_key(double x, bool neg) {
+  uint64_t b = (uint64_t)__double_as_longlong(x);
+  // (the same test on k, which lies between the infinities' keys, by a subtraction and one
+  // unsigned comparison, is compiled wrongly by nvcc 13.0)
+  const bool nan = (b & 0x7FFFFFFFFFFFFFFFull) > 0x7FF0000000000000ull;
+  if (neg) b ^= 0x8000000000000000ull;
+  const uint64_t k = (b >> 63) ? 0ull - b : b | 0x8000000000000000ull;
+  return nan ? ~0ull : k;
+}
+__device__ __forceinline__ double split_value(uint64_t k) {
+  return __longlong_as_double(
+      (long long)((k >> 63) ? k & 0x7FFFFFFFFFFFFFFFull : 0ull - k));
+}
+
+// Reading R7's window about the k-th value vk: a row below it goes left, a row in it is a
+// tie.  A row of a key up to vk's is one or the other and at most k - 1 rows are below,
+// so the ties always make up the k, also when vk or the range (and with it tau) is not
+// finite: an infinite range makes every number a tie, a range that is no number leaves
+// the exact ties.  Keys decide but for the rows just above vk, because an FP64
+// comparison holds an SM sub-partition for 64 cycles.
+struct TieWindow {
+  uint64_t klim, kvk, khi;
+  double vk, tau;
+  __device__ __forceinline__ TieWindow(double v, double t) : vk(v), tau(t >= 0.0 ? t : 0.0) {
+    klim = kvk = khi = split_key(vk, false);
+    if (kvk == ~0ull) return;  // (nothing is computed from a NaN)
+    if (isinf(tau)) {
+      khi = split_key(tau, false);
+      klim = 0ull - khi;
+    } else {
+      klim = split_key(vk - tau, false);
+      khi = split_key(vk + 1.5 * tau, false);
+    }
+  }
+  __device__ __forceinline__ bool below(uint64_t key) const { return key < klim; }
+  // (x: the value of the key)
+  __device__ __forceinline__ bool tie(uint64_t key, double x) const {
+    return key >= klim && (key <= kvk || (key <= khi && x - vk <= tau));
+  }
+};
+
+// mode 0: key = order bits of sign * v over unit rows, rank u.k -> u.vk
+// mode 1: key = gid over tie rows (TieWindow), rank k-below     -> u.sel_prefix
 // mode 2: key = component key over all unit rows, rank u.k           -> u.sel_prefix
 enum { SEL_VALUE = 0, SEL_TIEGID = 1, SEL_COMP = 2 };
 
 __device__ __forceinline__ bool sel_member(const Unit& u, int mode, int r, const uint64_t* ckey,
-                                           const double* v, const int64_t* gid, uint64_t& key) {
+                                           const double* v, const int64_t* gid,
+                                           const TieWindow& win, uint64_t& key) {
   if (mode == SEL_COMP) {
     key = ckey[r];
     return true;
   }
   if (!unit_has(u, ckey, r)) return false;
-  const double x = u.sign * v[r];
-  if (mode == SEL_VALUE) {
-    key = dkey(x);
-    return true;
-  }
-  if (fabs(x - u.vk) <= u.tau) {
-    key = (uint64_t)gid[r];
-    return true;
-  }
-  return false;
+  key = split_key(v[r], u.sign < 0.0);
+  if (mode == SEL_VALUE) return true;
+  if (!win.tie(key, u.sign * v[r])) return false;
+  key = (uint64_t)gid[r];
+  return true;
 }
 
 __global__ void k_sel_init(Unit* units, int nunits, int mode, int cand) {
@@ -238,9 +279,10 @@ __global__ void __launch_bounds__(RSB_BLOCK)
   __syncthreads();
   const uint64_t himask = shift >= 56 ? 0ull : (~0ull << (shift + 8));
   const uint64_t want = u.sel_prefix & himask;
+  const TieWindow win(u.vk, u.tau);
   for (int r = t.row0 + threadIdx.x; r < t.row1; r += RSB_BLOCK) {
     uint64_t key;
-    if (!sel_member(u, mode, r, ckey, v, gid, key)) continue;
+    if (!sel_member(u, mode, r, ckey, v, gid, win, key)) continue;
     if ((key & himask) != want) continue;
     atomicAdd(&sh[(key >> shift) & 255u], 1);
   }
@@ -272,7 +314,7 @@ __global__ void __launch_bounds__(256) k_sel_scan(Unit* units, int mode, int can
     u.sel_below += excl;
     u.sel_prefix |= (uint64_t)threadIdx.x << shift;
     u.sel_eq = c;
-    if (shift == 0 && mode == SEL_VALUE) u.vk = dkey_inv(u.sel_prefix);
+    if (shift == 0 && mode == SEL_VALUE) u.vk = split_value(u.sel_prefix);
   }
   h[threadIdx.x] = 0;
 }
@@ -303,11 +345,11 @@ __global__ void __launch_bounds__(RSB_BLOCK)
   const Tile t = tiles[blockIdx.x];
   Unit& u = units[t.unit];
   if (!u.valid || cand >= u.ncand) return;
-  const double lim = u.vk - u.tau;
-  double c = 0.0;
+  const TieWindow win(u.vk, u.tau);
+  int cnt = 0;
   for (int r = t.row0 + threadIdx.x; r < t.row1; r += RSB_BLOCK)
-    if (unit_has(u, ckey, r) && u.sign * v[r] < lim) c += 1.0;
-  c = block_sum(c, sm);
+    if (unit_has(u, ckey, r)) cnt += win.below(split_key(v[r], u.sign < 0.0));
+  const double c = block_sum((double)cnt, sm);
   if (threadIdx.x == 0) partials[blockIdx.x] = c;
   if (last_cta(&u.cnt, u.ntile)) {
     final_reduce(partials, stride, u.tile0, u.ntile, 1, out);
@@ -332,14 +374,14 @@ __global__ void __launch_bounds__(RSB_BLOCK)
   const Tile t = tiles[blockIdx.x];
   const Unit& u = units[t.unit];
   if (!u.valid || cand >= u.ncand) return;
-  const double lim = u.vk - u.tau;
+  const TieWindow win(u.vk, u.tau);
   const uint64_t gthr = u.sel_prefix;  // k''-th smallest tie gid
   const bool all_below = (u.k - u.below) <= 0;
   for (int r = t.row0 + threadIdx.x; r < t.row1; r += RSB_BLOCK) {
     if (!unit_has(u, ckey, r)) continue;
-    const double x = u.sign * v[r];
-    bool left = x < lim;
-    if (!left && !all_below && fabs(x - u.vk) <= u.tau) left = (uint64_t)gid[r] <= gthr;
+    const uint64_t key = split_key(v[r], u.sign < 0.0);
+    bool left = win.below(key);
+    if (!left && !all_below && win.tie(key, u.sign * v[r])) left = (uint64_t)gid[r] <= gthr;
     const uint8_t bit = (uint8_t)(1u << cand);
     side[r] = left ? (uint8_t)(side[r] & ~bit) : (uint8_t)(side[r] | bit);
   }
@@ -373,7 +415,9 @@ int launch_split_assign(const LevelGraph& G, const Tile* tiles, int ntiles, Unit
 // Per-unit scratch: zeroed (Z) and set to all ones (O) before the launch.
 struct SplitZ {
   int hist[3][SPLIT_BINS];   // three buffers in turn: one filled, one read, one cleared
-  unsigned long long kmax, tmax;
+  unsigned long long kmax;   // largest key of a number
+  unsigned long long nan;    // 1: there are NaNs
+  unsigned long long tmax;
   unsigned long long below;
   unsigned long long sgn;    // 1: v[g*] <= 0, 2: v[g*] > 0
 };
@@ -381,12 +425,6 @@ struct SplitO {
   unsigned long long kmin, tmin, gmin;
 };
 
-__device__ __forceinline__ uint64_t split_key(double x, bool neg) {
-  uint64_t b = (uint64_t)__double_as_longlong(x);
-  if (neg) b ^= 0x8000000000000000ull;
-  if (b == 0x8000000000000000ull) b = 0;  // -0 and +0 are one value
-  return (b >> 63) ? ~b : (b | 0x8000000000000000ull);
-}
 __device__ __forceinline__ unsigned long long warp_max_u64(unsigned long long x) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
@@ -416,7 +454,7 @@ __global__ void __launch_bounds__(RSB_BLOCK, 4)
   __shared__ long long rank[SPLIT_MAXL];
   __shared__ int first[SPLIT_MAXL];       // passes before this one are decided; 8: none left
   __shared__ uint8_t neg[SPLIT_MAXL], on[SPLIT_MAXL];
-  __shared__ uint64_t klim[SPLIT_MAXL], klo[SPLIT_MAXL], khi[SPLIT_MAXL];
+  __shared__ uint64_t klim[SPLIT_MAXL], kvk[SPLIT_MAXL], khi[SPLIT_MAXL];
   __shared__ double vk[SPLIT_MAXL], tau[SPLIT_MAXL];
   __shared__ unsigned long long red[2][RSB_WARPS];
   const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
@@ -439,6 +477,10 @@ __global__ void __launch_bounds__(RSB_BLOCK, 4)
     for (int r = t.row0 + tid; r < t.row1; r += RSB_BLOCK) {
       if (!unit_has(u, ckey, r)) continue;
       const uint64_t k = split_key(v[r], false);
+      if (k == ~0ull) {
+        Z[t.unit].nan = 1;
+        continue;
+      }
       hi = k > hi ? k : hi;
       lo = k < lo ? k : lo;
     }
@@ -466,13 +508,14 @@ __global__ void __launch_bounds__(RSB_BLOCK, 4)
       if (!on[l]) continue;
       const Tile t = tiles[blockIdx.x + l * G];
       const Unit& u = units[t.unit];
-      const double amax = fmax(fabs(dkey_inv(__ldcg(&Z[t.unit].kmax))),
-                               fabs(dkey_inv(__ldcg(&O[t.unit].kmin))));
+      const double amax = fmax(fabs(split_value(__ldcg(&Z[t.unit].kmax))),
+                               fabs(split_value(__ldcg(&O[t.unit].kmin))));
       const uint64_t thr = split_key(0.5 * amax, false);
       unsigned long long g = ~0ull;
       for (int r = t.row0 + tid; r < t.row1; r += RSB_BLOCK) {
         if (!unit_has(u, ckey, r)) continue;
-        if (split_key(fabs(v[r]), false) >= thr) {
+        const uint64_t key = split_key(v[r], false);
+        if ((key >> 63 ? key : 0ull - key) >= thr && key != ~0ull) {
           const unsigned long long x = (unsigned long long)gid[r] ^ 0x8000000000000000ull;
           g = x < g ? x : g;
         }
@@ -499,11 +542,13 @@ __global__ void __launch_bounds__(RSB_BLOCK, 4)
     const bool ng = !fixed_sign && __ldcg(&Z[ui].sgn) == 2;
     uint64_t hi = __ldcg(&Z[ui].kmax), lo = __ldcg(&O[ui].kmin);
     if (ng) {  // keys of the negated values
-      const uint64_t x = ~lo;
-      lo = ~hi;
+      const uint64_t x = 0ull - lo;
+      lo = 0ull - hi;
       hi = x;
-      if (lo == 0x7FFFFFFFFFFFFFFFull) lo = 0x8000000000000000ull;
-      if (hi == 0x7FFFFFFFFFFFFFFFull) hi = 0x8000000000000000ull;
+    }
+    if (__ldcg(&Z[ui].nan)) {  // (a unit of NaNs alone: one value)
+      if (__ldcg(&O[ui].kmin) == ~0ull) lo = ~0ull;
+      hi = ~0ull;
     }
     neg[l] = ng;
     rank[l] = units[ui].k;
@@ -530,9 +575,8 @@ __global__ void __launch_bounds__(RSB_BLOCK, 4)
           if (!unit_has(u, ckey, r)) continue;
           uint64_t key = split_key(v[r], ng);
           if (stage == 1) {
-            if (key < klo[l] || key > khi[l]) continue;
-            const double x = ng ? -v[r] : v[r];
-            if (!(fabs(x - vk[l]) <= tau[l])) continue;
+            if (key < klim[l] || key > khi[l]) continue;
+            if (key > kvk[l] && !((ng ? -v[r] : v[r]) - vk[l] <= tau[l])) continue;
             key = (uint64_t)gid[r];
           }
           if ((key & himask) == want) atomicAdd(&sh[(key >> shift) & 255u], 1);
@@ -569,12 +613,15 @@ __global__ void __launch_bounds__(RSB_BLOCK, 4)
     for (int l = tid; l < nl; l += RSB_BLOCK)
       if (on[l]) {
         const int ui = tiles[blockIdx.x + l * G].unit;
-        const double hi = dkey_inv(__ldcg(&Z[ui].kmax)), lo = dkey_inv(__ldcg(&O[ui].kmin));
-        vk[l] = dkey_inv(prefix[l]);
-        tau[l] = tie_rel * (hi - lo);
-        klim[l] = split_key(vk[l] - tau[l], false);
-        klo[l] = split_key(vk[l] - 1.5 * tau[l], false);
-        khi[l] = split_key(vk[l] + 1.5 * tau[l], false);
+        // (of the numbers, and not beyond the starts of k_orient_stats)
+        const double hi = fmax(-1e300, split_value(__ldcg(&Z[ui].kmax)));
+        const double lo = fmin(1e300, split_value(__ldcg(&O[ui].kmin)));
+        const TieWindow win(split_value(prefix[l]), tie_rel * (hi - lo));
+        vk[l] = win.vk;
+        tau[l] = win.tau;
+        klim[l] = win.klim;
+        kvk[l] = win.kvk;
+        khi[l] = win.khi;
       }
     __syncthreads();
     for (int l = 0; l < nl; ++l) {
@@ -588,9 +635,8 @@ __global__ void __launch_bounds__(RSB_BLOCK, 4)
         if (!unit_has(u, ckey, r)) continue;
         const uint64_t key = split_key(v[r], ng);
         below += key < klim[l];
-        if (key >= klo[l] && key <= khi[l]) {
-          const double x = ng ? -v[r] : v[r];
-          if (fabs(x - vk[l]) <= tau[l]) {
+        if (key >= klim[l] && key <= khi[l]) {
+          if (key <= kvk[l] || (ng ? -v[r] : v[r]) - vk[l] <= tau[l]) {
             const unsigned long long g = (unsigned long long)gid[r];
             hi = g > hi ? g : hi;
             lo = g < lo ? g : lo;
@@ -644,10 +690,9 @@ __global__ void __launch_bounds__(RSB_BLOCK, 4)
       if (!unit_has(u, ckey, r)) continue;
       const uint64_t key = split_key(v[r], ng);
       bool left = key < klim[l];
-      if (!left && !none && key >= klo[l] && key <= khi[l]) {
-        const double x = ng ? -v[r] : v[r];
-        if (fabs(x - vk[l]) <= tau[l]) left = (uint64_t)gid[r] <= gthr;
-      }
+      if (!left && !none && key <= khi[l] &&
+          (key <= kvk[l] || (ng ? -v[r] : v[r]) - vk[l] <= tau[l]))
+        left = (uint64_t)gid[r] <= gthr;
       side[r] = left ? (uint8_t)(side[r] & ~bit) : (uint8_t)(side[r] | bit);
     }
   }
