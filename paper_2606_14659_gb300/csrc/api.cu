@@ -46,7 +46,8 @@ int launch_choose(const LevelGraph& G, const Tile* tiles, int ntiles, Unit* unit
                   cudaStream_t s);
 int launch_finalize_side(const LevelGraph& G, const uint8_t* seg_split,
                          const uint64_t* seg_keystar, const int32_t* seg_unit, const Unit* units,
-                         const uint64_t* ckey, uint8_t* side, cudaStream_t s);
+                         const uint64_t* ckey, const int64_t* seg_row0, const int64_t* seg_nleft,
+                         const int* err, uint8_t* side, cudaStream_t s);
 int launch_cut(const LevelGraph& G, const Tile* tiles, int ntiles, Unit* units,
                const uint64_t* ckey, const uint8_t* side, int cand, double* partials,
                cudaStream_t s);
@@ -1084,7 +1085,9 @@ static int run_rsb(Ctx& c, const std::vector<MeshIn>& meshes, const std::vector<
                            cudaMemcpyHostToDevice, c.s));
     if ((rc = launch_finalize_side(G, dptr<uint8_t>(c.seg_split), dptr<uint64_t>(c.seg_keystar),
                                    dptr<int32_t>(c.seg_unit), dptr<Unit>(c.units),
-                                   dptr<uint64_t>(c.ckey), dptr<uint8_t>(c.side), c.s)))
+                                   dptr<uint64_t>(c.ckey), dptr<int64_t>(c.seg_row0),
+                                   dptr<int64_t>(c.seg_nleft), &cn->gb_split.err,
+                                   dptr<uint8_t>(c.side), c.s)))
       return rc;
     LevelGraph H;
     const int nxt = cur ^ 1;

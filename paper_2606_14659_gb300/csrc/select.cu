@@ -459,7 +459,7 @@ __global__ void __launch_bounds__(RSB_BLOCK, 4)
   __shared__ unsigned long long red[2][RSB_WARPS];
   const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
   const int G = gridDim.x;
-  UnitBar bar(counter, G, 0u, gb);
+  UnitBar bar(counter, G, __ldcg(&gb->count), gb);
   // tiles blockIdx, blockIdx + G, ... of this CTA
   const int nl = (ntiles - (int)blockIdx.x + G - 1) / G;
   for (int l = tid; l < nl; l += RSB_BLOCK) {
@@ -702,7 +702,10 @@ size_t split_scratch_bytes(int nunits) {
   return (sizeof(SplitZ) + sizeof(SplitO)) * (size_t)nunits + 256;
 }
 
-// scratch: split_scratch_bytes.  *done = 0 when the level has too many tiles for one
+// scratch: split_scratch_bytes.  gb: its error word outlives the launch (a wait that ran
+// out leaves the side bits unfinished; k_finalize_side then does not use them), its count
+// is where the barrier's arrivals are expected to start, out of reach under the test hook.
+// *done = 0 when the level has too many tiles for one
 // co-resident launch (the caller then takes the steps one by one).
 int launch_split(const LevelGraph& G, const Tile* tiles, int ntiles, Unit* units, int nunits,
                  const uint64_t* ckey, const double* v, int cand, double tie_rel, int fixed_sign,
@@ -723,6 +726,8 @@ int launch_split(const LevelGraph& G, const Tile* tiles, int ntiles, Unit* units
   SplitO* O = (SplitO*)(Z + nunits);
   RSB_CK(cudaMemsetAsync(scratch, 0, 256 + sizeof(SplitZ) * (size_t)nunits, s));
   RSB_CK(cudaMemsetAsync(O, 0xFF, sizeof(SplitO) * (size_t)nunits, s));
+  if (g_rsb_poison_barrier)
+    RSB_CK(cudaMemsetAsync(&gb->count, 0x40, sizeof(unsigned int), s));
   const int64_t* gid = G.gid;
   void* args[] = {(void*)&gid, (void*)&tiles, (void*)&ntiles, (void*)&units, (void*)&ckey, (void*)&v,
                   (void*)&cand, (void*)&tie_rel, (void*)&fixed_sign, (void*)&side, (void*)&Z,
@@ -819,16 +824,24 @@ int launch_choose(const LevelGraph& G, const Tile* tiles, int ntiles, Unit* unit
 // seg_keystar[s]: component key of the straddling (or last fitting) component of a
 // segment that fell apart.
 // seg_unit[s]: unit solving the straddler, or -1 when components fit exactly.
+// err: error word of the call's splits.  Once a wait of theirs ran out, the side bits may
+// be anything; the call will fail, but its levels still run to the end, so every segment
+// is then cut by row number, which gives the halves the sizes that the compaction relies on.
 __global__ void k_finalize_side(const int32_t* __restrict__ row_seg, int32_t n,
                                 const uint8_t* __restrict__ seg_split,
                                 const uint64_t* __restrict__ seg_keystar,
                                 const int32_t* __restrict__ seg_unit, const Unit* units,
-                                const uint64_t* __restrict__ ckey, uint8_t* side) {
+                                const uint64_t* __restrict__ ckey,
+                                const int64_t* __restrict__ seg_row0,
+                                const int64_t* __restrict__ seg_nleft,
+                                const int* __restrict__ err, uint8_t* side) {
   const int r = blockIdx.x * RSB_BLOCK + threadIdx.x;
   if (r >= n) return;
   const int s = row_seg[r];
   uint8_t out = 0;
-  if (seg_split[s]) {
+  if (*err) {
+    out = seg_split[s] && r - seg_row0[s] >= seg_nleft[s];
+  } else if (seg_split[s]) {
     const uint64_t k = seg_split[s] == 2 ? ckey[r] : 0, ks = seg_split[s] == 2 ? seg_keystar[s] : 0;
     if (k < ks) out = 0;
     else if (k > ks) out = 1;
@@ -842,10 +855,12 @@ __global__ void k_finalize_side(const int32_t* __restrict__ row_seg, int32_t n,
 
 int launch_finalize_side(const LevelGraph& G, const uint8_t* seg_split,
                          const uint64_t* seg_keystar, const int32_t* seg_unit, const Unit* units,
-                         const uint64_t* ckey, uint8_t* side, cudaStream_t s) {
+                         const uint64_t* ckey, const int64_t* seg_row0, const int64_t* seg_nleft,
+                         const int* err, uint8_t* side, cudaStream_t s) {
   if (G.n <= 0) return RSB_OK;
   k_finalize_side<<<(G.n + RSB_BLOCK - 1) / RSB_BLOCK, RSB_BLOCK, 0, s>>>(
-      G.row_seg, G.n, seg_split, seg_keystar, seg_unit, units, ckey, side);
+      G.row_seg, G.n, seg_split, seg_keystar, seg_unit, units, ckey, seg_row0, seg_nleft, err,
+      side);
   RSB_CKL("k_finalize_side");
   return RSB_OK;
 }
