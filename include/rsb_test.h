@@ -40,11 +40,12 @@ void rsb_profile_read(int family, double *ms, int64_t *launches, double *bytes);
 
 /*
  * Failure-path test hook (not part of the method).  While on != 0, the
- * persistent Lanczos launches (use_graph 2 and 3) and the cooperative split of a
- * level start their barrier from a corrupted arrival count, so no CTA sees the
- * last arrival: the first wait runs out (4 s of the GPU's global timer; later ones
- * end at once), the kernel ends, and the call returns RSB_ETIMEOUT.  Nothing faults or hangs; the next call with the hook
- * off starts from a clean barrier.  Process-wide, not thread-safe; for tests.
+ * persistent Lanczos launches (use_graph 2 and 3), the resident CG solves (3) and
+ * the cooperative split of a level start their barrier from a corrupted count, so
+ * no CTA sees the last arrival: the first wait runs out (4 s of the GPU's global
+ * timer; later ones end at once), the kernel ends, and the call returns
+ * RSB_ETIMEOUT.  Nothing faults or hangs; the next call with the hook off starts
+ * from a clean barrier.  Process-wide, not thread-safe; for tests.
  */
 void rsb_test_poison_barrier(int on);
 

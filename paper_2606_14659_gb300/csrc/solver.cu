@@ -3252,6 +3252,8 @@ static int inverse_run(const LevelGraph& G, const Tile* tiles, int ntiles, Unit*
       res = (long long)occ * nsm >= ntiles;
     }
     RSB_CK(cudaMemsetAsync(B.gb, 0, sizeof(GridBar), s));
+    if (g_rsb_poison_barrier && res)  // test hook: the units' arrivals are out of reach
+      RSB_CK(cudaMemsetAsync(&B.gb->count, 0x40, sizeof(unsigned int), s));
   }
   const int CGK = 8;
   cudaGraphExec_t exec = nullptr;
