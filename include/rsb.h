@@ -219,8 +219,8 @@ int rsb_fiedler(const rsb_csr *g, const rsb_options *o, double *lambda2, double 
  * y = L x with L = D - A of graph g (§4 weighted Laplacian, §5 action), in FP64
  * (x, y double[n]) or FP32 (x, y float[n]): a building block exposed for testing.
  * Rows are summed in entry order, as the solvers sum the library's sliced-ELL
- * form.  The graph is checked on the way; when it is malformed (RSB_EINVAL), a
- * device y is undefined.
+ * form.  The graph is checked on the way; when it is malformed (RSB_EINVAL), y is
+ * as it was once the call returns.
  */
 int rsb_laplacian_apply(const rsb_csr *g, const double *x, double *y, void *stream);
 int rsb_laplacian_apply_f32(const rsb_csr *g, const float *x, float *y, void *stream);

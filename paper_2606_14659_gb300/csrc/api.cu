@@ -288,7 +288,8 @@ struct Ctx {
   // gather-scatter (element -> vertex ids): buckets of elements per vertex
   DevBuf gs_count, gs_cnt, gs_bptr, gs_bucket, gs_ev32, gs_len, gs_rowptr, gs_w, gs_misc, gs_rows;
   DevBuf part_concat;
-  DevBuf lap_x, lap_y;  // device copies of a Laplacian action's host vectors
+  // Laplacian action: device copies of host vectors; of a device y, what it held before
+  DevBuf lap_x, lap_y;
   int trmax = 0;    // largest tile of the level being solved, rows
   int ntmax = 0;    // most tiles of one of its units
   std::vector<DevBuf> stage;  // staged host inputs
@@ -1559,15 +1560,13 @@ static int lap_apply(const rsb_csr* g, const void* x, void* y, int f32, void* st
     xd = c.lap_x.p;
   }
   const bool yh = !is_device_ptr(y);
-  if (yh) {
-    if ((rc = devbuf_reserve(c.lap_y, es * N))) return end_call(c, stream, rc);
-    yd = c.lap_y.p;
-  }
+  if ((rc = devbuf_reserve(c.lap_y, es * N))) return end_call(c, stream, rc);
+  if (yh) yd = c.lap_y.p;
   // faults are reported into pinned host words that the call reads once the kernel is
-  // done; a host y is left alone then
+  // done; y is then as it was
   int* err = c.h_pinned + 8;
   for (int i = 0; i < 5; ++i) err[i] = 0;
-  rc = launch_csr_apply(m.row_ptr, m.col, m.wt, N, f32, xd, yd, err, c.s);
+  rc = launch_csr_apply(m.row_ptr, m.col, m.wt, N, f32, xd, yd, yh ? nullptr : c.lap_y.p, err, c.s);
   auto faults = [&] {
     int f = 0;
     for (int i = 0; i < 5; ++i) f |= err[i] ? 1 << i : 0;
@@ -1581,7 +1580,14 @@ static int lap_apply(const rsb_csr* g, const void* x, void* y, int f32, void* st
   }
   rc = end_call(c, stream, rc);
   const int f = faults();
-  return !rc && f ? invalid_graph(f) : rc;
+  if (!rc && f) {
+    if (!yh) {
+      RSB_CK(cudaMemcpyAsync(y, c.lap_y.p, es * N, cudaMemcpyDeviceToDevice, c.s));
+      RSB_CK(cudaStreamSynchronize(c.s));
+    }
+    return invalid_graph(f);
+  }
+  return rc;
 }
 
 static int lap_bench(const rsb_csr* g, int f32, int reps, double* ms, double* bytes, void* stream) {

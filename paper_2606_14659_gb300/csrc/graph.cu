@@ -338,6 +338,8 @@ int launch_spmv_f32(const LevelGraph& G, const float* x, float* y, cudaStream_t 
 // err: five words the host sees (zero before the launch); a fault in the graph sets
 // the word of its kind, and y is then not to be used.  Reads stay inside
 // [0, row_ptr[n]) of col and wt and [0, n) of x whatever the graph holds.
+// old (optional): what y held before, for the caller to put back after a fault; the
+// rows' reads and writes travel beside the entries.
 // ----------------------------------------------------------------------------
 #define CSR_CAP 1024
 template <typename V>
@@ -345,7 +347,7 @@ __global__ void __launch_bounds__(RSB_BLOCK) k_csr_apply(const int64_t* __restri
                                                          const int32_t* __restrict__ col,
                                                          const int32_t* __restrict__ wt, int32_t n,
                                                          const V* __restrict__ x, V* __restrict__ y,
-                                                         volatile int* err) {
+                                                         V* __restrict__ old, volatile int* err) {
   __shared__ uint32_t sh[RSB_WARPS][CSR_CAP];
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t r0 = (int64_t)blockIdx.x * RSB_BLOCK + 32 * w;
@@ -354,9 +356,11 @@ __global__ void __launch_bounds__(RSB_BLOCK) k_csr_apply(const int64_t* __restri
   const int64_t r = r0 + lane;
   const int64_t nnz = row_ptr[n];
   int64_t b = 0, e = 0;
+  V was = V(0);
   if (lane < rows) {
     b = row_ptr[r];
     e = row_ptr[r + 1];
+    if (old) was = y[r];
   }
   // the warp's entries; rows that do not follow one another inside [0, nnz) are faults
   const int64_t w0 = __shfl_sync(0xffffffffu, b, 0);
@@ -365,6 +369,7 @@ __global__ void __launch_bounds__(RSB_BLOCK) k_csr_apply(const int64_t* __restri
   if (lane < rows && (e < b || (r == 0 && b != 0) || b < w0 || e > w1 || b < 0 || e > nnz)) f = 1;
   if (__any_sync(0xffffffffu, f)) {
     if (f) err[0] = 1;
+    if (old && lane < rows) old[r] = was;
     return;
   }
   uint32_t* ws = sh[w];
@@ -415,22 +420,25 @@ __global__ void __launch_bounds__(RSB_BLOCK) k_csr_apply(const int64_t* __restri
     __syncwarp();
   }
   if constexpr (sizeof(V) == 8) acc = fma((double)dsum, xr, -acc);
-  if (lane < rows) y[r] = acc;
+  if (lane < rows) {
+    if (old) old[r] = was;
+    y[r] = acc;
+  }
   if (f & 2) err[1] = 1;
   if (f & 4) err[2] = 1;
   if (f & 8) err[3] = 1;
 }
 
 int launch_csr_apply(const int64_t* row_ptr, const int32_t* col, const int32_t* wt, int64_t n,
-                     int f32, const void* x, void* y, int* err, cudaStream_t s) {
+                     int f32, const void* x, void* y, void* old, int* err, cudaStream_t s) {
   const unsigned nb = (unsigned)((n + RSB_BLOCK - 1) / RSB_BLOCK);
   const int pi = prof_before(PROF_SPMV, s);
   if (f32)
     k_csr_apply<float><<<nb, RSB_BLOCK, 0, s>>>(row_ptr, col, wt, (int32_t)n, (const float*)x,
-                                                (float*)y, err);
+                                                (float*)y, (float*)old, err);
   else
     k_csr_apply<double><<<nb, RSB_BLOCK, 0, s>>>(row_ptr, col, wt, (int32_t)n, (const double*)x,
-                                                 (double*)y, err);
+                                                 (double*)y, (double*)old, err);
   RSB_CKL("k_csr_apply");
   prof_after(pi, s);
   return RSB_OK;

@@ -835,7 +835,7 @@ int launch_spmv_f32(const LevelGraph& G, const float* x, float* y, cudaStream_t 
 int launch_fill_rows(const int64_t* gid_in, int64_t n, int64_t row_off, int64_t home_off, int32_t seg,
                      int64_t* gid, int64_t* home, int32_t* row_seg, cudaStream_t s);
 int launch_csr_apply(const int64_t* row_ptr, const int32_t* col, const int32_t* wt, int64_t n,
-                     int f32, const void* x, void* y, int* err, cudaStream_t s);
+                     int f32, const void* x, void* y, void* old, int* err, cudaStream_t s);
 int launch_cc(const LevelGraph& G, int32_t* parent, uint64_t* ckey, int* flag, cudaStream_t s);
 int launch_comp_count(const LevelGraph& G, const int32_t* parent, int32_t* seg_ncomp,
                       cudaStream_t s);
