@@ -314,7 +314,7 @@ static int ctx_get(Ctx** out) {
     RSB_CK(cudaStreamCreateWithFlags(&c->s, cudaStreamNonBlocking));
     RSB_CK(cudaEventCreateWithFlags(&c->ev_in, cudaEventDisableTiming));
     RSB_CK(cudaEventCreateWithFlags(&c->ev_out, cudaEventDisableTiming));
-    RSB_CK(cudaMallocHost(&c->h_pinned, 64));
+    RSB_CK(cudaMallocHost(&c->h_pinned, 128));
     g_ctx[dev] = c;
   }
   *out = g_ctx[dev];
@@ -1653,10 +1653,11 @@ extern "C" void rsb_test_poison_barrier(int on) { g_rsb_poison_barrier = on ? 1 
 // ----------------------------------------------------------------------------
 int gs_vertex_count(const int64_t* ev, int64_t cnt, unsigned long long* d_max,
                     unsigned long long* h_max, int64_t* V, cudaStream_t s);
-int gs_buckets(const int64_t* ev, int64_t ne, int nv, int64_t V, int64_t* count, int64_t* bptr,
-               int32_t* bucket, int32_t* ev32, void* scan_tmp, size_t scan_bytes, cudaStream_t s);
+int gs_buckets(const int64_t* ev, int64_t ne, int nv, int64_t V, const int32_t* counted,
+               int64_t* count, int64_t* bptr, int32_t* bucket, int32_t* ev32, void* scan_tmp,
+               size_t scan_bytes, cudaStream_t s);
 int gs_row_lengths(int64_t ne, int nv, const int32_t* ev32, const int64_t* bptr,
-                   const int32_t* bucket, int64_t* len, int* d_flag, cudaStream_t s);
+                   const int32_t* bucket, int64_t* len, int* flag, cudaStream_t s);
 int gs_fill_dual(int64_t ne, int nv, const int32_t* ev32, const int64_t* bptr,
                  const int32_t* bucket, const int64_t* row_ptr, int32_t* col, int32_t* wt,
                  cudaStream_t s);
@@ -1668,12 +1669,13 @@ size_t gs_slot_bytes(int64_t cap);
 size_t gs_cnt_bytes(int64_t cap);
 int gs_slots(const int64_t* ev, int64_t ne, int nv, int64_t cap, int32_t* cnt, int32_t* slot,
              cudaStream_t s);
-int gs_slot_apply(int f32, const int64_t* ev, int64_t ne, int nv, int64_t cap, const int32_t* cnt,
+int gs_slot_apply(int f32, const int64_t* ev, int64_t ne, int nv, int64_t cap, int32_t* cnt,
                   const int32_t* slot, const void* x, void* wc, void* y, int* err, cudaStream_t s);
 size_t gs_rows_bytes(int64_t ne);
 int gs_slot_rows(const int64_t* ev, int64_t ne, int nv, int64_t cap, int32_t* cnt, int32_t* slot,
                  uint32_t* ent, int64_t* len, int* err, cudaStream_t s);
-int gs_slot_write(int64_t ne, const uint32_t* ent, const int64_t* row_ptr, int32_t* col,
+int gs_slot_write(const int64_t* ev, int64_t ne, int nv, int64_t cap, int32_t* cnt,
+                  const int32_t* slot, const uint32_t* ent, const int64_t* row_ptr, int32_t* col,
                   int32_t* wt, cudaStream_t s);
 
 static int gs_check(int64_t ne, int nv, const void* ev) {
@@ -1682,15 +1684,18 @@ static int gs_check(int64_t ne, int nv, const void* ev) {
   return RSB_OK;
 }
 
-// Buckets of the elements at every vertex in the context's workspace; *V out.
-static int gs_setup(Ctx& c, int64_t ne, int nv, const int64_t* ev_in, int64_t* V) {
+// Buckets of the elements at every vertex in the context's workspace; *V: the number of
+// vertices, found here when it is zero.  counted (optional, with *V): the number of
+// elements at each of them.
+static int gs_setup(Ctx& c, int64_t ne, int nv, const int64_t* ev_in, int64_t* V,
+                    const int32_t* counted = nullptr) {
   int rc = gs_check(ne, nv, ev_in);
   if (rc) return rc;
   const int64_t* ev = nullptr;
   if ((rc = stage_in(c, ev_in, (size_t)(ne * nv), &ev))) return rc;
-  if ((rc = devbuf_reserve(c.gs_misc, 256))) return rc;
-  if ((rc = gs_vertex_count(ev, ne * nv, dptr<unsigned long long>(c.gs_misc),
-                            (unsigned long long*)(c.h_pinned + 12), V, c.s)))
+  if (!*V && ((rc = devbuf_reserve(c.gs_misc, 256)) ||
+              (rc = gs_vertex_count(ev, ne * nv, dptr<unsigned long long>(c.gs_misc),
+                                    (unsigned long long*)(c.h_pinned + 12), V, c.s))))
     return rc;
   const int64_t nV = *V;
   const size_t scan_bytes = scan_tmp_bytes(std::max<int64_t>(nV, ne) + 2);
@@ -1700,22 +1705,31 @@ static int gs_setup(Ctx& c, int64_t ne, int nv, const int64_t* ev_in, int64_t* V
       (rc = devbuf_reserve(c.gs_ev32, sizeof(int32_t) * (size_t)(ne * nv))) ||
       (rc = devbuf_reserve(c.scan_tmp, scan_bytes)))
     return rc;
-  return gs_buckets(ev, ne, nv, nV, dptr<int64_t>(c.gs_count), dptr<int64_t>(c.gs_bptr),
+  return gs_buckets(ev, ne, nv, nV, counted, dptr<int64_t>(c.gs_count), dptr<int64_t>(c.gs_bptr),
                     dptr<int32_t>(c.gs_bucket), dptr<int32_t>(c.gs_ev32), c.scan_tmp.p, c.scan_tmp.cap, c.s);
 }
 
-// gs_setup after the slot table was tried: its room is larger than the buckets', so it
-// is given back when the buckets find none.
-static int gs_setup_after_slots(Ctx& c, int64_t ne, int nv, const int64_t* ev, int64_t* V) {
-  int rc = gs_setup(c, ne, nv, ev, V);
+// The words that the slot table's kernels report into (pinned; see gs.cu).
+static int* gs_words(Ctx& c) { return c.h_pinned + 16; }
+
+// gs_setup after the slot table did not hold the mesh (tried) or found no room.  What the
+// attempt leaves is used: the largest id, for which the buckets would have to look and
+// wait, and the counts, when it lies below the table's bound.  The table's room is larger
+// than the buckets', so it is given back when they find none.
+static int gs_setup_after_slots(Ctx& c, int64_t ne, int nv, const int64_t* ev, bool tried,
+                                int64_t* V) {
+  *V = tried ? (int64_t)gs_words(c)[4] + 1 : 0;
+  int rc = gs_setup(c, ne, nv, ev, V,
+                    tried && *V <= gs_slot_cap(ne) ? dptr<int32_t>(c.gs_cnt) : nullptr);
   if (rc != RSB_ENOMEM) return rc;
   for (DevBuf* b : {&c.gs_cnt, &c.gs_bucket, &c.gs_w, &c.gs_rows}) free_buf(*b);
+  *V = 0;
   return gs_setup(c, ne, nv, ev, V);
 }
 
 // Row lengths and offsets of the dual graph in c.gs_rowptr, their total in *total: from
-// the slot table (with want_rows, the rows in c.gs_rows as well) when the mesh fits it
-// (*slots = 1), else from the buckets.
+// the slot table when the mesh fits it (*slots = 1; with want_rows, the rows in c.gs_rows
+// as well; 2: some are too long for that), else from the buckets.
 static int dual_rows(Ctx& c, int64_t ne, int nv, const int64_t* ev, bool want_rows, int64_t* total,
                      int* slots) {
   int rc;
@@ -1726,39 +1740,42 @@ static int dual_rows(Ctx& c, int64_t ne, int nv, const int64_t* ev, bool want_ro
     return rc;
   int64_t* len = dptr<int64_t>(c.gs_len);
   int64_t* rp = dptr<int64_t>(c.gs_rowptr);
-  int* err = c.h_pinned + 8;
-  err[0] = err[1] = err[2] = 0;
+  int64_t* h_total = (int64_t*)(c.h_pinned + 24);
+  int* err = gs_words(c);
+  for (int i = 0; i < 8; ++i) err[i] = 0;
+  bool tried = true;
   if ((rc = devbuf_reserve(c.gs_cnt, gs_cnt_bytes(cap))) ||
       (rc = devbuf_reserve(c.gs_bucket, gs_slot_bytes(cap))) ||
       (want_rows && (rc = devbuf_reserve(c.gs_rows, gs_rows_bytes(ne))))) {
     if (rc != RSB_ENOMEM) return rc;
     err[1] = 1;  // no room for the table: the buckets take less
+    tried = false;
   } else {
     if ((rc = gs_slots(ev, ne, nv, cap, dptr<int32_t>(c.gs_cnt), dptr<int32_t>(c.gs_bucket),
                        c.s)) ||
         (rc = gs_slot_rows(ev, ne, nv, cap, dptr<int32_t>(c.gs_cnt), dptr<int32_t>(c.gs_bucket),
                            want_rows ? dptr<uint32_t>(c.gs_rows) : nullptr, len, err, c.s)))
       return rc;
-    RSB_CK(cudaMemsetAsync(len + ne, 0, sizeof(int64_t), c.s));
     if ((rc = launch_scan_i64(len, rp, ne + 1, c.scan_tmp.p, c.scan_tmp.cap, c.s))) return rc;
-    RSB_CK(cudaMemcpyAsync(total, rp + ne, sizeof(int64_t), cudaMemcpyDeviceToHost, c.s));
+    RSB_CK(cudaMemcpyAsync(h_total, rp + ne, sizeof(int64_t), cudaMemcpyDeviceToHost, c.s));
     RSB_CK(cudaStreamSynchronize(c.s));
+    *total = *h_total;
   }
   if (err[0]) return rsb_set_error(RSB_EINVAL, "vertex ids must lie in [0, 2^31)");
   int flag = err[2] ? 4 : 0;
-  *slots = !err[1];
+  *slots = err[1] ? 0 : err[3] ? 2 : 1;
   if (!*slots) {
     int64_t V = 0;
-    if ((rc = gs_setup_after_slots(c, ne, nv, ev, &V))) return rc;
-    int* d_flag = (int*)(dptr<unsigned long long>(c.gs_misc) + 1);
+    if ((rc = gs_setup_after_slots(c, ne, nv, ev, tried, &V))) return rc;
+    err[0] = err[1] = 0;
     if ((rc = gs_row_lengths(ne, nv, dptr<int32_t>(c.gs_ev32), dptr<int64_t>(c.gs_bptr),
-                             dptr<int32_t>(c.gs_bucket), len, d_flag, c.s)))
+                             dptr<int32_t>(c.gs_bucket), len, err, c.s)))
       return rc;
-    RSB_CK(cudaMemsetAsync(len + ne, 0, sizeof(int64_t), c.s));
     if ((rc = launch_scan_i64(len, rp, ne + 1, c.scan_tmp.p, c.scan_tmp.cap, c.s))) return rc;
-    RSB_CK(cudaMemcpyAsync(total, rp + ne, sizeof(int64_t), cudaMemcpyDeviceToHost, c.s));
-    RSB_CK(cudaMemcpyAsync(&flag, d_flag, sizeof(int), cudaMemcpyDeviceToHost, c.s));
+    RSB_CK(cudaMemcpyAsync(h_total, rp + ne, sizeof(int64_t), cudaMemcpyDeviceToHost, c.s));
     RSB_CK(cudaStreamSynchronize(c.s));
+    *total = *h_total;
+    flag = (err[0] ? 2 : 0) | (err[1] ? 4 : 0);
   }
   if (flag & 2)
     return rsb_set_error(RSB_EINVAL, "an element meets more than 256 other elements at its "
@@ -1803,7 +1820,9 @@ extern "C" int rsb_dual_graph(int64_t ne, int nv, const int64_t* ev_in, int64_t*
     }
     if (!cd) colp = (int32_t*)tc.p;
     if (!wd) wtp = (int32_t*)tw.p;
-    rc = slots ? gs_slot_write(ne, dptr<uint32_t>(c.gs_rows), rp, colp, wtp, c.s)
+    rc = slots ? gs_slot_write(ev, ne, nv, gs_slot_cap(ne), dptr<int32_t>(c.gs_cnt),
+                               dptr<int32_t>(c.gs_bucket),
+                               slots == 1 ? dptr<uint32_t>(c.gs_rows) : nullptr, rp, colp, wtp, c.s)
                : gs_fill_dual(ne, nv, dptr<int32_t>(c.gs_ev32), dptr<int64_t>(c.gs_bptr),
                               dptr<int32_t>(c.gs_bucket), rp, colp, wtp, c.s);
     if (!rc && !cd)
@@ -1821,18 +1840,20 @@ extern "C" int rsb_dual_graph(int64_t ne, int nv, const int64_t* ev_in, int64_t*
 }
 
 // One application from the slot table; *fits = 0 when the mesh does not fit it (the
-// general path then answers) and y is as it was.  x, y and ev: device pointers.
+// general path then answers; *tried = 0 when there was no room to see) and y is as it was.
+// x, y and ev: device pointers.
 static int gs_lap_slots(Ctx& c, int64_t ne, int nv, const int64_t* ev, const void* x, void* y,
-                        int f32, int* fits) {
+                        int f32, int* fits, bool* tried) {
   const int64_t cap = gs_slot_cap(ne);
   int rc;
   *fits = 0;
+  *tried = false;
   if ((rc = devbuf_reserve(c.gs_cnt, gs_cnt_bytes(cap))) ||
       (rc = devbuf_reserve(c.gs_bucket, gs_slot_bytes(cap))) ||
       (rc = devbuf_reserve(c.gs_w, (f32 ? 8 : 16) * (size_t)cap)))
     return rc == RSB_ENOMEM ? RSB_OK : rc;  // (the buckets take less)
-  int* err = c.h_pinned + 8;  // words the kernels report into
-  err[0] = err[1] = 0;
+  int* err = gs_words(c);
+  err[0] = err[1] = err[4] = 0;
   if ((rc = gs_slots(ev, ne, nv, cap, dptr<int32_t>(c.gs_cnt), dptr<int32_t>(c.gs_bucket),
                      c.s)) ||
       (rc = gs_slot_apply(f32, ev, ne, nv, cap, dptr<int32_t>(c.gs_cnt),
@@ -1841,6 +1862,7 @@ static int gs_lap_slots(Ctx& c, int64_t ne, int nv, const int64_t* ev, const voi
   RSB_CK(cudaStreamSynchronize(c.s));
   if (err[0]) return rsb_set_error(RSB_EINVAL, "vertex ids must lie in [0, 2^31)");
   *fits = !err[1];
+  *tried = true;
   return RSB_OK;
 }
 
@@ -1873,10 +1895,11 @@ static int gs_lap_apply(int64_t ne, int nv, const int64_t* ev_in, const void* x,
     yd = ty.p;
   }
   int fits = 0;
-  if ((rc = gs_lap_slots(c, ne, nv, ev, xd, yd, f32, &fits))) return done(rc);
+  bool tried = false;
+  if ((rc = gs_lap_slots(c, ne, nv, ev, xd, yd, f32, &fits, &tried))) return done(rc);
   if (!fits) {
     int64_t V = 0;
-    if ((rc = gs_setup_after_slots(c, ne, nv, ev, &V)) ||
+    if ((rc = gs_setup_after_slots(c, ne, nv, ev, tried, &V)) ||
         (rc = devbuf_reserve(c.gs_w, es * (size_t)(V + 1))))
       return done(rc);
     if ((rc = gs_apply(f32, ne, nv, V, dptr<int32_t>(c.gs_ev32), dptr<int64_t>(c.gs_bptr),

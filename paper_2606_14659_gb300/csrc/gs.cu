@@ -48,6 +48,12 @@ __global__ void __launch_bounds__(RSB_BLOCK) k_gs_maxid(const int64_t* __restric
   }
 }
 
+// The counts of a slot table whose vertices are too full for it, widened (count[V] = 0).
+__global__ void k_gs_widen(const int32_t* __restrict__ cnt, int64_t V, int64_t* count) {
+  const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (v <= V) count[v] = v < V ? cnt[v] : 0;
+}
+
 __global__ void k_gs_count(const int64_t* __restrict__ ev, int64_t cnt, int64_t* count) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < cnt) atomicAdd((unsigned long long*)(count + ev[i]), 1ull);
@@ -111,13 +117,14 @@ __device__ int gs_neighbours(int64_t e, int nv, const int32_t* __restrict__ ev32
 
 __global__ void k_gs_rowlen(int64_t ne, int nv, const int32_t* __restrict__ ev32,
                             const int64_t* __restrict__ bptr, const int32_t* __restrict__ bucket,
-                            int64_t* len, int* flag) {
+                            int64_t* len, volatile int* flag) {
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (e == ne) len[ne] = 0;  // (the scan's last entry)
   if (e >= ne) return;
   int32_t cand[GS_MAXCAND];
   const int nc = gs_neighbours(e, nv, ev32, bptr, bucket, cand);
   if (nc < 0) {
-    atomicOr(flag, 2);
+    flag[0] = 1;
     len[e] = 0;
     return;
   }
@@ -127,7 +134,7 @@ __global__ void k_gs_rowlen(int64_t ne, int nv, const int32_t* __restrict__ ev32
     run = (p > 0 && cand[p] == cand[p - 1]) ? run + 1 : 1;
     if (p + 1 == nc || cand[p + 1] != cand[p]) {
       ++d;
-      if (run > 7) atomicOr(flag, 4);  // more than 7 shared vertices: duplicate elements
+      if (run > 7) flag[1] = 1;  // more than 7 shared vertices: duplicate elements
     }
   }
   len[e] = d;
@@ -191,15 +198,17 @@ __global__ void __launch_bounds__(RSB_BLOCK) k_gs_apply(int64_t ne, int nv,
 // below a bound known beforehand.  One pass over the ids takes the place of the pass
 // for the largest id (and the host's wait for it), the count, the scan and the fill of
 // the buckets above; a mesh that does not fit sets a word, the kernels that follow return
-// at once, and the caller takes the general path.  A vertex's slots hold its elements in
-// arrival order; their
-// readers sort the at most eight of them in registers, so results do not depend on it.
+// almost at once, leaving the largest id, and the caller takes the general path, which
+// need not look for it again, nor count when it is below the bound.  A vertex's slots hold its elements
+// in arrival order; their readers sort the at most eight of them in registers, so results
+// do not depend on it.
 // One Laplacian application at 1.9M hexes 168 us, 717 from the buckets.
 // Words behind the counts, cleared with them: [0] an id outside [0, 2^31), [1] the table
-// does not hold the mesh, [2] two elements share more than 7 vertices.
+// does not hold the mesh, [2] two elements share more than 7 vertices, [3] an element has
+// more than GS_ROW neighbours, [4] the largest id of a mesh that the table does not hold.
 // ----------------------------------------------------------------------------
 #define GS_SLOTS 8
-#define GS_WORDS 4
+#define GS_WORDS 8
 
 // The ids of element e (unused places: -1).
 template <bool HEX>
@@ -219,6 +228,14 @@ __device__ __forceinline__ void gs_ids(const int64_t* __restrict__ ev, int64_t e
   }
 }
 
+// Word 4 takes the largest m (not negative) of the threads that are here.
+__device__ __forceinline__ void gs_note_max(int32_t* cnt, int64_t cap, int m) {
+  const unsigned mask = __activemask();
+  m = __reduce_max_sync(mask, m);
+  if ((int)(threadIdx.x & 31) == __ffs(mask) - 1 && m > *(volatile int32_t*)(cnt + cap + 4))
+    atomicMax(cnt + cap + 4, m);
+}
+
 // Bound: the returned atomics (one per id, eight in flight a thread).
 template <bool HEX>
 __global__ void __launch_bounds__(RSB_BLOCK) k_gs_slots(const int64_t* __restrict__ ev, int64_t ne,
@@ -230,13 +247,14 @@ __global__ void __launch_bounds__(RSB_BLOCK) k_gs_slots(const int64_t* __restric
   int64_t id[8];
   gs_ids<HEX>(ev, e, nv, id);
   bool out = false, full = false;
+  int far = 0;
   int pos[8];
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
     pos[i] = GS_SLOTS;
     if (HEX || i < nv) {
       if (id[i] < 0 || id[i] >= (1ll << 31)) out = true;
-      else if (id[i] >= cap) full = true;
+      else if (id[i] >= cap) far = max(far, (int)id[i]);
       else pos[i] = atomicAdd(cnt + id[i], 1);
     }
   }
@@ -246,7 +264,8 @@ __global__ void __launch_bounds__(RSB_BLOCK) k_gs_slots(const int64_t* __restric
     else if ((HEX || i < nv) && id[i] >= 0 && id[i] < cap) full = true;
   }
   if (out && !err[0]) err[0] = 1;
-  if (full && !err[1]) err[1] = 1;
+  if ((full || far) && !err[1]) err[1] = 1;
+  if (far) gs_note_max(cnt, cap, far);
 }
 
 // Not zero: the table does not hold the mesh.  (Its readers load it beside their first
@@ -256,11 +275,12 @@ __device__ __forceinline__ int gs_unfit(const int32_t* cnt, int64_t cap) {
 }
 
 // The elements at vertex v in ascending order, INT_MAX in the places left (a sorting
-// network of 19 exchanges); returns their number (0 when the mesh does
-// not fit).
-__device__ __forceinline__ int gs_sorted_slots(const int32_t* cnt, int64_t cap, const int32_t* slot,
+// network of 19 exchanges); returns their number (0 when the mesh does not fit: the
+// largest vertex that has any is then noted).
+__device__ __forceinline__ int gs_sorted_slots(int32_t* cnt, int64_t cap, const int32_t* slot,
                                                int64_t v, int32_t (&f)[GS_SLOTS]) {
   const int here = cnt[v], unfit = gs_unfit(cnt, cap);
+  if (unfit && here) gs_note_max(cnt, cap, (int)v);
   const int n = unfit ? 0 : min(here, GS_SLOTS);
   const int4* p = reinterpret_cast<const int4*>(slot + v * GS_SLOTS);
   int4 lo = make_int4(0, 0, 0, 0), hi = lo;
@@ -292,7 +312,7 @@ struct alignas(2 * sizeof(V)) GsPair {
 };
 
 template <typename V>
-__global__ void __launch_bounds__(RSB_BLOCK) k_gs_vsum8(int64_t nvert, const int32_t* __restrict__ cnt,
+__global__ void __launch_bounds__(RSB_BLOCK) k_gs_vsum8(int64_t nvert, int32_t* cnt,
                                                       const int32_t* __restrict__ slot,
                                                       const V* __restrict__ x,
                                                       GsPair<V>* __restrict__ wc) {
@@ -323,7 +343,7 @@ __global__ void __launch_bounds__(RSB_BLOCK) k_gs_apply8(int64_t ne, int nv,
   int64_t id[8];
   gs_ids<HEX>(ev, e, nv, id);
   if (unfit) {  // told to the host, which then takes the buckets
-    if (e == 0) err[0] = cnt[cap], err[1] = cnt[cap + 1];
+    if (e == 0) err[0] = cnt[cap], err[1] = cnt[cap + 1], err[4] = cnt[cap + 4];
     return;
   }
   GsPair<V> p[8];
@@ -341,8 +361,7 @@ __global__ void __launch_bounds__(RSB_BLOCK) k_gs_apply8(int64_t ne, int nv,
 }
 
 // Every vertex's slots in ascending order, INT_MAX in the places left (in place).
-__global__ void __launch_bounds__(RSB_BLOCK) k_gs_sort8(int64_t nvert, const int32_t* __restrict__ cnt,
-                                                      int32_t* slot) {
+__global__ void __launch_bounds__(RSB_BLOCK) k_gs_sort8(int64_t nvert, int32_t* cnt, int32_t* slot) {
   const int64_t v = (int64_t)blockIdx.x * RSB_BLOCK + threadIdx.x;
   if (v >= nvert) return;
   int32_t f[GS_SLOTS];
@@ -354,29 +373,37 @@ __global__ void __launch_bounds__(RSB_BLOCK) k_gs_sort8(int64_t nvert, const int
 
 // Distinct neighbours of element e with their shared-vertex counts, ascending: a merge
 // of the sorted slots of its vertices, the heads in registers.  A neighbour's entry
-// (packed as in the sliced form) goes to ent[(32-row group * GS_ROW + k) * 32 + lane],
-// their number to len[e].  More than GS_ROW neighbours set word 1, which stops the CTAs
-// that start later.
+// (packed as in the sliced form) goes to ent[(32-row group * GS_ROW + k) * 32 + lane]
+// (MERGE_ROWS), their number to len[e].  An element of more than GS_ROW neighbours (of at
+// most 56) sets word 3, and the rows are merged once more, straight into CSR
+// (MERGE_CSR): the graph of 1M elements of 56 neighbours, counted and written by two calls,
+// 2.0 ms, from the buckets 4.6.
 // Bound: the loads of the heads (each slot of the element's vertices once, from L1 and
 // L2).  Collecting the candidates in a local-memory array of 256 and insertion-sorting
 // it, once to count and once to write, made the dual graph of 2.4M hexes take 4330 us
 // (two calls); it takes 589 (one).
 #define GS_ROW 32
-template <bool HEX, bool STORE>
+enum { MERGE_COUNT, MERGE_ROWS, MERGE_CSR };
+template <bool HEX, int MODE>
 __global__ void __launch_bounds__(RSB_BLOCK) k_gs_merge(int64_t ne, int nv,
                                                       const int64_t* __restrict__ ev, int64_t cap,
                                                       const int32_t* __restrict__ slot,
                                                       uint32_t* __restrict__ ent,
-                                                      int64_t* __restrict__ len, int32_t* cnt) {
+                                                      int64_t* __restrict__ len, int32_t* cnt,
+                                                      const int64_t* __restrict__ row_ptr,
+                                                      int32_t* __restrict__ col,
+                                                      int32_t* __restrict__ wt) {
   const int64_t e = (int64_t)blockIdx.x * RSB_BLOCK + threadIdx.x;
+  if (MODE != MERGE_CSR && e == ne) len[ne] = 0;  // (the scan's last entry)
   if (e >= ne) return;
   const int unfit = gs_unfit(cnt, cap);
   int64_t id[8];
   gs_ids<HEX>(ev, e, nv, id);
   if (unfit) {
-    len[e] = 0;
+    if (MODE != MERGE_CSR) len[e] = 0;
     return;
   }
+  const int64_t row = MODE == MERGE_CSR ? row_ptr[e] : 0;
   const int32_t* p[8];
   int32_t h[8];
 #pragma unroll
@@ -385,7 +412,7 @@ __global__ void __launch_bounds__(RSB_BLOCK) k_gs_merge(int64_t ne, int nv,
     p[i] = slot + (in ? id[i] * GS_SLOTS : 0);
     h[i] = in ? __ldg(p[i]) : INT_MAX;
   }
-  uint32_t* out = STORE ? ent + (e >> 5) * (GS_ROW * 32) + (e & 31) : nullptr;
+  uint32_t* out = MODE == MERGE_ROWS ? ent + (e >> 5) * (GS_ROW * 32) + (e & 31) : nullptr;
   uint32_t pos = 0;  // four bits a list
   int32_t prev = -1;
   int run = 0, d = 0, most = 0;
@@ -393,7 +420,12 @@ __global__ void __launch_bounds__(RSB_BLOCK) k_gs_merge(int64_t ne, int nv,
     const int32_t m = min(min(min(h[0], h[1]), min(h[2], h[3])), min(min(h[4], h[5]), min(h[6], h[7])));
     if (m != prev) {
       if (run > 0 && prev != (int32_t)e) {
-        if (STORE && d < GS_ROW) out[32 * d] = ((uint32_t)min(run, 7) << RSB_COLBITS) | (uint32_t)prev;
+        if (MODE == MERGE_ROWS && d < GS_ROW)
+          out[32 * d] = ((uint32_t)min(run, 7) << RSB_COLBITS) | (uint32_t)prev;
+        if (MODE == MERGE_CSR) {
+          col[row + d] = prev;
+          wt[row + d] = run;
+        }
         most = max(most, run);
         ++d;
       }
@@ -410,9 +442,10 @@ __global__ void __launch_bounds__(RSB_BLOCK) k_gs_merge(int64_t ne, int nv,
         h[i] = k < GS_SLOTS ? __ldg(p[i] + k) : INT_MAX;
       }
   }
+  if (MODE == MERGE_CSR) return;
   len[e] = d;
   volatile int32_t* err = cnt + cap;
-  if (d > GS_ROW && !err[1]) err[1] = 1;
+  if (d > GS_ROW && !err[3]) err[3] = 1;
   if (most > 7 && !err[2]) err[2] = 1;
 }
 
@@ -476,13 +509,18 @@ int gs_vertex_count(const int64_t* ev, int64_t cnt, unsigned long long* d_max,
 }
 
 // Buckets: bptr[V + 1], bucket[ne * nv], ev32[ne * nv]; count is int64[V + 1]
-// scratch.
-int gs_buckets(const int64_t* ev, int64_t ne, int nv, int64_t V, int64_t* count, int64_t* bptr,
-               int32_t* bucket, int32_t* ev32, void* scan_tmp, size_t scan_bytes,
-               cudaStream_t s) {
+// scratch.  counted (optional): the number of elements at each of the V vertices.
+int gs_buckets(const int64_t* ev, int64_t ne, int nv, int64_t V, const int32_t* counted,
+               int64_t* count, int64_t* bptr, int32_t* bucket, int32_t* ev32, void* scan_tmp,
+               size_t scan_bytes, cudaStream_t s) {
   const int64_t cnt = ne * nv;
-  RSB_CK(cudaMemsetAsync(count, 0, sizeof(int64_t) * (size_t)(V + 1), s));
-  if (cnt > 0) {
+  if (counted) {
+    k_gs_widen<<<grid_of(V + 1), RSB_BLOCK, 0, s>>>(counted, V, count);
+    RSB_CKL("k_gs_widen");
+  } else {
+    RSB_CK(cudaMemsetAsync(count, 0, sizeof(int64_t) * (size_t)(V + 1), s));
+  }
+  if (cnt > 0 && !counted) {
     k_gs_count<<<grid_of(cnt), RSB_BLOCK, 0, s>>>(ev, cnt, count);
     RSB_CKL("k_gs_count");
   }
@@ -497,11 +535,12 @@ int gs_buckets(const int64_t* ev, int64_t ne, int nv, int64_t V, int64_t* count,
   return RSB_OK;
 }
 
+// flag: two pinned host words (zero before): an element meets more than GS_MAXCAND others,
+// two elements share more than 7 vertices.  len: ne + 1 entries.
 int gs_row_lengths(int64_t ne, int nv, const int32_t* ev32, const int64_t* bptr,
-                   const int32_t* bucket, int64_t* len, int* d_flag, cudaStream_t s) {
-  RSB_CK(cudaMemsetAsync(d_flag, 0, sizeof(int), s));
+                   const int32_t* bucket, int64_t* len, int* flag, cudaStream_t s) {
   if (ne <= 0) return RSB_OK;
-  k_gs_rowlen<<<grid_of(ne, 128), 128, 0, s>>>(ne, nv, ev32, bptr, bucket, len, d_flag);
+  k_gs_rowlen<<<grid_of(ne + 1, 128), 128, 0, s>>>(ne, nv, ev32, bptr, bucket, len, flag);
   RSB_CKL("k_gs_rowlen");
   return RSB_OK;
 }
@@ -559,7 +598,7 @@ int gs_slots(const int64_t* ev, int64_t ne, int nv, int64_t cap, int32_t* cnt, i
 }
 
 template <typename V>
-static int gs_slot_apply_t(const int64_t* ev, int64_t ne, int nv, int64_t cap, const int32_t* cnt,
+static int gs_slot_apply_t(const int64_t* ev, int64_t ne, int nv, int64_t cap, int32_t* cnt,
                            const int32_t* slot, const V* x, void* wc, V* y, int* err,
                            cudaStream_t s) {
   GsPair<V>* p = (GsPair<V>*)wc;
@@ -574,8 +613,8 @@ static int gs_slot_apply_t(const int64_t* ev, int64_t ne, int nv, int64_t cap, c
 }
 
 // y = L x from the slot table (wc: 2 * cap values of the vector type); a mesh that does
-// not fit leaves y as it is and sets err[0] or err[1] (pinned host words).
-int gs_slot_apply(int f32, const int64_t* ev, int64_t ne, int nv, int64_t cap, const int32_t* cnt,
+// not fit leaves y as it is and sets err[0] or err[1], and err[4] (pinned host words).
+int gs_slot_apply(int f32, const int64_t* ev, int64_t ne, int nv, int64_t cap, int32_t* cnt,
                   const int32_t* slot, const void* x, void* wc, void* y, int* err, cudaStream_t s) {
   return f32 ? gs_slot_apply_t<float>(ev, ne, nv, cap, cnt, slot, (const float*)x, wc, (float*)y,
                                       err, s)
@@ -587,26 +626,41 @@ int gs_slot_apply(int f32, const int64_t* ev, int64_t ne, int nv, int64_t cap, c
 // themselves for gs_slot_write (ent: gs_rows_bytes).
 size_t gs_rows_bytes(int64_t ne) { return sizeof(uint32_t) * GS_ROW * 32 * (size_t)((ne + 31) / 32); }
 
-// err: pinned host words 0 to 2, valid once the stream is done.
+// err: GS_WORDS pinned host words, valid once the stream is done.  len: ne + 1 entries.
+template <int MODE>
+static int gs_merge(const int64_t* ev, int64_t ne, int nv, int64_t cap, int32_t* cnt,
+                    const int32_t* slot, uint32_t* ent, int64_t* len, const int64_t* row_ptr,
+                    int32_t* col, int32_t* wt, cudaStream_t s) {
+  const unsigned nb = grid_of(ne + 1);
+  if (hex_aligned(ev, nv))
+    k_gs_merge<true, MODE><<<nb, RSB_BLOCK, 0, s>>>(ne, nv, ev, cap, slot, ent, len, cnt, row_ptr,
+                                                   col, wt);
+  else
+    k_gs_merge<false, MODE><<<nb, RSB_BLOCK, 0, s>>>(ne, nv, ev, cap, slot, ent, len, cnt, row_ptr,
+                                                    col, wt);
+  RSB_CKL("k_gs_merge");
+  return RSB_OK;
+}
+
 int gs_slot_rows(const int64_t* ev, int64_t ne, int nv, int64_t cap, int32_t* cnt, int32_t* slot,
                  uint32_t* ent, int64_t* len, int* err, cudaStream_t s) {
   k_gs_sort8<<<grid_of(cap), RSB_BLOCK, 0, s>>>(cap, cnt, slot);
   RSB_CKL("k_gs_sort8");
-  const unsigned nb = grid_of(ne);
-  if (hex_aligned(ev, nv)) {
-    if (ent) k_gs_merge<true, true><<<nb, RSB_BLOCK, 0, s>>>(ne, nv, ev, cap, slot, ent, len, cnt);
-    else k_gs_merge<true, false><<<nb, RSB_BLOCK, 0, s>>>(ne, nv, ev, cap, slot, ent, len, cnt);
-  } else {
-    if (ent) k_gs_merge<false, true><<<nb, RSB_BLOCK, 0, s>>>(ne, nv, ev, cap, slot, ent, len, cnt);
-    else k_gs_merge<false, false><<<nb, RSB_BLOCK, 0, s>>>(ne, nv, ev, cap, slot, ent, len, cnt);
-  }
-  RSB_CKL("k_gs_merge");
-  RSB_CK(cudaMemcpyAsync(err, cnt + cap, 3 * sizeof(int), cudaMemcpyDeviceToHost, s));
+  int rc = ent ? gs_merge<MERGE_ROWS>(ev, ne, nv, cap, cnt, slot, ent, len, nullptr, nullptr,
+                                      nullptr, s)
+               : gs_merge<MERGE_COUNT>(ev, ne, nv, cap, cnt, slot, ent, len, nullptr, nullptr,
+                                       nullptr, s);
+  if (rc) return rc;
+  RSB_CK(cudaMemcpyAsync(err, cnt + cap, GS_WORDS * sizeof(int), cudaMemcpyDeviceToHost, s));
   return RSB_OK;
 }
 
-int gs_slot_write(int64_t ne, const uint32_t* ent, const int64_t* row_ptr, int32_t* col,
+// The rows into CSR: from ent, or where some are too long for it (ent null) merged again.
+int gs_slot_write(const int64_t* ev, int64_t ne, int nv, int64_t cap, int32_t* cnt,
+                  const int32_t* slot, const uint32_t* ent, const int64_t* row_ptr, int32_t* col,
                   int32_t* wt, cudaStream_t s) {
+  if (!ent)
+    return gs_merge<MERGE_CSR>(ev, ne, nv, cap, cnt, slot, nullptr, nullptr, row_ptr, col, wt, s);
   k_gs_write<<<grid_of(ne), RSB_BLOCK, 0, s>>>(ne, ent, row_ptr, col, wt);
   RSB_CKL("k_gs_write");
   return RSB_OK;
