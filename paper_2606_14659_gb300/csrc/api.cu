@@ -244,6 +244,9 @@ extern "C" void rsb_profile_read(int family, double* ms, int64_t* launches, doub
   if (bytes) *bytes = ok ? g_prof.bytes[family] : 0.0;
 }
 
+static bool free_idle_workspace();
+
+// A call that finds no memory first gives back what calls of another kind keep.
 int devbuf_reserve(DevBuf& b, size_t bytes) {
   if (bytes <= b.cap) return RSB_OK;
   if (b.p) cudaFree(b.p);
@@ -251,6 +254,10 @@ int devbuf_reserve(DevBuf& b, size_t bytes) {
   b.cap = 0;
   size_t want = bytes + bytes / 8 + 256;
   cudaError_t e = cudaMalloc(&b.p, want);
+  if (e == cudaErrorMemoryAllocation && free_idle_workspace()) {
+    cudaGetLastError();
+    e = cudaMalloc(&b.p, want);
+  }
   if (e != cudaSuccess) {
     cudaGetLastError();
     b.p = nullptr;
@@ -290,6 +297,7 @@ struct Ctx {
   DevBuf part_concat;
   // Laplacian action: device copies of host vectors; of a device y, what it held before
   DevBuf lap_x, lap_y;
+  bool gs_busy = false;  // the buffers of the gather-scatter and Laplacian calls are in use
   int trmax = 0;    // largest tile of the level being solved, rows
   int ntmax = 0;    // most tiles of one of its units
   std::vector<DevBuf> stage;  // staged host inputs
@@ -302,6 +310,22 @@ static void free_buf(DevBuf& b) {
   if (b.p) cudaFree(b.p);
   b.p = nullptr;
   b.cap = 0;
+}
+
+// The buffers that only the gather-scatter calls and the Laplacian action use (some 250 B
+// an element after a dual graph): kept for the next of them, not at a solve's expense.
+static bool free_idle_workspace() {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return false;
+  Ctx* c = g_ctx[dev];
+  if (!c || c->gs_busy) return false;
+  size_t held = 0;
+  for (DevBuf* b : {&c->gs_count, &c->gs_cnt, &c->gs_bptr, &c->gs_bucket, &c->gs_ev32, &c->gs_len,
+                    &c->gs_rowptr, &c->gs_w, &c->gs_rows, &c->lap_x, &c->lap_y}) {
+    held += b->cap;
+    free_buf(*b);
+  }
+  return held > 0;
 }
 
 static int ctx_get(Ctx** out) {
@@ -1145,6 +1169,7 @@ static int begin_call(Ctx** pc, void* stream) {
   int rc = ctx_get(pc);
   if (rc) return rc;
   Ctx& c = **pc;
+  c.gs_busy = false;
   RSB_CK(cudaEventRecord(c.ev_in, (cudaStream_t)stream));
   RSB_CK(cudaStreamWaitEvent(c.s, c.ev_in, 0));
   return RSB_OK;
@@ -1542,6 +1567,7 @@ static int lap_apply(const rsb_csr* g, const void* x, void* y, int f32, void* st
   int rc = begin_call(&pc, stream);
   if (rc) return rc;
   Ctx& c = *pc;
+  c.gs_busy = true;
   MeshIn m = {g->n, g->row_ptr, g->col, g->weight, nullptr, nullptr, 0};
   if (!g->col || !is_device_ptr(g->row_ptr) || !is_device_ptr(g->col) ||
       (g->weight && !is_device_ptr(g->weight))) {
@@ -1794,6 +1820,7 @@ extern "C" int rsb_dual_graph(int64_t ne, int nv, const int64_t* ev_in, int64_t*
   int rc = begin_call(&pc, stream);
   if (rc) return rc;
   Ctx& c = *pc;
+  c.gs_busy = true;
   const int64_t* ev = nullptr;
   if ((rc = gs_check(ne, nv, ev_in)) || (rc = stage_in(c, ev_in, (size_t)(ne * nv), &ev)))
     return end_call(c, stream, rc);
@@ -1873,6 +1900,7 @@ static int gs_lap_apply(int64_t ne, int nv, const int64_t* ev_in, const void* x,
   Ctx* pc = nullptr;
   if ((rc = begin_call(&pc, stream))) return rc;
   Ctx& c = *pc;
+  c.gs_busy = true;
   const size_t es = f32 ? 4 : 8;
   DevBuf tx, ty;
   auto done = [&](int r) {
@@ -1917,6 +1945,7 @@ static int gs_lap_bench(int64_t ne, int nv, const int64_t* ev, int f32, int reps
   int rc = begin_call(&pc, stream);
   if (rc) return rc;
   Ctx& c = *pc;
+  c.gs_busy = true;
   int64_t V = 0;
   if ((rc = gs_setup(c, ne, nv, ev, &V))) return end_call(c, stream, rc);
   const size_t es = f32 ? 4 : 8;

@@ -351,7 +351,8 @@ def rsb_laplacian_bench(g: Graph, f32: bool, reps: int = 20, stream=None):
 def rsb_dual_graph(ev, device: str = "cuda", stream=None):
     """Dual graph (n, row_ptr, col, weight) of elements given by their vertex
     ids ev (ne x nv integer array or tensor); arrays on `device` ("cuda" or
-    "host")."""
+    "host").  col and weight may be views of a little more room (an eighth at
+    most, or 256 KiB)."""
     lib = load()
     import torch
 
@@ -387,7 +388,7 @@ def rsb_dual_graph(ev, device: str = "cuda", stream=None):
         code, col, w = ask(cap)
     _check(code, "rsb_dual_graph")
     col, w = col[:nnz.value], w[:nnz.value]
-    if nnz.value < cap // 2:  # do not hold on to room that is mostly unused
+    if cap - nnz.value > max(nnz.value // 8, 1 << 16):  # do not hold on to unused room
         col, w = col.clone(), w.clone()
     return ne, rp, col, w
 
