@@ -570,12 +570,14 @@ static int max_unit_tiles(const std::vector<Unit>& units) {
 // units are parts of one mesh, whose rows they cover)
 // fp64_small: the one FP64 solve of rsb_fiedler by default tiles.  A small mesh then has
 // tiles of one row a thread, because an FP64 row takes 64 cycles of a sub-partition an
-// operation and twice the tiles put twice the SMs to work: Fiedler pair of 28k rows 13.8
-// -> 11.3 ms.  Up to RSB_SMALL_FP64 rows the tiles still fit the 152 SMs one each, so that
-// the solve stays resident; a unit of two tiles or fewer of two rows would pay more for
-// barriers than it gains.  Partitions keep two rows: they tile a mesh alike alone and in
-// a batch, whose other meshes use those SMs (eight of 28k rows: 96 ms so, 88 before).
-#define RSB_SMALL_FP64 31000
+// operation and twice the tiles put twice the SMs to work.  Up to RSB_SMALL_FP64 rows the
+// tiles fit the SMs one each (a fixed number: the tiles order the sums), so that the solve
+// stays resident; one tile of two rows has nothing to gain.  Two rows against one, ms,
+// vertex-adjacent boxes: 411 rows 3.00 : 3.05, 659 5.74 : 4.43, 5472 9.54 : 7.28, 28184
+// 15.5 : 12.6, 37049 17.7 : 14.0, 39368 17.8 : 24.2.  Partitions keep two rows: they tile a
+// mesh alike alone and in a batch, whose other meshes use those SMs (eight of 28k rows: 96
+// ms with one row, 88 with two).
+#define RSB_SMALL_FP64 (152 * RSB_BLOCK)
 static void make_tiles(std::vector<Unit>& units, std::vector<Tile>& tiles, int rmin = RSB_MINR,
                        const std::vector<int64_t>& mesh_rows = {}, bool fp64_small = false) {
   tiles.clear();
@@ -594,7 +596,7 @@ static void make_tiles(std::vector<Unit>& units, std::vector<Tile>& tiles, int r
                           ((int64_t)RSB_BLOCK * RSB_TARGET_TILES);
     int64_t R = (nr + (int64_t)RSB_BLOCK * RSB_MAXTILES_PER_UNIT - 1) /
                 ((int64_t)RSB_BLOCK * RSB_MAXTILES_PER_UNIT);
-    const bool one = fp64_small && nmesh <= RSB_SMALL_FP64 && nr > 2 * 2 * RSB_BLOCK;
+    const bool one = fp64_small && nmesh <= RSB_SMALL_FP64 && nr > 2 * RSB_BLOCK;
     if (R < rmin && !one) R = rmin;
     if (R < rmesh) R = rmesh;
     const int64_t tr = R * RSB_BLOCK;
