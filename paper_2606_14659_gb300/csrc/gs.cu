@@ -497,8 +497,11 @@ int gs_vertex_count(const int64_t* ev, int64_t cnt, unsigned long long* d_max,
                     unsigned long long* h_max, int64_t* V, cudaStream_t s) {
   RSB_CK(cudaMemsetAsync(d_max, 0, 2 * sizeof(unsigned long long), s));
   if (cnt > 0) {
-    k_gs_maxid<<<std::min(grid_of(cnt), 8u * 152u), RSB_BLOCK, 0, s>>>(ev, cnt, d_max,
-                                                                      (int*)(d_max + 1));
+    int dev = 0, nsm = 0;  // CTAs of one wave, so that the atomics are few
+    RSB_CK(cudaGetDevice(&dev));
+    RSB_CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+    k_gs_maxid<<<std::min(grid_of(cnt), 8u * (unsigned)nsm), RSB_BLOCK, 0, s>>>(
+        ev, cnt, d_max, (int*)(d_max + 1));
     RSB_CKL("k_gs_maxid");
   }
   RSB_CK(cudaMemcpyAsync(h_max, d_max, 2 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, s));

@@ -837,11 +837,9 @@ __global__ void __launch_bounds__(RSB_BLOCK) k_lz_close(LzArgs<V> a, int j, int 
 // thread, 48 registers and five CTAs the last, nearly empty wave of tiles made it 106.
 // The tiles are taken in the opposite order of D2, which has just streamed the same
 // vectors: what it read last is still in L2 (4 % at 1M rows, nothing at 3.7M).
-// T = 256 threads, or 128 where the tiles are more than the chip holds CTAs of 256: the
-// CTAs of short tiles live for a chain of loads and a reduction whatever their rows, so
-// one wave of sixteen a SM beats two of eight (batch of 1800 tiles 260 -> 255 ms,
-// with the scales and coefficients converted once by the closing kernel).  A thread of 128 keeps the sums of rows
-// t and t + 128 of every 256 apart, which are merged in the order of 256 threads.
+// T = 256 threads, or 128 (d3_half) where the tiles are short and more than the chip holds
+// CTAs of 256.  A thread of 128 keeps the sums of rows t and t + 128 of every 256 apart,
+// which are merged in the order of 256 threads, so both give the same bits.
 #define D3_KB 4  // basis vectors a round
 #define D3_RR 2  // rows a thread
 template <typename V, int T>
@@ -2445,10 +2443,22 @@ static int lz_start(LzArgs<V>& a, int ntiles, uint64_t sd, const double* from64,
   return RSB_OK;
 }
 
+// D3 in CTAs of 128 threads?  The CTA of a short tile lives for a chain of loads and a
+// reduction whatever its rows, so one wave of sixteen a SM beats two of eight, and half
+// the threads of 256 idle on tiles of up to 128 rows; long tiles, and full ones of more
+// than two waves, are better off with 256.  Sum of D3 over three cycles in CTAs of 256 and
+// 128, ms (8 x 152 = 1216 CTAs of 256 a wave): 1300 tiles of 512 rows 3.05 : 2.66, 2600
+// 5.11 : 5.29, 3200 4.72 : 5.08, 6000 9.64 : 9.23; 4000 of 240 rows 3.91 : 2.69; 6000 of
+// 351 on average 7.34 : 6.75; the levels of 3.7M rows (tiles of 1536 and more) 37.7 : 40.9,
+// of 15.9M rows 139 : 154.
+static bool d3_half(int64_t rows, int ntiles, int trmax, int nsm) {
+  const int64_t wave = 8ll * nsm;
+  return trmax <= 2 * RSB_BLOCK && ntiles > wave && (ntiles <= 2 * wave || rows < 384ll * ntiles);
+}
+
 template <typename V>
 static int lz_cycle(LzArgs<V>& a, int ntiles, int nunits, int M, double breakdown, int trmax,
-                    int ntmax, int nd, cudaStream_t s) {
-  constexpr int d3_one_wave = 8 * 152;  // CTAs of 256 threads at once
+                    int ntmax, int nd, bool half, cudaStream_t s) {
   // CTAs per tile of step D1
   const int nsub = std::max(1, (trmax + A1_ROWS - 1) / A1_ROWS);
   for (int j = 0; j < M; ++j) {
@@ -2465,7 +2475,7 @@ static int lz_cycle(LzArgs<V>& a, int ntiles, int nunits, int M, double breakdow
       RSB_CKL("k_lz_close<D2>");
       prof_after(pi, s);
       pi = prof_before(PROF_LZ_B, s);
-      if (ntiles > d3_one_wave) k_lz_d3<V, 128><<<ntiles, 128, 0, s>>>(a, j, breakdown);
+      if (half) k_lz_d3<V, 128><<<ntiles, 128, 0, s>>>(a, j, breakdown);
       else k_lz_d3<V, 256><<<ntiles, 256, 0, s>>>(a, j, breakdown);
       RSB_CKL("k_lz_d3");
       prof_after(pi, s);
@@ -2582,13 +2592,17 @@ static int lanczos_run(const LevelGraph& G, const Tile* tiles, int ntiles, Unit*
     }
     return rc;
   }
+  int dev = 0, nsm = 0;
+  RSB_CK(cudaGetDevice(&dev));
+  RSB_CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+  const bool half = d3_half(G.n, ntiles, B.trmax, nsm);
   cudaGraphExec_t exec = nullptr;
   std::vector<int> cap_pairs;
   if (use_graph) {
     cudaGraph_t graph = nullptr;
     RSB_CK(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
     prof_capture_begin();
-    rc = lz_cycle<V>(a, ntiles, nunits, M, breakdown, B.trmax, B.ntmax, nd, s);
+    rc = lz_cycle<V>(a, ntiles, nunits, M, breakdown, B.trmax, B.ntmax, nd, half, s);
     cap_pairs = prof_capture_end();
     cudaGraph_t g2 = nullptr;
     cudaError_t e = cudaStreamEndCapture(s, &g2);
@@ -2615,7 +2629,7 @@ static int lanczos_run(const LevelGraph& G, const Tile* tiles, int ntiles, Unit*
       }
       prof_replay(cap_pairs);
     } else {
-      rc = lz_cycle<V>(a, ntiles, nunits, M, breakdown, B.trmax, B.ntmax, nd, s);
+      rc = lz_cycle<V>(a, ntiles, nunits, M, breakdown, B.trmax, B.ntmax, nd, half, s);
       if (rc) return rc;
     }
     rc = read_active(B, s, &active);
