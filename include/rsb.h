@@ -274,10 +274,11 @@ int rsb_laplacian_apply_gs_f32(int64_t ne, int nv, const int64_t *ev, const floa
 
 /*
  * Times `reps` gather-scatter Laplacian applications (two kernels each; FP64
- * when f32 == 0) after building the vertex buckets once; *ms_per_apply gets
- * the mean device time of one application, *useful_bytes its algorithmic
- * bytes (bucket offsets twice, the bucket entries and vertex ids once each,
- * x read once, the vertex sums written and read once, y written once).
+ * when f32 == 0) after collecting the elements at every vertex once, as a call on
+ * this mesh does (slot table or buckets); *ms_per_apply gets the mean device time
+ * of one application, *useful_bytes its algorithmic bytes (the counts or twice the
+ * bucket offsets, the elements at every vertex and the vertex ids once each, x
+ * twice, the vertex sums written and read once, y written once).
  */
 int rsb_laplacian_bench_gs(int64_t ne, int nv, const int64_t *ev, int f32, int reps,
                            double *ms_per_apply, double *useful_bytes, void *stream);

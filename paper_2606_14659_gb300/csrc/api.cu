@@ -1941,22 +1941,43 @@ static int gs_lap_apply(int64_t ne, int nv, const int64_t* ev_in, const void* x,
   return done(rc);
 }
 
-static int gs_lap_bench(int64_t ne, int nv, const int64_t* ev, int f32, int reps, double* ms,
+// The two kernels of an application on the table or the buckets that a call on this mesh
+// would make.
+static int gs_lap_bench(int64_t ne, int nv, const int64_t* ev_in, int f32, int reps, double* ms,
                         double* bytes, void* stream) {
-  Ctx* pc = nullptr;
-  int rc = begin_call(&pc, stream);
+  int rc = gs_check(ne, nv, ev_in);
   if (rc) return rc;
+  Ctx* pc = nullptr;
+  if ((rc = begin_call(&pc, stream))) return rc;
   Ctx& c = *pc;
   c.gs_busy = true;
-  int64_t V = 0;
-  if ((rc = gs_setup(c, ne, nv, ev, &V))) return end_call(c, stream, rc);
   const size_t es = f32 ? 4 : 8;
-  if ((rc = devbuf_reserve(c.gs_w, es * (size_t)(V + 1)))) return end_call(c, stream, rc);
+  const int64_t cap = gs_slot_cap(ne);
   DevBuf tx, ty;  // operands of its own
-  if ((rc = devbuf_reserve(tx, es * (size_t)ne)) || (rc = devbuf_reserve(ty, es * (size_t)ne)))
-    return end_call(c, stream, rc);
+  auto done = [&](int r) {
+    r = end_call(c, stream, r);
+    free_buf(tx);
+    free_buf(ty);
+    return r;
+  };
+  const int64_t* ev = nullptr;
+  int64_t V = 0;
+  if ((rc = stage_in(c, ev_in, (size_t)(ne * nv), &ev)) || (rc = devbuf_reserve(c.gs_misc, 256)) ||
+      (rc = gs_vertex_count(ev, ne * nv, dptr<unsigned long long>(c.gs_misc),
+                            (unsigned long long*)(c.h_pinned + 12), &V, c.s)) ||
+      (rc = devbuf_reserve(tx, es * (size_t)ne)) || (rc = devbuf_reserve(ty, es * (size_t)ne)))
+    return done(rc);
   RSB_CK(cudaMemsetAsync(tx.p, 0, es * (size_t)ne, c.s));
+  int fits = 0;
+  bool tried = false;
+  if ((rc = gs_lap_slots(c, ne, nv, ev, tx.p, ty.p, f32, &fits, &tried)) ||
+      (!fits && ((rc = gs_setup(c, ne, nv, ev, &V)) ||
+                 (rc = devbuf_reserve(c.gs_w, es * (size_t)(V + 1))))))
+    return done(rc);
   auto apply = [&]() {
+    if (fits)
+      return gs_slot_apply(f32, ev, ne, nv, cap, dptr<int32_t>(c.gs_cnt),
+                           dptr<int32_t>(c.gs_bucket), tx.p, c.gs_w.p, ty.p, gs_words(c), c.s);
     return gs_apply(f32, ne, nv, V, dptr<int32_t>(c.gs_ev32), dptr<int64_t>(c.gs_bptr),
                     dptr<int32_t>(c.gs_bucket), tx.p, c.gs_w.p, ty.p, c.s);
   };
@@ -1973,15 +1994,15 @@ static int gs_lap_bench(int64_t ne, int nv, const int64_t* ev, int f32, int reps
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   if (ms) *ms = (double)t / reps;
-  // vertex sums: bucket offsets, bucket entries, x once, w written; element
-  // pass: vertex ids, bucket offsets, w and x read once, y written
+  // vertex sums: counts or bucket offsets, the elements at every vertex, x once, the sums
+  // (slots: with the counts) written; element pass: vertex ids, bucket offsets, the sums
+  // and x read once, y written
   if (bytes)
-    *bytes = 16.0 * (double)(V + 1) + 8.0 * (double)ne * nv + 3.0 * es * (double)ne +
-             2.0 * es * (double)V;
-  rc = end_call(c, stream, rc);
-  free_buf(tx);
-  free_buf(ty);
-  return rc;
+    *bytes = fits ? 4.0 * (double)V + 12.0 * (double)ne * nv + 3.0 * es * (double)ne +
+                        4.0 * es * (double)V
+                  : 16.0 * (double)(V + 1) + 8.0 * (double)ne * nv + 3.0 * es * (double)ne +
+                        2.0 * es * (double)V;
+  return done(rc);
 }
 
 extern "C" int rsb_laplacian_apply_gs(int64_t ne, int nv, const int64_t* ev, const double* x,
