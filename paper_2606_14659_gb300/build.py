@@ -32,7 +32,7 @@ def _stale(obj: str, src: str) -> bool:
         return True
     t = os.path.getmtime(obj)
     deps = [src, os.path.join(CSRC, "rsb_internal.cuh"), os.path.join(INCLUDE, "rsb.h"),
-            os.path.join(INCLUDE, "rsb_test.h")]
+            os.path.join(INCLUDE, "rsb_test.h"), os.path.join(INCLUDE, "rsb_probe.h")]
     return any(os.path.getmtime(d) > t for d in deps)
 
 

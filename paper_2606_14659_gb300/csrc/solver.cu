@@ -37,6 +37,7 @@
 #include <cfloat>
 
 #include "rsb_internal.cuh"
+#include "rsb_probe.h"
 
 int g_rsb_poison_barrier = 0;  // test hook, see rsb_test_poison_barrier
 
@@ -1383,6 +1384,40 @@ int launch_lz_eig(int f32, Unit* units, double* S, int nunits, cudaStream_t s) {
   if (f32) k_lz_eig<float><<<nunits, RSB_BLOCK, 0, s>>>(units, S, nunits);
   else k_lz_eig<double><<<nunits, RSB_BLOCK, 0, s>>>(units, S, nunits);
   RSB_CKL("k_lz_eig");
+  return RSB_OK;
+}
+
+extern "C" int rsb_probe_ritz(int f32, int K, int keep, const double* S, double* theta, double* Y) {
+  if (K < 1 || K > RSB_MAXM || keep < 0 || keep >= K || keep > RSB_MAXKEEP || !S || !theta || !Y)
+    return rsb_set_error(RSB_EINVAL, "ritz arguments");
+  Unit u;
+  memset(&u, 0, sizeof(u));
+  u.status = U_ACTIVE;
+  u.msteps = K;
+  u.keep = keep;
+  std::vector<double> h(RSB_SSTRIDE, 0.0);
+  for (int i = 0; i < K; ++i)
+    for (int k = 0; k < K; ++k) h[i * RSB_MAXM + k] = S[i * K + k];
+  DevBuf du, ds;
+  int rc;
+  if ((rc = devbuf_reserve(du, sizeof(Unit))) || (rc = devbuf_reserve(ds, sizeof(double) * h.size())))
+    return rc;
+  cudaError_t e = cudaMemcpy(du.p, &u, sizeof(Unit), cudaMemcpyHostToDevice);
+  if (!e) e = cudaMemcpy(ds.p, h.data(), sizeof(double) * h.size(), cudaMemcpyHostToDevice);
+  if (!e) {
+    rc = launch_lz_eig(f32, dptr<Unit>(du), dptr<double>(ds), 1, 0);
+    e = cudaDeviceSynchronize();
+  }
+  if (!e) e = cudaMemcpy(&u, du.p, sizeof(Unit), cudaMemcpyDeviceToHost);
+  if (!e) e = cudaMemcpy(h.data(), ds.p, sizeof(double) * h.size(), cudaMemcpyDeviceToHost);
+  cudaFree(du.p);
+  cudaFree(ds.p);
+  if (rc || e) return rc ? rc : rsb_set_cuda_error(e, "rsb_probe_ritz");
+  for (int i = 0; i <= keep; ++i) {
+    theta[i] = u.th[i];
+    for (int l = 0; l < K; ++l)
+      Y[l * (keep + 1) + i] = h[RSB_MAXM * RSB_MAXM + l * RSB_MAXM + i];
+  }
   return RSB_OK;
 }
 

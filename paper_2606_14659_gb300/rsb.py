@@ -26,7 +26,8 @@ EXPORTED = ["rsb_options_default", "rsb_partition", "rsb_partition_batch", "rsb_
             "rsb_strerror", "rsb_last_error_detail", "rsb_release", "rsb_profile_begin",
             "rsb_profile_end", "rsb_laplacian_apply_noalloc", "rsb_autotune",
             "rsb_test_poison_barrier", "rsb_profile_read", "rsb_dual_graph",
-            "rsb_laplacian_apply_gs", "rsb_laplacian_apply_gs_f32", "rsb_laplacian_bench_gs"]
+            "rsb_laplacian_apply_gs", "rsb_laplacian_apply_gs_f32", "rsb_laplacian_bench_gs",
+            "rsb_probe_ritz"]
 
 RSB_TUNE_CANDIDATES = 6
 TUNE_CANDIDATES = [(2, 3), (4, 3), (8, 3), (2, 1), (4, 1), (8, 1)]  # (tile_rows, use_graph)
@@ -93,6 +94,7 @@ def load():
     lib.rsb_laplacian_apply_gs_f32.argtypes = [C.c_int64, C.c_int, vp, vp, vp, vp]
     lib.rsb_laplacian_bench_gs.argtypes = [C.c_int64, C.c_int, vp, C.c_int, C.c_int,
                                            C.POINTER(C.c_double), C.POINTER(C.c_double), vp]
+    lib.rsb_probe_ritz.argtypes = [C.c_int, C.c_int, C.c_int, vp, vp, vp]
     lib.rsb_test_poison_barrier.argtypes = [C.c_int]
     lib.rsb_test_poison_barrier.restype = None
     lib.rsb_strerror.argtypes = [C.c_int]
@@ -113,7 +115,7 @@ def load():
                  "rsb_laplacian_apply",
                  "rsb_laplacian_apply_f32", "rsb_laplacian_bench", "rsb_laplacian_apply_noalloc",
                  "rsb_dual_graph", "rsb_laplacian_apply_gs", "rsb_laplacian_apply_gs_f32",
-                 "rsb_laplacian_bench_gs"):
+                 "rsb_laplacian_bench_gs", "rsb_probe_ritz"):
         getattr(lib, name).restype = C.c_int
     _lib = lib
     return lib
@@ -421,6 +423,17 @@ def rsb_laplacian_bench_gs(ev, f32: bool, reps: int = 20, stream=None):
 def rsb_test_poison_barrier(on: bool):
     """Failure-path test hook: the persistent launch modes' grid barrier times out."""
     load().rsb_test_poison_barrier(1 if on else 0)
+
+
+def rsb_probe_ritz(S, keep: int, f32: bool = False):
+    """(theta, Y): the keep + 1 smallest eigenpairs of a symmetric matrix of at most 40 rows, by
+    the kernel that ends a Lanczos cycle.  Probe for tests."""
+    S = np.ascontiguousarray(S, dtype=np.float64)
+    K = S.shape[0]
+    theta, Y = np.empty(keep + 1), np.empty((K, keep + 1))
+    _check(load().rsb_probe_ritz(int(bool(f32)), K, int(keep), _ptr(S), _ptr(theta), _ptr(Y)),
+           "rsb_probe_ritz")
+    return theta, Y
 
 
 def rsb_release():
