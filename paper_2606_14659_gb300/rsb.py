@@ -379,7 +379,7 @@ def rsb_dual_graph(ev, device: str = "cuda", stream=None):
     cap = 26 * ne
     try:
         code, col, w = ask(cap)
-    except torch.OutOfMemoryError:
+    except RuntimeError:  # (torch.OutOfMemoryError is one; the host allocator raises no other)
         code = RSB_ENOMEM
     if code == RSB_ENOMEM:
         col = w = None

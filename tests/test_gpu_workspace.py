@@ -63,3 +63,19 @@ def test_a_partition_takes_the_dual_graphs_room():
         torch.cuda.empty_cache()
         R.rsb_release()
     assert np.array_equal(np.bincount(ref.cpu().numpy()), [g.n // 2, g.n - g.n // 2])
+
+
+def test_dual_graph_on_the_host_without_the_large_room(monkeypatch):
+    """The host allocator's refusal is a plain RuntimeError; the exact room is taken then."""
+    ev = _hexes(6, 5, 4)
+    want = R.rsb.rsb_dual_graph(ev.cpu().numpy(), device="host")
+    empty = torch.empty
+
+    def small(n, **kw):
+        if n >= 26 * len(ev):
+            raise RuntimeError("DefaultCPUAllocator: can't allocate memory")
+        return empty(n, **kw)
+
+    monkeypatch.setattr(torch, "empty", small)
+    got = R.rsb.rsb_dual_graph(ev.cpu().numpy(), device="host")
+    assert got[0] == want[0] and all(torch.equal(a, b) for a, b in zip(got[1:], want[1:]))
