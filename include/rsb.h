@@ -239,9 +239,11 @@ int rsb_laplacian_bench(const rsb_csr *g, int f32, int reps, double *ms_per_appl
  * The element dual graph of a mesh given as element -> global vertex ids
  * (§2: elements are adjacent when they share a vertex, the weight omega is the
  * number of shared vertices; §5: the same graph is P^T Q Q^T P without its
- * diagonal).  Built on the GPU: the elements at every vertex are collected
- * (a counting sort by vertex id), then every element's distinct neighbours
- * are counted and written in ascending order.
+ * diagonal).  Built on the GPU: the elements at every vertex are collected (in
+ * eight slots a vertex, or by a counting sort when that does not hold the mesh), then
+ * every element's distinct neighbours are merged and written in ascending order.
+ * The workspace (some 250 bytes an element) stays with the library until
+ * rsb_release or until another call finds no memory.
  *   ne       number of elements, 1 <= ne < 2^29
  *   nv       vertices per element, 1..8 (8 for hexes)
  *   ev       int64[ne * nv], the vertex ids of element e at ev[e*nv .. e*nv+nv-1],

@@ -333,8 +333,8 @@ int launch_spmv_f32(const LevelGraph& G, const float* x, float* y, cudaStream_t 
 // entry).  The entries of a warp's 32 rows are contiguous, so the warp brings them to
 // shared memory packed as in the sliced form, coalesced and up to CSR_CAP at a time,
 // and every lane sums its row from there in entry order: the rows of spmv_row_ro bit
-// for bit.  192 x 128 x 96, 10 % deleted (54M entries): FP64 call 603 us with the
-// sliced copy (read and checked, lengths, scan, written, read again).
+// for bit.  192 x 128 x 96, 10 % deleted (54M entries): FP64 call 166 us; with the sliced
+// copy (read and checked, lengths, scan, written, read again) 603.
 // err: five words the host sees (zero before the launch); a fault in the graph sets
 // the word of its kind, and y is then not to be used.  Reads stay inside
 // [0, row_ptr[n]) of col and wt and [0, n) of x whatever the graph holds.

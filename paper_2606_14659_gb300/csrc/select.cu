@@ -401,10 +401,10 @@ int launch_split_assign(const LevelGraph& G, const Tile* tiles, int ntiles, Unit
 // k-th value, the tie window and the tie gid (R7), and the side bit of every row - the
 // steps of k_orient_*, k_sel_*, k_split_below and k_split_assign above, which take 36
 // launches and remain for levels of more tiles than SPLIT_MAXL a co-resident CTA.
-// Bound: the 12 to 20 grid barriers (about 2 us each) and, on large levels, one read of
-// v from L2 for each radix pass.  A CTA walks its tiles in every phase and keeps their
-// units' selection state; digits that all keys of a unit share (known from its smallest
-// and largest key) take no pass.  Values are compared as their integer keys, because an
+// Bound: 20 grid barriers, 18 with a fixed sign (about 2 us each, whether or not a unit
+// needs the pass), and, on large levels, one read of v from L2 for each radix pass.  A CTA
+// walks its tiles in every phase and keeps their units' selection state; leading digits
+// that all keys of a unit share (known from its smallest and largest key) take no read.  Values are compared as their integer keys, because an
 // FP64 comparison holds an SM sub-partition for 64 cycles; only rows near the tie
 // window take its FP64 test.  The split of a level of 512 rows 0.55 -> 0.12-0.26 ms (two
 // or three candidates), of 2.1M rows by coordinates 0.5-0.9 -> 0.27-0.3 ms.

@@ -728,9 +728,9 @@ __global__ void __launch_bounds__(D2_MAXTHREADS, 2) k_lz_d2(LzArgs<V> a, int j) 
 //   CLOSE_A: c1 (FP64 step A);  CLOSE_B: c2 and column j of S (FP64 step B);
 //   CLOSE_D2: d2_finish and the coefficients of D3.
 // The tiles' partials of one unit are nt x 2 (j + 2) FP64 values: at 973 tiles and
-// j = 39 their additions alone keep one SM's FP64 pipe busy for 20 us, which the
-// last CTA of the dots kernel used to spend while the chip idled (45 us with its
-// chain of loads).  So a kernel of its own spreads the coefficients over
+// j = 39 their additions alone keep one SM's FP64 pipe busy for 20 us (45 us with the
+// chain of loads, if the dots' last CTA does them while the chip idles).  So a kernel of
+// its own spreads the coefficients over
 // close_ctas() CTAs of the unit: one for a unit of few tiles, one per 32
 // coefficients (a warp sums four, as in final_reduce) up to 192 tiles, one per
 // four (final_reduce_few) above.  The order of every sum stays final_reduce's.
@@ -1433,10 +1433,9 @@ extern "C" int rsb_probe_ritz(int f32, int K, int keep, const double* S, double*
 // basis vector, read as broadcasts): a basis value is loaded once and updates NA
 // accumulators, RITZ_R rows per thread.  Every output sums over the basis vectors
 // in ascending order.
-// Before, every row thread fetched and converted each coefficient itself (an FP64
-// conversion per coefficient and warp): 2.36 ms for 40 FP32 vectors of 3.7M rows and
-// 9 outputs, 3.08 ms for 16 FP64 vectors; the Fiedler pair of that mesh took 437 ms
-// and takes 373 ms with this form.
+// 40 FP32 vectors of 3.7M rows and 9 outputs 0.17 ms, 16 FP64 vectors 0.90; with
+// every row thread converting each coefficient itself (an FP64 conversion per
+// coefficient and warp) 2.36 and 3.08 ms.
 // ----------------------------------------------------------------------------
 #define YSTR 20  // RSB_MAXKEEP + 1, rounded up to 16 bytes
 
@@ -1783,11 +1782,11 @@ __host__ __device__ constexpr size_t res_smem_bytes(int M, int trs) {
 // or three barriers) and of FP64 operations, each of which holds an SM sub-partition
 // for 64 cycles.  So units synchronise on their own barriers and run their cycles
 // independently of one another; FP64 work is done by whole warps, once (the closing
-// divisions of a step used to be done by every warp: 1.7 us); S_jj, which nothing
-// waits for, is computed while the norms travel; a unit of one tile exchanges nothing
-// through global memory but the SpMV operand.  FP32 step of the 512-row mesh 21.5 ->
-// about 11 us, the 131072-row box into 64 parts 167 -> 113 ms, the 512-row box into 8
-// parts 19.8 -> 13.7 ms.
+// divisions of a step by every warp take 1.7 us); S_jj, which nothing waits for, is
+// computed while the norms travel; a unit of one tile exchanges nothing through global
+// memory but the SpMV operand.  FP32 step of the 512-row mesh about 11 us, with whole-grid
+// barriers and the closing on single threads 21.5; the 131072-row box into 64 parts 113 and
+// 167 ms.
 //
 // Dots of [1, D, q_0..] with the tile's w: the coefficient split across warps
 // and the per-lane row order of tile_dots.
