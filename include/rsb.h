@@ -67,7 +67,8 @@ enum { RSB_DEGEN_NONE = 0, RSB_DEGEN_RESOLVE = 1 }; /* repeated lambda_2 (§9)  
  *            vectors, distinct within one graph; NULL means gid = row index
  *   coords   double[3 n], (x, y, z) of every element (e.g. its centroid), row
  *            by row; needed only by method RSB_RCB and by reorder = 1, else
- *            may be NULL
+ *            may be NULL.  NaNs sort behind every number; the parts have their
+ *            sizes whatever the coordinates hold
  */
 typedef struct rsb_csr {
   int64_t n;
